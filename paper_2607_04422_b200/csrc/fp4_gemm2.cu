@@ -799,7 +799,9 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
           sts128u(area + boff + lane * 32 + 16, hw_out[4], hw_out[5], hw_out[6], hw_out[7]);
           fence_proxy_async_smem();
           __syncwarp();
-          if (send && lane == 0) {
+          // the BF16 tensor has the padded work shape: its padding is read back by the next stage, so blocks
+          // outside the caller's matrix (zeros) are stored too
+          if (lane == 0) {
             tma_store_2d_s(&pr->tmH, xcol, y32, area + boff);
             bulk_commit();
           }

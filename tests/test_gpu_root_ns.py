@@ -669,3 +669,19 @@ def test_in_place_single_iteration(shape):
     inplace, _ = run_gpu(G, steps=1, in_place=True)
     assert np.array_equal(inplace, apart)
     assert rel(apart, oracle.root_ns(G, steps=1)) <= TOL_OUT
+
+
+@pytest.mark.parametrize("shape", [(496, 1008), (1008, 1456), (1008, 496)])
+def test_bf16_storage_of_shapes_that_pad_to_multiples_of_256(shape):
+    """Wide and tall shapes whose padded work shape takes 2-byte storage: the padding of the BF16 copy of X is
+    read by every later stage, so it must not keep what the workspace held before the call."""
+    m, n = shape
+    G = workloads.gradient_like(m, n, seed=23)
+    Gd = torch.from_numpy(G).cuda()
+    out = torch.empty_like(Gd)
+    ws = torch.full((fp4.fp4_root_ns_workspace_bytes(m, n, 3, FP4_FLAG_STORE_BF16),), 0xFF, dtype=torch.uint8,
+                    device="cuda")
+    fp4.fp4_root_ns(Gd, out, 3, fp4.NsParams.make(flags=FP4_FLAG_STORE_BF16), ws)
+    assert fp4.fp4_last_device_status(ws) == 0
+    want = oracle.root_ns(G, steps=3, store_bf16=True)
+    assert rel(out.cpu().numpy(), want) <= TOL_OUT
