@@ -253,12 +253,12 @@ __device__ __forceinline__ void mbar_arrive_s(uint32_t bar) {
 }
 #ifdef FP4_TRACE
 // Diagnostics build only: cycles each role spends waiting, summed per warp.
-__device__ unsigned long long g_trace[160 * 18 * 8];
+__device__ unsigned long long g_trace[160 * 19 * 8];
 #define TR_DECL unsigned long long tr_[8] = {0, 0, 0, 0, 0, 0, 0, 0}; long long tr_t0_ = clock64(), tr_s_ = 0;
 #define TR_BEGIN tr_s_ = clock64();
 #define TR_END(k) tr_[k] += (unsigned long long)(clock64() - tr_s_);
 #define TR_COUNT(k) tr_[k] += 1;
-#define TR_FLUSH if ((threadIdx.x & 31) == 0) { tr_[7] = (unsigned long long)(clock64() - tr_t0_); for (int k_ = 0; k_ < 8; ++k_) g_trace[(blockIdx.x * 18 + (threadIdx.x >> 5)) * 8 + k_] = tr_[k_]; }
+#define TR_FLUSH if ((threadIdx.x & 31) == 0) { tr_[7] = (unsigned long long)(clock64() - tr_t0_); for (int k_ = 0; k_ < 8; ++k_) g_trace[(blockIdx.x * 19 + (threadIdx.x >> 5)) * 8 + k_] = tr_[k_]; }
 #else
 #define TR_DECL
 #define TR_BEGIN
@@ -462,7 +462,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
     // column pass: lane = (column cq of the chunk, 16-row group g of this warp's 32 rows)
     const int cq = lane & 15, g = lane >> 4;
     const uint32_t area = smem_u32(smem + OFF_EPI + ew * WARP_AREA);
-    const uint32_t rq_st = area + XBUF * XBUF_BYTES;   // [32 rows][32 bytes]
+    const uint32_t rq_st = area + XBUF * XBUF_BYTES;   // [32 rows][32 bytes], 32-byte swizzle
     const int half = team >> 1;                         // the staging area this warp shares with seven others
     const uint32_t half_st = smem_u32(smem + OFF_HALF + half * HALF_AREA);
     const uint32_t half_done = smem_u32(&bars->half_done[half]), half_free = smem_u32(&bars->half_free[half]);
@@ -470,10 +470,15 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
     // row pass: this lane's row of a chunk buffer is 64 bytes whose 16-byte groups are XOR-swizzled with
     // bits 1-2 of the row; group j of the row sits at row_addr ^ (j << 4)
     const uint32_t row_addr = area + lane * 64 + (((lane >> 1) & 3) << 4);
-    // column pass: row k of the lane's 16-row group is at col_addr[(k >> 1) & 3] + k * 64
-    uint32_t col_addr[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) col_addr[k] = area + g * 16 * 64 + (cq & 3) * 4 + (((cq >> 2) ^ k) << 4);
+    // column pass: at step k the lane reads row k ^ g of its 16-row group g.  Two rows of a block share a
+    // 128-byte line and rows 16 apart share its half: with the groups in step the two half-warps would hit the same
+    // sixteen banks; swapping neighbouring rows in the second group keeps them apart.  The address of step k
+    // is col_base | (col_lane ^ (k << 6 | (k >> 1 & 3) << 4)), and 512 more for k + 8.  (Shared memory is the busiest
+    // part of the epilogue: operand copies, MMA operand reads and the blocks' four trips share 128 B per cycle.
+    // With the row codes' 32-byte swizzle and the branch-free quantiser: one 8192 x 2048 matrix, BF16 storage, 5
+    // iterations 490 -> 456 us, 2048 x 2048 247 -> 234 us.)
+    const uint32_t col_base = area + g * 16 * 64;
+    const uint32_t col_lane = (uint32_t)(g << 6 | cq << 2);
     const uint32_t tm_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
     const uint32_t acc_empty_leader0 = map_to_cta(&bars->acc_empty[0], 0);
     const uint32_t acc_empty_leader1 = map_to_cta(&bars->acc_empty[1], 0);
@@ -486,7 +491,6 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
     const bool hout = BH && STORE_F32 && MODE != kPlain && args.out_h == 1;           // the result is stored as BF16
 
     float scale = 0.0f, sg_out = 1.0f, inv_sg = 1.0f;
-    uint32_t rcp_base = 0;
     float ca = 0.0f, cb = 0.0f, cc = 0.0f;
     bool scale_pow2 = false;
     uint64_t scale2 = 0, ca2 = 0, cb2 = 0, ccs2 = 0;
@@ -566,7 +570,6 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         epilogue_scalars<MODE>(*pr, args, scale, sg_out,
                                leader && t == p * tiles_per_problem && threadIdx.x == ROLE_WARPS * 32);
         inv_sg = __frcp_rn(sg_out);  // exact: the predicted scales are powers of two
-        rcp_base = rcp_base_of(sg_out);
         ca = pr->ca; cb = pr->cb; cc = pr->cc;
         // a power-of-two scale (every tensor scale produced inside the loop is one) multiplies exactly
         scale_pow2 = (__float_as_uint(scale) & 0x007FFFFFu) == 0 && scale > 1e-30f && scale < 1e30f;
@@ -661,13 +664,13 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
           wait_or_abort(xfull0 + b * 8, (uint32_t)(i >> 1), abort_flag);
           TR_END(1)
         }
+        tc_wait_ld16(acc);
         // ---- combine the accumulator block with the FP32 tile
         if (BH && HAS_AUX && auxh) {
           // the tile is kept in BF16: this lane's row is 32 bytes of the first half of the buffer
           uint32_t hw[8];
           lds128u(area + boff + lane * 32, hw[0], hw[1], hw[2], hw[3]);
           lds128u(area + boff + lane * 32 + 16, hw[4], hw[5], hw[6], hw[7]);
-          tc_wait_ld16(acc);
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
             const float x = (q & 1) ? bf16_hi(hw[q >> 1]) : bf16_lo(hw[q >> 1]);
@@ -688,9 +691,6 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
             for (int j = 0; j < 4; ++j)
               lds128((row_addr + boff) ^ (j << 4), x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
           }
-          TR_BEGIN
-          tc_wait_ld16(acc);
-          TR_END(2)
           if (MODE == kG3 && raw) {
 #pragma unroll
             for (int q = 0; q < 16; ++q) x[q] = __fmul_rn(fminf(fmaxf(x[q], -tau), tau), inv);
@@ -724,7 +724,6 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
             }
           }
         } else {
-          tc_wait_ld16(acc);
 #pragma unroll
           for (int k = 0; k < 16; ++k) v[k] = __fmul_rn(__uint_as_float(acc[k]), scale);
         }
@@ -784,12 +783,16 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
           bulk_commit();
         }
         // ---- blocks of 16 down the rows of this warp's own 32 x 16 block (the transposed operand
-        // copy in G3, the mirrored triangle in G1/G2), read back from the buffer.  (The two
-        // half-warps read rows 16 apart, a two-way bank conflict on these sixteen 4-byte loads.)
+        // copy in G3, the mirrored triangle in G1/G2), read back from the buffer.
         float w[16];
         if (mirror) {
+          const uint32_t cb = col_base + boff;
 #pragma unroll
-          for (int k = 0; k < 16; ++k) w[k] = lds32(col_addr[(k >> 1) & 3] + boff + k * 64);
+          for (int k = 0; k < 8; ++k) {
+            const uint32_t at = cb | (col_lane ^ (uint32_t)(k << 6 | ((k >> 1) & 3) << 4));
+            w[k] = lds32(at);
+            w[k + 8] = lds32(at + 512);
+          }
         }
         if (BH && hout && store_out) {
           // BF16 storage: the rounded rows take the place of the FP32 block once it has been read back,
@@ -811,8 +814,8 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         if (do_q) {
           float bmax;
           uint32_t sb;
-          if (PF) sb = quantize_block16_opts<MODE != kG3>(v, args.q, sg_out, rlo, rhi, bmax);
-          else sb = quantize_block16_pow2(v, sg_out, inv_sg, rcp_base, rlo, rhi, bmax);
+          if (PF) sb = quantize_block16_opts_p2(v, args.q, inv_sg, rlo, rhi, bmax);
+          else sb = quantize_block16_p2(v, inv_sg, rlo, rhi, bmax);
           if (MODE == kG1 || MODE == kG3) amax = fmaxf(amax, bmax);
           sfw |= sb << (8 * e);
         }
@@ -838,15 +841,26 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
             // the stores of the previous tile have read the half's staging area
             wait_or_abort(half_free, (seq & 1) ^ 1, abort_flag);
           }
-          sts64u(rq_st + lane * 32 + e * 8, rlo, rhi);
+          sts64u(rq_st + lane * 32 + ((e * 8) ^ ((lane & 4) << 2)), rlo, rhi);   // 32-byte swizzle
         }
         // ---- quantise down the columns
         if (mirror) {
           uint32_t lo, hi;
           float bmax;
           uint32_t sb;
-          if (PF) sb = quantize_block16_opts<MODE != kG3>(w, args.q, sg_out, lo, hi, bmax);
-          else sb = quantize_block16_pow2(w, sg_out, inv_sg, rcp_base, lo, hi, bmax);
+          if (PF) {
+            // the transform and the error sums need the block in row order
+#pragma unroll
+            for (int k = 0; k < 16; k += 2) {
+              const float a = w[k], c = w[k + 1];
+              w[k] = g ? c : a;
+              w[k + 1] = g ? a : c;
+            }
+            sb = quantize_block16_opts_p2(w, args.q, inv_sg, lo, hi, bmax);
+          } else {
+            sb = quantize_block16_p2(w, inv_sg, lo, hi, bmax);
+            if (g) { lo = swap_nibbles(lo); hi = swap_nibbles(hi); }   // back into row order
+          }
           sts64u(cq_st + e * (CHUNK * 64), lo, hi);
           // tensor row = x64 + e * 16 + cq: e % 2 selects the upper 16 of 32 rows of its scale atom,
           // e / 2 the 32-row group
@@ -905,7 +919,7 @@ cudaError_t launch_pair_mode(const ProblemPack& pack, const GemmLaunch& L, int s
 extern "C" int fp4_trace_read(unsigned long long* dst, int clear) {
   if (cudaMemcpyFromSymbol(dst, g_trace, sizeof(g_trace)) != cudaSuccess) return 1;
   if (clear) {
-    static unsigned long long zero[160 * 18 * 8];
+    static unsigned long long zero[160 * 19 * 8];
     if (cudaMemcpyToSymbol(g_trace, zero, sizeof(zero)) != cudaSuccess) return 1;
   }
   return 0;
