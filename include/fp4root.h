@@ -176,8 +176,10 @@ fp4_status fp4_root_coeffs(int64_t m, int64_t n, int steps, float abc[3]);
  * Two calls that share a workspace must not overlap in time.
  * Launches: 6 kernels for clip, normalisation and the first quantisation plus 3 per iteration
  *   (and a transpose pass for a tall matrix on the routes that cannot write the result
- *   transposed from the last product).  Calls on small matrices (up to 8 M elements per group
- *   of equal shapes) chain their kernels with programmatic dependent launch; the environment
+ *   transposed from the last product).  Groups of up to a few million elements run all
+ *   iterations in one cooperative launch instead, whose blocks wait on one another (bounded
+ *   waits).  Calls on small matrices (up to 8 M elements per group
+ *   of equal shapes) chain their other kernels with programmatic dependent launch; the environment
  *   variable FP4ROOT_NO_PDL (any value) switches that off.  Kernels launched before or after
  *   the call on the same stream see ordinary stream order either way.
  */
@@ -381,7 +383,8 @@ fp4_status fp4_adamw_update(uint16_t* W, const uint16_t* G, int64_t n, uint8_t* 
 /* ---- measurement support (the paper has no counterpart) -----------------------------------
  * While profiling is enabled, every group of launches of the step is bracketed by a pair of
  * CUDA events on the caller's stream; fp4_profile_collect waits for them, adds the elapsed
- * times per class into ms[class] and the number of bracketed groups into groups[class]
+ * times per class into ms[class] (iterations that run in one launch count as FP4_PROF_G3) and
+ * the number of bracketed groups into groups[class]
  * (both host arrays of FP4_PROF_CLASSES entries), then forgets them.  Off by default; the
  * events add stream operations, so time whole calls with profiling off.
  * fp4_kernel_launches returns how many kernels this library has launched in this process.

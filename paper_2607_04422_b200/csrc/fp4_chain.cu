@@ -1,0 +1,701 @@
+// All iterations of the Newton-Schulz step (Section 3.4, display equations) for a small group of equal-shape
+// matrices in ONE cooperative launch.
+//
+// A matrix of up to a few million elements has fewer 256 x 256 tiles than the GPU has SM pairs, and with a
+// launch per product its time is launch latency, cold instruction fetches and the epilogue of one large tile.
+// Here one persistent block per SM walks the products of all iterations in order, in tiles of 128 x 64 or
+// 128 x 128 (chosen so that a product fills the SMs).  Nothing is launched between products: a tile of a
+// product waits, on a counter in the matrix's workspace header, until all tiles of the matrix's product
+// before it are stored.
+//
+// Work list: product 0, 1, 2, ... and within a product the tiles of all matrices; block b takes the tiles
+// b, b + grid, ... of every product.  Every dependency points to an earlier product and all blocks are
+// resident (cooperative launch), so the earliest unfinished tile can always run.  Since G1 and G2 list the
+// same tiles, and every G3 lists the same tiles, the FP32 values a tile combines with (A in G2, X in G3) were
+// written by the very thread that reads them: they need no ordering between blocks and are fetched
+// before the dependency is even looked at.
+//
+// Warp roles: 0-15 epilogue, 16 operand producer (TMA; also the only thread that polls the counter), 17 MMA
+// issuer and TMEM owner, 18 stores.  Epilogue warp w owns the TMEM lanes of quadrant w % 4 and the 16-column
+// (or two 16-column) pieces w / 4 of the tile; it moves its 32 x 16 FP32 blocks with its own TMA loads and
+// stores and shares nothing with the other epilogue warps but the staging area in which the tile's
+// quantised outputs are collected.  The store warp sends that area off, waits until it has arrived, publishes
+// the running maximum and counts the tile.
+//
+// Bounds: latency.  A 5-iteration call is a chain of 15 dependent products.  At 256 x 512 a product takes about 5 us:
+// the counter's round trip 1 us with its fences another 0.9, operand copies and MMAs 1, the one tile's epilogue 1.5-2.
+// Whole calls, before (three launches per iteration) and now: 256 x 512 175 -> 108 us, 1024 x 1024 190 -> 135,
+// 1040 x 2896 with the paper's quantiser options 307 -> 233.
+#include "fp4_gemm_common.cuh"
+
+namespace fp4 {
+
+namespace {
+
+constexpr int BM = 128, BK = 256, KSTEPS = BK / 64;
+constexpr int CHUNK = 16;
+constexpr int NACC = 2;
+constexpr int EPI_WARPS = 16;
+constexpr int W_LOAD = EPI_WARPS, W_MMA = EPI_WARPS + 1, W_STORE = EPI_WARPS + 2;
+constexpr int NTHREADS = (EPI_WARPS + 3) * 32;
+constexpr int DEP_RING = 16;
+constexpr int XBUF = 32 * 64;                 // a warp's 32 x 16 FP32 block: 64-byte rows, 64-byte swizzle
+constexpr int MAX_STAGES = 5;
+constexpr uint32_t TMEM_COLS = 512;
+constexpr uint32_t SF_COLS = KSTEPS * 8;      // per stage: 4 columns per MMA for each operand
+
+template <int BN>
+struct ChainLay {
+  static constexpr int STAGES = BN == 64 ? 5 : 3;
+  static constexpr int A_BYTES = BM * BK / 2, B_BYTES = BN * BK / 2, SF_BYTES = KSTEPS * 512;
+  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES + 2 * SF_BYTES;
+  static constexpr int CHUNKS = BN / 64;      // 16-column chunks per epilogue warp
+  // staging area of a tile's quantised outputs: row codes [64-column half][128 rows][32 bytes], column codes
+  // [BN columns][64 bytes] with a 64-byte swizzle, row scale atoms, column scales [2 atoms][32][BN / 32 words]
+  static constexpr int RQ = BM * BN / 2, CQ = BN * BM / 2, RSF = BN / 64 * 512, CSF = BN * 8;
+  static constexpr int OUT = RQ + CQ + 1024 * ((RSF + CSF + 1023) / 1024);
+  static constexpr int OFF_X = STAGES * STAGE_BYTES;         // two blocks per epilogue warp
+  static constexpr int OFF_OUT = OFF_X + EPI_WARPS * 2 * XBUF;  // two areas, used by alternate tiles
+  static constexpr int OFF_BAR = OFF_OUT + 2 * OUT;
+  static constexpr int SMEM = OFF_BAR + 2048 + 1024;
+  static constexpr uint32_t SF_COL = NACC * BN;
+  static_assert(SMEM <= 232448 && STAGE_BYTES % 1024 == 0 && OFF_OUT % 1024 == 0 && OUT % 1024 == 0, "shared memory");
+  static_assert(STAGES <= MAX_STAGES && SF_COL + STAGES * SF_COLS <= TMEM_COLS, "tensor memory columns");
+  // M = 128, N = BN, E2M1 x E2M1, UE4M3 scales, K-major operands
+  static constexpr uint32_t IDESC = (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+};
+
+struct ChainShared {
+  uint64_t full[MAX_STAGES], empty[MAX_STAGES];
+  uint64_t acc_full[NACC], acc_empty[NACC];
+  uint64_t dep[DEP_RING];          // the tile's dependency is met (one arrival by the producer per tile)
+  uint64_t xfull[EPI_WARPS * 2];   // an FP32 block has landed
+  uint64_t out_done[2], out_free[2];
+  alignas(16) uint32_t amax[2][4]; // running maximum of the tile in a staging area (bit pattern), at its place among four slots
+  uint32_t tmem_base, abort_flag;
+  uint32_t tiles[2][kChainTiles];  // this block's tiles of a symmetric product / of G3: p << 28 | ti << 16 | tj
+};
+static_assert(sizeof(ChainShared) <= 2048, "shared block");
+
+// Tile t of a product; the symmetric products list the tiles whose 128-column block is on or above the diagonal.
+template <int BN>
+__device__ __forceinline__ uint32_t chain_tile(int t, bool sym, int per_problem, int cols) {
+  const int p = t / per_problem;
+  t -= p * per_problem;
+  int ti, tj;
+  if (!sym) {
+    ti = t / cols;
+    tj = t - ti * cols;
+  } else {
+    constexpr int R = BM / BN;
+    int row = 0, len = cols;
+    while (t >= len) { t -= len; ++row; len -= R; }
+    ti = row;
+    tj = row * R + t;
+  }
+  return (uint32_t)p << 28 | (uint32_t)ti << 16 | (uint32_t)tj;
+}
+
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void red_release_add(uint32_t* p, uint32_t v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// running maxima (non-negative floats order like unsigned integers): four words at once, 16-byte aligned
+__device__ __forceinline__ void bulk_max16_s(void* dst, uint32_t src) {
+  asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.max.u32 [%0], [%1], 16;" ::"l"(dst), "r"(src) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// scalars written by other blocks of this launch: never from L1
+__device__ __forceinline__ float ld_scalar(const float* p) {
+  return __uint_as_float(ld_relaxed(reinterpret_cast<const uint32_t*>(p)));
+}
+__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
+__device__ __forceinline__ void sts_f4(uint32_t a, float x, float y, float z, float w) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+__device__ __forceinline__ void sts_u2(uint32_t a, uint32_t x, uint32_t y) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void sts_b(uint32_t a, uint32_t x) {
+  asm volatile("st.shared.b8 [%0], %1;" ::"r"(a), "r"(x) : "memory");
+}
+__device__ __forceinline__ float4 lds_f4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float lds_f1(uint32_t a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void tma_load_s(uint32_t dst, const void* tmap, int x, int y, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+      "l"(tmap), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void tma_store_s(const void* tmap, int x, int y, uint32_t src) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(tmap), "r"(x), "r"(y),
+               "r"(src)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_store_s(void* dst, uint32_t src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_expect_s(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
+// Root's parameter update of a tall matrix: the parameter has the caller's orientation, so the 16 values of this
+// lane's row lie a row of the parameter apart.
+__device__ __noinline__ void chain_update_tall(uint16_t* w, int64_t ld, const float (&v)[16], float decay, float step) {
+#pragma unroll 4
+  for (int i = 0; i < 16; ++i, w += ld)
+    *w = (uint16_t)cvt_bf16x2(param_update_value(bf16_lo(*w), v[i], decay, step), 0.0f);
+}
+
+template <int BN, bool PF>
+__global__ void __launch_bounds__(NTHREADS, 1)
+k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLaunch a) {
+  using L = ChainLay<BN>;
+  constexpr int STAGES = L::STAGES;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  ChainShared* sh = reinterpret_cast<ChainShared*>(smem + L::OFF_BAR);
+  volatile uint32_t* abort_flag = &sh->abort_flag;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const int nsym = a.nsym, nfull = (a.s / BM) * (a.l / BN);   // tiles per matrix of a symmetric product / of G3
+  const int grid = (int)gridDim.x;
+  // tiles of this block
+  const int my_sym = (nsym * a.count - (int)blockIdx.x + grid - 1) / grid;
+  const int my_full = (nfull * a.count - (int)blockIdx.x + grid - 1) / grid;
+  const int products = 3 * a.steps;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < STAGES; ++i) { mbar_init(&sh->full[i], 1); mbar_init(&sh->empty[i], 1); }
+    for (int i = 0; i < NACC; ++i) { mbar_init(&sh->acc_full[i], 1); mbar_init(&sh->acc_empty[i], EPI_WARPS); }
+    for (int i = 0; i < DEP_RING; ++i) mbar_init(&sh->dep[i], 1);
+    for (int i = 0; i < EPI_WARPS * 2; ++i) mbar_init(&sh->xfull[i], 1);
+    for (int i = 0; i < 2; ++i) { mbar_init(&sh->out_done[i], EPI_WARPS); mbar_init(&sh->out_free[i], 1); for (int q = 0; q < 4; ++q) sh->amax[i][q] = 0; }
+    sh->abort_flag = 0;
+    mbar_fence_init();
+  }
+  for (int i = (int)threadIdx.x - 64; i >= 0 && i < 2 * kChainTiles; i += NTHREADS) {
+    const int list = i / kChainTiles, j = i % kChainTiles;
+    if (j < (list ? my_full : my_sym))
+      sh->tiles[list][j] = chain_tile<BN>((int)blockIdx.x + j * grid, list == 0, list ? nfull : nsym, (list ? a.l : a.s) / BN);
+  }
+  if (warp == W_MMA) {
+    tmem_alloc(&sh->tmem_base, TMEM_COLS);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = sh->tmem_base;
+
+  if (warp == W_LOAD) {
+    // ------------------------------------------------------------ operand producer
+    if (elect_one()) {
+      int st = 0; uint32_t ph = 0, n = 0;
+      for (int pi = 0; pi < products; ++pi) {
+        const int k = pi / 3, mode = pi - 3 * k + kG1;
+        const bool sym = mode != kG3;
+        const int mine = sym ? my_sym : my_full;
+        const int K = mode == kG1 ? a.l : a.s;
+        const int num_kb = (K + BK - 1) / BK;
+        const uint32_t need = (uint32_t)(k * (2 * nsym + nfull) + (mode - kG1) * nsym);
+        int seen = -1;
+        for (int j = 0; j < mine; ++j, ++n) {
+          const uint32_t tile = sh->tiles[sym ? 0 : 1][j];
+          const int p = (int)(tile >> 28), ti = (int)(tile >> 16) & 0xFFF, tj = (int)(tile & 0xFFFF);
+          const ChainProblem& pr = pack.p[p];
+          if (p != seen && need != 0) {
+            // all tiles of the matrix's earlier products are stored
+            bool met = ld_acquire(pr.done) >= need;
+            if (!met) {
+              const uint64_t t0 = globaltimer_ns();
+              for (;;) {
+                for (int i = 0; i < 64 && !met; ++i) met = ld_acquire(pr.done) >= need;
+                if (met) break;
+                if (*abort_flag || globaltimer_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; break; }
+              }
+            }
+            fence_proxy_async_all();   // part of the operands was stored through the generic proxy, TMA reads them
+          }
+          seen = p;
+          mbar_arrive(&sh->dep[n % DEP_RING]);
+          const CUtensorMap* ma = mode == kG1 ? &pr.tm_qX : mode == kG2 ? &pr.tm_qA : &pr.tm_qB;
+          const CUtensorMap* mb = mode == kG1 ? &pr.tm_qX : mode == kG2 ? &pr.tm_qA : &pr.tm_qXt[k & 1];
+          const uint8_t* sfa = (mode == kG1 ? pr.qx_sf : mode == kG2 ? pr.qa_sf : pr.qb_sf) + (size_t)ti * (K / 64) * 512;
+          const uint8_t* sfb = (mode == kG1 ? pr.qx_sf : mode == kG2 ? pr.qa_sf : pr.qt_sf[k & 1]) +
+                               (size_t)(tj * BN / 128) * (K / 64) * 512;
+          for (int kb = 0; kb < num_kb; ++kb) {
+            wait_or_abort(&sh->empty[st], ph ^ 1, abort_flag);
+            // a half-full last stage: the operand boxes are zero-filled beyond K (and still credit their full
+            // size), only the scale atoms that exist are fetched
+            const int kvalid = K - kb * BK < BK ? K - kb * BK : BK;
+            const uint32_t sf_bytes = (uint32_t)(kvalid / 64) * 512;
+            uint8_t* d = smem + st * L::STAGE_BYTES;
+            mbar_expect_tx(&sh->full[st], L::A_BYTES + L::B_BYTES + 2 * sf_bytes);
+            tma_load_2d(d, ma, kb * (BK / 2), ti * BM, &sh->full[st]);
+            tma_load_2d(d + L::A_BYTES / 2, ma, kb * (BK / 2), ti * BM + 64, &sh->full[st]);
+#pragma unroll
+            for (int h = 0; h < BN / 64; ++h)
+              tma_load_2d(d + L::A_BYTES + h * (64 * BK / 2), mb, kb * (BK / 2), tj * BN + h * 64, &sh->full[st]);
+            bulk_load_1d(d + L::A_BYTES + L::B_BYTES, sfa + (size_t)kb * L::SF_BYTES, sf_bytes, &sh->full[st]);
+            bulk_load_1d(d + L::A_BYTES + L::B_BYTES + L::SF_BYTES, sfb + (size_t)kb * L::SF_BYTES, sf_bytes, &sh->full[st]);
+            if (++st == STAGES) { st = 0; ph ^= 1; }
+          }
+        }
+      }
+    }
+  } else if (warp == W_MMA) {
+    // ------------------------------------------------------------ MMA issuer
+    if (elect_one()) {
+      int st = 0; uint32_t ph = 0, n = 0;
+      for (int pi = 0; pi < products; ++pi) {
+        const int mode = pi % 3 + kG1;
+        const bool sym = mode != kG3;
+        const int mine = sym ? my_sym : my_full;
+        const int K = mode == kG1 ? a.l : a.s;
+        const int num_kb = (K + BK - 1) / BK;
+        for (int j = 0; j < mine; ++j, ++n) {
+          // scale atoms cover 128 rows of the column operand: an odd 64-column tile uses their upper half
+          const uint32_t sfb_shift = BN == 64 ? 2u * (sh->tiles[sym ? 0 : 1][j] & 1u) : 0u;
+          const uint32_t ab = n % NACC;
+          wait_or_abort(&sh->acc_empty[ab], ((n / NACC) & 1) ^ 1, abort_flag);
+          tc_fence_after();
+          const uint32_t d_tmem = tmem_base + ab * BN;
+          for (int kb = 0; kb < num_kb; ++kb) {
+            wait_or_abort(&sh->full[st], ph, abort_flag);
+            tc_fence_after();
+            const uint32_t sf_t = tmem_base + L::SF_COL + st * SF_COLS;
+            const uint32_t d = smem_u32(smem + st * L::STAGE_BYTES);
+            const int ksteps = (K - kb * BK < BK ? K - kb * BK : BK) / 64;
+            const uint64_t adesc = umma_desc(d, 1024, 2), bdesc = umma_desc(d + L::A_BYTES, 1024, 2);
+#pragma unroll
+            for (int i = 0; i < KSTEPS; ++i) {
+              if (i < ksteps) {
+                tc_cp_sf(sf_t + i * 4, umma_desc(d + L::A_BYTES + L::B_BYTES + i * 512, 128, 0));
+                tc_cp_sf(sf_t + KSTEPS * 4 + i * 4, umma_desc(d + L::A_BYTES + L::B_BYTES + L::SF_BYTES + i * 512, 128, 0));
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < KSTEPS; ++i) {
+              if (i < ksteps)
+                tc_mma_nvf4(d_tmem, adesc + 2 * i, bdesc + 2 * i, L::IDESC, sf_t + i * 4, sf_t + KSTEPS * 4 + i * 4 + sfb_shift,
+                            (kb | i) != 0 ? 1u : 0u);
+            }
+            tc_commit(&sh->empty[st]);
+            if (++st == STAGES) { st = 0; ph ^= 1; }
+          }
+          tc_commit(&sh->acc_full[ab]);
+        }
+      }
+    }
+  } else if (warp == W_STORE) {
+    // ------------------------------------------------------------ stores of the quantised outputs
+    uint32_t n = 0;
+    for (int pi = 0; pi < products; ++pi) {
+      const int k = pi / 3, mode = pi - 3 * k + kG1;
+      const bool sym = mode != kG3;
+      const int mine = sym ? my_sym : my_full;
+      if (pi == products - 1 && !a.keep) break;
+      const int rq_k = sym ? a.s : a.l;
+      for (int j = 0; j < mine; ++j, ++n) {
+        const uint32_t tile = sh->tiles[sym ? 0 : 1][j];
+        const int p = (int)(tile >> 28), ti = (int)(tile >> 16) & 0xFFF, tj = (int)(tile & 0xFFFF);
+        const ChainProblem& pr = pack.p[p];
+        const bool mirror = mode == kG3 || tj * BN / 128 != ti;
+        uint8_t* ob = smem + L::OFF_OUT + (n & 1) * L::OUT;
+        const uint32_t os = smem_u32(ob);
+        const CUtensorMap* mr = mode == kG1 ? &pr.st_qA : mode == kG2 ? &pr.st_qB : &pr.st_qX;
+        const CUtensorMap* mc = mode == kG1 ? &pr.st_qAc : mode == kG2 ? &pr.st_qBc : &pr.st_qXt[(k & 1) ^ 1];
+        uint8_t* sym_sf = mode == kG1 ? pr.qa_sf : pr.qb_sf;
+        uint8_t* rsf = (sym ? sym_sf : pr.qx_sf) + ((int64_t)ti * (rq_k / 64) + tj * (BN / 64)) * 512;
+        uint8_t* csf = (sym ? sym_sf : pr.qt_sf[(k & 1) ^ 1]) + ((int64_t)(tj * BN / 128) * (a.s / 64) + ti * 2) * 512;
+        const int slot = mode == kG1 ? a.ix.amax_A0 + k : a.ix.amax_X0 + k + 1;
+        float* maxima = pr.scalars + (slot & ~3);
+        uint32_t* done = pr.done;
+        wait_or_abort(&sh->out_done[n & 1], (n >> 1) & 1, abort_flag);
+        if (BN == 64 && mirror) {
+          // the scales of 64 rows are the 8-byte halves of the 16-byte rows of two atoms
+          uint8_t* dst = csf + lane * 16 + (tj & 1) * 8;
+          const uint8_t* src = ob + L::RQ + L::CQ + L::RSF + lane * 8;
+          *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src);
+          *reinterpret_cast<uint2*>(dst + 512) = *reinterpret_cast<const uint2*>(src + 256);
+        }
+        if (lane == 0) {
+#pragma unroll
+          for (int h = 0; h < BN / 64; ++h) tma_store_s(mr, tj * (BN / 2) + h * 32, ti * BM, os + h * 4096);
+          bulk_store_s(rsf, os + L::RQ + L::CQ, L::RSF);
+          if (mirror) {
+#pragma unroll
+            for (int h = 0; h < BN / 64; ++h) tma_store_s(mc, ti * 64, tj * BN + h * 64, os + L::RQ + h * 4096);
+            if (BN == 128) bulk_store_s(csf, os + L::RQ + L::CQ + L::RSF, L::CSF);
+          }
+          if (mode != kG2) bulk_max16_s(maxima, smem_u32(&sh->amax[n & 1][0]));
+          bulk_commit();
+          bulk_wait_all<0>();
+          sh->amax[n & 1][slot & 3] = 0;
+        }
+        __syncwarp();
+        if (lane == 0) {
+          red_release_add(done, 1u);
+          mbar_arrive(&sh->out_free[n & 1]);
+        }
+      }
+    }
+  } else {
+    // ------------------------------------------------------------ epilogue warps
+    const int quad = warp & 3, team = warp >> 2;
+    const int cq = lane & 15, g = lane >> 4;
+    const uint32_t area = smem_u32(smem + L::OFF_X + warp * 2 * XBUF);
+    const uint32_t xfull = smem_u32(&sh->xfull[warp * 2]);
+    // row-per-lane view of a block: 16-byte group j of this lane's row at row_addr ^ (j << 4)
+    const uint32_t row_addr = area + lane * 64 + (((lane >> 1) & 3) << 4);
+    // column view: at step k the lane reads row k ^ g of its 16-row group (in step the half-warps, whose rows are
+    // 16 apart, would hit the same banks), at col_base | (col_lane ^ (k << 6 | (k >> 1 & 3) << 4))
+    const uint32_t col_base = area + g * (16 * 64);
+    const uint32_t col_lane = (uint32_t)(g << 6 | cq << 2);
+    const uint32_t tm_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
+    // staging offsets of this lane's outputs (chunk 0 of the warp)
+    const uint32_t out0 = smem_u32(smem + L::OFF_OUT);
+    const int row = quad * 32 + lane;
+
+    // Lane 0 starts the copy of the FP32 block a unit (tile, chunk) combines with.
+    auto fetch = [&](int mode, int k, uint32_t tile, int c, int b) {
+      if (lane == 0) {
+        const ChainProblem& pr = pack.p[tile >> 28];
+        const int y = ((int)(tile >> 16) & 0xFFF) * BM + quad * 32;
+        const int x = (int)(tile & 0xFFFF) * BN + (team * L::CHUNKS + c) * CHUNK;
+        const CUtensorMap* m = mode == kG2 ? &pr.tm_A : k == 0 ? &pr.tm_G : &pr.tm_X;
+        const bool tr = mode == kG3 && k == 0 && pr.tall;
+        mbar_expect_s(xfull + b * 8, XBUF);
+        tma_load_s(area + b * XBUF, m, tr ? y : x, tr ? x : y, xfull + b * 8);
+      }
+    };
+
+    uint32_t n = 0, unit = 0, xph = 0;   // tiles, units, phases of the two block barriers
+    bool have = false;                   // the copy of the unit at hand is under way
+    for (int pi = 0; pi < products; ++pi) {
+      const int k = pi / 3, mode = pi - 3 * k + kG1;
+      const bool sym = mode != kG3;
+      const int mine = sym ? my_sym : my_full;
+      const bool last = pi == products - 1;
+      const bool do_q = !last || a.keep;
+      const bool raw = mode == kG3 && k == 0;
+      int cur_p = -1;
+      float scale = 0.0f, inv_sg = 1.0f, beta = 0.0f, gamma = 0.0f, tau = 0.0f, inv = 0.0f;
+      bool fused = false;
+      QuantOpts qo = a.q;
+      if (PF && a.q.rht) {
+        const int j = mode == kG1 ? 2 * k + 1 : mode == kG2 ? 2 * k : 2 * k + 2;
+        qo.mask = rht_signs(a.seed, (uint64_t)j);
+      }
+      for (int j = 0; j < mine; ++j, ++n) {
+        const uint32_t tile = sh->tiles[sym ? 0 : 1][j];
+        const int p = (int)(tile >> 28), ti = (int)(tile >> 16) & 0xFFF, tj = (int)(tile & 0xFFFF);
+        const ChainProblem& pr = pack.p[p];
+        const bool xposed = raw && pr.tall;
+        const bool mirror = do_q && (mode == kG3 || tj * BN / 128 != ti);
+        const bool out_t = last && pr.tall;              // the result of a tall matrix leaves transposed
+        wait_or_abort(&sh->dep[n % DEP_RING], (n / DEP_RING) & 1, abort_flag);
+        if (p != cur_p) {
+          cur_p = p;
+          const float* sc = pr.scalars;
+          float sg_out, bound;
+          if (mode == kG1) {
+            const float sgx = ld_scalar(sc + a.ix.sg_X0 + k), ax = ld_scalar(sc + a.ix.amax_X0 + k);
+            scale = __fmul_rn(sgx, sgx);
+            bound = fminf(__fmul_rn(__fmul_rn(__fmul_rn(2.0f, a.l_cols), ax), ax), 4.0f);
+          } else if (mode == kG2) {
+            const float sga = ld_scalar(sc + a.ix.sg_A0 + k), aa = ld_scalar(sc + a.ix.amax_A0 + k);
+            scale = __fmul_rn(sga, sga);
+            bound = __fmul_rn(__fadd_rn(fabsf(pr.cb), __fmul_rn(4.0f, fabsf(pr.cc))), aa);
+            beta = pr.cb;
+            gamma = __fmul_rn(pr.cc, scale);   // exact: sga is a power of two
+          } else {
+            const float sgb = ld_scalar(sc + a.ix.sg_B0 + k), sgx = ld_scalar(sc + a.ix.sg_X0 + k);
+            const float ax = ld_scalar(sc + a.ix.amax_X0 + k);
+            scale = __fmul_rn(sgb, sgx);
+            bound = __fmul_rn(__fmul_rn(4.0f, fabsf(pr.ca)), ax);
+            beta = pr.ca;
+            gamma = scale;
+            if (raw) {
+              tau = a.clip ? ld_scalar(sc + a.ix.tau) : __int_as_float(0x7f800000);
+              inv = ld_scalar(sc + a.ix.inv);
+            }
+          }
+          sg_out = scale_predicted(__fmul_rn(a.q.widen, bound));
+          inv_sg = __frcp_rn(sg_out);
+          // a power-of-two scale multiplies exactly, so fl(fl(a x) + fl(acc scale)) is one fused operation
+          fused = mode == kG3 && (__float_as_uint(scale) & 0x007FFFFFu) == 0 && scale > 1e-30f && scale < 1e30f;
+          // the matrix's first tile publishes its output scale (all epilogue warps of the block arrive on
+          // out_done after this, and the store warp counts the tile after that)
+          if (ti == 0 && tj == 0 && threadIdx.x == 0)
+            pr.scalars[mode == kG1 ? a.ix.sg_A0 + k : mode == kG2 ? a.ix.sg_B0 + k : a.ix.sg_X0 + k + 1] = sg_out;
+        }
+        const uint32_t ab = n % NACC;
+        const uint32_t os = out0 + (n & 1) * L::OUT;
+        float amax = 0.0f;
+#pragma unroll 1
+        for (int c = 0; c < L::CHUNKS; ++c, ++unit) {
+          const int ch = team * L::CHUNKS + c;             // chunk of the tile
+          const int y = ti * BM + quad * 32, x0 = tj * BN + ch * CHUNK;
+          const int b = (int)(unit & 1);
+          const uint32_t boff = (uint32_t)b * XBUF;
+          // both blocks' earlier stores have been read; the next unit of the same product is fetched now
+          if (lane == 0) bulk_wait_read<0>();
+          if (mode != kG1) {
+            if (!have) fetch(mode, k, tile, c, b);
+            const bool more = c + 1 < L::CHUNKS || j + 1 < mine;
+            if (more) fetch(mode, k, c + 1 < L::CHUNKS ? tile : sh->tiles[sym ? 0 : 1][j + 1], c + 1 < L::CHUNKS ? c + 1 : 0, b ^ 1);
+            have = more;
+          }
+          __syncwarp();
+          if (c == 0) {
+            wait_or_abort(&sh->acc_full[ab], (n / NACC) & 1, abort_flag);
+            tc_fence_after();
+          }
+          uint32_t acc[16];
+          tc_ld16_issue(tm_lane + ab * BN + ch * CHUNK, acc);
+          float x[16];
+          if (mode != kG1) {
+            wait_or_abort(xfull + b * 8, (xph >> b) & 1, abort_flag);
+            xph ^= 1u << b;
+            if (xposed) {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) x[i] = lds_f1(area + boff + i * 128 + lane * 4);
+              __syncwarp();  // every lane has its row before the result rows are staged over the block
+            } else {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const float4 f = lds_f4((row_addr + boff) ^ (i << 4));
+                x[4 * i] = f.x; x[4 * i + 1] = f.y; x[4 * i + 2] = f.z; x[4 * i + 3] = f.w;
+              }
+            }
+            if (raw) {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) x[i] = __fmul_rn(fminf(fmaxf(x[i], -tau), tau), inv);
+            }
+          }
+          tc_wait_ld16(acc);
+          if (c == L::CHUNKS - 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh->acc_empty[ab]);
+          }
+          float v[16];
+          if (mode == kG1) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = __fmul_rn(__uint_as_float(acc[i]), scale);
+          } else {
+            const uint64_t b2 = pack2(beta, beta), g2 = pack2(gamma, gamma);
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) {
+              const uint64_t ac2 = pack2(__uint_as_float(acc[i]), __uint_as_float(acc[i + 1]));
+              const uint64_t bx = mul2(b2, pack2(x[i], x[i + 1]));
+              if (fused) {
+                unpack2(fma2(ac2, g2, bx), v[i], v[i + 1]);
+              } else {
+                float t0, t1, u0, u1;
+                unpack2(bx, t0, t1);
+                unpack2(mul2(ac2, g2), u0, u1);
+                v[i] = __fadd_rn(t0, u0);
+                v[i + 1] = __fadd_rn(t1, u1);
+              }
+            }
+          }
+          // ---- stage the block (for the TMA store and for the pass down the columns) and send it off
+          if (out_t && !a.keep) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              asm volatile("st.shared.f32 [%0], %1;" ::"r"(area + boff + i * 128 + lane * 4), "f"(v[i]) : "memory");
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sts_f4((row_addr + boff) ^ (i << 4), v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+          }
+          const bool round = a.bf16 && !last && mode != kG2;  // stored rounded to BF16, after the pass down the columns
+          bool send = mode != kG2;
+          if (mode == kG3) {
+            // the caller's matrix has no padding; X of a tall matrix lies in the workspace and has
+            send = (y < a.s0 && x0 < a.l0) || (pr.tall && !out_t);
+            if (last && a.update && pr.W) {
+              const bool in = y + lane < a.s0 && x0 < a.l0;
+              if (pr.tall) {
+                if (in) chain_update_tall(pr.W + (int64_t)x0 * a.s0 + y + lane, a.s0, v, a.upd_decay, a.upd_step);
+              } else if (in) {
+                uint4* w = reinterpret_cast<uint4*>(pr.W + ((int64_t)y + lane) * a.l0 + x0);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  uint4 o = w[h];
+                  uint32_t* e = &o.x;
+#pragma unroll
+                  for (int i = 0; i < 4; ++i)
+                    e[i] = cvt_bf16x2(param_update_value(bf16_lo(e[i]), v[8 * h + 2 * i], a.upd_decay, a.upd_step),
+                                      param_update_value(bf16_hi(e[i]), v[8 * h + 2 * i + 1], a.upd_decay, a.upd_step));
+                  w[h] = o;
+                }
+              }
+              send = send && !a.no_out;
+            }
+          }
+          // The FP32 block leaves by TMA; only this warp reads it back.  With several units per product (BN = 128) it
+          // is sent now, so that its buffer is free in time; else after the outputs that other blocks wait for.
+          auto send_block = [&]() {
+            if (mode == kG1) tma_store_s(&pr.tm_A, x0, y, area + boff);
+            else if (!out_t || a.keep) tma_store_s(&pr.tm_X, x0, y, area + boff);
+            else tma_store_s(&pr.tm_outT, y, x0, area + boff);
+            bulk_commit();
+          };
+          const bool early = BN == 128 && !round;
+          if (send && early) fence_proxy_async_smem();
+          __syncwarp();
+          if (send && early && lane == 0) send_block();
+          float w[16];
+          if (mirror) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const uint32_t at = (col_base + boff) | (col_lane ^ (uint32_t)(i << 6 | ((i >> 1) & 3) << 4));
+              w[i] = lds_f1(at);
+              w[i + 8] = lds_f1(at + 512);
+            }
+            if (PF) {
+              // the transform and the error sums need the block in row order
+#pragma unroll
+              for (int i = 0; i < 16; i += 2) {
+                const float c0 = w[i], c1 = w[i + 1];
+                w[i] = g ? c1 : c0;
+                w[i + 1] = g ? c0 : c1;
+              }
+            }
+          }
+          if (round) {
+            // what is stored is rounded to BF16
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const uint32_t w0 = cvt_bf16x2(v[4 * i], v[4 * i + 1]), w1 = cvt_bf16x2(v[4 * i + 2], v[4 * i + 3]);
+              sts_f4((row_addr + boff) ^ (i << 4), bf16_lo(w0), bf16_hi(w0), bf16_lo(w1), bf16_hi(w1));
+            }
+          }
+          if (do_q) {
+            uint32_t lo, hi;
+            float bmax;
+            uint32_t sb;
+            if (PF) sb = quantize_block16_opts_p2(v, qo, inv_sg, lo, hi, bmax);
+            else sb = quantize_block16_p2(v, inv_sg, lo, hi, bmax);
+            amax = fmaxf(amax, bmax);
+            // the stores of the tile two back have read the staging area
+            if (c == 0) wait_or_abort(&sh->out_free[n & 1], ((n >> 1) & 1) ^ 1, abort_flag);
+            sts_u2(os + (ch >> 2) * 4096 + row * 32 + (((ch & 3) * 8) ^ ((lane & 4) << 2)), lo, hi);
+            sts_b(os + L::RQ + L::CQ + (ch >> 2) * 512 + lane * 16 + quad * 4 + (ch & 3), sb);
+            if (mirror) {
+              if (PF) sb = quantize_block16_opts_p2(w, qo, inv_sg, lo, hi, bmax);
+              else sb = quantize_block16_p2(w, inv_sg, lo, hi, bmax);
+              if (!PF && g) { lo = swap_nibbles(lo); hi = swap_nibbles(hi); }   // back into row order
+              const int col = ch * CHUNK + cq;
+              sts_u2(os + L::RQ + col * 64 + ((quad ^ ((col >> 1) & 3)) << 4) + g * 8, lo, hi);
+              sts_b(os + L::RQ + L::CQ + L::RSF + (quad >> 1) * (BN * 4) + (col & 31) * (BN / 8) + (col >> 5) * 4 + (quad & 1) * 2 + g, sb);
+            }
+          }
+          // The fence orders this lane's reads and writes of shared memory before what the copies (another proxy)
+          // read and write there.
+          fence_proxy_async_smem();
+          if (c == L::CHUNKS - 1 && do_q) {
+            if (mode != kG2) {
+              const int slot = mode == kG1 ? a.ix.amax_A0 + k : a.ix.amax_X0 + k + 1;
+              const uint32_t wm = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
+              if (lane == 0) atomicMax(&sh->amax[n & 1][slot & 3], wm);
+              fence_proxy_async_smem();
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh->out_done[n & 1]);
+          }
+          __syncwarp();
+          if (send && !early && lane == 0) send_block();
+        }
+      }
+      // The next product's first block: once this warp's own stores (its A, its X) have arrived.
+      if (mine > 0) for (int np = pi + 1; np < products && np <= pi + 3; ++np) {
+        const int nk = np / 3, nmode = np - 3 * nk + kG1;
+        const int nmine = nmode != kG3 ? my_sym : my_full;
+        if (nmine == 0) continue;
+        if (nmode != kG1) {
+          if (lane == 0) bulk_wait_all<0>();
+          fetch(nmode, nk, sh->tiles[nmode != kG3 ? 0 : 1][0], 0, (int)(unit & 1));
+          have = true;
+        }
+        break;
+      }
+    }
+    if (lane == 0) bulk_wait_all<0>();
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == W_MMA) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, TMEM_COLS);
+  }
+  if (threadIdx.x == 0 && sh->abort_flag) report_timeout(a.status);
+}
+
+template <int BN, bool PF>
+cudaError_t launch_one(const ChainPack& pack, const ChainLaunch& a, int grid, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = ChainLay<BN>::SMEM; cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  count_launches(1);
+  return cudaLaunchKernelEx(&cfg, k_chain<BN, PF>, pack, a);
+}
+
+int sym_tiles(int64_t s, int bn) {
+  int n = 0;
+  for (int64_t r = 0; r < s / BM; ++r) n += (int)((s - r * BM) / bn);
+  return n;
+}
+
+}  // namespace
+
+cudaError_t chain_set_attributes() {
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(k_chain<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<64>::SMEM))) return e;
+  if ((e = cudaFuncSetAttribute(k_chain<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<64>::SMEM))) return e;
+  if ((e = cudaFuncSetAttribute(k_chain<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<128>::SMEM))) return e;
+  if ((e = cudaFuncSetAttribute(k_chain<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<128>::SMEM))) return e;
+  return cudaSuccess;
+}
+
+cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st) {
+  if (launch.count < 1 || launch.count > kChainMax || launch.steps < 1) return cudaErrorInvalidValue;
+  ChainLaunch a = launch;
+  const int rows = a.s / BM;
+  const int64_t full64 = (int64_t)rows * (a.l / 64) * a.count, full128 = (int64_t)rows * (a.l / 128) * a.count;
+  // Narrow tiles while they shorten the longest block's work: rounds of 128 x 64 tiles against rounds of 128 x 128.
+  // (256 x 512, 5 iterations: 87 us against 121; 1536 x 2560, where both take four rounds of 64 columns: 202 / 184.)
+  const bool narrow = (full64 + sms - 1) / sms < 2 * ((full128 + sms - 1) / sms);
+  const int bn = narrow ? 64 : 128;
+  a.nsym = sym_tiles(a.s, bn);
+  const int64_t widest = narrow ? full64 : full128;
+  const int grid = (int)(widest < sms ? widest : sms);
+  const bool pf = a.q.rht || a.q.four_six;
+  if (narrow) return pf ? launch_one<64, true>(pack, a, grid, st) : launch_one<64, false>(pack, a, grid, st);
+  return pf ? launch_one<128, true>(pack, a, grid, st) : launch_one<128, false>(pack, a, grid, st);
+}
+
+}  // namespace fp4

@@ -25,7 +25,8 @@ struct NsHeader {
   uint32_t count_below;  // elements in the bins below it
   uint32_t cand_count;   // candidates appended by the second pass (may exceed the list's capacity)
   uint32_t overflow;     // 1: the candidate list overflowed, the fallback passes run
-  uint32_t pad[21];
+  uint32_t tiles_done;   // tiles of the matrix's products stored so far (single-launch iterations)
+  uint32_t pad[20];
 };
 
 // Indices into the FP32 `scalars` array of a workspace.
@@ -120,6 +121,48 @@ struct GemmLaunch {
   NsScalarIdx ix;
   uint32_t* status;
 };
+
+// One matrix of a single-launch run of all iterations (fp4_chain.cu).
+struct alignas(64) ChainProblem {
+  CUtensorMap tm_qX, tm_qXt[2], tm_qA, tm_qB;    // operand loads: NVFP4 codes, box = 256 elements of K x 64 rows
+  CUtensorMap st_qX, st_qA, st_qB;               // row-quantised codes: box = 32 bytes x 128 rows
+  CUtensorMap st_qXt[2], st_qAc, st_qBc;         // column-quantised codes: box = 64 bytes x 64 rows, 64-byte swizzle
+  CUtensorMap tm_A, tm_X;                        // FP32 A and X between iterations: box = 16 columns x 32 rows
+  CUtensorMap tm_G, tm_outT;                     // the caller's matrix (transposing box when tall); tall: the result
+  uint16_t* W;               // the BF16 parameter that takes the update, or null
+  float* scalars;
+  uint32_t* done;            // NsHeader::tiles_done
+  uint8_t *qx_sf, *qt_sf[2], *qa_sf, *qb_sf;
+  float ca, cb, cc;
+  int tall;
+};
+constexpr int kChainMax = 14;    // matrices of a launch
+constexpr int kChainTiles = 32;  // tiles of one product that a block takes at most
+struct ChainPack { ChainProblem p[kChainMax]; };
+struct ChainLaunch {
+  int count, steps;
+  int s, l, s0, l0;          // work shape, the caller's short and long side
+  int nsym;                  // tiles per matrix of a symmetric product (set by launch_chain)
+  int clip, keep, bf16;
+  int update, no_out;
+  float upd_decay, upd_step;
+  float l_cols;
+  QuantOpts q;               // mask unused: drawn per product from seed
+  uint64_t seed;
+  NsScalarIdx ix;
+  uint32_t* status;
+};
+static_assert(sizeof(ChainPack) + sizeof(ChainLaunch) <= 32764, "kernel parameter space");
+// The 16 signs of the j-th random Hadamard matrix of a call: splitmix64 on seed + j.
+__host__ __device__ inline uint32_t rht_signs(uint64_t seed, uint64_t j) {
+  uint64_t z = seed + 0x9E3779B97F4A7C15ull * (j + 1);
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  z ^= z >> 31;
+  return (uint32_t)(z & 0xFFFFu);
+}
+cudaError_t chain_set_attributes();
+cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st);
 
 // Measurement support: counts kernel launches and, when profiling is on, brackets a group of
 // launches with events.

@@ -83,6 +83,7 @@ const DeviceInfo* device_info() {
   }
   d.encode = reinterpret_cast<EncodeTiledFn>(fn);
   if (gemm_set_attributes() != cudaSuccess || gemm_pair_set_attributes() != cudaSuccess ||
+      chain_set_attributes() != cudaSuccess ||
       prologue_set_attributes() != cudaSuccess)
     d.status = FP4_ERR_CUDA;
   d.ready = true;
@@ -101,12 +102,13 @@ constexpr uint32_t kNsFlags =
     FP4_FLAG_OVERLAP_GROUPS;
 
 // 2-D map over a row-major byte matrix (NVFP4 codes): box = one operand stage of `stage_k` elements of K
-// (64 or 128 bytes x 128 rows), swizzled over the box width.
-bool make_codes_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int64_t rows, int64_t row_bytes, int stage_k) {
+// (64 or 128 bytes x box_rows rows), swizzled over the box width.
+bool make_codes_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int64_t rows, int64_t row_bytes, int stage_k,
+                    int box_rows = 128) {
   const cuuint32_t bw = (cuuint32_t)(stage_k / 2);
   cuuint64_t dims[2] = {(cuuint64_t)row_bytes, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)row_bytes};
-  cuuint32_t box[2] = {bw, 128};
+  cuuint32_t box[2] = {bw, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
   return d->encode(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, bw == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
@@ -162,7 +164,7 @@ bool make_bf16_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int64
 }
 
 // 2-D map over a row-major byte matrix (NVFP4 codes) for the stores of the CTA-pair kernel's epilogue
-// warps: box = box_bytes x box_rows.
+// warps: box = box_bytes x box_rows, no swizzle.
 bool make_code_store_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int64_t rows, int64_t row_bytes,
                          int box_bytes, int box_rows, CUtensorMapSwizzle swizzle) {
   cuuint64_t dims[2] = {(cuuint64_t)row_bytes, (cuuint64_t)rows};
@@ -216,15 +218,6 @@ void default_params(fp4_ns_params* p) {
   p->weights = nullptr;
   p->lr = p->weight_decay = 0.0f;
   p->update_scale = 1.0f;
-}
-
-// The 16 signs of the j-th random Hadamard matrix of a call: splitmix64 on seed + j.
-uint32_t rht_signs(uint64_t seed, uint64_t j) {
-  uint64_t z = seed + 0x9E3779B97F4A7C15ull * (j + 1);
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  z ^= z >> 31;
-  return (uint32_t)(z & 0xFFFFu);
 }
 
 // Quantiser options of the j-th product of a call.
@@ -338,7 +331,23 @@ struct MatrixCtx {
   // writes the caller's result through transposing boxes.
   bool native_tall;
   CUtensorMap tm_outT;
+  ChainProblem chain;         // for a run of all iterations in one launch
 };
+
+// Which groups run all their iterations in one launch (fp4_chain.cu).  Below the limit a product's time is
+// launch latency and one tile's epilogue, above it the CTA-pair kernel's larger tiles win.  Measured, 5
+// iterations, one launch against fifteen: 1024 x 1024 135 / 190 us, 1536 x 2560 and 4096 x 1024 equal, 2560 x 2560
+// 333 / 290 us; with the paper's quantiser options, whose longer epilogue gains from the narrower tiles,
+// 1024 x 1024 169 / 287 us, 2048 x 2048 327 / 339 us.  (Not for inspection of BF16-stored intermediates: there A and X
+// stay FP32 tensors with rounded values.)
+bool chain_group(const DeviceInfo* d, const NsPlan& pl, int count, const fp4_ns_params* p) {
+  if (count > kChainMax || (pl.bf16_mode == 1 && (p->flags & FP4_FLAG_KEEP_OPERANDS))) return false;
+  const bool pair = pl.s % 256 == 0 && pl.l % 256 == 0;
+  const bool opts = (p->flags & (FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)) != 0;
+  const int64_t elements = pl.s * pl.l * count;
+  const int64_t limit = (pair && !opts) ? (int64_t)7 << 19 : (int64_t)9 << 19;
+  return elements <= limit && elements / (128 * 64) <= (int64_t)d->sms * kChainTiles;
+}
 
 fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t m, int64_t n, int steps,
                         const fp4_ns_params* p, uint8_t* ws, MatrixCtx* c) {
@@ -430,6 +439,30 @@ fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t
     g.rq_codes = ws + L.qX_codes; g.rq_sf = ws + L.qX_scales;
     g.cq_codes = ws + L.qXt_codes[cur ^ 1]; g.cq_sf = ws + L.qXt_scales[cur ^ 1];
     g.tmRq = st_qX_r; g.tmCq = st_qXt_c[cur ^ 1];
+  }
+  {
+    ChainProblem& h = c->chain;
+    memset(&h, 0, sizeof(h));
+    const bool tall = c->pl.tall;
+    auto load = [&](CUtensorMap* m, size_t off, int64_t rows, int64_t k) { return make_codes_map(d, m, ws + off, rows, k / 2, 256, 64); };
+    auto rows32 = [&](CUtensorMap* m, size_t off, int64_t k) { return make_code_store_map(d, m, ws + off, s, k / 2, 32, 128, CU_TENSOR_MAP_SWIZZLE_32B); };
+    auto cols64 = [&](CUtensorMap* m, size_t off, int64_t rows) { return make_code_store_map(d, m, ws + off, rows, s / 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B); };
+    if (!load(&h.tm_qX, L.qX_codes, s, l) || !load(&h.tm_qXt[0], L.qXt_codes[0], l, s) || !load(&h.tm_qXt[1], L.qXt_codes[1], l, s) ||
+        !load(&h.tm_qA, L.qA_codes, s, s) || !load(&h.tm_qB, L.qB_codes, s, s) ||
+        !rows32(&h.st_qX, L.qX_codes, l) || !rows32(&h.st_qA, L.qA_codes, s) || !rows32(&h.st_qB, L.qB_codes, s) ||
+        !cols64(&h.st_qXt[0], L.qXt_codes[0], l) || !cols64(&h.st_qXt[1], L.qXt_codes[1], l) ||
+        !cols64(&h.st_qAc, L.qA_codes, s) || !cols64(&h.st_qBc, L.qB_codes, s) ||
+        !make_f32_map(d, &h.tm_A, ws + L.A, s, s, 32) || !make_f32_map(d, &h.tm_X, c->X, xr, xc, 32) ||
+        !(tall ? make_f32_tr_map(d, &h.tm_G, G, c->pl.l0, c->pl.s0) && make_f32_tr_map(d, &h.tm_outT, out, c->pl.l0, c->pl.s0)
+               : make_f32_map(d, &h.tm_G, G, c->pl.s0, c->pl.l0, 32)))
+      return FP4_ERR_CUDA;
+    h.scalars = base.scalars;
+    h.done = &reinterpret_cast<NsHeader*>(ws + L.header)->tiles_done;
+    h.qx_sf = ws + L.qX_scales;
+    for (int i = 0; i < 2; ++i) h.qt_sf[i] = ws + L.qXt_scales[i];
+    h.qa_sf = ws + L.qA_scales; h.qb_sf = ws + L.qB_scales;
+    h.ca = abc[0]; h.cb = abc[1]; h.cc = abc[2];
+    h.tall = tall;
   }
   c->g3_first = c->g3[0];
   c->native_tall = c->pl.tall && pair3;   // (rounded-FP32 storage, bmode 2, never runs in the CTA-pair kernel)
@@ -531,17 +564,41 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
   const NsPlan& pl0 = mats[0].pl;
   const int64_t s = pl0.s, l = pl0.l;
   pdl_select(s * l * count);
+  const bool chain = steps > 0 && chain_group(d, pl0, count, p);
   {
     std::vector<PrologueItem> items((size_t)count);
     for (int i = 0; i < count; ++i) {
       MatrixCtx& c = mats[i];
-      items[(size_t)i] = PrologueItem{c.G, c.X, c.ws, &c.pl, clear_first_status && i == 0, c.store_x0, c.x_rows, c.x_cols,
+      items[(size_t)i] = PrologueItem{c.G, c.X, c.ws, &c.pl, clear_first_status && i == 0, c.store_x0 && !chain, c.x_rows, c.x_cols,
                                       c.hist_top, &c.tm_G};
     }
     if (launch_prologue_group(items.data(), count, steps > 0 || keep, quant_opts(p, 0), status, st) != cudaSuccess)
       return FP4_ERR_CUDA;
   }
-  if (steps > 0) {
+  if (chain) {
+    ChainPack pack;
+    for (int j = 0; j < kChainMax; ++j) {
+      pack.p[j] = mats[j < count ? j : 0].chain;
+      pack.p[j].W = mats[j < count ? j : 0].W;
+    }
+    ChainLaunch a;
+    memset(&a, 0, sizeof(a));
+    a.count = count; a.steps = steps;
+    a.s = (int)s; a.l = (int)l; a.s0 = (int)pl0.s0; a.l0 = (int)pl0.l0;
+    a.clip = pl0.clip; a.keep = keep; a.bf16 = pl0.bf16_mode != 0;
+    a.update = any_update && !keep; a.no_out = upd.no_out; a.upd_decay = upd.decay; a.upd_step = upd.step;
+    a.l_cols = (float)l;
+    a.q = quant_opts(p, 0);
+    a.seed = p->seed;
+    a.ix = pl0.ix;
+    a.status = status;
+    for (int j = 0; j < count; ++j) {
+      // the results of tall matrices and the parameter updates are written there, too, unless operand copies are kept
+      if (!keep) { direct_out[(size_t)j] = mats[j].pl.tall; fused_update[(size_t)j] = 1; }
+    }
+    ProfScope ps(FP4_PROF_G3, st);
+    if (launch_chain(pack, a, d->sms, st) != cudaSuccess) return FP4_ERR_CUDA;
+  } else if (steps > 0) {
     // the problems of the five kinds of launches: G1, G2, G3 reading qXt[0] / qXt[1], the first G3
     std::vector<ProblemPack> packs(5);
     for (int kind = 0; kind < 5; ++kind) {

@@ -685,3 +685,41 @@ def test_bf16_storage_of_shapes_that_pad_to_multiples_of_256(shape):
     assert fp4.fp4_last_device_status(ws) == 0
     want = oracle.root_ns(G, steps=3, store_bf16=True)
     assert rel(out.cpu().numpy(), want) <= TOL_OUT
+
+
+@pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX, FP4_FLAG_STORE_BF16])
+@pytest.mark.parametrize("shape", [(16, 16), (128, 128), (144, 112), (128, 1040), (1040, 256), (1168, 1072), (1280, 1536)])
+def test_iterations_in_one_launch_at_the_edges_of_its_tiles(shape, flags):
+    """Small matrices run all iterations in one cooperative launch with 128 x 64 or 128 x 128 tiles: one tile, one
+    block per 128 rows, partial last tiles, more tiles than SMs (the last two; 1280 x 1536 takes the wide
+    tiles).  The result on a dirty workspace is the oracle's, twice the same."""
+    m, n = shape
+    G = workloads.gradient_like(m, n, seed=m + n)
+    Gd = torch.from_numpy(G).cuda()
+    out = torch.empty_like(Gd)
+    ws = torch.full((fp4.fp4_root_ns_workspace_bytes(m, n, 3, flags),), 0xFF, dtype=torch.uint8, device="cuda")
+    p = fp4.NsParams.make(flags=flags, seed=5)
+    before = fp4.fp4_kernel_launches()
+    fp4.fp4_root_ns(Gd, out, 3, p, ws)
+    assert fp4.fp4_kernel_launches() - before == 7      # prologue 6, iterations 1
+    assert fp4.fp4_last_device_status(ws) == 0
+    first = out.cpu().numpy()
+    pf = bool(flags & FP4_FLAG_RHT)
+    want = oracle.root_ns(G, steps=3, rht=pf, four_six=pf, seed=5, store_bf16=bool(flags & FP4_FLAG_STORE_BF16))
+    assert rel(first, want) <= TOL_OUT, rel(first, want)
+    fp4.fp4_root_ns(Gd, out, 3, p, ws)
+    assert np.array_equal(out.cpu().numpy(), first)
+
+
+def test_iterations_in_one_launch_for_a_group_are_those_of_single_calls():
+    """Fourteen equal shapes, wide and tall, share one launch; a fifteenth makes the group take the other route."""
+    for count in (14, 15):
+        mats = [workloads.gradient_like(*((256, 384) if i % 3 else (384, 256)), seed=40 + i) for i in range(count)]
+        Gs = [torch.from_numpy(g).cuda() for g in mats]
+        outs = [torch.empty_like(g) for g in Gs]
+        ws = torch.empty(fp4.fp4_root_ns_batched_workspace_bytes([g.shape for g in mats], 4), dtype=torch.uint8, device="cuda")
+        fp4.fp4_root_ns_batched(Gs, outs, 4, None, ws)
+        assert fp4.fp4_last_device_status(ws) == 0
+        for g, o in zip(mats, outs):
+            single, _ = run_gpu(g, steps=4)
+            assert np.array_equal(o.cpu().numpy(), single)
