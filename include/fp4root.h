@@ -76,9 +76,8 @@ typedef enum {
  * precision; FP32 is the default): A_k and X_k (k >= 1) are kept in BF16, round to nearest
  * even, which halves the FP32 traffic of the fused epilogues.  The NVFP4 operand copies and the
  * running maxima are still derived from the FP32 values in the epilogue, X_0 stays FP32 and
- * the result is FP32.  When every dimension of the work shape is a multiple of 256 the copies
- * really are 2-byte tensors; otherwise they stay FP32 tensors that hold BF16-rounded values
- * (same results, no traffic saved). */
+ * the result is FP32.  The copies are 2-byte tensors, except in a group small enough to run all
+ * its iterations in one launch, where they are FP32 tensors that hold the rounded values. */
 #define FP4_FLAG_STORE_BF16 8u
 /* With fp4_ns_params.weights: the FP32 result is not written (the parameter update is all the caller
  * wants).  `out` is still required - it is the working copy of X during the iterations of a wide matrix -
@@ -264,7 +263,7 @@ typedef struct {
   int32_t idx_sg_X0;                /* scalars[idx + k] = tensor scale of qX_k      */
   int32_t idx_sg_A0, idx_sg_B0;     /* likewise for qA_k, qB_k                      */
   size_t total;
-  size_t Xh;          /* FP4_FLAG_STORE_BF16 with 2-byte storage: BF16 s x l, X_k (k >= 1); the A
+  size_t Xh;          /* FP4_FLAG_STORE_BF16: BF16 s x l, X_k (k >= 1); the A
                          region then holds A as BF16 s x s.  0 otherwise.                  */
 } fp4_ws_layout;
 fp4_status fp4_root_ns_workspace_layout(int64_t m, int64_t n, int steps, uint32_t flags,

@@ -1,9 +1,11 @@
 // The block-scaled NVFP4 GEMM with the fused Newton-Schulz epilogues (Section 3.4, display
-// equations) for shapes whose dimensions are multiples of 256: a pair of CTAs on two SMs (a
+// equations): a pair of CTAs on two SMs (a
 // cluster of 2) computes one 256 x 256 output tile with tcgen05.mma.cta_group::2.  Each CTA
 // holds 128 rows of the row operand and 128 of the 256 rows of the column operand in its
 // shared memory, so every byte fetched from L2 and every byte the tensor core reads from
-// shared memory feeds twice as many multiply-adds as in the 128 x 128 single-CTA kernel.
+// shared memory feeds twice as many multiply-adds as in a 128 x 128 tile of one CTA.  Dimensions are
+// multiples of 128: of a last tile that sticks out, TMA fills the operands with zeros and the blocks outside the
+// matrix are neither combined nor stored; a last stage of 128 elements of K takes two MMAs instead of four.
 //
 // Per CTA: accumulator 128 lanes x 256 FP32 columns in tensor memory, drained by sixteen
 // epilogue warps that share nothing with one another.  A warp owns the 32 accumulator lanes
@@ -308,7 +310,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
   const bool sym = (MODE == kG1 || MODE == kG2) && args.symmetric != 0;
   const int tiles_per_problem = sym ? args.tiles_n * (args.tiles_n + 1) / 2 : args.tiles_m * args.tiles_n;
   const int num_tiles = tiles_per_problem * args.num_problems;
-  const int num_kb = args.K / BK;
+  const int num_kb = (args.K + BK - 1) / BK;
   constexpr bool HAS_AUX = (MODE == kG2 || MODE == kG3);
   constexpr bool STORE_F32 = (MODE == kPlain || MODE == kG1 || MODE == kG3);
   const bool do_q = (MODE != kPlain) && !UPD && args.write_q;  // the update variant is launched without quantised outputs
@@ -405,8 +407,10 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
           const uint8_t* sf = smem + OFF_SF + st * SF_BYTES;
           const uint64_t adesc = umma_desc(smem_u32(smem + OFF_A + st * OPER_BYTES), OPER_SBO, OPER_SWIZZLE);
           const uint64_t bdesc = umma_desc(smem_u32(smem + OFF_B + st * OPER_BYTES), OPER_SBO, OPER_SWIZZLE);
+          const bool half_stage = (kb + 1) * BK > args.K;   // K is a multiple of 128
 #pragma unroll
           for (int k = 0; k < KSTEPS; ++k) {
+            if (k == KSTEPS / 2 && half_stage) break;
             tc_cp_sf2(sf_t, umma_desc(smem_u32(sf + k * 512), 128, 0));
             tc_cp_sf2(sf_t + 4, umma_desc(smem_u32(sf + SF_ATOMS + k * 512), 128, 0));
             tc_cp_sf2(sf_t + 8, umma_desc(smem_u32(sf + 2 * SF_ATOMS + k * 512), 128, 0));
@@ -434,7 +438,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         for (int h = 0; h < 2; ++h) {
           const int hcol = (seq & 1) ? h : 1 - h;          // which 128 columns of the tile this half holds
           const int bj = tj * 2 + hcol;
-          const bool below = sym && bj < bi;
+          const bool below = (sym && bj < bi) || bi >= args.blocks_m || bj >= args.blocks_n;
           const bool mirror = !below && (MODE == kG3 || (sym && bi != bj));
           wait_or_abort(&bars->half_done[h], seq & 1, abort_flag);
           if (!below) {
@@ -488,7 +492,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
     // an FP32 copy of X0 nor a final transpose pass is needed (per-problem flags aux_tr / out_tr).
     constexpr bool TR = (MODE == kG3);
     const bool auxh = BH && HAS_AUX && args.aux_h != 0;                               // the combined tile is BF16
-    const bool hout = BH && STORE_F32 && MODE != kPlain && args.out_h == 1;           // the result is stored as BF16
+    const bool hout = BH && STORE_F32 && MODE != kPlain && args.out_h != 0;           // the result is stored as BF16
 
     float scale = 0.0f, sg_out = 1.0f, inv_sg = 1.0f;
     float ca = 0.0f, cb = 0.0f, cc = 0.0f;
@@ -531,7 +535,11 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
       const int bi_ = q.ti * 2 + (int)rank;
       q.x64 = q.tj * PN + cgx * (TEAM_CHUNKS * CHUNK);
       q.y32 = bi_ * BM + quad * 32;
-      q.below = sym && (q.tj * 2 + (cgx >> 1)) < bi_;              // redundant block of a diagonal tile
+      const int bj_ = q.tj * 2 + (cgx >> 1);
+      // A redundant block of a diagonal tile, or one outside the matrix.  (Blocks outside run through G3's epilogue as
+      // zeros and TMA drops what they store: the path that skips a block costs G3 registers, 9 % of its time with
+      // BF16 storage.)
+      q.below = sym && (bj_ < bi_ || bi_ >= args.blocks_m || bj_ >= args.blocks_n);
       return q;
     };
 
@@ -957,14 +965,16 @@ int gemm_pair_stage_k(GemmMode mode) {
   }
 }
 
-// `launch` carries tile counts in 128-blocks; all of M, N, K must be multiples of 256.
+// `launch` carries tile counts in 128-blocks; M, N and K are multiples of 128.
 cudaError_t launch_gemm_pair(GemmMode mode, const ProblemPack& pack, const GemmLaunch& launch, int sms,
                              cudaStream_t st) {
-  if ((launch.tiles_m & 1) || (launch.tiles_n & 1) || (launch.K % 256)) return cudaErrorInvalidValue;
+  if (launch.K % 128) return cudaErrorInvalidValue;
   if (launch.num_problems < 1 || launch.num_problems > kPackMax) return cudaErrorInvalidValue;
   GemmLaunch L = launch;
-  L.tiles_m = launch.tiles_m / 2;
-  L.tiles_n = launch.tiles_n / 2;
+  L.blocks_m = launch.tiles_m;
+  L.blocks_n = launch.tiles_n;
+  L.tiles_m = (launch.tiles_m + 1) / 2;
+  L.tiles_n = (launch.tiles_n + 1) / 2;
   const bool pf = launch.q.rht || launch.q.four_six;
   const bool bh = launch.aux_h != 0 || launch.out_h != 0;
 #define FP4_PAIR_CASE(M)                                                                \

@@ -1,4 +1,4 @@
-// Device helpers shared by the two GEMM kernels (one CTA per tile / a pair of CTAs per tile).
+// Device helpers shared by the kernels that run the products.
 #pragma once
 
 #include "fp4_kernels.h"
@@ -11,31 +11,9 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
   return t;
 }
 
-// Wait on an mbarrier phase for at most limit_ns; false on give-up (own time-out or another
-// thread's abort flag).
-static __device__ __noinline__ bool wait_limited(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag,
-                                                 uint64_t limit_ns) {
-  const uint64_t t0 = globaltimer_ns();
-  for (;;) {
-    for (int i = 0; i < 256; ++i)
-      if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (globaltimer_ns() - t0 > limit_ns) {
-      *abort_flag = 1;
-      return false;
-    }
-  }
-}
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // two seconds
-static __device__ __forceinline__ bool wait_slow(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag) {
-  return wait_limited(bar, parity, abort_flag, kWaitLimitNs);
-}
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag) {
-  if (mbar_try_wait(bar, parity)) return true;
-  return wait_slow(bar, parity, abort_flag);
-}
 
-// The same wait for callers that do not branch on the outcome: when a wait gives up (its own
+// Bounded wait on an mbarrier phase.  When a wait gives up (its own
 // time-out, or another thread of the CTA gave up before) the abort flag is set and every later
 // wait of the CTA falls through at once, so the kernel runs to its end on whatever data it has
 // and the host reads FP4_ERR_DEVICE_TIMEOUT from the status word.  The polls carry a suspend-time
@@ -50,13 +28,14 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar_addr, uint32_t p
       : "memory");
   return ok != 0;
 }
-static __device__ __noinline__ void wait_slow_abort(uint32_t bar_addr, uint32_t parity, volatile uint32_t* abort_flag) {
+static __device__ __noinline__ void wait_limited_abort(uint32_t bar_addr, uint32_t parity, volatile uint32_t* abort_flag,
+                                                       uint64_t limit_ns) {
   const uint64_t t0 = globaltimer_ns();
   for (;;) {
     if (*abort_flag) return;
     for (int i = 0; i < 64; ++i)
       if (mbar_try_wait_hint(bar_addr, parity, 4000u)) return;
-    if (globaltimer_ns() - t0 > kWaitLimitNs) {
+    if (globaltimer_ns() - t0 > limit_ns) {
       *abort_flag = 1;
       return;
     }
@@ -70,7 +49,7 @@ __device__ __forceinline__ void wait_or_abort(uint32_t bar_addr, uint32_t parity
       : "=r"(ok)
       : "r"(bar_addr), "r"(parity)
       : "memory");
-  if (!ok) wait_slow_abort(bar_addr, parity, abort_flag);
+  if (!ok) wait_limited_abort(bar_addr, parity, abort_flag, kWaitLimitNs);
 }
 __device__ __forceinline__ void wait_or_abort(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag) {
   wait_or_abort(smem_u32(bar), parity, abort_flag);
@@ -91,10 +70,6 @@ __device__ __forceinline__ void decode_tile(int t, const GemmLaunch& L, int tile
     ti = row;
     tj = row + rem;
   }
-}
-__device__ __forceinline__ void decode_tile(int t, const GemmLaunch& L, int tiles_per_problem, int& p, int& ti,
-                                            int& tj) {
-  decode_tile(t, L, tiles_per_problem, p, ti, tj, L.symmetric != 0);
 }
 
 // Per-call scalars of an epilogue: the factor that turns the accumulator into the

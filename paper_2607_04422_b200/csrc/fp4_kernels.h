@@ -44,8 +44,8 @@ struct NsPlan {
   int64_t s, l;      // work shape: s0, l0 rounded up to multiples of 128 (zero padding)
   int tall;
   int clip;
-  int bf16_mode;     // 0: FP32 storage of X_k / A_k; 1: BF16 tensors; 2: FP32 tensors holding BF16-rounded values
-  size_t off_Xh;     // bf16_mode 1: BF16 X in the workspace
+  int bf16;          // X_k / A_k are kept as BF16 tensors
+  size_t off_Xh;     // bf16: BF16 X in the workspace
   int64_t clip_rank;
   float eps;
   int sms;
@@ -63,31 +63,26 @@ enum GemmMode : int {
 };
 
 // One matrix product of a launch.  A launch runs the same stage for a group of matrices
-// of one shape; the problems of a group sit in an array in device memory (or, for a single
-// problem, in the kernel's parameter space).
+// of one shape.
 struct alignas(64) GemmProblem {
   CUtensorMap tmA, tmB;      // NVFP4 codes of the row and the column operand
-  CUtensorMap tmAux, tmOut;  // FP32 tile combined in the epilogue / FP32 result (box: 16 columns x 128 rows in
-                             // the single-CTA kernel, 16 x 32 - one epilogue warp's block - in the CTA-pair kernel)
-  CUtensorMap tmSfa, tmSfb;  // scale atoms of the two operands as 2-D maps (CTA-pair kernel)
+  CUtensorMap tmAux, tmOut;  // FP32 tile combined in the epilogue / FP32 result (box: 16 columns x 32 rows, one
+                             // epilogue warp's block)
+  CUtensorMap tmSfa, tmSfb;  // scale atoms of the two operands as 2-D maps
   CUtensorMap tmH;           // BF16 storage: the 2-byte tensor this stage reads its tile from and / or stores its
                              // result to (A for G1 / G2, X for G3); box 16 columns x 32 rows, no swizzle
-  CUtensorMap tmRq, tmCq;    // CTA-pair kernel: byte maps over rq_codes (box 32 bytes x 32 rows: one warp's part of a
-                             // tile) and cq_codes (box 64 bytes x 128 rows, 64-byte swizzle: a CTA's 128 rows of
+  CUtensorMap tmRq, tmCq;    // byte maps over the row-quantised codes (box 32 bytes x 32 rows: one warp's part of a
+                             // tile) and the column-quantised codes (box 64 bytes x 128 rows, 64-byte swizzle: a CTA's 128 rows of
                              // 128 tile columns) for the stores of the quantised outputs
-  const uint8_t* sfa;        // scale atoms of the row operand
-  const uint8_t* sfb;        // scale atoms of the column operand
   float* scalars;            // workspace scalars of this matrix (device)
-  uint8_t* rq_codes; uint8_t* rq_sf;  // quantised output, blocks along the tile's columns
-  uint8_t* cq_codes; uint8_t* cq_sf;  // quantised output, blocks along the tile's rows
+  uint8_t* rq_sf;            // scales of the quantised output, blocks along the tile's columns
+  uint8_t* cq_sf;            // likewise, blocks along the tile's rows
   float ca, cb, cc;          // coefficients
   float sg_a, sg_b;          // kPlain: tensor scales from the host
   int aux_raw;               // kG3: tmAux maps the raw input G; X0 = clamp(G, tau) * inv is formed on the fly
-  int aux_tr;                // kG3, CTA-pair kernel: tmAux maps a matrix stored as the transpose of the tile grid (box = 32 x 16)
-  int out_tr;                // kG3, CTA-pair kernel: so does tmOut (the caller's result of a tall input)
+  int aux_tr;                // kG3: tmAux maps a matrix stored as the transpose of the tile grid (box = 32 x 16)
+  int out_tr;                // kG3: so does tmOut (the caller's result of a tall input)
   int out_rows, out_cols;    // extent of the matrix behind tmOut (chunks that start outside it are not stored)
-  void* out_direct;          // out_h == 2: the FP32 tensor the epilogue warps store the rounded result to
-  int64_t out_direct_ld;     //   (row-major, leading dimension in elements)
   uint16_t* W;               // kG3 with launch.update: the BF16 parameter (same shape and orientation as the
   int64_t W_ld;              //   result, row-major, leading dimension in elements) updated with the result; or null
 };
@@ -102,7 +97,8 @@ static_assert(sizeof(ProblemPack) + 256 <= 32764, "kernel parameter space");
 struct GemmLaunch {
   int num_problems;
   int K;               // contraction length in elements (multiple of 128)
-  int tiles_m, tiles_n;
+  int tiles_m, tiles_n;        // callers: in blocks of 128; inside the kernel: 256 x 256 tiles, rounded up
+  int blocks_m, blocks_n;      // extent in blocks of 128 (set by launch_gemm_pair)
   int symmetric;       // only tiles with tile_n >= tile_m; mirrored quantised output
   int iter;            // Newton-Schulz iteration index k
   int write_q;         // emit the quantised outputs
@@ -111,13 +107,12 @@ struct GemmLaunch {
   QuantOpts q;         // how this stage's output is quantised (q.widen = 1 in the base mode)
   int clip;            // kG3 on a problem with aux_raw: whether tau applies
   int aux_h;           // the combined tile is read from tmH (BF16)
-  int out_h;           // 0: FP32 result by TMA store; 1: rounded to BF16, staged and stored through tmH (CTA-pair
-                       // kernel); 2: rounded to BF16, stored as FP32 by the epilogue warps (single-CTA kernel)
-  int update;          // kG3, CTA-pair kernel, last iteration: Root's parameter update W <- BF16(W * upd_decay -
+  int out_h;           // 0: FP32 result by TMA store; 1: rounded to BF16, staged and stored through tmH
+  int update;          // kG3, last iteration: Root's parameter update W <- BF16(W * upd_decay -
   float upd_decay;     //   upd_step * X+) on every problem whose W is set, in the epilogue
   float upd_step;
   int no_out;          // with update: the FP32 result is not stored
-  int dry_operands;    // kPlain, CTA-pair kernel: measurement of the tensor-pipe ceiling - no operand is fetched
+  int dry_operands;    // kPlain: measurement of the tensor-pipe ceiling - no operand is fetched
   NsScalarIdx ix;
   uint32_t* status;
 };
@@ -242,13 +237,10 @@ cudaError_t launch_transpose_out(const float* X, int64_t s, int64_t l, float* ou
 cudaError_t launch_param_update(const float* O, int64_t n, const ParamUpdate& upd, int sms, cudaStream_t st);
 cudaError_t prologue_set_attributes();
 
-cudaError_t gemm_set_attributes();
 cudaError_t gemm_pair_set_attributes();
 // pack: the launch.num_problems (<= kPackMax) problems of the launch
 cudaError_t launch_gemm_pair(GemmMode mode, const ProblemPack& pack, const GemmLaunch& launch, int sms,
                              cudaStream_t st);
-int gemm_stage_k();  // elements of K per operand stage (the codes maps' box is this / 2 bytes wide)
 int gemm_pair_stage_k(GemmMode mode);  // the same for a mode of the CTA-pair kernel
-cudaError_t launch_gemm(GemmMode mode, const ProblemPack& pack, const GemmLaunch& launch, int sms, cudaStream_t st);
 
 }  // namespace fp4

@@ -82,7 +82,7 @@ const DeviceInfo* device_info() {
     d.status = FP4_ERR_CUDA; d.ready = true; return &d;
   }
   d.encode = reinterpret_cast<EncodeTiledFn>(fn);
-  if (gemm_set_attributes() != cudaSuccess || gemm_pair_set_attributes() != cudaSuccess ||
+  if (gemm_pair_set_attributes() != cudaSuccess ||
       chain_set_attributes() != cudaSuccess ||
       prologue_set_attributes() != cudaSuccess)
     d.status = FP4_ERR_CUDA;
@@ -115,12 +115,11 @@ bool make_codes_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int6
                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-// 2-D map over a row-major FP32 matrix: box = 16 columns x box_rows rows (128: a chunk of the single-CTA
-// kernel; 32: one epilogue warp's block in the CTA-pair kernel), 64-byte swizzle.
-bool make_f32_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int box_rows) {
+// 2-D map over a row-major FP32 matrix: box = 16 columns x 32 rows, one epilogue warp's block, 64-byte swizzle.
+bool make_f32_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int64_t rows, int64_t cols) {
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
-  cuuint32_t box[2] = {16, (cuuint32_t)box_rows};
+  cuuint32_t box[2] = {16, 32};
   cuuint32_t estr[2] = {1, 1};
   return d->encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -181,7 +180,6 @@ constexpr int kDefaultMaxGroup = kPackMax;
 // 2-D map over the scale atoms of a rows x K operand: one map row per 128-row block, 64-bit
 // elements, box = the atoms of one operand stage (`stage_k` elements of 8 bytes: 1 or 2 KB), no swizzle.
 bool make_sf_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int64_t rows, int64_t K, int stage_k) {
-  if (K < 256) { memset(tm, 0, sizeof(*tm)); return true; }   // never used by the CTA-pair kernel
   cuuint64_t dims[2] = {(cuuint64_t)(K / 64) * 64, (cuuint64_t)(rows / 128)};
   cuuint64_t strides[1] = {(cuuint64_t)(K / 64) * 512};
   cuuint32_t box[2] = {(cuuint32_t)stage_k, 1};
@@ -189,22 +187,6 @@ bool make_sf_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int64_t
   return d->encode(tm, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// The CTA-pair kernel takes every product whose dimensions are all multiples of 256 (tile counts in 128-blocks).
-// The descriptors of a problem are built for the kernel that runs it (pair_kernel decides both).
-bool pair_kernel(int64_t tiles_m, int64_t tiles_n, int64_t K, int sms, bool force_single = false) {
-#ifndef FP4_DISABLE_PAIR
-  return !force_single && !(tiles_m & 1) && !(tiles_n & 1) && K % 256 == 0 && sms >= 2;
-#else
-  (void)tiles_m; (void)tiles_n; (void)K; (void)sms; (void)force_single;
-  return false;
-#endif
-}
-cudaError_t launch_gemm_auto(GemmMode mode, const ProblemPack& pack, const GemmLaunch& L, int sms, cudaStream_t st,
-                             bool force_single = false) {
-  if (pair_kernel(L.tiles_m, L.tiles_n, L.K, sms, force_single)) return launch_gemm_pair(mode, pack, L, sms, st);
-  return launch_gemm(mode, pack, L, sms, st);
 }
 
 void default_params(fp4_ns_params* p) {
@@ -264,12 +246,7 @@ fp4_status make_plan(int64_t m, int64_t n, int steps, const fp4_ns_params* p, in
   // maximum; since the dimensions are multiples of 16 no block mixes data and padding.
   pl->s = pad128(pl->s0);
   pl->l = pad128(pl->l0);
-  // BF16 storage: 2-byte tensors when all three stages run in the CTA-pair kernel, else FP32
-  // tensors that hold rounded values (and all stages in the single-CTA kernel)
-  if (p->flags & FP4_FLAG_STORE_BF16) pl->bf16_mode = (pl->s % 256 == 0 && pl->l % 256 == 0) ? 1 : 2;
-#ifdef FP4_DISABLE_PAIR
-  if (pl->bf16_mode == 1) pl->bf16_mode = 2;
-#endif
+  pl->bf16 = (p->flags & FP4_FLAG_STORE_BF16) != 0;
   const int64_t s = pl->s, l = pl->l;
   pl->clip = p->clip_quantile > 0.0f && p->clip_quantile < 1.0f;
   pl->clip_rank = pl->clip ? quantile_rank(m * n, p->clip_quantile) : 0;
@@ -305,7 +282,7 @@ fp4_status make_plan(int64_t m, int64_t n, int steps, const fp4_ns_params* p, in
   L.qB_codes = off; off += align_up((size_t)s * s / 2, 1024);
   L.qB_scales = off; off += align_up((size_t)s * s / 16, 1024);
   L.Xh = 0;
-  if (pl->bf16_mode == 1) { pl->off_Xh = off; L.Xh = off; off += align_up((size_t)s * l * 2, 1024); }
+  if (pl->bf16) { pl->off_Xh = off; L.Xh = off; off += align_up((size_t)s * l * 2, 1024); }
   L.idx_tau = ix.tau; L.idx_nu = ix.nu; L.idx_inv = ix.inv;
   L.idx_amax_X0 = ix.amax_X0; L.idx_amax_A0 = ix.amax_A0;
   L.idx_sg_X0 = ix.sg_X0; L.idx_sg_A0 = ix.sg_A0; L.idx_sg_B0 = ix.sg_B0;
@@ -327,10 +304,7 @@ struct MatrixCtx {
   uint32_t* hist_top;         // the caller's first-pass histogram of G, or null
   uint16_t* W;                // the BF16 parameter that takes Root's update in this call, or null
   CUtensorMap tm_G;           // the caller's matrix for the operand preparation (tiles of 128 x 128)
-  // A tall input in the CTA-pair kernel: the first G3 stage reads the caller's matrix and the last one
-  // writes the caller's result through transposing boxes.
-  bool native_tall;
-  CUtensorMap tm_outT;
+  CUtensorMap tm_outT;        // tall: the caller's result through transposing boxes
   ChainProblem chain;         // for a run of all iterations in one launch
 };
 
@@ -341,11 +315,10 @@ struct MatrixCtx {
 // 1024 x 1024 169 / 287 us, 2048 x 2048 327 / 339 us.  (Not for inspection of BF16-stored intermediates: there A and X
 // stay FP32 tensors with rounded values.)
 bool chain_group(const DeviceInfo* d, const NsPlan& pl, int count, const fp4_ns_params* p) {
-  if (count > kChainMax || (pl.bf16_mode == 1 && (p->flags & FP4_FLAG_KEEP_OPERANDS))) return false;
-  const bool pair = pl.s % 256 == 0 && pl.l % 256 == 0;
+  if (count > kChainMax || (pl.bf16 && (p->flags & FP4_FLAG_KEEP_OPERANDS))) return false;
   const bool opts = (p->flags & (FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)) != 0;
   const int64_t elements = pl.s * pl.l * count;
-  const int64_t limit = (pair && !opts) ? (int64_t)7 << 19 : (int64_t)9 << 19;
+  const int64_t limit = opts ? (int64_t)9 << 19 : (int64_t)7 << 19;
   return elements <= limit && elements / (128 * 64) <= (int64_t)d->sms * kChainTiles;
 }
 
@@ -363,21 +336,15 @@ fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t
   // lies outside with zeros on loads and drops it on stores)
   const int64_t xr = c->pl.tall ? s : c->pl.s0, xc = c->pl.tall ? l : c->pl.l0;
   c->x_rows = xr; c->x_cols = xc;
-  c->store_x0 = c->pl.tall || steps == 0;
-  c->native_tall = false;
+  c->store_x0 = steps == 0;   // else the first G3 stage reads the caller's matrix
   if (!make_f32_tile_map(d, &c->tm_G, G, m, n)) return FP4_ERR_CUDA;
   if (steps == 0) return FP4_OK;
   float abc[3] = {p->a, p->b, p->c};
   if (std::isnan(p->a)) coeffs(m, n, abc);
-  // which kernel runs each stage (rounded-FP32 storage is implemented by the single-CTA kernel only)
-  const bool fs = c->pl.bf16_mode == 2;
-  const bool pair1 = pair_kernel(s / 128, s / 128, l, d->sms, fs), pair2 = pair_kernel(s / 128, s / 128, s, d->sms, fs),
-             pair3 = pair_kernel(s / 128, l / 128, s, d->sms, fs);
-  CUtensorMap tm_qX, tm_qXt[2], tm_qA, tm_qB, tm_A1, tm_A2, tm_X;
+  CUtensorMap tm_qX, tm_qXt[2], tm_qA, tm_qB, tm_A, tm_X;
   CUtensorMap sf_qX, sf_qXt[2], sf_qA, sf_qB;
   // every operand is read by exactly one stage: its descriptors take that stage's depth in K
-  const int k1 = pair1 ? gemm_pair_stage_k(kG1) : gemm_stage_k(), k2 = pair2 ? gemm_pair_stage_k(kG2) : gemm_stage_k(),
-            k3 = pair3 ? gemm_pair_stage_k(kG3) : gemm_stage_k();
+  const int k1 = gemm_pair_stage_k(kG1), k2 = gemm_pair_stage_k(kG2), k3 = gemm_pair_stage_k(kG3);
   bool ok = make_sf_map(d, &sf_qX, ws + L.qX_scales, s, l, k1) && make_sf_map(d, &sf_qXt[0], ws + L.qXt_scales[0], l, s, k3) &&
             make_sf_map(d, &sf_qXt[1], ws + L.qXt_scales[1], l, s, k3) && make_sf_map(d, &sf_qA, ws + L.qA_scales, s, s, k2) &&
             make_sf_map(d, &sf_qB, ws + L.qB_scales, s, s, k3) &&
@@ -386,9 +353,7 @@ fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t
             make_codes_map(d, &tm_qXt[1], ws + L.qXt_codes[1], l, s / 2, k3) &&
             make_codes_map(d, &tm_qA, ws + L.qA_codes, s, s / 2, k2) &&
             make_codes_map(d, &tm_qB, ws + L.qB_codes, s, s / 2, k3) &&
-            make_f32_map(d, &tm_A1, ws + L.A, s, s, pair1 ? 32 : 128) &&
-            make_f32_map(d, &tm_A2, ws + L.A, s, s, pair2 ? 32 : 128) &&
-            make_f32_map(d, &tm_X, c->X, xr, xc, pair3 ? 32 : 128);
+            make_f32_map(d, &tm_A, ws + L.A, s, s) && make_f32_map(d, &tm_X, c->X, xr, xc);
   if (!ok) return FP4_ERR_CUDA;
   // stores of the quantised outputs by the CTA-pair kernel's epilogue warps
   CUtensorMap st_qA_r, st_qA_c, st_qB_r, st_qB_c, st_qX_r, st_qXt_c[2];
@@ -405,39 +370,34 @@ fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t
   base.scalars = reinterpret_cast<float*>(ws + L.scalars);
   base.ca = abc[0]; base.cb = abc[1]; base.cc = abc[2];
   base.out_rows = (int)s; base.out_cols = (int)s;
-  const int bmode = c->pl.bf16_mode;
+  const bool bf16 = c->pl.bf16 != 0;
   CUtensorMap tm_Ah, tm_Xh;
-  uint8_t* Xh = bmode == 1 ? ws + c->pl.off_Xh : nullptr;
-  if (bmode == 1 && (!make_bf16_map(d, &tm_Ah, ws + L.A, s, s) || !make_bf16_map(d, &tm_Xh, Xh, s, l))) return FP4_ERR_CUDA;
+  uint8_t* Xh = bf16 ? ws + c->pl.off_Xh : nullptr;
+  if (bf16 && (!make_bf16_map(d, &tm_Ah, ws + L.A, s, s) || !make_bf16_map(d, &tm_Xh, Xh, s, l))) return FP4_ERR_CUDA;
   // G1: A = qX qX^T (upper-triangle tiles), qA in both triangles
   c->g1 = base;
-  c->g1.tmA = c->g1.tmB = tm_qX; c->g1.tmAux = c->g1.tmOut = tm_A1;
+  c->g1.tmA = c->g1.tmB = tm_qX; c->g1.tmAux = c->g1.tmOut = tm_A;
   c->g1.tmRq = st_qA_r; c->g1.tmCq = st_qA_c;
   c->g1.tmSfa = c->g1.tmSfb = sf_qX;
-  c->g1.sfa = c->g1.sfb = ws + L.qX_scales;
-  c->g1.rq_codes = c->g1.cq_codes = ws + L.qA_codes; c->g1.rq_sf = c->g1.cq_sf = ws + L.qA_scales;
-  if (bmode == 1) c->g1.tmH = tm_Ah;                                           // A as a BF16 tensor
-  if (bmode == 2) { c->g1.out_direct = ws + L.A; c->g1.out_direct_ld = s; }   // A as rounded FP32
+  c->g1.rq_sf = c->g1.cq_sf = ws + L.qA_scales;
+  if (bf16) c->g1.tmH = tm_Ah;                                           // A as a BF16 tensor
   // G2: B = bA + c qA qA^T, qB in both triangles
   c->g2 = base;
-  c->g2.tmA = c->g2.tmB = tm_qA; c->g2.tmAux = c->g2.tmOut = tm_A2;
+  c->g2.tmA = c->g2.tmB = tm_qA; c->g2.tmAux = c->g2.tmOut = tm_A;
   c->g2.tmRq = st_qB_r; c->g2.tmCq = st_qB_c;
   c->g2.tmSfa = c->g2.tmSfb = sf_qA;
-  c->g2.sfa = c->g2.sfb = ws + L.qA_scales;
-  if (bmode == 1) c->g2.tmH = tm_Ah;
-  c->g2.rq_codes = c->g2.cq_codes = ws + L.qB_codes; c->g2.rq_sf = c->g2.cq_sf = ws + L.qB_scales;
+  if (bf16) c->g2.tmH = tm_Ah;
+  c->g2.rq_sf = c->g2.cq_sf = ws + L.qB_scales;
   // G3: X+ = aX + qB qXt^T in place on X; new operand copies
   for (int cur = 0; cur < 2; ++cur) {
     GemmProblem& g = c->g3[cur];
     g = base;
     g.tmA = tm_qB; g.tmB = tm_qXt[cur]; g.tmAux = g.tmOut = tm_X;
     g.out_rows = (int)xr; g.out_cols = (int)xc;
-    if (bmode == 1) g.tmH = tm_Xh;
-    if (bmode == 2) { g.out_direct = c->X; g.out_direct_ld = xc; }
+    if (bf16) g.tmH = tm_Xh;
     g.tmSfa = sf_qB; g.tmSfb = sf_qXt[cur];
-    g.sfa = ws + L.qB_scales; g.sfb = ws + L.qXt_scales[cur];
-    g.rq_codes = ws + L.qX_codes; g.rq_sf = ws + L.qX_scales;
-    g.cq_codes = ws + L.qXt_codes[cur ^ 1]; g.cq_sf = ws + L.qXt_scales[cur ^ 1];
+    g.rq_sf = ws + L.qX_scales;
+    g.cq_sf = ws + L.qXt_scales[cur ^ 1];
     g.tmRq = st_qX_r; g.tmCq = st_qXt_c[cur ^ 1];
   }
   {
@@ -452,9 +412,9 @@ fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t
         !rows32(&h.st_qX, L.qX_codes, l) || !rows32(&h.st_qA, L.qA_codes, s) || !rows32(&h.st_qB, L.qB_codes, s) ||
         !cols64(&h.st_qXt[0], L.qXt_codes[0], l) || !cols64(&h.st_qXt[1], L.qXt_codes[1], l) ||
         !cols64(&h.st_qAc, L.qA_codes, s) || !cols64(&h.st_qBc, L.qB_codes, s) ||
-        !make_f32_map(d, &h.tm_A, ws + L.A, s, s, 32) || !make_f32_map(d, &h.tm_X, c->X, xr, xc, 32) ||
+        !make_f32_map(d, &h.tm_A, ws + L.A, s, s) || !make_f32_map(d, &h.tm_X, c->X, xr, xc) ||
         !(tall ? make_f32_tr_map(d, &h.tm_G, G, c->pl.l0, c->pl.s0) && make_f32_tr_map(d, &h.tm_outT, out, c->pl.l0, c->pl.s0)
-               : make_f32_map(d, &h.tm_G, G, c->pl.s0, c->pl.l0, 32)))
+               : make_f32_map(d, &h.tm_G, G, c->pl.s0, c->pl.l0)))
       return FP4_ERR_CUDA;
     h.scalars = base.scalars;
     h.done = &reinterpret_cast<NsHeader*>(ws + L.header)->tiles_done;
@@ -465,19 +425,17 @@ fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t
     h.tall = tall;
   }
   c->g3_first = c->g3[0];
-  c->native_tall = c->pl.tall && pair3;   // (rounded-FP32 storage, bmode 2, never runs in the CTA-pair kernel)
-  if (c->native_tall) {
+  if (c->pl.tall) {
     // the caller's matrices are l0 x s0
     CUtensorMap tm_Gt;
     if (!make_f32_tr_map(d, &tm_Gt, G, c->pl.l0, c->pl.s0) || !make_f32_tr_map(d, &c->tm_outT, out, c->pl.l0, c->pl.s0))
       return FP4_ERR_CUDA;
-    c->store_x0 = false;
     c->g3_first.tmAux = tm_Gt;
     c->g3_first.aux_raw = 1;
     c->g3_first.aux_tr = 1;
-  } else if (!c->store_x0) {
+  } else {
     CUtensorMap tm_G;
-    if (!make_f32_map(d, &tm_G, G, c->pl.s0, c->pl.l0, pair3 ? 32 : 128)) return FP4_ERR_CUDA;
+    if (!make_f32_map(d, &tm_G, G, c->pl.s0, c->pl.l0)) return FP4_ERR_CUDA;
     c->g3_first.tmAux = tm_G;
     c->g3_first.aux_raw = 1;
   }
@@ -560,7 +518,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
   std::vector<char> direct_out((size_t)count, 0);
   bool any_direct = false;
   for (int i = 0; i < count; ++i)
-    if (steps > 0 && mats[i].native_tall && !keep && !any_update) { direct_out[(size_t)i] = 1; any_direct = true; }
+    if (steps > 0 && mats[i].pl.tall && !keep && !any_update) { direct_out[(size_t)i] = 1; any_direct = true; }
   const NsPlan& pl0 = mats[0].pl;
   const int64_t s = pl0.s, l = pl0.l;
   pdl_select(s * l * count);
@@ -569,7 +527,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     std::vector<PrologueItem> items((size_t)count);
     for (int i = 0; i < count; ++i) {
       MatrixCtx& c = mats[i];
-      items[(size_t)i] = PrologueItem{c.G, c.X, c.ws, &c.pl, clear_first_status && i == 0, c.store_x0 && !chain, c.x_rows, c.x_cols,
+      items[(size_t)i] = PrologueItem{c.G, c.X, c.ws, &c.pl, clear_first_status && i == 0, c.store_x0, c.x_rows, c.x_cols,
                                       c.hist_top, &c.tm_G};
     }
     if (launch_prologue_group(items.data(), count, steps > 0 || keep, quant_opts(p, 0), status, st) != cudaSuccess)
@@ -585,7 +543,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     memset(&a, 0, sizeof(a));
     a.count = count; a.steps = steps;
     a.s = (int)s; a.l = (int)l; a.s0 = (int)pl0.s0; a.l0 = (int)pl0.l0;
-    a.clip = pl0.clip; a.keep = keep; a.bf16 = pl0.bf16_mode != 0;
+    a.clip = pl0.clip; a.keep = keep; a.bf16 = pl0.bf16;
     a.update = any_update && !keep; a.no_out = upd.no_out; a.upd_decay = upd.decay; a.upd_step = upd.step;
     a.l_cols = (float)l;
     a.q = quant_opts(p, 0);
@@ -607,11 +565,10 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
         packs[(size_t)kind].p[j] = kind == 0 ? c.g1 : kind == 1 ? c.g2 : kind == 4 ? c.g3_first : c.g3[kind - 2];
       }
     }
-    // Root's parameter update: fused into the last G3 stage where the CTA-pair kernel runs it on a
-    // matrix in the caller's orientation and no operand copies are wanted from that stage; into the
-    // final transpose for a tall matrix; a separate elementwise pass otherwise (below).
-    const bool g3_pair = pair_kernel(s / 128, l / 128, s, d->sms, pl0.bf16_mode == 2);
-    if (g3_pair && !keep) {
+    // Root's parameter update: fused into the last G3 stage of a matrix in the caller's orientation when no
+    // operand copies are wanted from that stage; into the final transpose for a tall matrix; a separate
+    // elementwise pass otherwise (below).
+    if (!keep) {
       for (int kind = 2; kind < 5; ++kind)
         for (int j = 0; j < count; ++j)
           if (mats[j].W && !mats[j].pl.tall) {
@@ -627,8 +584,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     base.l_cols = (float)l;
     base.status = status;
     base.clip = pl0.clip;
-    const int bmode = pl0.bf16_mode;
-    const bool fs = bmode == 2;  // rounded-FP32 storage is implemented by the single-CTA kernel only
+    const int bf16 = pl0.bf16;
     for (int k = 0; k < steps; ++k) {
       const int cur = k & 1;
       const bool last = (k == steps - 1);
@@ -636,19 +592,19 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       L1.iter = k; L1.K = (int)l; L1.tiles_m = L1.tiles_n = (int)(s / 128); L1.symmetric = 1;
       L1.rq_K = L1.cq_K = (int)s; L1.write_q = 1;
       L1.q = quant_opts(p, 2 * (uint64_t)k + 1);  // qA_k
-      L1.out_h = bmode;
+      L1.out_h = bf16;
       {
         ProfScope ps(FP4_PROF_G1, st);
-        if (launch_gemm_auto(kG1, packs[0], L1, d->sms, st, fs) != cudaSuccess)
+        if (launch_gemm_pair(kG1, packs[0], L1, d->sms, st) != cudaSuccess)
           return FP4_ERR_CUDA;
       }
       GemmLaunch L2 = L1;
       L2.K = (int)s;
       L2.q = quant_opts(p, 2 * (uint64_t)k);      // qB_k meets qX_k^{16x1}
-      L2.out_h = 0; L2.aux_h = bmode == 1;
+      L2.out_h = 0; L2.aux_h = bf16;
       {
         ProfScope ps(FP4_PROF_G2, st);
-        if (launch_gemm_auto(kG2, packs[1], L2, d->sms, st, fs) != cudaSuccess)
+        if (launch_gemm_pair(kG2, packs[1], L2, d->sms, st) != cudaSuccess)
           return FP4_ERR_CUDA;
       }
       GemmLaunch L3 = base;
@@ -656,9 +612,9 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       L3.rq_K = (int)l; L3.cq_K = (int)s;
       L3.write_q = (!last || keep) ? 1 : 0;
       L3.q = quant_opts(p, 2 * (uint64_t)k + 2);  // both copies of X_{k+1}
-      L3.aux_h = (bmode == 1 && k > 0) ? 1 : 0;   // X_0 is FP32 (or the raw input)
-      L3.out_h = last ? 0 : bmode;                 // the result itself is FP32
-      if (last && g3_pair && !keep && any_update) {
+      L3.aux_h = k > 0 ? bf16 : 0;   // X_0 is FP32 (or the raw input)
+      L3.out_h = last ? 0 : bf16;                 // the result itself is FP32
+      if (last && !keep && any_update) {
         L3.update = 1;
         L3.upd_decay = upd.decay; L3.upd_step = upd.step;
         L3.no_out = upd.no_out;
@@ -679,7 +635,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       }
       {
         ProfScope ps(FP4_PROF_G3, st);
-        if (launch_gemm_auto(kG3, *pk, L3, d->sms, st, fs) != cudaSuccess)
+        if (launch_gemm_pair(kG3, *pk, L3, d->sms, st) != cudaSuccess)
           return FP4_ERR_CUDA;
       }
     }
@@ -996,14 +952,12 @@ static fp4_status gemm_nt_impl(int dry, const uint8_t* a_codes, const uint8_t* a
   ProblemPack pack;
   memset(&pack, 0, sizeof(pack));
   GemmProblem& pr = pack.p[0];
-  const bool pair = pair_kernel(M / 128, N / 128, K, d->sms);
-  const int sk = pair ? gemm_pair_stage_k(kPlain) : gemm_stage_k();
+  const int sk = gemm_pair_stage_k(kPlain);
   if (!make_codes_map(d, &pr.tmA, a_codes, M, K / 2, sk) || !make_codes_map(d, &pr.tmB, b_codes, N, K / 2, sk) ||
-      !make_f32_map(d, &pr.tmOut, D, M, N, pair ? 32 : 128) || !make_sf_map(d, &pr.tmSfa, a_scales, M, K, sk) ||
+      !make_f32_map(d, &pr.tmOut, D, M, N) || !make_sf_map(d, &pr.tmSfa, a_scales, M, K, sk) ||
       !make_sf_map(d, &pr.tmSfb, b_scales, N, K, sk))
     return FP4_ERR_CUDA;
   pr.tmAux = pr.tmOut;
-  pr.sfa = a_scales; pr.sfb = b_scales;
   pr.sg_a = a_tensor_scale; pr.sg_b = b_tensor_scale;
   pr.out_rows = (int)M; pr.out_cols = (int)N;
   GemmLaunch L;
@@ -1012,8 +966,8 @@ static fp4_status gemm_nt_impl(int dry, const uint8_t* a_codes, const uint8_t* a
   L.K = (int)K; L.tiles_m = (int)(M / 128); L.tiles_n = (int)(N / 128);
   L.status = device_status;
   L.dry_operands = dry;
-  if (dry && !pair_kernel(L.tiles_m, L.tiles_n, L.K, d->sms)) return FP4_ERR_SHAPE;
-  return launch_gemm_auto(kPlain, pack, L, d->sms, stream) == cudaSuccess ? FP4_OK : FP4_ERR_CUDA;
+  if (dry && (M % 256 || N % 256 || K % 256)) return FP4_ERR_SHAPE;
+  return launch_gemm_pair(kPlain, pack, L, d->sms, stream) == cudaSuccess ? FP4_OK : FP4_ERR_CUDA;
 }
 
 fp4_status fp4_gemm_nt(const uint8_t* a_codes, const uint8_t* a_scales, float a_tensor_scale,
@@ -1046,9 +1000,10 @@ static __global__ void __launch_bounds__(32) k_selftest_wait(uint32_t* status, u
   __syncwarp();
   if (threadIdx.x == 1) fp4::mbar_arrive(&bar_seen);
   if (threadIdx.x == 0) {
-    const bool first = fp4::wait_bar(&bar_seen, 0, &abort_flag);                 // lane 1 arrives: must succeed
-    const bool second = fp4::wait_limited(&bar_never, 0, &abort_flag, limit_ns);  // nobody arrives: must give up
-    *status = (first && !second && abort_flag == 1) ? (uint32_t)FP4_ERR_DEVICE_TIMEOUT : (uint32_t)FP4_ERR_INVALID_ARG;
+    fp4::wait_or_abort(&bar_seen, 0, &abort_flag);                                  // lane 1 arrives: must succeed
+    const bool first = *(volatile uint32_t*)&abort_flag == 0;
+    fp4::wait_limited_abort(fp4::smem_u32(&bar_never), 0, &abort_flag, limit_ns);   // nobody arrives: must give up
+    *status = (first && abort_flag == 1) ? (uint32_t)FP4_ERR_DEVICE_TIMEOUT : (uint32_t)FP4_ERR_INVALID_ARG;
   }
 }
 }  // namespace fp4

@@ -723,3 +723,18 @@ def test_iterations_in_one_launch_for_a_group_are_those_of_single_calls():
         for g, o in zip(mats, outs):
             single, _ = run_gpu(g, steps=4)
             assert np.array_equal(o.cpu().numpy(), single)
+
+
+@pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX, FP4_FLAG_STORE_BF16])
+@pytest.mark.parametrize("shape", [(1664, 2928), (2928, 1648), (128, 37120)])
+def test_pair_tiles_that_stick_out_of_the_matrix(shape, flags):
+    """Work dimensions that are odd multiples of 128, beyond the single-launch sizes: last 256 x 256 tiles with one half
+    outside, a last stage of 128 elements of K; with 128 rows one CTA of every pair has nothing to do."""
+    m, n = shape
+    G = workloads.gradient_like(m, n, seed=m)
+    pf = bool(flags & FP4_FLAG_RHT)
+    before = fp4.fp4_kernel_launches()
+    got, _ = run_gpu(G, steps=2, flags=flags, seed=3)
+    assert fp4.fp4_kernel_launches() - before == 12
+    want = oracle.root_ns(G, steps=2, rht=pf, four_six=pf, seed=3, store_bf16=bool(flags & FP4_FLAG_STORE_BF16))
+    assert rel(got, want) <= TOL_OUT, rel(got, want)
