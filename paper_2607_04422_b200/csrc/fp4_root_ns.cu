@@ -84,7 +84,7 @@ const DeviceInfo* device_info() {
   d.encode = reinterpret_cast<EncodeTiledFn>(fn);
   if (gemm_pair_set_attributes() != cudaSuccess ||
       chain_set_attributes() != cudaSuccess ||
-      prologue_set_attributes() != cudaSuccess)
+      prologue_set_attributes() != cudaSuccess || quantize_set_attributes() != cudaSuccess)
     d.status = FP4_ERR_CUDA;
   d.ready = true;
   return &d;
@@ -123,6 +123,17 @@ bool make_f32_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int64_
   cuuint32_t estr[2] = {1, 1};
   return d->encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// A contiguous FP32 tensor as rows of 16 elements (one block each): box = 128 blocks, 64-byte swizzle.
+bool make_blocks_map(const DeviceInfo* d, CUtensorMap* tm, const void* base, int64_t blocks) {
+  cuuint64_t dims[2] = {16, (cuuint64_t)blocks};
+  cuuint64_t strides[1] = {64};
+  cuuint32_t box[2] = {16, 128};
+  cuuint32_t estr[2] = {1, 1};
+  return d->encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -716,9 +727,13 @@ fp4_status fp4_quantize(const float* x, int64_t rows, int64_t cols, uint8_t* cod
   const DeviceInfo* d;
   fp4_status rc = check_common(&d);
   if (rc != FP4_OK) return rc;
+  CUtensorMap tm;
+  const bool small = quantize_fits_smem(rows * cols, d->sms);
+  if (small && !make_blocks_map(d, &tm, x, rows * cols / 16)) return FP4_ERR_CUDA;
   ProfScope ps(FP4_PROF_QUANTIZE, stream);
-  return launch_quantize(x, rows, cols, codes, scales, tensor_scale, q, d->sms, stream) == cudaSuccess ? FP4_OK
-                                                                                                      : FP4_ERR_CUDA;
+  return launch_quantize(small ? &tm : nullptr, x, rows, cols, codes, scales, tensor_scale, q, d->sms, stream) == cudaSuccess
+             ? FP4_OK
+             : FP4_ERR_CUDA;
 }
 
 fp4_status fp4_momentum_update(const float* G, int64_t rows, int64_t cols, uint8_t* codes, uint16_t* scales,

@@ -131,3 +131,27 @@ def test_argument_errors():
     with pytest.raises(fp4.Fp4Error) as e:       # sign bits without the transform flag
         fp4.fp4_quantize(x, codes, scales, ts, flags=FP4_FLAG_FOUR_SIX | (0x1234 << 16))
     assert e.value.code == 1
+
+
+@pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX])
+@pytest.mark.parametrize("shape", [(128, 128), (128, 384), (640, 2432), (128, 56832), (128, 56960)])
+def test_single_launch_quantiser_at_its_limits(shape, flags):
+    """Tensors that fit the shared memories of all SMs are quantised in one launch: fewer units than SMs, a partial last
+    round, the largest on 148 SMs (6 units in each of 4 groups), and the first size beyond; twice the same on
+    dirty outputs."""
+    rows, cols = shape
+    x_np = workloads.row_lognormal(rows, cols, seed=cols)
+    mask = 0x5A3C if flags else 0
+    x = torch.from_numpy(x_np).cuda()
+    oc, os_, osg = oracle.quantize(x_np, rht=True, mask=mask, four_six=True) if flags else oracle.quantize(x_np)
+    for _ in range(2):
+        codes = torch.full((rows, cols // 2), 0xEE, dtype=torch.uint8, device="cuda")
+        scales = torch.full((fp4.fp4_scale_bytes(rows, cols),), 0xEE, dtype=torch.uint8, device="cuda")
+        ts = torch.full((1,), float("nan"), device="cuda")
+        before = fp4.fp4_kernel_launches()
+        fp4.fp4_quantize(x, codes, scales, ts, flags=flags | mask << 16)
+        assert fp4.fp4_kernel_launches() - before == (3 if shape == (128, 56960) else 1)
+        assert np.float32(ts.item()) == np.float32(osg)
+        got = sf_from_atoms(scales.cpu().numpy(), rows, cols // 16)
+        assert np.array_equal(got, os_), mismatch_report(got, os_)
+        assert np.array_equal(codes.cpu().numpy(), oc), mismatch_report(codes.cpu().numpy(), oc)
