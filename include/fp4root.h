@@ -173,7 +173,8 @@ fp4_status fp4_root_coeffs(int64_t m, int64_t n, int steps, float abc[3]);
  *   an NVFP4 quantisation with 16-element blocks along the contraction axis; the
  *   result is X_steps (transposed back when m > n).
  * Two calls that share a workspace must not overlap in time.
- * Launches: 6 kernels for clip, normalisation and the first quantisation plus 3 per iteration
+ * Launches: 6 kernels for clip, normalisation and the first quantisation (one, cooperative, when
+ *   the group's matrices fit the shared memories of all SMs: 7.2 M elements) plus 3 per iteration
  *   (and a transpose pass for a tall matrix on the routes that cannot write the result
  *   transposed from the last product).  Groups of up to a few million elements run all
  *   iterations in one cooperative launch instead, whose blocks wait on one another (bounded

@@ -1,7 +1,8 @@
 // Prologue of the Root step for a group of equal-size matrices (Section 3.4: "p99 outlier
 // clipping"; normalisation; the first operand copies qX = Q_1x16(X), qX^{16x1} = Q_16x1(X)).
 // Every kernel covers the whole group (gridDim.y = matrix, or a tile list over all matrices), so a
-// group needs six launches instead of six per matrix.
+// group needs six launches instead of six per matrix; a group that fits the shared memories of all SMs
+// needs one (kp_resident, at the end).
 //
 // Clip threshold tau = nearest-rank quantile of |g|, found exactly with two passes over
 // the data where three were needed before:
@@ -257,15 +258,20 @@ __device__ __forceinline__ double sum_partials(const double* partial, int nparts
   return sh[0];
 }
 
-__device__ __forceinline__ void write_norm_scalars(float* scalars, const NsScalarIdx& ix, double sumsq, float maxabs,
-                                                   float eps, float widen) {
-  const float nu = (float)sqrt(sumsq);
-  const float inv = __fdiv_rn(1.0f, __fadd_rn(nu, eps));
-  const float amax0 = __fmul_rn(maxabs, inv);
-  scalars[ix.nu] = nu;
-  scalars[ix.inv] = inv;
-  scalars[ix.amax_X0] = amax0;
-  scalars[ix.sg_X0] = scale_exact(__fmul_rn(widen, amax0));
+struct NormScalars { float nu, inv, amax0, sg; };
+__device__ __forceinline__ NormScalars norm_scalars(double sumsq, float maxabs, float eps, float widen) {
+  NormScalars n;
+  n.nu = (float)sqrt(sumsq);
+  n.inv = __fdiv_rn(1.0f, __fadd_rn(n.nu, eps));
+  n.amax0 = __fmul_rn(maxabs, n.inv);
+  n.sg = scale_exact(__fmul_rn(widen, n.amax0));
+  return n;
+}
+__device__ __forceinline__ void write_norm_scalars(float* scalars, const NsScalarIdx& ix, const NormScalars& n) {
+  scalars[ix.nu] = n.nu;
+  scalars[ix.inv] = n.inv;
+  scalars[ix.amax_X0] = n.amax0;
+  scalars[ix.sg_X0] = n.sg;
 }
 
 // ---- fallback when the candidate list overflowed (so many equal magnitudes that the picked bin holds more
@@ -321,7 +327,7 @@ __device__ void fallback_select_and_stats(const PrepGroup& g, const PrepMatrix& 
   if (threadIdx.x == 0) {
     hdr->sel_prefix = s_fb_prefix;
     m.scalars[g.ix.tau] = tau;
-    write_norm_scalars(m.scalars, g.ix, shd[0], tau, g.eps, g.q.widen);
+    write_norm_scalars(m.scalars, g.ix, norm_scalars(shd[0], tau, g.eps, g.q.widen));
   }
 }
 
@@ -338,8 +344,8 @@ __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ Prep
   NsHeader* hdr = m.hdr;
   if (!g.clip) {
     const double total = sum_partials(m.partial, g.stat_blocks, shd);
-    if (threadIdx.x == 0) write_norm_scalars(m.scalars, g.ix, total, __uint_as_float(hdr->maxabs_bits), g.eps,
-                                               g.q.widen);
+    if (threadIdx.x == 0)
+      write_norm_scalars(m.scalars, g.ix, norm_scalars(total, __uint_as_float(hdr->maxabs_bits), g.eps, g.q.widen));
     return;
   }
   const uint32_t count = hdr->cand_count;
@@ -462,7 +468,7 @@ __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ Prep
     const double n_clipped = n_total - (double)hdr->count_below - (double)hdr->bin_count + (double)s_above;
     const double total = below + cand_sq + n_clipped * (double)tau * (double)tau;
     m.scalars[g.ix.tau] = tau;
-    write_norm_scalars(m.scalars, g.ix, total, tau, g.eps, g.q.widen);
+    write_norm_scalars(m.scalars, g.ix, norm_scalars(total, tau, g.eps, g.q.widen));
     hdr->overflow = 0;
   }
 }
@@ -619,6 +625,204 @@ __device__ __forceinline__ void prep_quant_col2(uint64_t (&y2)[16], const PrepSc
   rare = rare0 || rare1;
 }
 
+// Lane-dependent parts of the shared-memory addresses of a thread's blocks, fixed for a whole kernel.
+struct PrepLane {
+  bool row_warp;
+  int rr, box;         // row pass: a warp takes 8 rows, a thread one 32-column box of a row (two blocks)
+  int band, cp;        // column pass: a warp takes a band of 16 rows and 64 columns, a thread two columns (pair cp)
+  uint32_t base_off, sw;
+};
+__device__ __forceinline__ PrepLane prep_lane() {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cwp = warp & 15;
+  PrepLane p;
+  p.row_warp = warp < kPrepWarps / 2;
+  p.rr = cwp * 8 + (lane & 7); p.box = lane >> 3;
+  p.band = cwp >> 1; p.cp = (cwp & 1) * 32 + lane;
+  if (p.row_warp) { p.base_off = (uint32_t)(p.box * kPrepBox + p.rr * 128); p.sw = (uint32_t)(p.rr & 7) << 4; }
+  else { p.base_off = (uint32_t)((p.cp >> 4) * kPrepBox + p.band * 16 * 128 + (p.cp & 1) * 8); p.sw = (uint32_t)((p.cp >> 1) & 7) << 4; }
+  return p;
+}
+// Scalars of a matrix; sg = its tensor scale, rcp_tab = the shared-memory address of its eight reciprocals.
+__device__ __forceinline__ PrepScalars prep_scalars(float tau, float inv, float sg, uint32_t rcp_tab) {
+  PrepScalars ps;
+  ps.tau = tau;
+  ps.inv = inv;
+  ps.tinv = __fmul_rn(ps.tau, ps.inv);
+  ps.sg = sg;
+  ps.six_sg = __fmul_rn(6.0f, ps.sg);
+  ps.rcp_six_sg = __frcp_rn(ps.six_sg);
+  ps.rcp_tab = rcp_tab;
+  const uint32_t esg = (__float_as_uint(ps.sg) >> 23) & 0xFFu;
+  bool ok = esg >= 67u && esg <= 187u;   // 2^-60 .. 2^60
+  if (ps.tinv < __int_as_float(0x7f800000)) {
+    // a block with clipped elements has amax = tinv: is the clip level quantised to 6 there?
+    const float dc = __fmul_rn(ue4m3_to_float(cvt_ue4m3(__fdiv_rn(ps.tinv, ps.six_sg))), ps.sg);
+    ok = ok && dc != 0.0f && __fmul_rn(ps.tinv, __frcp_rn(dc)) > 5.0f;
+  }
+  ps.near_limit = ok ? 4u : 0xFFFFFFFFu;
+  return ps;
+}
+// One tile: its origin in G is (gr0, gc0), its elements lie at `tile`.  Row codes (and X0 where it is wanted) are stored,
+// column codes and scale bytes are staged.
+template <bool PF>
+__device__ __forceinline__ void prep_tile(const PrepGroup& g, const PrepMatrix& m, const PrepScalars& ps, const PrepLane& pl,
+                                          uint32_t tile, uint8_t* stage, int gr0, int gc0) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool row_warp = pl.row_warp;
+  const int rr = pl.rr, box = pl.box, band = pl.band, cp = pl.cp;
+  const uint32_t base_off = pl.base_off, sw = pl.sw;
+  auto x0 = [&](float gval) { return __fmul_rn(fminf(fmaxf(gval, -ps.tau), ps.tau), ps.inv); };
+  const int tall = m.tall;
+
+  if (m.store_x) {
+    if (!tall) {
+      // X = G: rows of the tile are rows of X
+#pragma unroll 4
+      for (int r = warp; r < 128; r += kPrepWarps) {
+        const float4 v = lds128f(prep_piece(tile, r, lane));
+        if ((gr0 + r) < m.x_rows && (gc0 + lane * 4) < m.x_cols)
+          *reinterpret_cast<float4*>(m.X + (int64_t)(gr0 + r) * m.x_cols + gc0 + lane * 4) =
+              make_float4(x0(v.x), x0(v.y), x0(v.z), x0(v.w));
+      }
+    } else {
+      // X = G^T: a lane group of 8 consecutive tile rows writes one 32-byte sector of a row of X;
+      // the 8 rows x 4 columns a warp reads at once lie in 32 different banks
+      const int r8 = lane & 7, cq = lane >> 3;
+#pragma unroll 4
+      for (int k = 0; k < 512 / kPrepWarps; ++k) {
+        const int p = warp * (512 / kPrepWarps) + k;
+        const int row = (p & 15) * 8 + r8, col = (p >> 4) * 4 + cq;
+        const float v = lds32f(prep_piece(tile, row, col >> 2) + (uint32_t)(col & 3) * 4u);
+        if ((gc0 + col) < m.x_rows && (gr0 + row) < m.x_cols) m.X[(int64_t)(gc0 + col) * m.x_cols + gr0 + row] = x0(v);
+      }
+    }
+  }
+
+  const int64_t rp_k = tall ? g.s : g.l;  // blocks along the rows of G are qX for a wide G, qX^T for a tall one
+  if (g.write_q) {
+    uint8_t* sf_stage = stage + 8 * kQtSlot;
+    const uint32_t tb = tile + base_off;
+    if (row_warp) {
+      uint32_t code[4];
+      uint32_t sfw = 0;
+      bool redo = false;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        uint64_t g2[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];"
+                       : "=l"(g2[2 * i]), "=l"(g2[2 * i + 1])
+                       : "r"(tb + (((uint32_t)(q * 4 + i) << 4) ^ sw)));
+        uint32_t sb;
+        if (PF) {
+          float v[16], unused;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            float a, b2;
+            unpack2(g2[i], a, b2);
+            v[2 * i] = x0(a); v[2 * i + 1] = x0(b2);
+          }
+          sb = quantize_block16_opts(v, g.q, ps.sg, code[2 * q], code[2 * q + 1], unused);
+        } else {
+          bool rare;
+          sb = prep_quant_row(g2, ps, code[2 * q], code[2 * q + 1], rare);
+          redo = redo || rare;
+        }
+        sfw |= sb << (8 * q);
+      }
+      if (!PF && redo) {   // rare: both blocks again from the tile, with the plain quantiser
+        sfw = 0;
+#pragma unroll 1
+        for (int q = 0; q < 2; ++q) {
+          float gv[16];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 f = lds128f(tb + (((uint32_t)(q * 4 + i) << 4) ^ sw));
+            gv[4 * i] = f.x; gv[4 * i + 1] = f.y; gv[4 * i + 2] = f.z; gv[4 * i + 3] = f.w;
+          }
+          sfw |= prep_quant_exact(gv, ps.tau, ps.inv, ps.six_sg, ps.sg, code[2 * q], code[2 * q + 1]) << (8 * q);
+        }
+      }
+      // the four lanes of a row write 64 contiguous bytes
+      uint8_t* rp_codes = tall ? m.qt_codes : m.qx_codes;
+      *reinterpret_cast<uint4*>(rp_codes + (int64_t)(gr0 + rr) * (rp_k / 2) + gc0 / 2 + box * 16) =
+          make_uint4(code[0], code[1], code[2], code[3]);
+      *reinterpret_cast<uint16_t*>(sf_stage + (box >> 1) * 512 + (rr & 31) * 16 + (rr >> 5) * 4 + (box & 1) * 2) =
+          (uint16_t)sfw;
+    } else {
+      uint64_t g2[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        // row band * 16 + i of the tile: its low three bits are those of i
+        const uint32_t a = tb + (uint32_t)(i * 128) + (sw ^ ((uint32_t)(i & 7) << 4));
+        asm volatile("ld.shared.b64 %0, [%1];" : "=l"(g2[i]) : "r"(a));
+      }
+      uint32_t cw[4], sb0 = 0, sb1 = 0;
+      if (PF) {
+        float unused;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          float v[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            float a, b2;
+            unpack2(g2[i], a, b2);
+            v[i] = x0(j == 0 ? a : b2);
+          }
+          const uint32_t sb = quantize_block16_opts(v, g.q, ps.sg, cw[2 * j], cw[2 * j + 1], unused);
+          if (j == 0) sb0 = sb; else sb1 = sb;
+        }
+      } else {
+        bool rare;
+        prep_quant_col2(g2, ps, cw, sb0, sb1, rare);
+        if (rare) {   // redo both blocks from the tile with the plain quantiser
+#pragma unroll 1
+          for (int j = 0; j < 2; ++j) {
+            float gv[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              gv[i] = lds32f(tb + (uint32_t)(i * 128 + j * 4) + (sw ^ ((uint32_t)(i & 7) << 4)));
+            const uint32_t sb = prep_quant_exact(gv, ps.tau, ps.inv, ps.six_sg, ps.sg, cw[2 * j], cw[2 * j + 1]);
+            if (j == 0) sb0 = sb; else sb1 = sb;
+          }
+        }
+      }
+      uint8_t* sfc = sf_stage + 1024 + (band >> 2) * 512 + (band & 3);
+      const int c = cp * 2;
+      sfc[(c & 31) * 16 + (c >> 5) * 4] = (uint8_t)sb0;
+      sfc[((c + 1) & 31) * 16 + ((c + 1) >> 5) * 4] = (uint8_t)sb1;
+      *reinterpret_cast<uint4*>(stage + band * kQtSlot + cp * 16) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
+    }
+  }
+
+}
+// The staged bytes of a tile go out (after a block-wide barrier).
+__device__ __forceinline__ void prep_copy_out(const PrepGroup& g, const PrepMatrix& m, const uint8_t* stage, int gr0, int gc0) {
+  const int tall = m.tall;
+  const int64_t rp_k = tall ? g.s : g.l, cp_k = tall ? g.l : g.s;  // contraction length of the passes' destinations
+  if (g.write_q) {
+    const int tid = threadIdx.x;
+    if (tid < 512) {
+      // column-pass codes: row (gc0 + c) of the destination, 64 bytes from byte gr0 / 2; four lanes per row
+      uint8_t* cp_codes = tall ? m.qx_codes : m.qt_codes;
+      const int c = tid >> 2, h = tid & 3;
+      const uint8_t* src = stage + c * 8;
+      const uint2 a = *reinterpret_cast<const uint2*>(src + (2 * h) * kQtSlot);
+      const uint2 d = *reinterpret_cast<const uint2*>(src + (2 * h + 1) * kQtSlot);
+      *reinterpret_cast<uint4*>(cp_codes + (int64_t)(gc0 + c) * (cp_k / 2) + gr0 / 2 + h * 16) = make_uint4(a.x, a.y, d.x, d.y);
+    } else if (tid < 640) {
+      // scale atoms: two adjacent 512-byte atoms per pass
+      const bool rowpass = tid < 576;
+      uint8_t* sf_base = rowpass ? (tall ? m.qt_sf : m.qx_sf) : (tall ? m.qx_sf : m.qt_sf);
+      const int64_t row0 = rowpass ? gr0 : gc0, k0 = rowpass ? gc0 : gr0, kk = rowpass ? rp_k : cp_k;
+      const int j = tid & 63;
+      const uint4 w = *reinterpret_cast<const uint4*>(stage + 8 * kQtSlot + (rowpass ? 0 : 1024) + j * 16);
+      *reinterpret_cast<uint4*>(sf_base + sf_offset(row0, k0 / 16, kk / 16) + j * 16) = w;
+    }
+  }
+}
+
 template <bool PF>
 __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid_constant__ PrepGroup g) {
   extern __shared__ uint8_t prep_smem_raw[];
@@ -626,7 +830,6 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
   uint8_t* stage_base = smem + kPrepBufs * kPrepTile;
   PrepShared* sh = reinterpret_cast<PrepShared*>(stage_base + kPrepBufs * kPrepStage);
   volatile uint32_t* abort_flag = &sh->abort_flag;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tiles_per_matrix = (int)((g.s >> 7) * (g.l >> 7));
   const int total = tiles_per_matrix * g.count;
   const int my_tiles = (total - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // tiles of this block
@@ -668,16 +871,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
   }
   __syncthreads();
 
-  // lane-dependent parts of the shared-memory addresses, fixed for the whole kernel
-  const bool row_warp = warp < kPrepWarps / 2;
-  //   row pass: a warp takes 8 rows, a thread one 32-column box of a row (two blocks)
-  const int rr = (warp & 15) * 8 + (lane & 7), box = lane >> 3;
-  //   column pass: a warp takes a band of 16 rows and 64 columns, a thread two columns
-  const int cwp = warp & 15, band = cwp >> 1, cp = (cwp & 1) * 32 + lane;  // cp: column pair 0..63
-  uint32_t base_off, sw;
-  if (row_warp) { base_off = (uint32_t)(box * kPrepBox + rr * 128); sw = (uint32_t)(rr & 7) << 4; }
-  else { base_off = (uint32_t)((cp >> 4) * kPrepBox + band * 16 * 128 + (cp & 1) * 8); sw = (uint32_t)((cp >> 1) & 7) << 4; }
-
+  const PrepLane pl = prep_lane();
   int cur = -1;
   PrepScalars ps;
   ps.tau = ps.inv = ps.tinv = ps.six_sg = ps.rcp_six_sg = ps.sg = 0.0f; ps.rcp_tab = 0; ps.near_limit = 0;
@@ -689,149 +883,11 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
     const PrepMatrix& m = g.mat[mi];
     if (mi != cur) {
       cur = mi;
-      ps.tau = g.clip ? m.scalars[g.ix.tau] : __int_as_float(0x7f800000);
-      ps.inv = m.scalars[g.ix.inv];
-      ps.tinv = __fmul_rn(ps.tau, ps.inv);
-      ps.sg = m.scalars[g.ix.sg_X0];
-      ps.six_sg = __fmul_rn(6.0f, ps.sg);
-      ps.rcp_six_sg = __frcp_rn(ps.six_sg);
-      ps.rcp_tab = smem_u32(&sh->rcp_tab[mi][0]);
-      const uint32_t esg = (__float_as_uint(ps.sg) >> 23) & 0xFFu;
-      bool ok = esg >= 67u && esg <= 187u;   // 2^-60 .. 2^60
-      if (ps.tinv < __int_as_float(0x7f800000)) {
-        // a block with clipped elements has amax = tinv: is the clip level quantised to 6 there?
-        const float dc = __fmul_rn(ue4m3_to_float(cvt_ue4m3(__fdiv_rn(ps.tinv, ps.six_sg))), ps.sg);
-        ok = ok && dc != 0.0f && __fmul_rn(ps.tinv, __frcp_rn(dc)) > 5.0f;
-      }
-      ps.near_limit = ok ? 4u : 0xFFFFFFFFu;
+      ps = prep_scalars(g.clip ? m.scalars[g.ix.tau] : __int_as_float(0x7f800000), m.scalars[g.ix.inv], m.scalars[g.ix.sg_X0],
+                        smem_u32(&sh->rcp_tab[mi][0]));
     }
-    auto x0 = [&](float gval) { return __fmul_rn(fminf(fmaxf(gval, -ps.tau), ps.tau), ps.inv); };
-    const uint32_t tile = smem_u32(smem + b * kPrepTile);
     uint8_t* stage = stage_base + b * kPrepStage;
-    const int tall = m.tall;
-
-    if (m.store_x) {
-      if (!tall) {
-        // X = G: rows of the tile are rows of X
-#pragma unroll 4
-        for (int r = warp; r < 128; r += kPrepWarps) {
-          const float4 v = lds128f(prep_piece(tile, r, lane));
-          if ((gr0 + r) < m.x_rows && (gc0 + lane * 4) < m.x_cols)
-            *reinterpret_cast<float4*>(m.X + (int64_t)(gr0 + r) * m.x_cols + gc0 + lane * 4) =
-                make_float4(x0(v.x), x0(v.y), x0(v.z), x0(v.w));
-        }
-      } else {
-        // X = G^T: a lane group of 8 consecutive tile rows writes one 32-byte sector of a row of X;
-        // the 8 rows x 4 columns a warp reads at once lie in 32 different banks
-        const int r8 = lane & 7, cq = lane >> 3;
-#pragma unroll 4
-        for (int k = 0; k < 512 / kPrepWarps; ++k) {
-          const int p = warp * (512 / kPrepWarps) + k;
-          const int row = (p & 15) * 8 + r8, col = (p >> 4) * 4 + cq;
-          const float v = lds32f(prep_piece(tile, row, col >> 2) + (uint32_t)(col & 3) * 4u);
-          if ((gc0 + col) < m.x_rows && (gr0 + row) < m.x_cols) m.X[(int64_t)(gc0 + col) * m.x_cols + gr0 + row] = x0(v);
-        }
-      }
-    }
-
-    // destinations of the two passes: blocks along the rows of G are qX for a wide G, qX^T for a tall one
-    const int64_t rp_k = tall ? g.s : g.l, cp_k = tall ? g.l : g.s;  // contraction length of each destination
-    if (g.write_q) {
-      uint8_t* sf_stage = stage + 8 * kQtSlot;
-      const uint32_t tb = tile + base_off;
-      if (row_warp) {
-        uint32_t code[4];
-        uint32_t sfw = 0;
-        bool redo = false;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          uint64_t g2[8];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];"
-                         : "=l"(g2[2 * i]), "=l"(g2[2 * i + 1])
-                         : "r"(tb + (((uint32_t)(q * 4 + i) << 4) ^ sw)));
-          uint32_t sb;
-          if (PF) {
-            float v[16], unused;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              float a, b2;
-              unpack2(g2[i], a, b2);
-              v[2 * i] = x0(a); v[2 * i + 1] = x0(b2);
-            }
-            sb = quantize_block16_opts(v, g.q, ps.sg, code[2 * q], code[2 * q + 1], unused);
-          } else {
-            bool rare;
-            sb = prep_quant_row(g2, ps, code[2 * q], code[2 * q + 1], rare);
-            redo = redo || rare;
-          }
-          sfw |= sb << (8 * q);
-        }
-        if (!PF && redo) {   // rare: both blocks again from the tile, with the plain quantiser
-          sfw = 0;
-#pragma unroll 1
-          for (int q = 0; q < 2; ++q) {
-            float gv[16];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const float4 f = lds128f(tb + (((uint32_t)(q * 4 + i) << 4) ^ sw));
-              gv[4 * i] = f.x; gv[4 * i + 1] = f.y; gv[4 * i + 2] = f.z; gv[4 * i + 3] = f.w;
-            }
-            sfw |= prep_quant_exact(gv, ps.tau, ps.inv, ps.six_sg, ps.sg, code[2 * q], code[2 * q + 1]) << (8 * q);
-          }
-        }
-        // the four lanes of a row write 64 contiguous bytes
-        uint8_t* rp_codes = tall ? m.qt_codes : m.qx_codes;
-        *reinterpret_cast<uint4*>(rp_codes + (int64_t)(gr0 + rr) * (rp_k / 2) + gc0 / 2 + box * 16) =
-            make_uint4(code[0], code[1], code[2], code[3]);
-        *reinterpret_cast<uint16_t*>(sf_stage + (box >> 1) * 512 + (rr & 31) * 16 + (rr >> 5) * 4 + (box & 1) * 2) =
-            (uint16_t)sfw;
-      } else {
-        uint64_t g2[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          // row band * 16 + i of the tile: its low three bits are those of i
-          const uint32_t a = tb + (uint32_t)(i * 128) + (sw ^ ((uint32_t)(i & 7) << 4));
-          asm volatile("ld.shared.b64 %0, [%1];" : "=l"(g2[i]) : "r"(a));
-        }
-        uint32_t cw[4], sb0 = 0, sb1 = 0;
-        if (PF) {
-          float unused;
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            float v[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              float a, b2;
-              unpack2(g2[i], a, b2);
-              v[i] = x0(j == 0 ? a : b2);
-            }
-            const uint32_t sb = quantize_block16_opts(v, g.q, ps.sg, cw[2 * j], cw[2 * j + 1], unused);
-            if (j == 0) sb0 = sb; else sb1 = sb;
-          }
-        } else {
-          bool rare;
-          prep_quant_col2(g2, ps, cw, sb0, sb1, rare);
-          if (rare) {   // redo both blocks from the tile with the plain quantiser
-#pragma unroll 1
-            for (int j = 0; j < 2; ++j) {
-              float gv[16];
-#pragma unroll
-              for (int i = 0; i < 16; ++i)
-                gv[i] = lds32f(tb + (uint32_t)(i * 128 + j * 4) + (sw ^ ((uint32_t)(i & 7) << 4)));
-              const uint32_t sb = prep_quant_exact(gv, ps.tau, ps.inv, ps.six_sg, ps.sg, cw[2 * j], cw[2 * j + 1]);
-              if (j == 0) sb0 = sb; else sb1 = sb;
-            }
-          }
-        }
-        uint8_t* sfc = sf_stage + 1024 + (band >> 2) * 512 + (band & 3);
-        const int c = cp * 2;
-        sfc[(c & 31) * 16 + (c >> 5) * 4] = (uint8_t)sb0;
-        sfc[((c + 1) & 31) * 16 + ((c + 1) >> 5) * 4] = (uint8_t)sb1;
-        *reinterpret_cast<uint4*>(stage + band * kQtSlot + cp * 16) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
-      }
-    }
+    prep_tile<PF>(g, m, ps, pl, smem_u32(smem + b * kPrepTile), stage, gr0, gc0);
 
     // Every warp has read the tile and staged its output: the buffer takes the tile three ahead, the
     // staged bytes go out.
@@ -840,28 +896,419 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
       fence_proxy_async_smem();
       fetch(it + kPrepBufs);
     }
-    if (g.write_q) {
-      const int tid = threadIdx.x;
-      if (tid < 512) {
-        // column-pass codes: row (gc0 + c) of the destination, 64 bytes from byte gr0 / 2; four lanes per row
-        uint8_t* cp_codes = tall ? m.qx_codes : m.qt_codes;
-        const int c = tid >> 2, h = tid & 3;
-        const uint8_t* src = stage + c * 8;
-        const uint2 a = *reinterpret_cast<const uint2*>(src + (2 * h) * kQtSlot);
-        const uint2 d = *reinterpret_cast<const uint2*>(src + (2 * h + 1) * kQtSlot);
-        *reinterpret_cast<uint4*>(cp_codes + (int64_t)(gc0 + c) * (cp_k / 2) + gr0 / 2 + h * 16) = make_uint4(a.x, a.y, d.x, d.y);
-      } else if (tid < 640) {
-        // scale atoms: two adjacent 512-byte atoms per pass
-        const bool rowpass = tid < 576;
-        uint8_t* sf_base = rowpass ? (tall ? m.qt_sf : m.qx_sf) : (tall ? m.qx_sf : m.qt_sf);
-        const int64_t row0 = rowpass ? gr0 : gc0, k0 = rowpass ? gc0 : gr0, kk = rowpass ? rp_k : cp_k;
-        const int j = tid & 63;
-        const uint4 w = *reinterpret_cast<const uint4*>(stage + 8 * kQtSlot + (rowpass ? 0 : 1024) + j * 16);
-        *reinterpret_cast<uint4*>(sf_base + sf_offset(row0, k0 / 16, kk / 16) + j * 16) = w;
-      }
-    }
+    if (g.write_q) prep_copy_out(g, m, stage, gr0, gc0);
   }
   if (threadIdx.x == 0 && sh->abort_flag) report_timeout(g.status);
+}
+
+// ---- the whole prologue of a group whose matrices fit the shared memories of all SMs, in one cooperative launch.
+//
+// Every block brings up to three 128 x 128 tiles into shared memory once and keeps them there: it counts them into the
+// histogram, compacts candidates and squares from them, and quantises them.  Between those phases the blocks
+// meet at (bounded) grid barriers; what a single block did between two launches - the bin of the rank, the select
+// among the candidates, the normalisation scalars - every block now computes for its own matrices, which costs less
+// than another exchange.  Same sums in another order: nu is a sum of FP64 partials per tile.
+//
+// Bounds: latency - three barriers, 3200 cycles of shared-memory counting and 4500 of FP64 sums per tile, two radix rounds,
+// one tile's quantisation (18 us for one tile per SM, 42 us for three).  Whole 5-iteration calls, six launches before
+// and this one now: 512 x 512 121 -> 110-120 us, 1024 x 1024 134 -> 124-128, 2048 x 2048 232 -> 223, 384 x 12160
+// 272 -> 262.
+constexpr int kResTiles = 3;
+constexpr int kResUnion = kTopBins * 4;     // histogram / candidate buffer / select arrays / staged output of a tile
+static_assert(kResUnion >= kPrepStage && kResUnion >= 4096 + 1024 * 8, "union area");
+struct ResidentShared {
+  uint64_t full[kResTiles];
+  PrepTileInfo info[kResTiles];              // pad: index of the tile within its matrix
+  uint32_t prefix[kResTiles], rank[kResTiles], bin_count[kResTiles], below[kResTiles];   // of the tile's matrix
+  float tau[kResTiles], inv[kResTiles], sg[kResTiles];
+  float rcp_tab[8];
+  double wsum[32];
+  float wmax[32];
+  uint32_t wtot[32];
+  unsigned long long wlo[32], whi[32];
+  uint32_t wabove[32];
+  uint32_t sel_prefix, sel_rank, cnt, base;
+  uint32_t abort_flag;
+};
+constexpr int kResSmem = kResTiles * kPrepTile + kResUnion + (int)sizeof(ResidentShared) + 1024;
+static_assert(kResSmem + 64 <= 232448, "at most 227 KB of shared memory (64 bytes of it static, in the fallback)");
+
+// Exclusive prefix of one value per thread over a block of 1024 threads; `wtot`: 32 words.
+__device__ __forceinline__ uint32_t block_prefix(uint32_t v, uint32_t* wtot) {
+  uint32_t incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    if ((int)(threadIdx.x & 31) >= o) incl += t;
+  }
+  if ((threadIdx.x & 31) == 31) wtot[threadIdx.x >> 5] = incl;
+  __syncthreads();
+  uint32_t w = wtot[threadIdx.x & 31], s = w;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, s, o);
+    if ((int)(threadIdx.x & 31) >= o) s += t;
+  }
+  const uint32_t before = __shfl_sync(0xffffffffu, s - w, (int)(threadIdx.x >> 5));
+  __syncthreads();
+  return before + incl - v;
+}
+
+template <bool PF>
+__global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_constant__ PrepGroup g) {
+  extern __shared__ uint8_t prep_smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(prep_smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* uni = smem + kResTiles * kPrepTile;
+  ResidentShared* sh = reinterpret_cast<ResidentShared*>(uni + kResUnion);
+  volatile uint32_t* abort_flag = &sh->abort_flag;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tiles_per_matrix = (int)((g.s >> 7) * (g.l >> 7));
+  const int total = tiles_per_matrix * g.count;
+  const int mine = (total - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // 1 .. kResTiles
+  uint32_t* counter = &g.mat[0].hdr->barrier;
+  uint32_t round = 0;
+  if (tid == 0) {
+    for (int i = 0; i < kResTiles; ++i) mbar_init(&sh->full[i], 1);
+    sh->abort_flag = 0;
+    mbar_fence_init();
+    for (int it = 0; it < mine; ++it) {
+      const int t = (int)blockIdx.x + it * (int)gridDim.x;
+      PrepTileInfo ti;
+      ti.mi = t / tiles_per_matrix;
+      ti.pad = t - ti.mi * tiles_per_matrix;
+      const int tiles_x = (int)((g.mat[ti.mi].tall ? g.s : g.l) >> 7);
+      const int ty = ti.pad / tiles_x;
+      ti.gr0 = ty * 128;
+      ti.gc0 = (ti.pad - ty * tiles_x) * 128;
+      sh->info[it] = ti;
+      mbar_expect_tx(&sh->full[it], kPrepTile);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        tma_load_2d(smem + it * kPrepTile + q * kPrepBox, &g.tmG[ti.mi], ti.gc0 + 32 * q, ti.gr0, &sh->full[it]);
+    }
+  }
+  // clear headers (all but the status word of all but the call's first matrix, and the barrier), scalars, histograms
+  constexpr int kBarrierWord = (int)(offsetof(NsHeader, barrier) / 4);
+  for (int j = 0; j < g.count; ++j) {
+    uint32_t* w = reinterpret_cast<uint32_t*>(g.mat[j].hdr);
+    for (int i = (g.mat[j].clear_status ? 0 : 4) + (int)blockIdx.x * kPrepThreads + tid; i < g.zero_words;
+         i += (int)gridDim.x * kPrepThreads)
+      if (i != kBarrierWord) w[i] = 0;
+  }
+  __syncthreads();
+  // a thread's four 16-byte pieces of a tile: row tid / 8 of each 32-column box; f(values, in the caller's matrix)
+  auto pieces = [&](int it, auto&& f) {
+    const PrepTileInfo ti = sh->info[it];
+    const PrepMatrix& m = g.mat[ti.mi];
+    const int row = tid >> 3, c = ((tid & 7) ^ (row & 7)) * 4;
+    const bool row_in = ti.gr0 + row < (m.tall ? g.l0 : g.s0);
+    const int cols = (int)(m.tall ? g.s0 : g.l0) - ti.gc0;
+    const uint32_t at = smem_u32(smem + it * kPrepTile) + tid * 16;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 v = lds128f(at + k * kPrepBox);
+      if (row_in && k * 32 + c < cols) { f(v.x); f(v.y); f(v.z); f(v.w); }
+    }
+  };
+  for (int it = 0; it < mine; ++it) wait_or_abort(&sh->full[it], 0, abort_flag);
+
+  if (g.clip) {
+    // ---- histogram of the top magnitude bits
+    uint32_t* hist = reinterpret_cast<uint32_t*>(uni);
+    for (int it = 0; it < mine; ++it) {
+      const int mi = sh->info[it].mi;
+      const bool first = it == 0 || sh->info[it - 1].mi != mi, last = it == mine - 1 || sh->info[it + 1].mi != mi;
+      if (!g.mat[mi].hist_top) {
+        if (first) {
+          for (int i = tid; i < kTopBins; i += kPrepThreads) hist[i] = 0;
+          __syncthreads();
+        }
+        pieces(it, [&](float x) { atomicAdd(&hist[mag_bits(x) >> kTopShift], 1u); });
+        __syncthreads();
+      }
+      if (round == 0) grid_barrier(counter, ++round, abort_flag);   // everything is cleared
+      if (last && !g.mat[mi].hist_top) {
+        for (int i = tid; i < kTopBins; i += kPrepThreads)
+          if (hist[i]) atomicAdd(&g.mat[mi].hist[i], hist[i]);
+        __syncthreads();
+      }
+    }
+    grid_barrier(counter, ++round, abort_flag);
+    // ---- the bin that holds the rank
+    for (int it = 0; it < mine; ++it) {
+      const int mi = sh->info[it].mi;
+      if (it > 0 && sh->info[it - 1].mi == mi) {
+        if (tid == 0) {
+          sh->prefix[it] = sh->prefix[it - 1]; sh->rank[it] = sh->rank[it - 1];
+          sh->bin_count[it] = sh->bin_count[it - 1]; sh->below[it] = sh->below[it - 1];
+        }
+        __syncthreads();
+        continue;
+      }
+      // a warp takes 256 bins, a lane two groups of four; the warp that holds the rank looks closer
+      const uint32_t* h = (g.mat[mi].hist_top ? g.mat[mi].hist_top : g.mat[mi].hist) + warp * 256 + lane * 4;
+      uint32_t c[8];
+      if ((reinterpret_cast<uintptr_t>(h) & 15) == 0) {
+        const uint4 a = __ldcg(reinterpret_cast<const uint4*>(h)), b = __ldcg(reinterpret_cast<const uint4*>(h + 128));
+        c[0] = a.x; c[1] = a.y; c[2] = a.z; c[3] = a.w; c[4] = b.x; c[5] = b.y; c[6] = b.z; c[7] = b.w;
+      } else {   // a caller's histogram need only be 4-byte aligned
+#pragma unroll
+        for (int q = 0; q < 8; ++q) c[q] = __ldcg(h + (q >> 2) * 128 + (q & 3));
+      }
+      const uint32_t s0 = c[0] + c[1] + c[2] + c[3], s1 = c[4] + c[5] + c[6] + c[7];
+      const uint32_t all = __reduce_add_sync(0xffffffffu, s0 + s1);
+      if (lane == 0) sh->wtot[warp] = all;
+      __syncthreads();
+      const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? sh->wtot[lane] : 0u);
+      if (g.clip_rank > before && g.clip_rank <= before + all) {
+        uint32_t run = before;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          const uint32_t v = half ? s1 : s0;
+          uint32_t incl = v;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+          }
+          uint32_t at = run + incl - v;
+          if (g.clip_rank > at && g.clip_rank <= at + v) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const uint32_t n = c[half * 4 + q];
+              if (g.clip_rank > at && g.clip_rank <= at + n) {
+                sh->prefix[it] = (uint32_t)(warp * 256 + half * 128 + lane * 4 + q) << kTopShift;
+                sh->rank[it] = g.clip_rank - at;
+                sh->bin_count[it] = n;
+                sh->below[it] = at;
+              }
+              at += n;
+            }
+          }
+          run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+      }
+      __syncthreads();
+    }
+  } else {
+    grid_barrier(counter, ++round, abort_flag);
+  }
+
+  // ---- squares below the bin, candidates of the bin
+  for (int it = 0; it < mine; ++it) {
+    const PrepTileInfo ti = sh->info[it];
+    const PrepMatrix& m = g.mat[ti.mi];
+    const uint32_t bin = g.clip ? sh->prefix[it] >> kTopShift : 0xFFFFFFFFu;
+    uint32_t* buf = reinterpret_cast<uint32_t*>(uni);
+    constexpr uint32_t kBuf = kResUnion / 4;
+    if (tid == 0) sh->cnt = 0;
+    __syncthreads();
+    double acc = 0.0;
+    float mx = 0.0f;
+    pieces(it, [&](float x) {
+      const uint32_t k = mag_bits(x), kb = k >> kTopShift;
+      if (kb < bin) {
+        acc += (double)x * (double)x;
+        mx = fmaxf(mx, __uint_as_float(k));
+      } else if (kb == bin) {
+        const uint32_t pos = atomicAdd(&sh->cnt, 1u);
+        if (pos < kBuf) {
+          buf[pos] = k;
+        } else {
+          const uint32_t gpos = atomicAdd(&m.hdr->cand_count, 1u);
+          if (gpos < g.cand_cap) m.cand[gpos] = k;
+        }
+      }
+    });
+#pragma unroll
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
+    if (lane == 0) { sh->wsum[warp] = acc; sh->wmax[warp] = mx; }
+    __syncthreads();
+    const uint32_t nbuf = sh->cnt < kBuf ? sh->cnt : kBuf;
+    if (warp == 0) {
+      acc = sh->wsum[lane];
+#pragma unroll
+      for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sh->wmax[lane])));
+      if (lane == 0) {
+        m.partial[ti.pad] = acc;
+        atomicMax(&m.hdr->maxabs_bits, __float_as_uint(mx));
+        sh->base = nbuf ? atomicAdd(&m.hdr->cand_count, nbuf) : 0u;
+      }
+    }
+    __syncthreads();
+    for (uint32_t j = tid; j < nbuf; j += kPrepThreads) {
+      const uint32_t gpos = sh->base + j;
+      if (gpos < g.cand_cap) m.cand[gpos] = buf[j];
+    }
+    __syncthreads();
+  }
+  grid_barrier(counter, ++round, abort_flag);
+
+  // ---- tau among the candidates, normalisation scalars: every block for its own matrices; the block of a matrix's
+  // first tile writes them
+  for (int it = 0; it < mine; ++it) {
+    const int mi = sh->info[it].mi;
+    const PrepMatrix& m = g.mat[mi];
+    NsHeader* hdr = m.hdr;
+    if (it > 0 && sh->info[it - 1].mi == mi) {
+      if (tid == 0) { sh->tau[it] = sh->tau[it - 1]; sh->inv[it] = sh->inv[it - 1]; sh->sg[it] = sh->sg[it - 1]; }
+      __syncthreads();
+      continue;
+    }
+    const bool owner = sh->info[it].pad == 0;
+    const uint32_t count = g.clip ? __ldcg(&hdr->cand_count) : 0u;
+    if (count > g.cand_cap) {
+      // so many equal magnitudes that the list overflowed: the owner finishes alone, the others wait for it
+      if (owner) {
+        if (tid == 0) { hdr->sel_prefix = sh->prefix[it]; hdr->sel_rank = sh->rank[it]; }
+        __syncthreads();
+        fallback_select_and_stats(g, m, reinterpret_cast<uint32_t*>(uni), reinterpret_cast<double*>(uni + 8192));
+        __syncthreads();
+        if (tid == 0) {
+          __threadfence();
+          asm volatile("st.release.gpu.global.u32 [%0], 1;" ::"l"(&hdr->overflow) : "memory");
+        }
+      } else if (tid == 0) {
+        const uint64_t t0 = globaltimer_ns();
+        for (;;) {
+          uint32_t v;
+          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&hdr->overflow) : "memory");
+          if (v) break;
+          if (*abort_flag || globaltimer_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; break; }
+        }
+      }
+      __syncthreads();
+      if (tid == 0) {
+        sh->tau[it] = __ldcg(m.scalars + g.ix.tau);
+        sh->inv[it] = __ldcg(m.scalars + g.ix.inv);
+        sh->sg[it] = __ldcg(m.scalars + g.ix.sg_X0);
+      }
+      __syncthreads();
+      continue;
+    }
+    uint32_t* hist = reinterpret_cast<uint32_t*>(uni);     // 512 counters
+    if (tid == 0) {
+      sh->sel_prefix = sh->prefix[it]; sh->sel_rank = sh->rank[it];
+    }
+    unsigned long long lo = 0, hi = 0;
+    uint32_t above = 0, tau_bits = 0;
+    const uint32_t efield = g.clip ? sh->prefix[it] >> 23 : 0u;
+    const uint32_t implicit = efield ? 0x800000u : 0u;
+    if (g.clip) {
+      // two radix rounds over the low 18 bits of the candidates; the second also gathers exact squares of those
+      // below the sub-bin and counts those above (see kp_finalize)
+      for (int r = 0; r < 2; ++r) {
+        const int shift = r == 0 ? 9 : 0;
+        const uint32_t high_mask = ~((1u << (shift + 9)) - 1u) & 0x7FFFFFFFu;
+        if (tid < 512) hist[tid] = 0;
+        __syncthreads();
+        const uint32_t prefix = sh->sel_prefix, rank = sh->sel_rank;
+        for (uint32_t i0 = tid; i0 < count; i0 += 8 * kPrepThreads) {
+          uint32_t k[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) k[u] = i0 + u * kPrepThreads < count ? __ldcg(m.cand + i0 + u * kPrepThreads) : 0xFFFFFFFFu;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            if (k[u] == 0xFFFFFFFFu) continue;
+            if ((k[u] & high_mask) == (prefix & high_mask)) {
+              atomicAdd(&hist[(k[u] >> shift) & 511u], 1u);
+            } else if (r == 1) {
+              if (k[u] < prefix) {
+                const unsigned long long mant = (k[u] & 0x7FFFFFu) | implicit, sq = mant * mant;
+                lo += sq & 0xFFFFFFull;
+                hi += sq >> 24;
+              } else {
+                above += 1;
+              }
+            }
+          }
+        }
+        __syncthreads();
+        const uint32_t c = tid < 512 ? hist[tid] : 0u;
+        const uint32_t before = block_prefix(c, sh->wtot);
+        if (c && rank > before && rank <= before + c) {
+          sh->sel_prefix = prefix | ((uint32_t)tid << shift);
+          sh->sel_rank = rank - before;
+        }
+        __syncthreads();
+      }
+      tau_bits = sh->sel_prefix;
+      // a counter of the second round stands for one exact magnitude
+      if (tid < 512 && hist[tid]) {
+        const uint32_t cnt = hist[tid], kk = (tau_bits & ~511u) | (uint32_t)tid;
+        if (kk <= tau_bits) {
+          const unsigned long long mant = (kk & 0x7FFFFFu) | implicit, sq = mant * mant;
+          lo += (unsigned long long)cnt * (sq & 0xFFFFFFull);
+          hi += (unsigned long long)cnt * (sq >> 24);
+        } else {
+          above += cnt;
+        }
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        lo += __shfl_xor_sync(0xffffffffu, lo, o);
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        above += __shfl_xor_sync(0xffffffffu, above, o);
+      }
+      if (lane == 0) { sh->wlo[warp] = lo; sh->whi[warp] = hi; sh->wabove[warp] = above; }
+    }
+    // fixed-order sum of the tiles' partials
+    double acc = 0.0;
+    for (int i = tid; i < tiles_per_matrix; i += kPrepThreads) acc += __ldcg(m.partial + i);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) sh->wsum[warp] = acc;
+    __syncthreads();
+    if (warp == 0) {
+      acc = sh->wsum[lane];
+      if (g.clip) { lo = sh->wlo[lane]; hi = sh->whi[lane]; above = sh->wabove[lane]; }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        lo += __shfl_xor_sync(0xffffffffu, lo, o);
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        above += __shfl_xor_sync(0xffffffffu, above, o);
+      }
+      if (lane == 0) {
+        float maxabs = __uint_as_float(__ldcg(&hdr->maxabs_bits)), tau = __int_as_float(0x7f800000);
+        if (g.clip) {
+          tau = __uint_as_float(tau_bits);
+          maxabs = tau;
+          const int e2 = 2 * ((int)(efield ? efield : 1u) - 150);
+          const double cand_sq = ldexp((double)hi * 16777216.0 + (double)lo, e2);
+          // clamped to tau: everything in the bins above the picked one, and the candidates above tau
+          const double n_clipped = (double)g.n4 * 4.0 - (double)sh->below[it] - (double)sh->bin_count[it] + (double)above;
+          acc = acc + cand_sq + n_clipped * (double)tau * (double)tau;
+        }
+        const NormScalars ns = norm_scalars(acc, maxabs, g.eps, g.q.widen);
+        sh->tau[it] = tau; sh->inv[it] = ns.inv; sh->sg[it] = ns.sg;
+        if (owner) {
+          if (g.clip) m.scalars[g.ix.tau] = tau;
+          write_norm_scalars(m.scalars, g.ix, ns);
+        }
+      }
+    }
+    __syncthreads();
+    if (owner && g.clip && m.hist_top)                    // the caller's counters are consumed
+      for (int i = tid; i < kTopBins; i += kPrepThreads) m.hist_top[i] = 0;
+  }
+
+  // ---- operand copies of X0 from the resident tiles
+  const PrepLane pl = prep_lane();
+  for (int it = 0; it < mine; ++it) {
+    const PrepTileInfo ti = sh->info[it];
+    const PrepMatrix& m = g.mat[ti.mi];
+    if (tid < 8) sh->rcp_tab[tid] = __frcp_rn(__fmul_rn((float)(8 + tid), sh->sg[it]));
+    __syncthreads();
+    const PrepScalars ps = prep_scalars(sh->tau[it], sh->inv[it], sh->sg[it], smem_u32(&sh->rcp_tab[0]));
+    prep_tile<PF>(g, m, ps, pl, smem_u32(smem + it * kPrepTile), uni, ti.gr0, ti.gc0);
+    __syncthreads();
+    if (g.write_q) prep_copy_out(g, m, uni, ti.gr0, ti.gc0);
+    __syncthreads();
+  }
+  if (tid == 0 && sh->abort_flag) report_timeout(g.status);
 }
 
 }  // namespace
@@ -869,7 +1316,9 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
 cudaError_t prologue_set_attributes() {
   cudaError_t e = cudaFuncSetAttribute(kp_prep_operands<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepSmem);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(kp_prep_operands<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepSmem);
+  if ((e = cudaFuncSetAttribute(kp_prep_operands<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepSmem))) return e;
+  if ((e = cudaFuncSetAttribute(kp_resident<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem))) return e;
+  return cudaFuncSetAttribute(kp_resident<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
 }
 
 // Enqueue the prologue for `count` matrices of one shape (s, l) and one parameter set.
@@ -922,6 +1371,24 @@ cudaError_t launch_prologue_group(const PrologueItem* items, int count, int writ
       g.tmG[j] = *it.tmG;
     }
     const int sms = pl.sms;
+    const int64_t tiles = (pl.l / 128) * (pl.s / 128) * nn;
+    if (tiles <= (int64_t)kResTiles * sms) {
+      // everything fits the shared memories: one launch
+      ProfScope ps(FP4_PROF_PREP, st);
+      cudaError_t e = cudaMemsetAsync(&g.mat[0].hdr->barrier, 0, 4, st);
+      if (e != cudaSuccess) return e;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(tiles < sms ? tiles : sms)); cfg.blockDim = dim3(kPrepThreads);
+      cfg.dynamicSmemBytes = kResSmem; cfg.stream = st;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeCooperative;
+      attr[0].val.cooperative = 1;
+      cfg.attrs = attr; cfg.numAttrs = 1;
+      count_launches(1);
+      e = cudaLaunchKernelEx(&cfg, q.rht || q.four_six ? kp_resident<true> : kp_resident<false>, g);
+      if (e != cudaSuccess) return e;
+      continue;
+    }
     int64_t hb = (g.n4 + 512 * 4 - 1) / (512 * 4);
     const int hist_blocks = (int)(hb < (int64_t)sms * 4 ? (hb < 1 ? 1 : hb) : (int64_t)sms * 4);
     const dim3 gy1(1, (unsigned)nn), gh((unsigned)hist_blocks, (unsigned)nn), gs((unsigned)g.stat_blocks, (unsigned)nn);
@@ -943,7 +1410,6 @@ cudaError_t launch_prologue_group(const PrologueItem* items, int count, int writ
     }
     {
       ProfScope ps(FP4_PROF_PREP, st);
-      const int64_t tiles = (pl.l / 128) * (pl.s / 128) * nn;
       const unsigned gp = (unsigned)(tiles < sms ? tiles : sms);
       if (q.rht || q.four_six) launch_chained(kp_prep_operands<true>, dim3(gp), dim3(kPrepThreads), kPrepSmem, st, g);
       else launch_chained(kp_prep_operands<false>, dim3(gp), dim3(kPrepThreads), kPrepSmem, st, g);

@@ -131,23 +131,6 @@ struct QuantShared {
 };
 constexpr int kQSmem = kQGroups * kQHold * kQUnitBytes + (int)sizeof(QuantShared) + 1024;
 
-// All blocks have arrived `round` times; bounded like the other waits (the launch is cooperative: all are resident).
-__device__ __forceinline__ void quant_barrier(uint32_t* counter, uint32_t round, volatile uint32_t* abort_flag) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
-    const uint32_t want = round * gridDim.x;
-    const uint64_t t0 = globaltimer_ns();
-    for (;;) {
-      uint32_t v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
-      if (v >= want) break;
-      if (globaltimer_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; break; }
-    }
-  }
-  __syncthreads();
-}
-
 template <bool PF>
 __global__ void __launch_bounds__(kQThreads, 1)
 k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols, uint8_t* __restrict__ codes, uint8_t* scales,
@@ -196,7 +179,7 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
     for (int w = 0; w < kQThreads / 32; ++w) mx = fmaxf(mx, sh->wmax[w]);
     scratch[blockIdx.x] = __float_as_uint(mx);
   }
-  quant_barrier(scratch + kQCounterWord, 1, abort_flag);
+  grid_barrier(scratch + kQCounterWord, 1, abort_flag);
   uint32_t bits = 0;
   for (int i = threadIdx.x & 31; i < (int)gridDim.x; i += 32) {
     uint32_t v;
@@ -206,7 +189,7 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
   bits = __reduce_max_sync(0xffffffffu, bits);
   const float sg = scale_exact(__fmul_rn(q.widen, __uint_as_float(bits)));
   const float six_sg = __fmul_rn(6.0f, sg);
-  quant_barrier(scratch + kQCounterWord, 2, abort_flag);   // everyone has read the maxima: scales may be written
+  grid_barrier(scratch + kQCounterWord, 2, abort_flag);   // everyone has read the maxima: scales may be written
   if (blockIdx.x == 0 && threadIdx.x == 0) *tensor_scale = sg;
   const uint32_t kblocks = (uint32_t)(cols >> 4);
   for (int i = 0; i < m; ++i) {
