@@ -23,9 +23,10 @@
 // the running maximum and counts the tile.
 //
 // Bounds: latency.  A 5-iteration call is a chain of 15 dependent products.  At 256 x 512 a product takes about 5 us:
-// the counter's round trip 1 us with its fences another 0.9, operand copies and MMAs 1, the one tile's epilogue 1.5-2.
-// Whole calls, before (three launches per iteration) and now: 256 x 512 175 -> 108 us, 1024 x 1024 190 -> 135,
-// 1040 x 2896 with the paper's quantiser options 307 -> 233.
+// the counter's round trip and the release 1.5, operand copies and MMAs 1, the one tile's epilogue 2.
+// With the proxy fence on the reading side and one lane storing everything the iterations of 256 x 512 took 87 us
+// instead of 78, of 1408 x 2176 156 instead of 141.  Whole calls against three launches per iteration: 256 x 512
+// 175 -> 97 us, 1024 x 1024 190 -> 118, 1040 x 2896 with the paper's quantiser options 307 -> 223.
 #include "fp4_gemm_common.cuh"
 
 namespace fp4 {
@@ -117,7 +118,7 @@ __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
 __device__ __forceinline__ float ld_scalar(const float* p) {
   return __uint_as_float(ld_relaxed(reinterpret_cast<const uint32_t*>(p)));
 }
-__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void sts_f4(uint32_t a, float x, float y, float z, float w) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
@@ -194,6 +195,8 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
     if (j < (list ? my_full : my_sym))
       sh->tiles[list][j] = chain_tile<BN>((int)blockIdx.x + j * grid, list == 0, list ? nfull : nsym, (list ? a.l : a.s) / BN);
   }
+  for (int i = (int)threadIdx.x; i < a.count * kChainMaps; i += NTHREADS)   // descriptors come first in a problem
+    tma_prefetch_desc(reinterpret_cast<const CUtensorMap*>(&pack.p[i / kChainMaps]) + i % kChainMaps);
   if (warp == W_MMA) {
     tmem_alloc(&sh->tmem_base, TMEM_COLS);
     tmem_relinquish();
@@ -230,7 +233,6 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
                 if (*abort_flag || globaltimer_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; break; }
               }
             }
-            fence_proxy_async_all();   // part of the operands was stored through the generic proxy, TMA reads them
           }
           seen = p;
           mbar_arrive(&sh->dep[n % DEP_RING]);
@@ -328,13 +330,6 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
         float* maxima = pr.scalars + (slot & ~3);
         uint32_t* done = pr.done;
         wait_or_abort(&sh->out_done[n & 1], (n >> 1) & 1, abort_flag);
-        if (BN == 64 && mirror) {
-          // the scales of 64 rows are the 8-byte halves of the 16-byte rows of two atoms
-          uint8_t* dst = csf + lane * 16 + (tj & 1) * 8;
-          const uint8_t* src = ob + L::RQ + L::CQ + L::RSF + lane * 8;
-          *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src);
-          *reinterpret_cast<uint2*>(dst + 512) = *reinterpret_cast<const uint2*>(src + 256);
-        }
         if (lane == 0) {
 #pragma unroll
           for (int h = 0; h < BN / 64; ++h) tma_store_s(mr, tj * (BN / 2) + h * 32, ti * BM, os + h * 4096);
@@ -346,6 +341,19 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
           }
           if (mode != kG2) bulk_max16_s(maxima, smem_u32(&sh->amax[n & 1][0]));
           bulk_commit();
+        } else if (BN == 64 && mirror && lane >= 16) {
+          // The scales of 64 rows are the 8-byte halves of the 16-byte rows of two atoms: stored by other lanes than
+          // the one that waits for the copies (its release would wait for its own stores again), and fenced here,
+          // because the next product's TMA loads read what the generic proxy wrote.
+          uint8_t* dst = csf + (lane - 16) * 16 + (tj & 1) * 8;
+          const uint8_t* src = ob + L::RQ + L::CQ + L::RSF + (lane - 16) * 8;
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            *reinterpret_cast<uint2*>(dst + (q >> 1) * 512 + (q & 1) * 256) = *reinterpret_cast<const uint2*>(src + q * 128);
+          fence_proxy_async_global();
+        }
+        __syncwarp();
+        if (lane == 0) {
           bulk_wait_all<0>();
           sh->amax[n & 1][slot & 3] = 0;
         }

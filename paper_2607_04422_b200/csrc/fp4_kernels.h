@@ -132,6 +132,7 @@ struct alignas(64) ChainProblem {
   float ca, cb, cc;
   int tall;
 };
+constexpr int kChainMaps = 16;   // tensor maps at the start of a ChainProblem
 constexpr int kChainMax = 14;    // matrices of a launch
 constexpr int kChainTiles = 32;  // tiles of one product that a block takes at most
 struct ChainPack { ChainProblem p[kChainMax]; };
