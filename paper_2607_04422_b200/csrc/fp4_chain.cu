@@ -672,10 +672,17 @@ cudaError_t launch_one(const ChainPack& pack, const ChainLaunch& a, int grid, cu
   return cudaLaunchKernelEx(&cfg, k_chain<BN, PF>, pack, a);
 }
 
-int sym_tiles(int64_t s, int bn) {
-  int n = 0;
-  for (int64_t r = 0; r < s / BM; ++r) n += (int)((s - r * BM) / bn);
+int64_t sym_tiles(int64_t s, int bn) {
+  int64_t n = 0;
+  for (int64_t r = 0; r < s / BM; ++r) n += (s - r * BM) / bn;
   return n;
+}
+int64_t rounds(int64_t tiles, int sms) { return (tiles + sms - 1) / sms; }
+// Narrow tiles while they shorten the longest block's work: rounds of 128 x 64 tiles against rounds of 128 x 128.
+// (256 x 512, 5 iterations: 87 us against 121; 1536 x 2560, where both take four rounds of 64 columns: 202 / 184.)
+bool narrow_tiles(int64_t s, int64_t l, int count, int sms) {
+  const int64_t full128 = s / BM * (l / 128) * count;
+  return rounds(2 * full128, sms) < 2 * rounds(full128, sms);
 }
 
 }  // namespace
@@ -689,17 +696,29 @@ cudaError_t chain_set_attributes() {
   return cudaSuccess;
 }
 
+// Estimated time of one iteration in us: per product a dependency round trip, and rounds of tiles that take an epilogue
+// or a main loop each, whichever is longer (0 when a block would take more tiles than its list holds).  The constants of
+// this estimate and of the CTA-pair kernel's beside its caller are fitted to both kernels' times at 75 shapes and
+// groups, 256 to 3072 wide, plain and with the quantiser options; choosing by them loses 0.6 % on average against
+// always knowing the faster one, 8 % at worst.
+double chain_iteration_us(int64_t s, int64_t l, int count, bool opts, int sms) {
+  const bool narrow = narrow_tiles(s, l, count, sms);
+  const int bn = narrow ? 64 : 128;
+  const int64_t rs = rounds(sym_tiles(s, bn) * count, sms), rf = rounds(s / BM * (l / bn) * count, sms);
+  if (rf > kChainTiles) return 0.0;
+  const double epi = 2.5 * (narrow ? 1.0 : 2.0) * (opts ? 1.6 : 1.0), kb = 0.4;
+  const double k1 = kb * (double)((l + 255) / 256), k2 = kb * (double)((s + 255) / 256);
+  const double r1 = (double)rs, r3 = (double)rf;
+  return 3 * 4.0 + r1 * (epi > k1 ? epi : k1) + (r1 + r3) * (epi > k2 ? epi : k2);
+}
+
 cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st) {
   if (launch.count < 1 || launch.count > kChainMax || launch.steps < 1) return cudaErrorInvalidValue;
   ChainLaunch a = launch;
-  const int rows = a.s / BM;
-  const int64_t full64 = (int64_t)rows * (a.l / 64) * a.count, full128 = (int64_t)rows * (a.l / 128) * a.count;
-  // Narrow tiles while they shorten the longest block's work: rounds of 128 x 64 tiles against rounds of 128 x 128.
-  // (256 x 512, 5 iterations: 87 us against 121; 1536 x 2560, where both take four rounds of 64 columns: 202 / 184.)
-  const bool narrow = (full64 + sms - 1) / sms < 2 * ((full128 + sms - 1) / sms);
+  const bool narrow = narrow_tiles(a.s, a.l, a.count, sms);
   const int bn = narrow ? 64 : 128;
-  a.nsym = sym_tiles(a.s, bn);
-  const int64_t widest = narrow ? full64 : full128;
+  a.nsym = (int)sym_tiles(a.s, bn);
+  const int64_t widest = (int64_t)(a.s / BM) * (a.l / bn) * a.count;
   const int grid = (int)(widest < sms ? widest : sms);
   const bool pf = a.q.rht || a.q.four_six;
   if (narrow) return pf ? launch_one<64, true>(pack, a, grid, st) : launch_one<64, false>(pack, a, grid, st);

@@ -159,6 +159,7 @@ __host__ __device__ inline uint32_t rht_signs(uint64_t seed, uint64_t j) {
   return (uint32_t)(z & 0xFFFFu);
 }
 cudaError_t chain_set_attributes();
+double chain_iteration_us(int64_t s, int64_t l, int count, bool opts, int sms);
 cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st);
 
 // Measurement support: counts kernel launches and, when profiling is on, brackets a group of

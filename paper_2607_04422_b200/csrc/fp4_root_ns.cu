@@ -319,18 +319,28 @@ struct MatrixCtx {
   ChainProblem chain;         // for a run of all iterations in one launch
 };
 
-// Which groups run all their iterations in one launch (fp4_chain.cu).  Below the limit a product's time is
-// launch latency and one tile's epilogue, above it the CTA-pair kernel's larger tiles win.  Measured, 5
-// iterations, one launch against fifteen: 1024 x 1024 135 / 190 us, 1536 x 2560 and 4096 x 1024 equal, 2560 x 2560
-// 333 / 290 us; with the paper's quantiser options, whose longer epilogue gains from the narrower tiles,
-// 1024 x 1024 169 / 287 us, 2048 x 2048 327 / 339 us.  (Not for inspection of BF16-stored intermediates: there A and X
-// stay FP32 tensors with rounded values.)
+// Estimated time of one iteration in three launches of the CTA-pair kernel, in us (see chain_iteration_us): a launch
+// and, per round of 256 x 256 tiles over the SM pairs, an epilogue or a main loop; a partly filled last round
+// costs half of what it lacks.
+double pair_iteration_us(int64_t s, int64_t l, int count, bool opts, int sms) {
+  const double ts = (double)((s + 255) / 256), tl = (double)((l + 255) / 256), pairs = (double)(sms / 2);
+  auto rounds = [](double r) { return (std::ceil(r) + (r > 1.0 ? r : 1.0)) / 2; };
+  const double epi = 6.0 * (opts ? 1.7 : 1.0), kb = 0.3;
+  const double k1 = kb * tl, k2 = kb * ts;
+  const double rs = rounds(ts * (ts + 1) / 2 * count / pairs), rf = rounds(ts * tl * count / pairs);
+  return 3 * 8.0 + rs * (epi > k1 ? epi : k1) + (rs + rf) * (epi > k2 ? epi : k2);
+}
+
+// Which groups run all their iterations in one launch (fp4_chain.cu): those for which that is estimated to be faster -
+// single matrices up to about 4 M elements, groups of short ones up to 15 M.  Measured, 5 iterations, one launch
+// against fifteen: 4 x 512 x 512 106 / 178 us, 2 x 1024 x 2816 194 / 249, 2048 x 2048 220 / 222, 2560 x 2560 330 / 285,
+// 8 x 1536 x 1536 643 / 537; with the quantiser options 2048 x 2048 306 / 338.  (Not for inspection of
+// BF16-stored intermediates: there A and X stay FP32 tensors with rounded values.)
 bool chain_group(const DeviceInfo* d, const NsPlan& pl, int count, const fp4_ns_params* p) {
   if (count > kChainMax || (pl.bf16 && (p->flags & FP4_FLAG_KEEP_OPERANDS))) return false;
   const bool opts = (p->flags & (FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)) != 0;
-  const int64_t elements = pl.s * pl.l * count;
-  const int64_t limit = opts ? (int64_t)9 << 19 : (int64_t)7 << 19;
-  return elements <= limit && elements / (128 * 64) <= (int64_t)d->sms * kChainTiles;
+  const double t = chain_iteration_us(pl.s, pl.l, count, opts, d->sms);
+  return t > 0.0 && t <= pair_iteration_us(pl.s, pl.l, count, opts, d->sms);
 }
 
 fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t m, int64_t n, int steps,
