@@ -193,6 +193,8 @@ cudaError_t launch_momentum_update(const float* G, int64_t rows, int64_t cols, f
 struct AdamwConsts {
   float b1, b2, omb1, omb2, eps, rsb2, step_size, decay;
   uint64_t seed;
+  float one;   // 1, kept from the compiler (fp4_adamw.cu)
+  bool plain;  // rsb2 and eps leave sqrt(v) rsb2 + eps in the range of the unguarded square root and division
 };
 AdamwConsts adamw_consts(float lr, float beta1, float beta2, float eps, float weight_decay, int step, uint64_t seed);
 cudaError_t launch_adamw_update(uint16_t* W, const uint16_t* G, int64_t n, const AdamwConsts& k, bool sr,

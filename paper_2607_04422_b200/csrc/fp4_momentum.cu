@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(256) k_momentum_update(const float* __restrict
     float g[16], m[16];
     ldg_f32x8(G + b * 16, g);
     ldg_f32x8(G + b * 16 + 8, g + 8);
-    mom_decode(c_in, s_in, m);
+    mom_decode<!HIST>(c_in, s_in, m);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       float a0, a1, b0, b1;
@@ -68,7 +68,8 @@ __global__ void __launch_bounds__(256) k_momentum_update(const float* __restrict
     }
     uint2 c_out;
     uint32_t s_out;
-    mom_encode<SR>(m, seed, (uint64_t)b * 16, c_out, s_out);
+    hadamard16_pairs(m);
+    state_encode<SR>(m, seed, (uint64_t)b * 16, c_out, s_out);
     *reinterpret_cast<uint2*>(codes + b * 8) = c_out;
     scales[b] = (uint16_t)s_out;
   }
@@ -85,7 +86,7 @@ __global__ void __launch_bounds__(256) k_momentum_decode(const uint8_t* __restri
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nblocks; b += stride) {
     float m[16];
-    mom_decode(__ldg(reinterpret_cast<const uint2*>(codes + b * 8)), __ldg(scales + b), m);
+    mom_decode<false>(__ldg(reinterpret_cast<const uint2*>(codes + b * 8)), __ldg(scales + b), m);
     stg_f32x8(M_out + b * 16, m);
     stg_f32x8(M_out + b * 16 + 8, m + 8);
   }

@@ -135,3 +135,22 @@ def test_argument_errors():
         fp4.fp4_adamw_update(W[8:264], G[:256], mc, ms, vc, vs, vm, lr=1e-3)      # W 16- but not 32-byte aligned
     fp4.fp4_adamw_update(W, G, mc, ms, vc, vs, vm, lr=1e-3)                       # and the good call works
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("exp", [-45, -38, -37, -30, 14, 16, 17, 38])
+def test_square_root_and_quotient_range_limits(exp):
+    # v and m around the limits of the unguarded square root and division (2^-80, 2^30), mixed within a block and with zeros;
+    # eps = 0 leaves the denominator to v alone
+    n = 256 * 8
+    rng = np.random.default_rng(exp & 255)
+    W = _weights(n, seed=4)
+    g = rng.standard_normal(n) * np.exp2(rng.integers(exp - 2, exp + 3, n).astype(np.float64))
+    g[256:512] *= np.repeat(np.exp2(rng.integers(-20, 20, 16).astype(np.float64)), 16)
+    g[512:768][rng.random(256) < 0.1] = 0.0
+    gb = oracle.bf16_bits(g.astype(np.float32))
+    gpu, st = GpuAdam(W), None
+    for t, eps in ((1, 1e-8), (2, 0.0 if exp > -40 else 1e-30), (3, 1e-8)):
+        hp = {**HP, "eps": eps}
+        gpu.step(gb, t, sr=t == 2, seed=t, **hp)
+        W, st, _, _ = oracle.adamw_update(W, gb, st, step=t, sr=t == 2, seed=t, **hp)
+        _compare(gpu, W, st)
