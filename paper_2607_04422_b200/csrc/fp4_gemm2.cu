@@ -68,8 +68,10 @@ constexpr uint32_t ACC1_COL = PN - CHUNK;      // 240
 // SMs keeps in flight (the plain product runs at 2.9 / 3.9 / 4.7 PFLOP/s with 2 / 3 / 4 stages), so every
 // mode takes as many stages as its epilogue leaves room for: the modes that combine with an FP32 tile
 // (G2, G3) need two chunk buffers per warp - one in work, one being fetched - and fit three stages; the
-// others (G1, the plain product) stage their result in one buffer and fit four.
-template <int MODE>
+// others (G1, the plain product) stage their result in one buffer and fit four.  DEEP gives G2 and G3 four stages, too: one
+// buffer per warp, into which the next chunk is fetched when this one has left it, so the epilogue of a tile waits for four
+// fetches - worth it where the main loop of the next tile is longer still (launch_pair_mode).
+template <int MODE, bool DEEP = false>
 struct Lay {
   static constexpr bool HAS_AUX = (MODE == kG2 || MODE == kG3);
   static constexpr int BK = HAS_AUX ? FP4_BK_AUX : 256;        // elements of K per stage: 64- or 128-byte operand rows
@@ -81,8 +83,8 @@ struct Lay {
   static constexpr int SF_ATOMS = KSTEPS * 512;                // scale atoms of one 128-row block and stage
   static constexpr int SF_BYTES = 3 * SF_ATOMS;                // row operand: own block; column operand: both blocks
   static constexpr uint32_t STAGE_BYTES_CTA = 2 * OPER_BYTES + SF_BYTES;
-  static constexpr int STAGES = HAS_AUX ? FP4_STAGES_AUX : FP4_STAGES_NOAUX;
-  static constexpr int XBUF = HAS_AUX ? 2 : 1;                 // FP32 chunk buffers per warp
+  static constexpr int STAGES = HAS_AUX && !DEEP ? FP4_STAGES_AUX : FP4_STAGES_NOAUX;
+  static constexpr int XBUF = HAS_AUX && !DEEP ? 2 : 1;                 // FP32 chunk buffers per warp
   static constexpr int WARP_AREA = XBUF * XBUF_BYTES + RQ_BYTES;
   static constexpr int OFF_A = 0;
   static constexpr int OFF_B = OFF_A + STAGES * OPER_BYTES;
@@ -286,10 +288,10 @@ __device__ __forceinline__ void stg256(void* p, const uint32_t (&r)[8]) {
 // UPD: the last G3 stage of a call that also applies Root's parameter update (args.update): every lane
 //   loads the 16 BF16 weights under its row of a chunk (one 32-byte sector, fetched a chunk ahead),
 //   forms W * decay - step * X+ from the values it holds and stores the sector back.
-template <int MODE, bool PF, bool BH, bool UPD = false>
+template <int MODE, bool PF, bool BH, bool UPD, bool DEEP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ GemmLaunch args) {
-  using L = Lay<MODE>;
+  using L = Lay<MODE, DEEP>;
   constexpr int STAGES = L::STAGES, XBUF = L::XBUF, WARP_AREA = L::WARP_AREA;
   constexpr int BK = L::BK, KSTEPS = L::KSTEPS, OPER_BYTES = L::OPER_BYTES, SF_ATOMS = L::SF_ATOMS, SF_BYTES = L::SF_BYTES;
   constexpr uint32_t STAGE_BYTES_CTA = L::STAGE_BYTES_CTA, OPER_SBO = L::OPER_SBO, OPER_SWIZZLE = L::OPER_SWIZZLE;
@@ -552,7 +554,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
       if (HAS_AUX) {
         // chunk position e of slot i: i on buffer 1, 3 - i on buffer 0 (seq = 0 uses buffer 0)
         fetch(probs + cur.p, cur.x64, cur.y32, 3, cur.below, 0);
-        fetch(probs + cur.p, cur.x64, cur.y32, 2, cur.below, 1);
+        if (XBUF == 2) fetch(probs + cur.p, cur.x64, cur.y32, 2, cur.below, 1);
       }
     }
     for (; t < num_tiles; t += num_pairs, ++seq) {
@@ -628,9 +630,9 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         if (HAS_AUX) {
 #pragma unroll
           for (int i = 0; i < TEAM_CHUNKS; ++i) {
-            wait_or_abort(xfull0 + (i & 1) * 8, (uint32_t)(i >> 1), abort_flag);
-            if (i < 2) fetch(pr, x64, y32, (i + 2) ^ flip, true, i & 1);
-            else if (has_next) fetch(probs + nxt.p, nxt.x64, nxt.y32, (i - 2) ^ (flip ^ 3), nxt.below, i & 1);
+            wait_or_abort(xfull0 + i % XBUF * 8, (uint32_t)(i / XBUF & 1), abort_flag);
+            if (i < TEAM_CHUNKS - XBUF) fetch(pr, x64, y32, (i + XBUF) ^ flip, true, i % XBUF);
+            else if (has_next) fetch(probs + nxt.p, nxt.x64, nxt.y32, (i + XBUF - TEAM_CHUNKS) ^ (flip ^ 3), nxt.below, i % XBUF);
           }
         }
         cur = nxt;
@@ -663,13 +665,13 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
 #pragma unroll
       for (int i = 0; i < TEAM_CHUNKS; ++i) {
         const int e = i ^ flip;                         // position of this chunk among the warp's 64 columns
-        const int b = i & 1;
-        const uint32_t boff = (XBUF == 2 ? b : 0) * XBUF_BYTES;   // without a fetched tile: one staging buffer
+        const int b = i % XBUF;
+        const uint32_t boff = b * XBUF_BYTES;
         const int xcol = x64 + e * CHUNK;
         float v[16];
         if (HAS_AUX) {
           TR_BEGIN
-          wait_or_abort(xfull0 + b * 8, (uint32_t)(i >> 1), abort_flag);
+          wait_or_abort(xfull0 + b * 8, (uint32_t)(i / XBUF & 1), abort_flag);
           TR_END(1)
         }
         tc_wait_ld16(acc);
@@ -840,8 +842,8 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         TR_END(3)
         if (XBUF == 1) __syncwarp();  // one buffer: the next chunk is staged over this one, after the store's read
         if (HAS_AUX) {
-          if (i < 2) fetch(pr, x64, y32, (i + 2) ^ flip, false, b);
-          else if (has_next) fetch(probs + nxt.p, nxt.x64, nxt.y32, (i - 2) ^ (flip ^ 3), nxt.below, b);
+          if (i < TEAM_CHUNKS - XBUF) fetch(pr, x64, y32, (i + XBUF) ^ flip, false, b);
+          else if (has_next) fetch(probs + nxt.p, nxt.x64, nxt.y32, (i + XBUF - TEAM_CHUNKS) ^ (flip ^ 3), nxt.below, b);
         }
         if (do_q) {
           if (i == 0) {
@@ -910,15 +912,27 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
   if (threadIdx.x == 0 && bars->abort_flag) report_timeout(args.status);
 }
 
-template <int MODE, bool PF, bool BH, bool UPD = false>
-cudaError_t launch_pair_mode(const ProblemPack& pack, const GemmLaunch& L, int sms, cudaStream_t st) {
+template <int MODE, bool PF, bool BH, bool UPD, bool DEEP>
+cudaError_t launch_pair_variant(const ProblemPack& pack, const GemmLaunch& L, int sms, cudaStream_t st) {
   const int tpp = L.symmetric ? L.tiles_n * (L.tiles_n + 1) / 2 : L.tiles_m * L.tiles_n;
   const int num_tiles = tpp * L.num_problems;
   int pairs = sms / 2;
   if (pairs > num_tiles) pairs = num_tiles;
   count_launches(1);
-  launch_chained(k_gemm_pair<MODE, PF, BH, UPD>, dim3(2 * pairs), dim3(NTHREADS), Lay<MODE>::SMEM_BYTES, st, pack, L);
+  launch_chained(k_gemm_pair<MODE, PF, BH, UPD, DEEP>, dim3(2 * pairs), dim3(NTHREADS), Lay<MODE, DEEP>::SMEM_BYTES, st, pack, L);
   return cudaGetLastError();
+}
+
+// G2 and G3 with a long contraction take the deep layout: there the main loop of a tile outlasts its epilogue, even one that
+// waits for every block of the FP32 tile.  Measured, G2 + G3 of 5 iterations, without / with: 16384 x 16384 20.1 / 18.0 ms,
+// 8192 x 8192 2.72 / 2.42, 4096 x 14336 1.10 / 0.99, 3072 x 8192 0.50 / 0.50.  The quantiser options double the
+// epilogue: 8192 x 8192 2.60 / 2.30, 4096 x 16384 1.28 / 1.34 ms.
+template <int MODE, bool PF, bool BH, bool UPD = false>
+cudaError_t launch_pair_mode(const ProblemPack& pack, const GemmLaunch& L, int sms, cudaStream_t st) {
+  if constexpr (MODE == kG2 || MODE == kG3) {
+    if (L.K >= (PF ? 5120 : 4096)) return launch_pair_variant<MODE, PF, BH, UPD, true>(pack, L, sms, st);
+  }
+  return launch_pair_variant<MODE, PF, BH, UPD, false>(pack, L, sms, st);
 }
 
 }  // namespace
@@ -934,24 +948,31 @@ extern "C" int fp4_trace_read(unsigned long long* dst, int clear) {
 }
 #endif
 
+template <int MODE, bool PF, bool BH, bool UPD, bool DEEP>
+static cudaError_t set_attribute() {
+  return cudaFuncSetAttribute(k_gemm_pair<MODE, PF, BH, UPD, DEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              Lay<MODE, DEEP>::SMEM_BYTES);
+}
+template <int MODE, bool DEEP>
+static cudaError_t set_attributes() {
+  cudaError_t e;
+  if ((e = set_attribute<MODE, false, false, false, DEEP>())) return e;
+  if ((e = set_attribute<MODE, false, true, false, DEEP>())) return e;
+  if ((e = set_attribute<MODE, true, false, false, DEEP>())) return e;
+  return set_attribute<MODE, true, true, false, DEEP>();
+}
 cudaError_t gemm_pair_set_attributes() {
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kPlain, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kPlain>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG1>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG1>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG1>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG1, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG1>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG2>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG2, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG2>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG2, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG2>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG2, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG2>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG3, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG3>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG3, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG3>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG3, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG3>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG3, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG3>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG3, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG3>::SMEM_BYTES))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_pair<kG3, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<kG3>::SMEM_BYTES))) return e;
-  return cudaSuccess;
+  if ((e = set_attribute<kPlain, false, false, false, false>())) return e;
+  if ((e = set_attributes<kG1, false>())) return e;
+  if ((e = set_attributes<kG2, false>())) return e;
+  if ((e = set_attributes<kG2, true>())) return e;
+  if ((e = set_attributes<kG3, false>())) return e;
+  if ((e = set_attributes<kG3, true>())) return e;
+  if ((e = set_attribute<kG3, false, false, true, false>())) return e;
+  if ((e = set_attribute<kG3, false, true, true, false>())) return e;
+  if ((e = set_attribute<kG3, false, false, true, true>())) return e;
+  return set_attribute<kG3, false, true, true, true>();
 }
 
 // Elements of K per operand stage of a mode: the operand and scale descriptors of a problem are built
@@ -975,6 +996,11 @@ cudaError_t launch_gemm_pair(GemmMode mode, const ProblemPack& pack, const GemmL
   L.blocks_n = launch.tiles_n;
   L.tiles_m = (launch.tiles_m + 1) / 2;
   L.tiles_n = (launch.tiles_n + 1) / 2;
+  // Row order reads the whole column operand once per row of tiles, which is cheap as long as it stays in the L2 (126 MB, shared
+  // with the streaming FP32 tile); beyond that, bands of 8 rows keep the 74 tiles in flight near a square.  Measured, 5
+  // iterations, row order / bands: 16384 x 16384 24.9 / 21.1 ms, 12288 x 12288 10.9 / 10.0, 8192 x 16384 6.3 / 5.75, 8192 x 8192
+  // (a column operand of 32 MB) 3.45 / 3.36, 6144 x 6144 (18 MB) 1.68 / 1.73.  Bands of 6 and 12 rows: +1 %.
+  L.band = (int64_t)L.blocks_n * 128 * L.K / 2 >= (int64_t)32 << 20 ? 8 : 1;
   const bool pf = launch.q.rht || launch.q.four_six;
   const bool bh = launch.aux_h != 0 || launch.out_h != 0;
 #define FP4_PAIR_CASE(M)                                                                \

@@ -73,20 +73,38 @@ __device__ __forceinline__ void grid_barrier(uint32_t* counter, uint32_t round, 
   __syncthreads();
 }
 
-// tile index of a launch -> (problem, tile row, tile column)
+// tile index of a launch -> (problem, tile row, tile column): bands of L.band tile rows, each walked column by column
+// (only the tiles on and above the diagonal of a symmetric product); a band of one row is plain row order
 __device__ __forceinline__ void decode_tile(int t, const GemmLaunch& L, int tiles_per_problem, int& p, int& ti,
                                             int& tj, bool sym) {
   p = t / tiles_per_problem;
   t -= p * tiles_per_problem;
-  const int tiles_n = L.tiles_n;
+  const int tiles_n = L.tiles_n, band = L.band;
   if (!sym) {
-    ti = t / tiles_n;
-    tj = t - ti * tiles_n;
+    const int b = t / (band * tiles_n);
+    t -= b * band * tiles_n;
+    const int h = min(band, L.tiles_m - b * band);   // the last band may be lower
+    tj = t / h;
+    ti = b * band + (t - tj * h);
   } else {
-    int row = 0, rem = t;
-    while (rem >= tiles_n - row) { rem -= tiles_n - row; ++row; }
-    ti = row;
-    tj = row + rem;
+    int row = 0, h = min(band, tiles_n);
+    for (;;) {
+      // h rows from `row` on: a triangle of h columns, then whole columns
+      const int in_band = h * (h + 1) / 2 + (tiles_n - row - h) * h;
+      if (t < in_band) break;
+      t -= in_band;
+      row += h;
+      h = min(band, tiles_n - row);
+    }
+    int col = 0;
+    while (col < h && t > col) { t -= col + 1; ++col; }
+    if (col == h) {
+      const int c = t / h;
+      col += c;
+      t -= c * h;
+    }
+    ti = row + t;
+    tj = row + col;
   }
 }
 

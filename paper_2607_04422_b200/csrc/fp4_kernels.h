@@ -100,6 +100,7 @@ struct GemmLaunch {
   int K;               // contraction length in elements (multiple of 128)
   int tiles_m, tiles_n;        // callers: in blocks of 128; inside the kernel: 256 x 256 tiles, rounded up
   int blocks_m, blocks_n;      // extent in blocks of 128 (set by launch_gemm_pair)
+  int band;            // tile rows per band of the tile order (set by launch_gemm_pair)
   int symmetric;       // only tiles with tile_n >= tile_m; mirrored quantised output
   int iter;            // Newton-Schulz iteration index k
   int write_q;         // emit the quantised outputs
