@@ -26,7 +26,8 @@ struct NsHeader {
   uint32_t cand_count;   // candidates appended by the second pass (may exceed the list's capacity)
   uint32_t overflow;     // 1: the candidate list overflowed, the fallback passes run
   uint32_t tiles_done;   // tiles of the matrix's products stored so far (single-launch iterations)
-  uint32_t pad[19];
+  uint32_t ticket;       // blocks of the select that are through
+  uint32_t pad[18];
   uint32_t barrier;      // of the single-launch prologue (first matrix of a group); cleared by the host
 };
 

@@ -4,19 +4,17 @@
 // group needs six launches instead of six per matrix; a group that fits the shared memories of all SMs
 // needs one (kp_resident, at the end).
 //
-// Clip threshold tau = nearest-rank quantile of |g|, found exactly with two passes over
-// the data where three were needed before:
+// Clip threshold tau = nearest-rank quantile of |g|, found exactly with two passes over the data:
 //   pass 1  histogram of the top 13 magnitude bits (exponent + 5 mantissa bits);
 //   pick    the bin that holds the wanted rank;
 //   pass 2  elements of that bin are appended to a candidate list (they are about 1 % of a
-//           continuous distribution); in the same pass the squares of all elements below
-//           the bin are summed in FP64 (they are certainly not clipped);
-//   finish  one block per matrix selects tau among the candidates (two shared-memory radix
-//           rounds over the remaining 18 bits), adds the candidates' squares exactly (they
-//           share an exponent, so their squares add as integers) and tau^2 for every clipped
-//           element, and derives nu, 1/(nu+eps), amax(X0) and the tensor scale of X0.
+//           continuous distribution) and counted by their next 9 bits; in the same pass the squares of all
+//           elements below the bin are summed in FP64 (they are certainly not clipped);
+//   finish  the candidates are gone through once more, for their last 9 bits: tau, the candidates' squares
+//           exactly (they share an exponent, so their squares add as integers) and tau^2 for every clipped
+//           element give nu, 1/(nu+eps), amax(X0) and the tensor scale of X0.
 // If the bin holds more candidates than the list can take (many equal values, e.g. a
-// constant matrix) the finishing block itself continues the radix select with two more passes
+// constant matrix) one finishing block continues the radix select with two more passes
 // over the matrix and a statistics pass (slow, rare, no extra launch).
 #include <stddef.h>
 
@@ -85,6 +83,75 @@ constexpr int kTopBits = 13;                 // bits of the first radix pass
 constexpr int kTopShift = 31 - kTopBits;     // 18
 constexpr int kTopBins = 1 << kTopBits;      // 8192
 
+// True in every thread of the last of `blocks` thread blocks that get here: it sees what the others wrote before.
+__device__ __forceinline__ bool last_block(uint32_t* ticket, uint32_t blocks) {
+  __shared__ uint32_t s_ticket;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_ticket = atomicAdd(ticket, 1u);
+    __threadfence();
+  }
+  __syncthreads();
+  return s_ticket == blocks - 1;
+}
+
+// The bin of the 8192 counters that holds rank hdr->sel_rank: becomes the prefix; the rank is reduced to one within
+// the bin and the counters are cleared.  For 512 threads.
+__device__ __forceinline__ void pick_top_bin(NsHeader* hdr, uint32_t* hist) {
+  constexpr int PER = kTopBins / 512;
+  __shared__ uint32_t wtot[16];
+  uint32_t local[PER];
+  uint32_t sum = 0;
+  if ((reinterpret_cast<uintptr_t>(hist) & 15) == 0) {
+#pragma unroll
+    for (int j = 0; j < PER; j += 4) {
+      const uint4 v = __ldcg(reinterpret_cast<const uint4*>(hist + threadIdx.x * PER + j));
+      local[j] = v.x; local[j + 1] = v.y; local[j + 2] = v.z; local[j + 3] = v.w;
+    }
+  } else {   // a caller's histogram need only be 4-byte aligned
+#pragma unroll
+    for (int j = 0; j < PER; ++j) local[j] = __ldcg(hist + threadIdx.x * PER + j);
+  }
+#pragma unroll
+  for (int j = 0; j < PER; ++j) sum += local[j];
+  // exclusive prefix of the chunk sums: scan inside each warp, then add the totals of the warps before
+  uint32_t incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    if ((int)(threadIdx.x & 31) >= o) incl += t;
+  }
+  if ((threadIdx.x & 31) == 31) wtot[threadIdx.x >> 5] = incl;
+  const uint32_t rank = hdr->sel_rank;
+  __syncthreads();
+  uint32_t before = incl - sum;
+  for (int w = 0; w < (int)(threadIdx.x >> 5); ++w) before += wtot[w];
+  if (rank > before && rank <= before + sum) {
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      if (rank > before && rank <= before + local[j]) {
+        hdr->sel_prefix = (uint32_t)(threadIdx.x * PER + j) << kTopShift;
+        hdr->sel_rank = rank - before;
+        hdr->bin_count = local[j];
+        hdr->count_below = before;
+      }
+      before += local[j];
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < PER; ++j) hist[threadIdx.x * PER + j] = 0;
+}
+
+// (The last block of the histogram could do this, too: then every block waits for its counts to arrive before it takes its
+// ticket, and the histogram of sixteen 3072 x 3072 took 144 us instead of 116 + 10.)
+__global__ void __launch_bounds__(512) kp_pick_top(const __grid_constant__ PrepGroup g) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const PrepMatrix& m = g.mat[blockIdx.y];
+  pick_top_bin(m.hdr, m.hist_top ? m.hist_top : m.hist);
+}
+
 // ---- pass 1: histogram of the top 13 magnitude bits
 __global__ void __launch_bounds__(512) kp_hist_top(const __grid_constant__ PrepGroup g) {
   pdl_launch_dependents();
@@ -120,72 +187,20 @@ __global__ void __launch_bounds__(512) kp_hist_top(const __grid_constant__ PrepG
     if (sh[j]) atomicAdd(&m.hist[j], sh[j]);
 }
 
-// ---- pick: the bin (of NB bins of a histogram) that holds rank hdr->sel_rank; extends the
-// prefix by bin << SHIFT, reduces the rank, clears the histogram
-template <int NB>
-__device__ __forceinline__ void pick_bin(NsHeader* hdr, uint32_t* hist, int shift, uint32_t* bin_count_out,
-                                         uint32_t* below_out) {
-  constexpr int PER = NB / 256;
-  static_assert(PER % 4 == 0, "a thread reads its counters as 16-byte pieces");
-  __shared__ uint32_t wtot[8];
-  uint32_t local[PER];
-  uint32_t sum = 0;
-  if ((reinterpret_cast<uintptr_t>(hist) & 15) == 0) {
-#pragma unroll
-    for (int j = 0; j < PER; j += 4) {
-      const uint4 v = *reinterpret_cast<const uint4*>(hist + threadIdx.x * PER + j);
-      local[j] = v.x; local[j + 1] = v.y; local[j + 2] = v.z; local[j + 3] = v.w;
-    }
-  } else {   // a caller's histogram need only be 4-byte aligned
-#pragma unroll
-    for (int j = 0; j < PER; ++j) local[j] = hist[threadIdx.x * PER + j];
-  }
-#pragma unroll
-  for (int j = 0; j < PER; ++j) sum += local[j];
-  // exclusive prefix of the 256 chunk sums: scan inside each warp, then add the totals of the warps before
-  uint32_t incl = sum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-    if ((int)(threadIdx.x & 31) >= o) incl += t;
-  }
-  if ((threadIdx.x & 31) == 31) wtot[threadIdx.x >> 5] = incl;
-  __syncthreads();
-  uint32_t before = incl - sum;
-  for (int w = 0; w < (int)(threadIdx.x >> 5); ++w) before += wtot[w];
-  const uint32_t rank = hdr->sel_rank;
-  __syncthreads();
-  if (rank > before && rank <= before + sum) {
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      if (rank > before && rank <= before + local[j]) {
-        hdr->sel_prefix |= (uint32_t)(threadIdx.x * PER + j) << shift;
-        hdr->sel_rank = rank - before;
-        if (bin_count_out) *bin_count_out = local[j];
-        if (below_out) *below_out = before;
-      }
-      before += local[j];
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < PER; ++j) hist[threadIdx.x * PER + j] = 0;
-}
-
-__global__ void __launch_bounds__(256) kp_pick_top(const __grid_constant__ PrepGroup g) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const PrepMatrix& m = g.mat[blockIdx.y];
-  pick_bin<kTopBins>(m.hdr, m.hist_top ? m.hist_top : m.hist, kTopShift, &m.hdr->bin_count, &m.hdr->count_below);
-}
+constexpr int kSubBins = 512;                 // counters of bits 17..9 and of bits 8..0 of the candidates
 
 // ---- pass 2: candidates of the picked bin, FP64 sum of squares below the bin, max |g|.
 // Candidates are rare: they are collected in a shared-memory buffer per block and copied to
-// the global list with one reservation per block (or directly when the buffer is full).
-__global__ void __launch_bounds__(256) kp_compact_stats(const __grid_constant__ PrepGroup g) {
+// the global list with one reservation per block (or directly when the buffer is full); on the way there the next 9
+// bits of each are counted, in the counters the first pass has left cleared.
+// Eight blocks per SM: the 1024 blocks of a matrix are resident at once.  (With 40 registers and six blocks an eighth of them
+// ran as a second wave: 16384 x 16384 248 us against 178, 6.0 TB/s; 4096 x 8192 36 against 27.5.)
+__global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant__ PrepGroup g) {
   pdl_launch_dependents();
   pdl_wait();
   constexpr uint32_t kBuf = 2048;
   __shared__ uint32_t s_buf[kBuf];
+  __shared__ uint32_t s_sub[kSubBins];
   __shared__ uint32_t s_cnt, s_base;
   const PrepMatrix& m = g.mat[blockIdx.y];
   const uint32_t bin = g.clip ? (m.hdr->sel_prefix >> kTopShift) : 0xFFFFFFFFu;
@@ -208,6 +223,7 @@ __global__ void __launch_bounds__(256) kp_compact_stats(const __grid_constant__ 
       } else {
         const uint32_t gpos = atomicAdd(&m.hdr->cand_count, 1u);
         if (gpos < g.cand_cap) m.cand[gpos] = k;
+        atomicAdd(&m.hist[(k >> 9) & (kSubBins - 1)], 1u);
       }
     }
   };
@@ -242,6 +258,16 @@ __global__ void __launch_bounds__(256) kp_compact_stats(const __grid_constant__ 
   for (uint32_t j = threadIdx.x; j < nbuf; j += blockDim.x) {
     const uint32_t gpos = s_base + j;
     if (gpos < g.cand_cap) m.cand[gpos] = s_buf[j];
+  }
+  if (nbuf <= kSubBins) {
+    for (uint32_t j = threadIdx.x; j < nbuf; j += blockDim.x) atomicAdd(&m.hist[(s_buf[j] >> 9) & (kSubBins - 1)], 1u);
+  } else {   // fewer global atomics by way of shared counters
+    for (int j = threadIdx.x; j < kSubBins; j += blockDim.x) s_sub[j] = 0;
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < nbuf; j += blockDim.x) atomicAdd(&s_sub[(s_buf[j] >> 9) & (kSubBins - 1)], 1u);
+    __syncthreads();
+    for (int j = threadIdx.x; j < kSubBins; j += blockDim.x)
+      if (s_sub[j]) atomicAdd(&m.hist[j], s_sub[j]);
   }
 }
 
@@ -331,117 +357,103 @@ __device__ void fallback_select_and_stats(const PrepGroup& g, const PrepMatrix& 
   }
 }
 
-// ---- finish: select tau among the candidates and derive the normalisation scalars
+// What the select's blocks of a matrix add up (in the matrix's counters behind the 512 of bits 17..9).
+struct SelectSums {
+  uint32_t low[kSubBins];          // candidates of the picked sub-bin by their last 9 bits
+  unsigned long long lo, hi;       // exact squares of the candidates below the sub-bin, in two parts
+  uint32_t above;                  // candidates above it
+};
+
+// Exclusive prefix of one value per thread over a block of 1024 threads; `wtot`: 32 words.
+__device__ __forceinline__ uint32_t block_prefix(uint32_t v, uint32_t* wtot) {
+  uint32_t incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    if ((int)(threadIdx.x & 31) >= o) incl += t;
+  }
+  if ((threadIdx.x & 31) == 31) wtot[threadIdx.x >> 5] = incl;
+  __syncthreads();
+  uint32_t w = wtot[threadIdx.x & 31], s = w;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, s, o);
+    if ((int)(threadIdx.x & 31) >= o) s += t;
+  }
+  const uint32_t before = __shfl_sync(0xffffffffu, s - w, (int)(threadIdx.x >> 5));
+  __syncthreads();
+  return before + incl - v;
+}
+
+// ---- finish: select tau among the candidates and derive the normalisation scalars.
+// The candidates share their top 13 bits.  Every block finds the sub-bin of bits 17..9 from the counters of the second
+// pass and goes through its share of the list: members of the sub-bin are counted by their last 9 bits, and the
+// squares of those below it (certainly not clipped) are summed as exact integers -- all candidates share the
+// exponent field, so x = mant * 2^(e-150) with a 24-bit integer mant.  The last block picks tau.
+// (One block alone, counting both halves of the bits itself, took 135 us for the candidates of 16384 x 16384 and 26 us for
+// those of 4096 x 8192; now 12 us each.)
 __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ PrepGroup g) {
   pdl_launch_dependents();
   pdl_wait();
   const PrepMatrix& m = g.mat[blockIdx.y];
   __shared__ double shd[1024];
-  __shared__ uint32_t hist[1024];
+  __shared__ uint32_t hist[kSubBins];
+  __shared__ uint32_t wtot[32];
   __shared__ uint32_t s_prefix, s_rank;
   __shared__ unsigned long long s_lo, s_hi;
   __shared__ uint32_t s_above;
   NsHeader* hdr = m.hdr;
+  const int tid = threadIdx.x;
   if (!g.clip) {
+    if (blockIdx.x) return;
     const double total = sum_partials(m.partial, g.stat_blocks, shd);
-    if (threadIdx.x == 0)
+    if (tid == 0)
       write_norm_scalars(m.scalars, g.ix, norm_scalars(total, __uint_as_float(hdr->maxabs_bits), g.eps, g.q.widen));
     return;
   }
   const uint32_t count = hdr->cand_count;
   if (count > g.cand_cap) {
-    if (threadIdx.x == 0) hdr->overflow = 1;
+    if (blockIdx.x) return;
+    if (tid == 0) hdr->overflow = 1;
     __shared__ uint32_t fb_hist[2048];
     fallback_select_and_stats(g, m, fb_hist, shd);
     return;
   }
-  // two radix rounds over the low 18 bits of the candidates: 9 bits each.  The second round
-  // also gathers what the norm needs: squares of the candidates below the sub-bin picked by
-  // the first round (certainly not clipped) as exact integers -- all candidates share the
-  // exponent field, so x = mant * 2^(e-150) with a 24-bit integer mant -- and the number above it.
-  if (threadIdx.x == 0) { s_prefix = hdr->sel_prefix; s_rank = hdr->sel_rank; s_lo = 0; s_hi = 0; s_above = 0; }
+  SelectSums* sums = reinterpret_cast<SelectSums*>(m.hist + kSubBins);
+  const uint32_t top = hdr->sel_prefix, top_rank = hdr->sel_rank;
+  const uint32_t efield = top >> 23;
+  const uint32_t implicit = efield ? 0x800000u : 0u;
+  if (tid == 0) { s_lo = 0; s_hi = 0; s_above = 0; }
+  if (tid < kSubBins) hist[tid] = 0;
+  {
+    const uint32_t c = tid < kSubBins ? m.hist[tid] : 0u;
+    const uint32_t before = block_prefix(c, wtot);
+    if (c && top_rank > before && top_rank <= before + c) {
+      s_prefix = top | ((uint32_t)tid << 9);
+      s_rank = top_rank - before;
+    }
+  }
+  __syncthreads();
+  const uint32_t prefix = s_prefix, rank = s_rank;
   unsigned long long lo = 0, hi = 0;
   uint32_t above = 0;
-  const uint32_t efield = hdr->sel_prefix >> 23;
-  const uint32_t implicit = efield ? 0x800000u : 0u;
-  for (int round = 0; round < 2; ++round) {
-    const int shift = round == 0 ? 9 : 0;
-    const uint32_t high_mask = ~((1u << (shift + 9)) - 1u) & 0x7FFFFFFFu;
-    hist[threadIdx.x] = 0;
-    __syncthreads();
-    const uint32_t prefix = s_prefix;
-    for (uint32_t i0 = threadIdx.x; i0 < count; i0 += 8 * blockDim.x) {
-      uint32_t k[8];
+  const uint32_t stride = gridDim.x * blockDim.x;
+  for (uint32_t i0 = blockIdx.x * blockDim.x + tid; i0 < count; i0 += 8 * stride) {
+    uint32_t k[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const uint32_t i = i0 + u * blockDim.x;
-        k[u] = i < count ? m.cand[i] : 0xFFFFFFFFu;
-      }
+    for (int u = 0; u < 8; ++u) k[u] = i0 + u * (uint64_t)stride < count ? m.cand[i0 + u * stride] : 0xFFFFFFFFu;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        if (k[u] == 0xFFFFFFFFu) continue;
-        if ((k[u] & high_mask) == (prefix & high_mask)) {
-          atomicAdd(&hist[(k[u] >> shift) & 511u], 1u);
-        } else if (round == 1) {
-          if (k[u] < prefix) {
-            const unsigned long long mant = (k[u] & 0x7FFFFFu) | implicit;
-            const unsigned long long sq = mant * mant;
-            lo += sq & 0xFFFFFFull;
-            hi += sq >> 24;
-          } else {
-            above += 1;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    // the bin that holds the rank: inclusive scan of the 512 counters by the first warps
-    if (threadIdx.x < 512) {
-      // each of 16 warps scans 32 bins; warp totals are then scanned by thread 0
-      uint32_t v = hist[threadIdx.x], incl = v;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-        if ((threadIdx.x & 31) >= o) incl += t;
-      }
-      hist[512 + threadIdx.x] = incl;            // inclusive within the warp's 32 bins
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t run = 0;
-      const uint32_t rank = s_rank;
-      for (int w = 0; w < 16; ++w) {
-        const uint32_t wt = hist[512 + w * 32 + 31];
-        if (rank <= run + wt) {
-          for (int b = 0; b < 32; ++b) {
-            const uint32_t incl = run + hist[512 + w * 32 + b];
-            if (rank <= incl) {
-              s_prefix = prefix | ((uint32_t)(w * 32 + b) << shift);
-              s_rank = rank - (incl - hist[w * 32 + b]);
-              break;
-            }
-          }
-          break;
-        }
-        run += wt;
-      }
-    }
-    __syncthreads();
-  }
-  const uint32_t tau_bits = s_prefix;
-  // candidates inside the last sub-bin: a counter of the second round stands for one exact
-  // magnitude (all 31 bits known), so its members' squares are count * mant^2
-  if (threadIdx.x < 512) {
-    const uint32_t cnt = hist[threadIdx.x];
-    const uint32_t kk = (tau_bits & ~511u) | threadIdx.x;
-    if (cnt) {
-      if (kk <= tau_bits) {
-        const unsigned long long mant = (kk & 0x7FFFFFu) | implicit;
+    for (int u = 0; u < 8; ++u) {
+      if (k[u] == 0xFFFFFFFFu) continue;
+      if ((k[u] & ~511u) == prefix) {
+        atomicAdd(&hist[k[u] & 511u], 1u);
+      } else if (k[u] < prefix) {
+        const unsigned long long mant = (k[u] & 0x7FFFFFu) | implicit;
         const unsigned long long sq = mant * mant;
-        lo += (unsigned long long)cnt * (sq & 0xFFFFFFull);
-        hi += (unsigned long long)cnt * (sq >> 24);
+        lo += sq & 0xFFFFFFull;
+        hi += sq >> 24;
       } else {
-        above += cnt;
+        above += 1;
       }
     }
   }
@@ -452,14 +464,58 @@ __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ Prep
     hi += __shfl_xor_sync(0xffffffffu, hi, o);
     above += __shfl_xor_sync(0xffffffffu, above, o);
   }
-  if ((threadIdx.x & 31) == 0) {
+  if ((tid & 31) == 0) {
+    atomicAdd(&s_lo, lo);
+    atomicAdd(&s_hi, hi);
+    atomicAdd(&s_above, above);
+  }
+  __syncthreads();
+  if (gridDim.x > 1) {
+    if (tid < kSubBins && hist[tid]) atomicAdd(&sums->low[tid], hist[tid]);
+    if (tid == 0) {
+      atomicAdd(&sums->lo, s_lo);
+      atomicAdd(&sums->hi, s_hi);
+      atomicAdd(&sums->above, s_above);
+    }
+    if (!last_block(&hdr->ticket, gridDim.x)) return;
+    if (tid < kSubBins) hist[tid] = __ldcg(&sums->low[tid]);
+    if (tid == 0) { s_lo = __ldcg(&sums->lo); s_hi = __ldcg(&sums->hi); s_above = __ldcg(&sums->above); }
+    __syncthreads();
+  }
+  const uint32_t cnt = tid < kSubBins ? hist[tid] : 0u;
+  {
+    const uint32_t before = block_prefix(cnt, wtot);
+    if (cnt && rank > before && rank <= before + cnt) s_prefix = prefix | (uint32_t)tid;
+  }
+  __syncthreads();
+  const uint32_t tau_bits = s_prefix;
+  // a counter stands for one exact magnitude (all 31 bits known), so its members' squares are count * mant^2
+  lo = 0; hi = 0; above = 0;
+  if (cnt) {
+    const uint32_t kk = prefix | (uint32_t)tid;
+    if (kk <= tau_bits) {
+      const unsigned long long mant = (kk & 0x7FFFFFu) | implicit;
+      const unsigned long long sq = mant * mant;
+      lo = (unsigned long long)cnt * (sq & 0xFFFFFFull);
+      hi = (unsigned long long)cnt * (sq >> 24);
+    } else {
+      above = cnt;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    lo += __shfl_xor_sync(0xffffffffu, lo, o);
+    hi += __shfl_xor_sync(0xffffffffu, hi, o);
+    above += __shfl_xor_sync(0xffffffffu, above, o);
+  }
+  if (tid < kSubBins && (tid & 31) == 0) {
     atomicAdd(&s_lo, lo);
     atomicAdd(&s_hi, hi);
     atomicAdd(&s_above, above);
   }
   __syncthreads();
   const double below = sum_partials(m.partial, g.stat_blocks, shd);
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     const float tau = __uint_as_float(tau_bits);
     const int e2 = 2 * ((int)(efield ? efield : 1u) - 150);
     const double cand_sq = ldexp((double)s_hi * 16777216.0 + (double)s_lo, e2);
@@ -933,27 +989,6 @@ struct ResidentShared {
 constexpr int kResSmem = kResTiles * kPrepTile + kResUnion + (int)sizeof(ResidentShared) + 1024;
 static_assert(kResSmem + 64 <= 232448, "at most 227 KB of shared memory (64 bytes of it static, in the fallback)");
 
-// Exclusive prefix of one value per thread over a block of 1024 threads; `wtot`: 32 words.
-__device__ __forceinline__ uint32_t block_prefix(uint32_t v, uint32_t* wtot) {
-  uint32_t incl = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-    if ((int)(threadIdx.x & 31) >= o) incl += t;
-  }
-  if ((threadIdx.x & 31) == 31) wtot[threadIdx.x >> 5] = incl;
-  __syncthreads();
-  uint32_t w = wtot[threadIdx.x & 31], s = w;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, s, o);
-    if ((int)(threadIdx.x & 31) >= o) s += t;
-  }
-  const uint32_t before = __shfl_sync(0xffffffffu, s - w, (int)(threadIdx.x >> 5));
-  __syncthreads();
-  return before + incl - v;
-}
-
 template <bool PF>
 __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_constant__ PrepGroup g) {
   extern __shared__ uint8_t prep_smem_raw[];
@@ -1398,14 +1433,16 @@ cudaError_t launch_prologue_group(const PrologueItem* items, int count, int writ
       count_launches(1);
       if (g.clip) {
         if (!all_counted) launch_chained(kp_hist_top, gh, dim3(512), 0, st, g);
-        launch_chained(kp_pick_top, gy1, dim3(256), 0, st, g);
+        launch_chained(kp_pick_top, gy1, dim3(512), 0, st, g);
         count_launches(all_counted ? 1 : 2);
       }
     }
     {
       ProfScope ps(FP4_PROF_STATS, st);
       launch_chained(kp_compact_stats, gs, dim3(256), 0, st, g);
-      launch_chained(kp_finalize, gy1, dim3(1024), 0, st, g);
+      // a block of the select per 4 M elements: some 10 k candidates of a Gaussian matrix
+      const int64_t fb = g.n4 >> 20;
+      launch_chained(kp_finalize, dim3((unsigned)(fb < 1 ? 1 : fb < 64 ? fb : 64), (unsigned)nn), dim3(1024), 0, st, g);
       count_launches(2);
     }
     {

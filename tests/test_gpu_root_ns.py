@@ -754,3 +754,29 @@ def test_prologue_waits_for_the_block_that_finishes_an_overflowed_select(kind):
     G = rng.choice([-3.0, 3.0] if kind == "constant" else [-1.0, 0.5, 2.0], (m, n)).astype(np.float32)
     got, _ = run_gpu(G, steps=1)
     assert rel(got, oracle.root_ns(G, steps=1)) <= TOL_OUT
+
+
+@pytest.mark.parametrize("shape", [(2048, 4096), (2048, 4080)])
+@pytest.mark.parametrize("spread", [0.0, 1e-3, 1.0])
+def test_select_by_several_blocks(shape, spread):
+    """From 8 M elements on several blocks go through the candidates.  A tenth of the elements lies in the bin of the
+    threshold (thousands per block of the statistics pass), on few values, within one sub-bin or over all of them."""
+    m, n = shape
+    rng = np.random.default_rng(int(spread * 1000) + n)
+    G = rng.standard_normal((m, n)).astype(np.float32) * np.float32(0.1)
+    top = rng.random((m, n)) < 0.1
+    G[top] = (np.float32(2.0) + np.float32(0.06 * spread) * rng.random(int(top.sum()), dtype=np.float32)) if spread else \
+        rng.choice([2.0, 2.01, 2.05], int(top.sum())).astype(np.float32)
+    flags = FP4_FLAG_KEEP_OPERANDS
+    Gd = torch.from_numpy(G).cuda()
+    out = torch.empty_like(Gd)
+    ws = torch.full((fp4.fp4_root_ns_workspace_bytes(m, n, 1, flags),), 0xFF, dtype=torch.uint8, device="cuda")
+    fp4.fp4_root_ns(Gd, out, 1, fp4.NsParams.make(flags=flags), ws)
+    assert fp4.fp4_last_device_status(ws) == 0
+    lay = fp4_root_ns_workspace_layout(m, n, 1, flags)
+    sc = ws[lay.scalars:lay.scalars + 4096].cpu().numpy().view(np.float32)
+    a = np.abs(G).ravel()
+    rank = -(-99 * a.size // 100)
+    tau = np.partition(a, rank - 1)[rank - 1]
+    assert sc[lay.idx_tau] == tau
+    assert sc[lay.idx_nu] == np.float32(np.sqrt(np.square(np.minimum(a, tau).astype(np.float64)).sum()))
