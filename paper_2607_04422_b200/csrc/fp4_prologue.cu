@@ -758,6 +758,7 @@ __device__ __forceinline__ void prep_tile(const PrepGroup& g, const PrepMatrix& 
   if (g.write_q) {
     uint8_t* sf_stage = stage + 8 * kQtSlot;
     const uint32_t tb = tile + base_off;
+    const uint64_t inv2 = pack2(ps.inv, ps.inv);
     if (row_warp) {
       uint32_t code[4];
       uint32_t sfw = 0;
@@ -772,14 +773,14 @@ __device__ __forceinline__ void prep_tile(const PrepGroup& g, const PrepMatrix& 
                        : "r"(tb + (((uint32_t)(q * 4 + i) << 4) ^ sw)));
         uint32_t sb;
         if (PF) {
-          float v[16], unused;
+          float v[16];
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             float a, b2;
-            unpack2(g2[i], a, b2);
-            v[2 * i] = x0(a); v[2 * i + 1] = x0(b2);
+            unpack2(mul2(g2[i], inv2), a, b2);
+            v[2 * i] = fminf(fmaxf(a, -ps.tinv), ps.tinv); v[2 * i + 1] = fminf(fmaxf(b2, -ps.tinv), ps.tinv);
           }
-          sb = quantize_block16_opts(v, g.q, ps.sg, code[2 * q], code[2 * q + 1], unused);
+          sb = quantize_block16_opts(v, g.q, ps.sg, code[2 * q], code[2 * q + 1]);
         } else {
           bool rare;
           sb = prep_quant_row(g2, ps, code[2 * q], code[2 * q + 1], rare);
@@ -816,7 +817,8 @@ __device__ __forceinline__ void prep_tile(const PrepGroup& g, const PrepMatrix& 
       }
       uint32_t cw[4], sb0 = 0, sb1 = 0;
       if (PF) {
-        float unused;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) g2[i] = mul2(g2[i], inv2);   // clamped to tinv below: fl(clamp(g, tau) inv)
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           float v[16];
@@ -824,9 +826,9 @@ __device__ __forceinline__ void prep_tile(const PrepGroup& g, const PrepMatrix& 
           for (int i = 0; i < 16; ++i) {
             float a, b2;
             unpack2(g2[i], a, b2);
-            v[i] = x0(j == 0 ? a : b2);
+            v[i] = fminf(fmaxf(j == 0 ? a : b2, -ps.tinv), ps.tinv);
           }
-          const uint32_t sb = quantize_block16_opts(v, g.q, ps.sg, cw[2 * j], cw[2 * j + 1], unused);
+          const uint32_t sb = quantize_block16_opts(v, g.q, ps.sg, cw[2 * j], cw[2 * j + 1]);
           if (j == 0) sb0 = sb; else sb1 = sb;
         }
       } else {

@@ -98,8 +98,7 @@ __global__ void __launch_bounds__(256) k_quantize_rows_opts(const float* __restr
     v[4 * j] = t.x; v[4 * j + 1] = t.y; v[4 * j + 2] = t.z; v[4 * j + 3] = t.w;
   }
   uint32_t lo, hi;
-  float unused;
-  const uint32_t sb = quantize_block16_opts(v, q, sg, lo, hi, unused);
+  const uint32_t sb = quantize_block16_opts(v, q, sg, lo, hi);
   *reinterpret_cast<uint2*>(codes + r * (cols / 2) + kb * 8) = make_uint2(lo, hi);
   scales[sf_offset(r, kb, cols >> 4)] = (uint8_t)sb;
 }
@@ -197,8 +196,7 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
     read(i, v);
     const uint32_t b = (uint32_t)(first + i * step) * 128 + row;   // block of the tensor
     uint32_t lo, hi, sb;
-    float unused;
-    if (PF) sb = quantize_block16_opts(v, q, sg, lo, hi, unused);
+    if (PF) sb = quantize_block16_opts(v, q, sg, lo, hi);
     else sb = quantize_block16(v, six_sg, sg, lo, hi);
     *reinterpret_cast<uint2*>(codes + (int64_t)b * 8) = make_uint2(lo, hi);
     const uint32_t r = b / kblocks;

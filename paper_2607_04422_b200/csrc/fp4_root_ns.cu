@@ -220,6 +220,7 @@ QuantOpts quant_opts(const fp4_ns_params* p, uint64_t j) {
   q.four_six = (p->flags & FP4_FLAG_FOUR_SIX) ? 1u : 0u;
   q.mask = q.rht ? rht_signs(p->seed, j) : 0u;
   q.widen = q.rht ? 4.0f : 1.0f;
+  q.minus_one = -1.0f;
   return q;
 }
 
@@ -731,6 +732,7 @@ fp4_status fp4_quantize(const float* x, int64_t rows, int64_t cols, uint8_t* cod
   q.four_six = (flags & FP4_FLAG_FOUR_SIX) ? 1u : 0u;
   q.mask = flags >> 16;
   q.widen = q.rht ? 4.0f : 1.0f;
+  q.minus_one = -1.0f;
   if (!shape_ok(rows) || !shape_ok(cols)) return FP4_ERR_SHAPE;
   if (!aligned(x, 16) || !aligned(codes, 16) || !aligned(scales, 16) || !aligned(tensor_scale, 4))
     return FP4_ERR_ALIGNMENT;

@@ -86,9 +86,6 @@ __device__ __forceinline__ uint32_t cvt_rs_e2m1x4(float v0, float v1, float v2, 
   return r;
 }
 
-__device__ __forceinline__ void half2_to_float2(uint32_t h, float& a, float& b) {
-  asm("{\n\t.reg .f16 x, y;\n\tmov.b32 {x, y}, %2;\n\tcvt.f32.f16 %0, x;\n\tcvt.f32.f16 %1, y;\n\t}" : "=f"(a), "=f"(b) : "r"(h));
-}
 __device__ __forceinline__ uint32_t hadd2(uint32_t a, uint32_t b) {
   uint32_t r;
   asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
