@@ -602,7 +602,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
             uint32_t lo, hi;
             float bmax;
             uint32_t sb;
-            if (PF) sb = quantize_block16_opts_p2(v, qo, inv_sg, lo, hi, bmax);
+            if (PF) sb = quantize_block16_opts_p2<false>(v, qo, inv_sg, lo, hi, bmax);
             else sb = quantize_block16_p2(v, inv_sg, lo, hi, bmax);
             amax = fmaxf(amax, bmax);
             // the stores of the tile two back have read the staging area
@@ -610,7 +610,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
             sts_u2(os + (ch >> 2) * 4096 + row * 32 + (((ch & 3) * 8) ^ ((lane & 4) << 2)), lo, hi);
             sts_b(os + L::RQ + L::CQ + (ch >> 2) * 512 + lane * 16 + quad * 4 + (ch & 3), sb);
             if (mirror) {
-              if (PF) sb = quantize_block16_opts_p2(w, qo, inv_sg, lo, hi, bmax);
+              if (PF) sb = quantize_block16_opts_p2<false>(w, qo, inv_sg, lo, hi, bmax);
               else sb = quantize_block16_p2(w, inv_sg, lo, hi, bmax);
               if (!PF && g) { lo = swap_nibbles(lo); hi = swap_nibbles(hi); }   // back into row order
               const int col = ch * CHUNK + cq;

@@ -824,7 +824,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         if (do_q) {
           float bmax;
           uint32_t sb;
-          if (PF) sb = quantize_block16_opts_p2(v, args.q, inv_sg, rlo, rhi, bmax);
+          if (PF) sb = quantize_block16_opts_p2<true>(v, args.q, inv_sg, rlo, rhi, bmax);
           else sb = quantize_block16_p2(v, inv_sg, rlo, rhi, bmax);
           if (MODE == kG1 || MODE == kG3) amax = fmaxf(amax, bmax);
           sfw |= sb << (8 * e);
@@ -866,7 +866,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
               w[k] = g ? c : a;
               w[k + 1] = g ? a : c;
             }
-            sb = quantize_block16_opts_p2(w, args.q, inv_sg, lo, hi, bmax);
+            sb = quantize_block16_opts_p2<true>(w, args.q, inv_sg, lo, hi, bmax);
           } else {
             sb = quantize_block16_p2(w, inv_sg, lo, hi, bmax);
             if (g) { lo = swap_nibbles(lo); hi = swap_nibbles(hi); }   // back into row order

@@ -221,6 +221,7 @@ QuantOpts quant_opts(const fp4_ns_params* p, uint64_t j) {
   q.mask = q.rht ? rht_signs(p->seed, j) : 0u;
   q.widen = q.rht ? 4.0f : 1.0f;
   q.minus_one = -1.0f;
+  set_signs(q);
   return q;
 }
 
@@ -733,6 +734,7 @@ fp4_status fp4_quantize(const float* x, int64_t rows, int64_t cols, uint8_t* cod
   q.mask = flags >> 16;
   q.widen = q.rht ? 4.0f : 1.0f;
   q.minus_one = -1.0f;
+  set_signs(q);
   if (!shape_ok(rows) || !shape_ok(cols)) return FP4_ERR_SHAPE;
   if (!aligned(x, 16) || !aligned(codes, 16) || !aligned(scales, 16) || !aligned(tensor_scale, 4))
     return FP4_ERR_ALIGNMENT;
