@@ -178,7 +178,8 @@ fp4_status fp4_root_coeffs(int64_t m, int64_t n, int steps, float abc[3]);
  *   (and a transpose pass for a tall matrix on the routes that cannot write the result
  *   transposed from the last product).  Groups of up to a few million elements run all
  *   iterations in one cooperative launch instead, whose blocks wait on one another (bounded
- *   waits).  Calls on small matrices (up to 8 M elements per group
+ *   waits); somewhat larger ones (short sides up to 2048) run two of the three products of an
+ *   iteration in such a launch.  Calls on small matrices (up to 8 M elements per group
  *   of equal shapes) chain their other kernels with programmatic dependent launch; the environment
  *   variable FP4ROOT_NO_PDL (any value) switches that off.  Kernels launched before or after
  *   the call on the same stream see ordinary stream order either way.
@@ -383,7 +384,7 @@ fp4_status fp4_adamw_update(uint16_t* W, const uint16_t* G, int64_t n, uint8_t* 
 /* ---- measurement support (the paper has no counterpart) -----------------------------------
  * While profiling is enabled, every group of launches of the step is bracketed by a pair of
  * CUDA events on the caller's stream; fp4_profile_collect waits for them, adds the elapsed
- * times per class into ms[class] (iterations that run in one launch count as FP4_PROF_G3) and
+ * times per class into ms[class] (iterations that run in one launch count as FP4_PROF_G3, G1 and G2 in one launch as FP4_PROF_G1) and
  * the number of bracketed groups into groups[class]
  * (both host arrays of FP4_PROF_CLASSES entries), then forgets them.  Off by default; the
  * events add stream operations, so time whole calls with profiling off.

@@ -164,7 +164,8 @@ __device__ __noinline__ void chain_update_tall(uint16_t* w, int64_t ld, const fl
     *w = (uint16_t)cvt_bf16x2(param_update_value(bf16_lo(*w), v[i], decay, step), 0.0f);
 }
 
-template <int BN, bool PF>
+// SYM: the products [a.first, a.end) only, G1 and G2 of an iteration (loop bounds the compiler cannot unroll by); else all products of all iterations
+template <int BN, bool PF, bool SYM>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLaunch a) {
   using L = ChainLay<BN>;
@@ -180,6 +181,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
   const int my_sym = (nsym * a.count - (int)blockIdx.x + grid - 1) / grid;
   const int my_full = (nfull * a.count - (int)blockIdx.x + grid - 1) / grid;
   const int products = 3 * a.steps;
+  const int first = SYM ? a.first : 0, end = SYM ? a.end : products;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < STAGES; ++i) { mbar_init(&sh->full[i], 1); mbar_init(&sh->empty[i], 1); }
@@ -210,13 +212,15 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
     // ------------------------------------------------------------ operand producer
     if (elect_one()) {
       int st = 0; uint32_t ph = 0, n = 0;
-      for (int pi = 0; pi < products; ++pi) {
+      for (int pi = first; pi < end; ++pi) {
         const int k = pi / 3, mode = pi - 3 * k + kG1;
         const bool sym = mode != kG3;
         const int mine = sym ? my_sym : my_full;
         const int K = mode == kG1 ? a.l : a.s;
         const int num_kb = (K + BK - 1) / BK;
-        const uint32_t need = (uint32_t)(k * (2 * nsym + nfull) + (mode - kG1) * nsym);
+        // tiles of the matrix's earlier products (SYM: what the launches before have left is complete)
+        const uint32_t need = SYM ? (mode == kG1 ? 0u : (uint32_t)((2 * k + 1) * nsym))
+                                  : (uint32_t)(k * (2 * nsym + nfull) + (mode - kG1) * nsym);
         int seen = -1;
         for (int j = 0; j < mine; ++j, ++n) {
           const uint32_t tile = sh->tiles[sym ? 0 : 1][j];
@@ -265,7 +269,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
     // ------------------------------------------------------------ MMA issuer
     if (elect_one()) {
       int st = 0; uint32_t ph = 0, n = 0;
-      for (int pi = 0; pi < products; ++pi) {
+      for (int pi = first; pi < end; ++pi) {
         const int mode = pi % 3 + kG1;
         const bool sym = mode != kG3;
         const int mine = sym ? my_sym : my_full;
@@ -308,7 +312,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
   } else if (warp == W_STORE) {
     // ------------------------------------------------------------ stores of the quantised outputs
     uint32_t n = 0;
-    for (int pi = 0; pi < products; ++pi) {
+    for (int pi = first; pi < end; ++pi) {
       const int k = pi / 3, mode = pi - 3 * k + kG1;
       const bool sym = mode != kG3;
       const int mine = sym ? my_sym : my_full;
@@ -396,7 +400,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
 
     uint32_t n = 0, unit = 0, xph = 0;   // tiles, units, phases of the two block barriers
     bool have = false;                   // the copy of the unit at hand is under way
-    for (int pi = 0; pi < products; ++pi) {
+    for (int pi = first; pi < end; ++pi) {
       const int k = pi / 3, mode = pi - 3 * k + kG1;
       const bool sym = mode != kG3;
       const int mine = sym ? my_sym : my_full;
@@ -636,7 +640,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
         }
       }
       // The next product's first block: once this warp's own stores (its A, its X) have arrived.
-      if (mine > 0) for (int np = pi + 1; np < products && np <= pi + 3; ++np) {
+      if (mine > 0) for (int np = pi + 1; np < end && np <= pi + 3; ++np) {
         const int nk = np / 3, nmode = np - 3 * nk + kG1;
         const int nmine = nmode != kG3 ? my_sym : my_full;
         if (nmine == 0) continue;
@@ -660,7 +664,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
   if (threadIdx.x == 0 && sh->abort_flag) report_timeout(a.status);
 }
 
-template <int BN, bool PF>
+template <int BN, bool PF, bool SYM = false>
 cudaError_t launch_one(const ChainPack& pack, const ChainLaunch& a, int grid, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = ChainLay<BN>::SMEM; cfg.stream = st;
@@ -669,7 +673,7 @@ cudaError_t launch_one(const ChainPack& pack, const ChainLaunch& a, int grid, cu
   attr[0].val.cooperative = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
   count_launches(1);
-  return cudaLaunchKernelEx(&cfg, k_chain<BN, PF>, pack, a);
+  return cudaLaunchKernelEx(&cfg, k_chain<BN, PF, SYM>, pack, a);
 }
 
 int64_t sym_tiles(int64_t s, int bn) {
@@ -678,51 +682,76 @@ int64_t sym_tiles(int64_t s, int bn) {
   return n;
 }
 int64_t rounds(int64_t tiles, int sms) { return (tiles + sms - 1) / sms; }
-// Narrow tiles while they shorten the longest block's work: rounds of 128 x 64 tiles against rounds of 128 x 128.
-// (256 x 512, 5 iterations: 87 us against 121; 1536 x 2560, where both take four rounds of 64 columns: 202 / 184.)
-bool narrow_tiles(int64_t s, int64_t l, int count, int sms) {
-  const int64_t full128 = s / BM * (l / 128) * count;
-  return rounds(2 * full128, sms) < 2 * rounds(full128, sms);
-}
-
 }  // namespace
 
 cudaError_t chain_set_attributes() {
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_chain<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<64>::SMEM))) return e;
-  if ((e = cudaFuncSetAttribute(k_chain<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<64>::SMEM))) return e;
-  if ((e = cudaFuncSetAttribute(k_chain<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<128>::SMEM))) return e;
-  if ((e = cudaFuncSetAttribute(k_chain<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<128>::SMEM))) return e;
+  if ((e = cudaFuncSetAttribute(k_chain<64, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<64>::SMEM))) return e;
+  if ((e = cudaFuncSetAttribute(k_chain<64, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<64>::SMEM))) return e;
+  if ((e = cudaFuncSetAttribute(k_chain<128, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<128>::SMEM))) return e;
+  if ((e = cudaFuncSetAttribute(k_chain<128, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<128>::SMEM))) return e;
+  if ((e = cudaFuncSetAttribute(k_chain<128, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<128>::SMEM))) return e;
+  if ((e = cudaFuncSetAttribute(k_chain<128, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<128>::SMEM))) return e;
   return cudaSuccess;
 }
 
-// Estimated time of one iteration in us: per product a dependency round trip, and rounds of tiles that take an epilogue
-// or a main loop each, whichever is longer (0 when a block would take more tiles than its list holds).  The constants of
-// this estimate and of the CTA-pair kernel's beside its caller are fitted to both kernels' times at 75 shapes and
-// groups, 256 to 3072 wide, plain and with the quantiser options; choosing by them loses 0.6 % on average against
-// always knowing the faster one, 8 % at worst.
-double chain_iteration_us(int64_t s, int64_t l, int count, bool opts, int sms) {
-  const bool narrow = narrow_tiles(s, l, count, sms);
-  const int bn = narrow ? 64 : 128;
+// Estimated times in us.  A product costs a dependency round trip and rounds of tiles that take an epilogue or a main
+// loop each, whichever is longer.  The constants here and of the CTA-pair kernel's estimate beside the caller are fitted to
+// the times of all routes at 54 shapes and groups, 128 to 2560 wide, plain and with the quantiser options; choosing by
+// them loses 0.5 % on average against always knowing the fastest, 4 % at worst.
+struct TileUs {
+  double epi, k1, k2;   // epilogue; main loop of G1; of G2 and G3
+  TileUs(int bn, int64_t s, int64_t l, bool opts)
+      : epi(2.5 * (bn / 64) * (opts ? 1.6 : 1.0)), k1(0.4 * (double)((l + 255) / 256)), k2(0.4 * (double)((s + 255) / 256)) {}
+  double g1() const { return epi > k1 ? epi : k1; }
+  double g23() const { return epi > k2 ? epi : k2; }
+};
+// one iteration of a single launch with tiles of bn columns; 0 when a block would take more tiles than its list holds
+static double width_us(int bn, int64_t s, int64_t l, int count, bool opts, int sms) {
   const int64_t rs = rounds(sym_tiles(s, bn) * count, sms), rf = rounds(s / BM * (l / bn) * count, sms);
   if (rf > kChainTiles) return 0.0;
-  const double epi = 2.5 * (narrow ? 1.0 : 2.0) * (opts ? 1.6 : 1.0), kb = 0.4;
-  const double k1 = kb * (double)((l + 255) / 256), k2 = kb * (double)((s + 255) / 256);
-  const double r1 = (double)rs, r3 = (double)rf;
-  return 3 * 4.0 + r1 * (epi > k1 ? epi : k1) + (r1 + r3) * (epi > k2 ? epi : k2);
+  const TileUs t(bn, s, l, opts);
+  return 3 * 4.0 + (double)rs * t.g1() + (double)(rs + rf) * t.g23();
+}
+// The width of a single launch's tiles.  Measured, 5 iterations, 64 / 128 columns: 256 x 512 95 / 126 us, 1024 x 4096
+// 185 / 212 (with the quantiser options 240 / 293), 8 x 768 x 768 176 / 211, 1536 x 4096 264 / 261, 2048 x 2048 228 / 224.
+static bool narrow_tiles(int64_t s, int64_t l, int count, bool opts, int sms) {
+  const double n = width_us(64, s, l, count, opts, sms), w = width_us(128, s, l, count, opts, sms);
+  return n > 0.0 && n <= w;
+}
+double chain_iteration_us(int64_t s, int64_t l, int count, bool opts, int sms) {
+  return width_us(narrow_tiles(s, l, count, opts, sms) ? 64 : 128, s, l, count, opts, sms);
+}
+// G1 and G2 of an iteration in a launch of their own, where every SM has at most one tile (else 0)
+double chain_symmetric_us(int64_t s, int64_t l, int count, bool opts, int sms) {
+  if (sym_tiles(s, 128) * count > sms) return 0.0;
+  const TileUs t(128, s, l, opts);
+  return 12.0 + t.g1() + t.g23();
 }
 
 cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st) {
   if (launch.count < 1 || launch.count > kChainMax || launch.steps < 1) return cudaErrorInvalidValue;
   ChainLaunch a = launch;
-  const bool narrow = narrow_tiles(a.s, a.l, a.count, sms);
+  const bool pf = a.q.rht || a.q.four_six;
+  const bool narrow = narrow_tiles(a.s, a.l, a.count, pf, sms);
   const int bn = narrow ? 64 : 128;
   a.nsym = (int)sym_tiles(a.s, bn);
   const int64_t widest = (int64_t)(a.s / BM) * (a.l / bn) * a.count;
   const int grid = (int)(widest < sms ? widest : sms);
-  const bool pf = a.q.rht || a.q.four_six;
   if (narrow) return pf ? launch_one<64, true>(pack, a, grid, st) : launch_one<64, false>(pack, a, grid, st);
   return pf ? launch_one<128, true>(pack, a, grid, st) : launch_one<128, false>(pack, a, grid, st);
+}
+
+// G1 and G2 of iteration `step` in one launch with a 128 x 128 tile per SM.
+cudaError_t launch_chain_symmetric(const ChainPack& pack, const ChainLaunch& launch, int step, int sms, cudaStream_t st) {
+  if (launch.count < 1 || launch.count > kChainMax || launch.steps < 1) return cudaErrorInvalidValue;
+  ChainLaunch a = launch;
+  a.nsym = (int)sym_tiles(a.s, 128);
+  a.first = 3 * step; a.end = a.first + 2;
+  const int64_t widest = (int64_t)a.nsym * a.count;
+  if (widest > sms) return cudaErrorInvalidValue;
+  const int grid = (int)widest;
+  return a.q.rht || a.q.four_six ? launch_one<128, true, true>(pack, a, grid, st) : launch_one<128, false, true>(pack, a, grid, st);
 }
 
 }  // namespace fp4

@@ -141,7 +141,8 @@ struct ChainPack { ChainProblem p[kChainMax]; };
 struct ChainLaunch {
   int count, steps;
   int s, l, s0, l0;          // work shape, the caller's short and long side
-  int nsym;                  // tiles per matrix of a symmetric product (set by launch_chain)
+  int first, end;            // launch_chain_symmetric: its products
+  int nsym;                  // tiles per matrix of a symmetric product (set by the launch)
   int clip, keep, bf16;
   int update, no_out;
   float upd_decay, upd_step;
@@ -162,7 +163,9 @@ __host__ __device__ inline uint32_t rht_signs(uint64_t seed, uint64_t j) {
 }
 cudaError_t chain_set_attributes();
 double chain_iteration_us(int64_t s, int64_t l, int count, bool opts, int sms);
+double chain_symmetric_us(int64_t s, int64_t l, int count, bool opts, int sms);
 cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st);
+cudaError_t launch_chain_symmetric(const ChainPack& pack, const ChainLaunch& launch, int step, int sms, cudaStream_t st);
 
 // Measurement support: counts kernel launches and, when profiling is on, brackets a group of
 // launches with events.

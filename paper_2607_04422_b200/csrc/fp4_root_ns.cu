@@ -321,28 +321,40 @@ struct MatrixCtx {
   ChainProblem chain;         // for a run of all iterations in one launch
 };
 
-// Estimated time of one iteration in three launches of the CTA-pair kernel, in us (see chain_iteration_us): a launch
-// and, per round of 256 x 256 tiles over the SM pairs, an epilogue or a main loop; a partly filled last round
-// costs half of what it lacks.
-double pair_iteration_us(int64_t s, int64_t l, int count, bool opts, int sms) {
-  const double ts = (double)((s + 255) / 256), tl = (double)((l + 255) / 256), pairs = (double)(sms / 2);
-  auto rounds = [](double r) { return (std::ceil(r) + (r > 1.0 ? r : 1.0)) / 2; };
-  const double epi = 6.0 * (opts ? 1.7 : 1.0), kb = 0.3;
-  const double k1 = kb * tl, k2 = kb * ts;
-  const double rs = rounds(ts * (ts + 1) / 2 * count / pairs), rf = rounds(ts * tl * count / pairs);
-  return 3 * 8.0 + rs * (epi > k1 ? epi : k1) + (rs + rf) * (epi > k2 ? epi : k2);
-}
+// Estimated times in us of the CTA-pair kernel's launches (see chain_iteration_us): a launch and, per round of 256 x 256
+// tiles over the SM pairs, an epilogue or a main loop; a partly filled last round costs half of what it lacks.
+struct PairUs {
+  double g1, g2, g3;
+  PairUs(int64_t s, int64_t l, int count, bool opts, int sms) {
+    const double ts = (double)((s + 255) / 256), tl = (double)((l + 255) / 256), pairs = (double)(sms / 2);
+    auto rounds = [](double r) { return (std::ceil(r) + (r > 1.0 ? r : 1.0)) / 2; };
+    const double epi = 6.0 * (opts ? 1.7 : 1.0), kb = 0.3;
+    const double k1 = kb * tl, k2 = kb * ts;
+    const double rs = rounds(ts * (ts + 1) / 2 * count / pairs), rf = rounds(ts * tl * count / pairs);
+    g1 = 8.0 + rs * (epi > k1 ? epi : k1);
+    g2 = 8.0 + rs * (epi > k2 ? epi : k2);
+    g3 = 8.0 + rf * (epi > k2 ? epi : k2);
+  }
+};
 
-// Which groups run all their iterations in one launch (fp4_chain.cu): those for which that is estimated to be faster -
-// single matrices up to about 4 M elements, groups of short ones up to 15 M.  Measured, 5 iterations, one launch
-// against fifteen: 4 x 512 x 512 106 / 178 us, 2 x 1024 x 2816 194 / 249, 2048 x 2048 220 / 222, 2560 x 2560 330 / 285,
-// 8 x 1536 x 1536 643 / 537; with the quantiser options 2048 x 2048 306 / 338.  (Not for inspection of
-// BF16-stored intermediates: there A and X stay FP32 tensors with rounded values.)
-bool chain_group(const DeviceInfo* d, const NsPlan& pl, int count, const fp4_ns_params* p) {
-  if (count > kChainMax || (pl.bf16 && (p->flags & FP4_FLAG_KEEP_OPERANDS))) return false;
+// How a group runs its iterations: all of them in one launch (fp4_chain.cu), three launches of the CTA-pair kernel per
+// iteration, or two - G1 and G2 as one launch with a 128 x 128 tile per SM where their 256 x 256 tiles would leave half of
+// the SM pairs idle, and the pairs' G3.  What is estimated to be fastest.  Measured, 5 iterations, one launch / two / three
+// per iteration: 1024 x 1024 119 / 174 / 179 us, 2048 x 2048 224 / 221 / 231, 2048 x 4096 318 / 287 / 307, 1536 x 6144
+// 339 / 305 / 330, 2048 x 8192 492 / 446 / 450 (with the quantiser options 669 / 604 / 619), 2304 x 2304 295 / - / 264,
+// 4 x 512 x 512 106 / 170 / 179, 2 x 1024 x 2816 200 / 248 / 260.  (Not for inspection of BF16-stored intermediates: in
+// single launches A and X stay FP32 tensors with rounded values.)
+enum Route { kOneLaunch, kTwoLaunches, kThreeLaunches };
+Route route_of(const DeviceInfo* d, const NsPlan& pl, int count, const fp4_ns_params* p) {
+  if (count > kChainMax || (pl.bf16 && (p->flags & FP4_FLAG_KEEP_OPERANDS))) return kThreeLaunches;
   const bool opts = (p->flags & (FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)) != 0;
-  const double t = chain_iteration_us(pl.s, pl.l, count, opts, d->sms);
-  return t > 0.0 && t <= pair_iteration_us(pl.s, pl.l, count, opts, d->sms);
+  const PairUs pair(pl.s, pl.l, count, opts, d->sms);
+  const double three = pair.g1 + pair.g2 + pair.g3;
+  const double sym = chain_symmetric_us(pl.s, pl.l, count, opts, d->sms);
+  const double best = sym > 0.0 && sym + pair.g3 < three ? sym + pair.g3 : three;
+  const double one = chain_iteration_us(pl.s, pl.l, count, opts, d->sms);
+  if (one > 0.0 && one <= best) return kOneLaunch;
+  return best < three ? kTwoLaunches : kThreeLaunches;
 }
 
 fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t m, int64_t n, int steps,
@@ -545,7 +557,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
   const NsPlan& pl0 = mats[0].pl;
   const int64_t s = pl0.s, l = pl0.l;
   pdl_select(s * l * count);
-  const bool chain = steps > 0 && chain_group(d, pl0, count, p);
+  const Route route = steps > 0 ? route_of(d, pl0, count, p) : kThreeLaunches;
   {
     std::vector<PrologueItem> items((size_t)count);
     for (int i = 0; i < count; ++i) {
@@ -556,13 +568,13 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     if (launch_prologue_group(items.data(), count, steps > 0 || keep, quant_opts(p, 0), status, st) != cudaSuccess)
       return FP4_ERR_CUDA;
   }
-  if (chain) {
-    ChainPack pack;
+  ChainPack pack;
+  ChainLaunch a;
+  if (route != kThreeLaunches) {
     for (int j = 0; j < kChainMax; ++j) {
       pack.p[j] = mats[j < count ? j : 0].chain;
       pack.p[j].W = mats[j < count ? j : 0].W;
     }
-    ChainLaunch a;
     memset(&a, 0, sizeof(a));
     a.count = count; a.steps = steps;
     a.s = (int)s; a.l = (int)l; a.s0 = (int)pl0.s0; a.l0 = (int)pl0.l0;
@@ -573,6 +585,8 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     a.seed = p->seed;
     a.ix = pl0.ix;
     a.status = status;
+  }
+  if (route == kOneLaunch) {
     for (int j = 0; j < count; ++j) {
       // the results of tall matrices and the parameter updates are written there, too, unless operand copies are kept
       if (!keep) { direct_out[(size_t)j] = mats[j].pl.tall; fused_update[(size_t)j] = 1; }
@@ -616,7 +630,10 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       L1.rq_K = L1.cq_K = (int)s; L1.write_q = 1;
       L1.q = quant_opts(p, 2 * (uint64_t)k + 1);  // qA_k
       L1.out_h = bf16;
-      {
+      if (route == kTwoLaunches) {
+        ProfScope ps(FP4_PROF_G1, st);
+        if (launch_chain_symmetric(pack, a, k, d->sms, st) != cudaSuccess) return FP4_ERR_CUDA;
+      } else {
         ProfScope ps(FP4_PROF_G1, st);
         if (launch_gemm_pair(kG1, packs[0], L1, d->sms, st) != cudaSuccess)
           return FP4_ERR_CUDA;
@@ -625,7 +642,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       L2.K = (int)s;
       L2.q = quant_opts(p, 2 * (uint64_t)k);      // qB_k meets qX_k^{16x1}
       L2.out_h = 0; L2.aux_h = bf16;
-      {
+      if (route == kThreeLaunches) {
         ProfScope ps(FP4_PROF_G2, st);
         if (launch_gemm_pair(kG2, packs[1], L2, d->sms, st) != cudaSuccess)
           return FP4_ERR_CUDA;

@@ -725,8 +725,9 @@ def test_iterations_in_one_launch_for_a_group_are_those_of_single_calls():
             assert np.array_equal(o.cpu().numpy(), single)
 
 
-@pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX, FP4_FLAG_STORE_BF16])
-@pytest.mark.parametrize("shape", [(2176, 2928), (2928, 2160), (128, 53760)])
+@pytest.mark.parametrize("shape,flags", [(shape, flags) for shape in ((2176, 2928), (2928, 2160))
+                                         for flags in (0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX, FP4_FLAG_STORE_BF16)] +
+                         [((128, 56784), flags) for flags in (0, FP4_FLAG_STORE_BF16)])
 def test_pair_tiles_that_stick_out_of_the_matrix(shape, flags):
     """Work dimensions that are odd multiples of 128, beyond the single-launch sizes: last 256 x 256 tiles with one half
     outside, a last stage of 128 elements of K; with 128 rows one CTA of every pair has nothing to do."""
@@ -780,3 +781,35 @@ def test_select_by_several_blocks(shape, spread):
     tau = np.partition(a, rank - 1)[rank - 1]
     assert sc[lay.idx_tau] == tau
     assert sc[lay.idx_nu] == np.float32(np.sqrt(np.square(np.minimum(a, tau).astype(np.float64)).sum()))
+
+
+@pytest.mark.parametrize("shape,flags", [((2048, 4096), 0), ((2032, 4080), FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX),
+                                         ((4096, 2048), FP4_FLAG_STORE_BF16), ((1520, 6128), 0)])
+def test_symmetric_products_in_one_launch(shape, flags):
+    """G1 and G2 in one cooperative launch with a 128 x 128 tile per SM (136 of 148, and 78), G3 on the CTA pairs: whole tiles,
+    padding, a tall matrix with BF16 storage."""
+    m, n = shape
+    G = workloads.gradient_like(m, n, seed=n)
+    Gd = torch.from_numpy(G).cuda()
+    out = torch.empty_like(Gd)
+    ws = torch.full((fp4.fp4_root_ns_workspace_bytes(m, n, 2, flags),), 0xFF, dtype=torch.uint8, device="cuda")
+    p = fp4.NsParams.make(flags=flags, seed=6)
+    before = fp4.fp4_kernel_launches()
+    fp4.fp4_root_ns(Gd, out, 2, p, ws)
+    assert fp4.fp4_kernel_launches() - before == 6 + 2 * 2      # prologue, 2 per iteration
+    assert fp4.fp4_last_device_status(ws) == 0
+    pf = bool(flags & FP4_FLAG_RHT)
+    want = oracle.root_ns(G, steps=2, rht=pf, four_six=pf, seed=6, store_bf16=bool(flags & FP4_FLAG_STORE_BF16))
+    assert rel(out.cpu().numpy(), want) <= TOL_OUT
+
+
+def test_symmetric_products_in_one_launch_for_a_group():
+    mats = [workloads.gradient_like(*((1280, 5120) if i else (5120, 1280)), seed=60 + i) for i in range(2)]
+    Gs = [torch.from_numpy(g).cuda() for g in mats]
+    outs = [torch.empty_like(g) for g in Gs]
+    ws = torch.empty(fp4.fp4_root_ns_batched_workspace_bytes([g.shape for g in mats], 3), dtype=torch.uint8, device="cuda")
+    fp4.fp4_root_ns_batched(Gs, outs, 3, None, ws)
+    assert fp4.fp4_last_device_status(ws) == 0
+    for g, o in zip(mats, outs):
+        single, _ = run_gpu(g, steps=3)
+        assert np.array_equal(o.cpu().numpy(), single)
