@@ -1195,6 +1195,8 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       continue;
     }
     const bool owner = sh->info[it].pad == 0;
+    if (owner && g.clip && m.hist_top)   // the caller's counters are consumed, whichever way tau is found: every block has read them
+      for (int i = tid; i < kTopBins; i += kPrepThreads) m.hist_top[i] = 0;
     const uint32_t count = g.clip ? __ldcg(&hdr->cand_count) : 0u;
     if (count > g.cand_cap) {
       // so many equal magnitudes that the list overflowed: the owner finishes alone, the others wait for it
@@ -1328,8 +1330,6 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       }
     }
     __syncthreads();
-    if (owner && g.clip && m.hist_top)                    // the caller's counters are consumed
-      for (int i = tid; i < kTopBins; i += kPrepThreads) m.hist_top[i] = 0;
   }
 
   // ---- operand copies of X0 from the resident tiles

@@ -7,6 +7,7 @@ import torch
 import oracle
 import paper_2607_04422_b200 as fp4
 from paper_2607_04422_b200 import workloads
+from paper_2607_04422_b200.binding import fp4_root_ns_workspace_layout
 from helpers import mismatch_report
 
 pytestmark = pytest.mark.gpu
@@ -231,6 +232,37 @@ def test_momentum_histograms_in_a_batched_call():
     for h in hists:
         if h is not None:
             assert int(h.abs().sum().item()) == 0
+
+
+@pytest.mark.parametrize("shape", [(256, 512), (1136, 400), (128, 57088)])
+def test_momentum_histogram_is_consumed_whichever_way_the_clip_level_is_found(shape):
+    """The same counters over three steps: an all-zero momentum and one of few values (more elements in the clip's bin than its
+    candidate list takes), then a dense one.  After every step the counters are zero, and clip level and result are those of the
+    step that counts for itself.  One cooperative prologue launch for the first two shapes, several launches for the last."""
+    rows, cols = shape
+    rng = np.random.default_rng(rows)
+    grads = [np.zeros(shape, np.float32), rng.choice([-1.0, 0.5, 2.0], shape).astype(np.float32), _gradient(rows, cols, seed=4)]
+    st = GpuState(rows, cols)
+    M = torch.empty(shape, device="cuda")
+    hist = torch.zeros(8192, dtype=torch.int32, device="cuda")
+    ws = torch.empty(fp4.fp4_root_ns_workspace_bytes(rows, cols, 1), dtype=torch.uint8, device="cuda")
+    lay = fp4_root_ns_workspace_layout(rows, cols, 1)
+
+    def step(top_hist):
+        out = torch.full(shape, float("nan"), device="cuda")
+        fp4.fp4_root_ns(M, out, 1, fp4.NsParams.make(top_hist=top_hist), ws)
+        assert fp4.fp4_last_device_status(ws) == 0
+        return out, ws[lay.scalars:lay.scalars + 4096].cpu().numpy().view(np.float32)[lay.idx_tau]
+
+    for g in grads:
+        fp4.fp4_momentum_update(torch.from_numpy(g).cuda(), st.codes, st.scales, M, hist, 0.95, 1.0)
+        assert int(hist.sum().item()) == rows * cols
+        got, tau = step([hist])
+        assert int(hist.abs().sum().item()) == 0
+        a = M.abs().flatten()
+        assert tau == a.kthvalue(-(-99 * a.numel() // 100)).values.item()
+        ref, ref_tau = step(None)
+        assert tau == ref_tau and torch.equal(got, ref)
 
 
 def test_optimizer_chain_in_a_cuda_graph():
