@@ -115,13 +115,15 @@ __global__ void __launch_bounds__(256) k_quantize_rows_opts(const float* __restr
 // 512 x 512 15.8 -> 10.  (A ring that streams larger tensors through the same kernel was slower than the two
 // passes below, 185 against 178 us at 16384 x 8192: a quarter of their threads hides less latency.)
 //
-// The barrier's counter and the blocks' maxima lie in the scale buffer (at least 1 KB), which is written only
-// after a second barrier; the counter is cleared by the host.
+// The blocks' maxima lie in the scale buffer (at least 1 KB), which is written only after a second barrier: all have
+// read them by then.  The barriers' counter, cleared by the host, is the word of the tensor scale, which takes the place of
+// the count while slower blocks may still poll it: as an unsigned number a normal FP32 value is larger than any count, so it
+// releases them, too.  A tensor scale so small that its bits are not (below 512 2^-149) is stored by the last
+// of the blocks to count themselves out.  (Counting out always: 13.6 us at 1152 x 2688 instead of 13.2.)
 // ----------------------------------------------------------------------------------
 constexpr int kQUnit = 2048;
 constexpr int kQUnitBytes = kQUnit * 4;
-constexpr int kQMaxBlocks = 240;      // maxima in words 0 .. 239 of the scale buffer
-constexpr int kQCounterWord = 255;
+constexpr int kQMaxBlocks = 256;      // maxima in words 0 .. 255 of the scale buffer
 constexpr int kQGroups = 4, kQHold = 6, kQThreads = kQGroups * 128;
 struct QuantShared {
   uint64_t full[kQGroups][kQHold];
@@ -133,7 +135,7 @@ constexpr int kQSmem = kQGroups * kQHold * kQUnitBytes + (int)sizeof(QuantShared
 template <bool PF>
 __global__ void __launch_bounds__(kQThreads, 1)
 k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols, uint8_t* __restrict__ codes, uint8_t* scales,
-                 float* __restrict__ tensor_scale, const QuantOpts q) {
+                 float* tensor_scale, const QuantOpts q) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   QuantShared* sh = reinterpret_cast<QuantShared*>(smem + kQGroups * kQHold * kQUnitBytes);
@@ -178,7 +180,8 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
     for (int w = 0; w < kQThreads / 32; ++w) mx = fmaxf(mx, sh->wmax[w]);
     scratch[blockIdx.x] = __float_as_uint(mx);
   }
-  grid_barrier(scratch + kQCounterWord, 1, abort_flag);
+  uint32_t* counter = reinterpret_cast<uint32_t*>(tensor_scale);
+  grid_barrier(counter, 1, abort_flag);
   uint32_t bits = 0;
   for (int i = threadIdx.x & 31; i < (int)gridDim.x; i += 32) {
     uint32_t v;
@@ -188,8 +191,11 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
   bits = __reduce_max_sync(0xffffffffu, bits);
   const float sg = scale_exact(__fmul_rn(q.widen, __uint_as_float(bits)));
   const float six_sg = __fmul_rn(6.0f, sg);
-  grid_barrier(scratch + kQCounterWord, 2, abort_flag);   // everyone has read the maxima: scales may be written
-  if (blockIdx.x == 0 && threadIdx.x == 0) *tensor_scale = sg;
+  grid_barrier(counter, 2, abort_flag);   // everyone has read the maxima: scales may be written
+  if (threadIdx.x == 0) {
+    const uint32_t sg_bits = __float_as_uint(sg);
+    if (sg_bits >= 2 * gridDim.x ? blockIdx.x == 0 : atomicAdd(counter, 1u) == 3 * gridDim.x - 1) *counter = sg_bits;
+  }
   const uint32_t kblocks = (uint32_t)(cols >> 4);
   for (int i = 0; i < m; ++i) {
     float v[16];
@@ -282,7 +288,7 @@ cudaError_t launch_quantize(const CUtensorMap* tm, const float* x, int64_t rows,
   const bool pf = q.rht || q.four_six;
   if (tm) {
     const int units = (int)(rows * cols / kQUnit);
-    cudaError_t e = cudaMemsetAsync(scales + kQCounterWord * 4, 0, 4, st);
+    cudaError_t e = cudaMemsetAsync(tensor_scale, 0, 4, st);
     if (e != cudaSuccess) return e;
     int grid = sms < kQMaxBlocks ? sms : kQMaxBlocks;
     if (units < grid) grid = units;

@@ -1,4 +1,6 @@
 """fp4_quantize against the oracle: codes, scales and tensor scale bit for bit."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -155,3 +157,33 @@ def test_single_launch_quantiser_at_its_limits(shape, flags):
         got = sf_from_atoms(scales.cpu().numpy(), rows, cols // 16)
         assert np.array_equal(got, os_), mismatch_report(got, os_)
         assert np.array_equal(codes.cpu().numpy(), oc), mismatch_report(codes.cpu().numpy(), oc)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-41])    # the second: a tensor scale of a few units of 2^-149
+@pytest.mark.parametrize("shape", [(128, 128), (1024, 1152), (1152, 2688)])
+def test_single_launch_quantiser_waits_for_no_word_that_it_overwrites(shape, scale):
+    """Blocks of the single launch go on to write scales while others may still be at its last barrier.  Zero scale bytes
+    throughout the first two atoms - whatever the blocks could share there - must stall nobody: a wait that nothing ends takes
+    two seconds to give up, 200 calls take a few milliseconds."""
+    rows, cols = shape
+    x_np = workloads.gaussian(rows, cols, seed=cols) * np.float32(scale)
+    # below 2^-128 the reciprocal of a block's scale is infinite: 0 times it is a NaN, whose code is nowhere defined
+    x_np[x_np == 0] = scale
+    x_np[:128, :128] = 0
+    if shape == (128, 128):
+        x_np[0, :16] = scale
+    x = torch.from_numpy(x_np).cuda()
+    codes = torch.empty((rows, cols // 2), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(fp4.fp4_scale_bytes(rows, cols), dtype=torch.uint8, device="cuda")
+    ts = torch.empty(1, device="cuda")
+    fp4.fp4_quantize(x, codes, scales, ts)
+    torch.cuda.synchronize()
+    t0 = time.monotonic()
+    for _ in range(200):
+        fp4.fp4_quantize(x, codes, scales, ts)
+    torch.cuda.synchronize()
+    assert time.monotonic() - t0 < 1.0
+    oc, os_, osg = oracle.quantize(x_np)
+    assert np.float32(ts.item()) == np.float32(osg)
+    assert np.array_equal(sf_from_atoms(scales.cpu().numpy(), rows, cols // 16), os_)
+    assert np.array_equal(codes.cpu().numpy(), oc)
