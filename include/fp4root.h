@@ -141,7 +141,9 @@ const char* fp4_status_string(fp4_status s);
  *   consecutive blocks; the scale of (row r, block kb) is at
  *     ((r/128) * (cols/64) + kb/4) * 512 + (r%32)*16 + ((r%128)/32)*4 + kb%4.
  * tensor_scale: device, out, one FP32: s_g = amax(x)/2688 (1 if x is all zero).  It is
- *   also used as scratch while the call runs.
+ *   also used as scratch while the call runs, and so are the scales.  A tensor that fits the shared
+ *   memories of all SMs (7.2 M elements) is quantised in one cooperative launch, whose blocks wait
+ *   on one another (bounded waits): if one gives up, the tensor scale is a NaN, and only then.
  * Decoded value of an element = E2M1 value * E4M3 scale * s_g.  Rounding is to nearest,
  * ties to even, saturating.  Block scale = E4M3(amax_block / (6 s_g)); elements are
  * multiplied by the FP32 reciprocal of (scale * s_g) before conversion.
@@ -408,6 +410,11 @@ uint64_t fp4_kernel_launches(void);
  * The kernel neither traps nor spins past the limit; the context stays usable.
  */
 fp4_status fp4_selftest_bounded_wait(uint32_t* device_status, uint32_t limit_us, cudaStream_t stream);
+/* The single launch of fp4_quantize (no options) with a limit of limit_us microseconds (1 .. 100000) and barriers that expect one
+ * block more than there are: every block gives up.  tensor_scale must be a NaN afterwards; codes and scales have
+ * unspecified values.  Arguments as for fp4_quantize; a tensor too large for one launch: FP4_ERR_SHAPE. */
+fp4_status fp4_selftest_quantize_wait(const float* x, int64_t rows, int64_t cols, uint8_t* codes, uint8_t* scales,
+                                      float* tensor_scale, uint32_t limit_us, cudaStream_t stream);
 
 #ifdef __cplusplus
 }

@@ -32,7 +32,7 @@ EXPORTS = ("fp4_status_string", "fp4_scale_bytes", "fp4_quantize", "fp4_root_coe
            "fp4_root_ns_batched", "fp4_last_device_status", "fp4_root_ns_workspace_layout", "fp4_gemm_nt",
            "fp4_gemm_nt_resident",
            "fp4_profile_enable", "fp4_profile_collect", "fp4_kernel_launches", "fp4_root_ns_static",
-           "fp4_selftest_bounded_wait")
+           "fp4_selftest_bounded_wait", "fp4_selftest_quantize_wait")
 PROF_CLASSES = ("clip", "stats", "prep", "G1", "G2", "G3", "transpose", "quantize", "momentum", "adamw")
 
 
@@ -146,6 +146,8 @@ def load_library():
     L.fp4_adamw_update.restype = C.c_int
     L.fp4_momentum_decode.argtypes = [vp, vp, i64, i64, vp, vp]; L.fp4_momentum_decode.restype = C.c_int
     L.fp4_selftest_bounded_wait.argtypes = [vp, u32, vp]; L.fp4_selftest_bounded_wait.restype = C.c_int
+    L.fp4_selftest_quantize_wait.argtypes = [vp, i64, i64, vp, vp, vp, u32, vp]
+    L.fp4_selftest_quantize_wait.restype = C.c_int
     _lib = L
     return L
 
@@ -304,6 +306,14 @@ def fp4_profile_collect():
 def fp4_selftest_bounded_wait(status: torch.Tensor, limit_us: int, stream=None) -> None:
     _check(load_library().fp4_selftest_bounded_wait(status.data_ptr(), int(limit_us), _stream(stream)),
            "fp4_selftest_bounded_wait")
+
+
+def fp4_selftest_quantize_wait(x: torch.Tensor, codes: torch.Tensor, scales: torch.Tensor, tensor_scale: torch.Tensor,
+                               limit_us: int, stream=None) -> None:
+    rows, cols = x.shape
+    _check(load_library().fp4_selftest_quantize_wait(x.data_ptr(), rows, cols, codes.data_ptr(), scales.data_ptr(),
+                                                     tensor_scale.data_ptr(), int(limit_us), _stream(stream)),
+           "fp4_selftest_quantize_wait")
 
 
 def fp4_kernel_launches() -> int:

@@ -55,19 +55,19 @@ __device__ __forceinline__ void wait_or_abort(uint64_t* bar, uint32_t parity, vo
   wait_or_abort(smem_u32(bar), parity, abort_flag);
 }
 
-// Barrier over all blocks of a cooperative launch: `counter` (zero before the launch) has been incremented by all of
-// them `round` times.  Bounded like the other waits.
-__device__ __forceinline__ void grid_barrier(uint32_t* counter, uint32_t round, volatile uint32_t* abort_flag) {
+// Barrier over all blocks of a cooperative launch: this block increments `counter` (zero before the launch) and waits until
+// it is at least `want`, the number of blocks times that of the barrier.  Bounded like the other waits.
+__device__ __forceinline__ void grid_barrier(uint32_t* counter, uint32_t want, volatile uint32_t* abort_flag,
+                                             uint64_t limit_ns = kWaitLimitNs) {
   __syncthreads();
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
-    const uint32_t want = round * gridDim.x;
     const uint64_t t0 = globaltimer_ns();
     for (;;) {
       uint32_t v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
       if (v >= want) break;
-      if (*abort_flag || globaltimer_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; break; }
+      if (*abort_flag || globaltimer_ns() - t0 > limit_ns) { *abort_flag = 1; break; }
     }
   }
   __syncthreads();

@@ -217,7 +217,7 @@ cudaError_t quantize_set_attributes();
 bool quantize_fits_smem(int64_t elements, int sms);
 // tm: x as rows of 16 floats, box = 128 rows, 64-byte swizzle - given when the tensor fits the shared memories, else null
 cudaError_t launch_quantize(const CUtensorMap* tm, const float* x, int64_t rows, int64_t cols, uint8_t* codes, uint8_t* scales,
-                            float* tensor_scale, const QuantOpts& q, int sms, cudaStream_t st);
+                            float* tensor_scale, const QuantOpts& q, int sms, cudaStream_t st, uint64_t give_up_ns = 0);
 struct PrologueItem {
   const float* G;
   float* X;

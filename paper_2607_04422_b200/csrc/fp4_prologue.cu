@@ -1063,14 +1063,14 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
         pieces(it, [&](float x) { atomicAdd(&hist[mag_bits(x) >> kTopShift], 1u); });
         __syncthreads();
       }
-      if (round == 0) grid_barrier(counter, ++round, abort_flag);   // everything is cleared
+      if (round == 0) grid_barrier(counter, ++round * gridDim.x, abort_flag);   // everything is cleared
       if (last && !g.mat[mi].hist_top) {
         for (int i = tid; i < kTopBins; i += kPrepThreads)
           if (hist[i]) atomicAdd(&g.mat[mi].hist[i], hist[i]);
         __syncthreads();
       }
     }
-    grid_barrier(counter, ++round, abort_flag);
+    grid_barrier(counter, ++round * gridDim.x, abort_flag);
     // ---- the bin that holds the rank
     for (int it = 0; it < mine; ++it) {
       const int mi = sh->info[it].mi;
@@ -1128,7 +1128,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       __syncthreads();
     }
   } else {
-    grid_barrier(counter, ++round, abort_flag);
+    grid_barrier(counter, ++round * gridDim.x, abort_flag);
   }
 
   // ---- squares below the bin, candidates of the bin
@@ -1181,7 +1181,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
     }
     __syncthreads();
   }
-  grid_barrier(counter, ++round, abort_flag);
+  grid_barrier(counter, ++round * gridDim.x, abort_flag);
 
   // ---- tau among the candidates, normalisation scalars: every block for its own matrices; the block of a matrix's
   // first tile writes them

@@ -120,10 +120,14 @@ __global__ void __launch_bounds__(256) k_quantize_rows_opts(const float* __restr
 // the count while slower blocks may still poll it: as an unsigned number a normal FP32 value is larger than any count, so it
 // releases them, too.  A tensor scale so small that its bits are not (below 512 2^-149) is stored by the last
 // of the blocks to count themselves out.  (Counting out always: 13.6 us at 1152 x 2688 instead of 13.2.)
+// There is no workspace to report in: a block that gave up on a wait turns the word into a NaN, which no tensor has as its scale.
+// The bits it sets stay set: a count does not reach them, and the tensor scale takes the count's place as the larger number.
+// (An exchange there, whose answer the block waits for: 13.4 us.)
 // ----------------------------------------------------------------------------------
 constexpr int kQUnit = 2048;
 constexpr int kQUnitBytes = kQUnit * 4;
 constexpr int kQMaxBlocks = 256;      // maxima in words 0 .. 255 of the scale buffer
+constexpr uint32_t kQGaveUp = 0xFFC00000u;
 constexpr int kQGroups = 4, kQHold = 6, kQThreads = kQGroups * 128;
 struct QuantShared {
   uint64_t full[kQGroups][kQHold];
@@ -135,7 +139,7 @@ constexpr int kQSmem = kQGroups * kQHold * kQUnitBytes + (int)sizeof(QuantShared
 template <bool PF>
 __global__ void __launch_bounds__(kQThreads, 1)
 k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols, uint8_t* __restrict__ codes, uint8_t* scales,
-                 float* tensor_scale, const QuantOpts q) {
+                 float* tensor_scale, const QuantOpts q, const uint32_t blocks, const uint64_t limit_ns) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   QuantShared* sh = reinterpret_cast<QuantShared*>(smem + kQGroups * kQHold * kQUnitBytes);
@@ -181,7 +185,7 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
     scratch[blockIdx.x] = __float_as_uint(mx);
   }
   uint32_t* counter = reinterpret_cast<uint32_t*>(tensor_scale);
-  grid_barrier(counter, 1, abort_flag);
+  grid_barrier(counter, blocks, abort_flag, limit_ns);
   uint32_t bits = 0;
   for (int i = threadIdx.x & 31; i < (int)gridDim.x; i += 32) {
     uint32_t v;
@@ -191,11 +195,7 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
   bits = __reduce_max_sync(0xffffffffu, bits);
   const float sg = scale_exact(__fmul_rn(q.widen, __uint_as_float(bits)));
   const float six_sg = __fmul_rn(6.0f, sg);
-  grid_barrier(counter, 2, abort_flag);   // everyone has read the maxima: scales may be written
-  if (threadIdx.x == 0) {
-    const uint32_t sg_bits = __float_as_uint(sg);
-    if (sg_bits >= 2 * gridDim.x ? blockIdx.x == 0 : atomicAdd(counter, 1u) == 3 * gridDim.x - 1) *counter = sg_bits;
-  }
+  grid_barrier(counter, 2 * blocks, abort_flag, limit_ns);   // everyone has read the maxima: scales may be written
   const uint32_t kblocks = (uint32_t)(cols >> 4);
   for (int i = 0; i < m; ++i) {
     float v[16];
@@ -207,6 +207,12 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
     *reinterpret_cast<uint2*>(codes + (int64_t)b * 8) = make_uint2(lo, hi);
     const uint32_t r = b / kblocks;
     scales[sf_offset(r, b - r * kblocks, kblocks)] = (uint8_t)sb;
+  }
+  if (threadIdx.x == 0) {
+    const uint32_t sg_bits = __float_as_uint(sg);
+    if (sh->abort_flag) atomicOr(counter, kQGaveUp);
+    else if (sg_bits >= 2 * blocks) { if (blockIdx.x == 0) atomicMax(counter, sg_bits); }
+    else if (atomicAdd(counter, 1u) == 3 * blocks - 1) atomicCAS(counter, 3 * blocks, sg_bits);
   }
 }
 
@@ -282,9 +288,10 @@ cudaError_t quantize_set_attributes() {
   return cudaFuncSetAttribute(k_quantize_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kQSmem);
 }
 
-// tm: x as rows of 16 floats, box = 128 rows, 64-byte swizzle (tensors small enough for one launch)
+// tm: x as rows of 16 floats, box = 128 rows, 64-byte swizzle (tensors small enough for one launch).  give_up_ns: not 0 in the
+// self-test, whose barriers expect a block that is not launched.
 cudaError_t launch_quantize(const CUtensorMap* tm, const float* x, int64_t rows, int64_t cols, uint8_t* codes, uint8_t* scales,
-                            float* tensor_scale, const QuantOpts& q, int sms, cudaStream_t st) {
+                            float* tensor_scale, const QuantOpts& q, int sms, cudaStream_t st, uint64_t give_up_ns) {
   const bool pf = q.rht || q.four_six;
   if (tm) {
     const int units = (int)(rows * cols / kQUnit);
@@ -300,7 +307,7 @@ cudaError_t launch_quantize(const CUtensorMap* tm, const float* x, int64_t rows,
     cfg.attrs = attr; cfg.numAttrs = 1;
     count_launches(1);
     return cudaLaunchKernelEx(&cfg, pf ? k_quantize_small<true> : k_quantize_small<false>, *tm, units, cols, codes, scales,
-                              tensor_scale, q);
+                              tensor_scale, q, (uint32_t)grid + (give_up_ns ? 1u : 0u), give_up_ns ? give_up_ns : kWaitLimitNs);
   }
   const int64_t n4 = rows * cols / 4;
   cudaError_t e = cudaMemsetAsync(tensor_scale, 0, 4, st);

@@ -767,6 +767,26 @@ fp4_status fp4_quantize(const float* x, int64_t rows, int64_t cols, uint8_t* cod
              : FP4_ERR_CUDA;
 }
 
+fp4_status fp4_selftest_quantize_wait(const float* x, int64_t rows, int64_t cols, uint8_t* codes, uint8_t* scales,
+                                      float* tensor_scale, uint32_t limit_us, cudaStream_t stream) {
+  if (!x || !codes || !scales || !tensor_scale || limit_us < 1 || limit_us > 100000) return FP4_ERR_INVALID_ARG;
+  if (!shape_ok(rows) || !shape_ok(cols)) return FP4_ERR_SHAPE;
+  if (!aligned(x, 16) || !aligned(codes, 16) || !aligned(scales, 16) || !aligned(tensor_scale, 4)) return FP4_ERR_ALIGNMENT;
+  const DeviceInfo* d;
+  fp4_status rc = check_common(&d);
+  if (rc != FP4_OK) return rc;
+  if (!quantize_fits_smem(rows * cols, d->sms)) return FP4_ERR_SHAPE;
+  QuantOpts q;
+  memset(&q, 0, sizeof(q));
+  q.widen = 1.0f;
+  CUtensorMap tm;
+  if (!make_blocks_map(d, &tm, x, rows * cols / 16)) return FP4_ERR_CUDA;
+  return launch_quantize(&tm, x, rows, cols, codes, scales, tensor_scale, q, d->sms, stream, (uint64_t)limit_us * 1000ull) ==
+                 cudaSuccess
+             ? FP4_OK
+             : FP4_ERR_CUDA;
+}
+
 fp4_status fp4_momentum_update(const float* G, int64_t rows, int64_t cols, uint8_t* codes, uint16_t* scales,
                                float* M_out, uint32_t* hist, const fp4_momentum_params* params,
                                cudaStream_t stream) {

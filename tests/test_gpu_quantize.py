@@ -187,3 +187,22 @@ def test_single_launch_quantiser_waits_for_no_word_that_it_overwrites(shape, sca
     assert np.float32(ts.item()) == np.float32(osg)
     assert np.array_equal(sf_from_atoms(scales.cpu().numpy(), rows, cols // 16), os_)
     assert np.array_equal(codes.cpu().numpy(), oc)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-41])
+@pytest.mark.parametrize("shape", [(128, 128), (1152, 2688)])
+def test_single_launch_quantiser_reports_that_it_gave_up(shape, scale):
+    """Barriers that expect a block which is not launched give up after the limit, and the tensor scale says so; the
+    next call on the same buffers is whole."""
+    rows, cols = shape
+    x_np = workloads.gaussian(rows, cols, seed=2) * np.float32(scale)
+    x = torch.from_numpy(x_np).cuda()
+    codes = torch.empty((rows, cols // 2), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(fp4.fp4_scale_bytes(rows, cols), dtype=torch.uint8, device="cuda")
+    ts = torch.ones(1, device="cuda")
+    fp4.fp4_selftest_quantize_wait(x, codes, scales, ts, 200)
+    assert np.isnan(ts.item())
+    fp4.fp4_quantize(x, codes, scales, ts)
+    oc, os_, osg = oracle.quantize(x_np)
+    assert np.float32(ts.item()) == np.float32(osg)
+    assert np.array_equal(sf_from_atoms(scales.cpu().numpy(), rows, cols // 16), os_)
