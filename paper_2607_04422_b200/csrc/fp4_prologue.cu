@@ -187,14 +187,27 @@ __global__ void __launch_bounds__(512) kp_hist_top(const __grid_constant__ PrepG
     if (sh[j]) atomicAdd(&m.hist[j], sh[j]);
 }
 
+// Sum of a warp's values, the same in every lane: pairs 16 lanes apart first.
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 constexpr int kSubBins = 512;                 // counters of bits 17..9 and of bits 8..0 of the candidates
 
 // ---- pass 2: candidates of the picked bin, FP64 sum of squares below the bin, max |g|.
 // Candidates are rare: they are collected in a shared-memory buffer per block and copied to
 // the global list with one reservation per block (or directly when the buffer is full); on the way there the next 9
 // bits of each are counted, in the counters the first pass has left cleared.
+//
+// The sum of squares must not depend on how many matrices a call has, so it is the same sum in kp_resident: a matrix small
+// enough to be resident is summed tile by tile (a lane 4 columns of 4 rows, a warp its lanes, then the 32 row sums), larger
+// ones as their elements lie in memory.
+//
 // Eight blocks per SM: the 1024 blocks of a matrix are resident at once.  (With 40 registers and six blocks an eighth of them
 // ran as a second wave: 16384 x 16384 248 us against 178, 6.0 TB/s; 4096 x 8192 36 against 27.5.)
+template <bool TILED>
 __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant__ PrepGroup g) {
   pdl_launch_dependents();
   pdl_wait();
@@ -227,29 +240,52 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
       }
     }
   };
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  for (; i + stride < g.n4; i += 2 * stride) {
-    const float4 v = __ldg(src + i), w = __ldg(src + i + stride);
-    visit(v.x); visit(v.y); visit(v.z); visit(v.w);
-    visit(w.x); visit(w.y); visit(w.z); visit(w.w);
-  }
-  for (; i < g.n4; i += stride) {
-    const float4 v = __ldg(src + i);
-    visit(v.x); visit(v.y); visit(v.z); visit(v.w);
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  }
-  __shared__ double wa[8];
+  __shared__ double wa[32];
   __shared__ float wm[8];
-  if (lane == 0) { wa[threadIdx.x >> 5] = acc; wm[threadIdx.x >> 5] = mx; }
+  const int warp = threadIdx.x >> 5;
+  if (TILED) {
+    const int rows = (int)(m.tall ? g.l0 : g.s0), cols = (int)(m.tall ? g.s0 : g.l0);
+    const int tiles_x = (int)((m.tall ? g.s : g.l) >> 7), ty = (int)blockIdx.x / tiles_x;
+    const int row0 = ty * 128, col = ((int)blockIdx.x - ty * tiles_x) * 128 + lane * 4;
+#pragma unroll 1
+    for (int r = warp; r < 32; r += 8) {
+      acc = 0.0;
+      if (col < cols) {
+#pragma unroll 1
+        for (int k = 0; k < 128; k += 64) {
+          const int ra = row0 + r + k, rb = ra + 32;
+          const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          const float4 v = ra < rows ? __ldg(src + ((int64_t)ra * cols + col) / 4) : zero;
+          const float4 w = rb < rows ? __ldg(src + ((int64_t)rb * cols + col) / 4) : zero;
+          if (ra < rows) { visit(v.x); visit(v.y); visit(v.z); visit(v.w); }
+          if (rb < rows) { visit(w.x); visit(w.y); visit(w.z); visit(w.w); }
+        }
+      }
+      acc = warp_sum(acc);
+      if (lane == 0) wa[r] = acc;
+    }
+  } else {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (; i + stride < g.n4; i += 2 * stride) {
+      const float4 v = __ldg(src + i), w = __ldg(src + i + stride);
+      visit(v.x); visit(v.y); visit(v.z); visit(v.w);
+      visit(w.x); visit(w.y); visit(w.z); visit(w.w);
+    }
+    for (; i < g.n4; i += stride) {
+      const float4 v = __ldg(src + i);
+      visit(v.x); visit(v.y); visit(v.z); visit(v.w);
+    }
+    acc = warp_sum(acc);
+    if (lane < 4) wa[warp + 8 * lane] = lane == 0 ? acc : 0.0;
+  }
+  mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
+  if (lane == 0) wm[warp] = mx;
   __syncthreads();
+  if (warp == 0) acc = warp_sum(wa[lane]);
   const uint32_t nbuf = s_cnt < kBuf ? s_cnt : kBuf;
   if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) { acc += wa[w]; mx = fmaxf(mx, wm[w]); }
+    for (int w = 1; w < 8; ++w) mx = fmaxf(mx, wm[w]);
     m.partial[blockIdx.x] = acc;
     atomicMax(&m.hdr->maxabs_bits, __float_as_uint(mx));
     s_base = nbuf ? atomicAdd(&m.hdr->cand_count, nbuf) : 0u;
@@ -271,17 +307,21 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
   }
 }
 
-// fixed-order sum of the per-block partials by one block of 1024 threads
-__device__ __forceinline__ double sum_partials(const double* partial, int nparts, double* sh) {
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += partial[i];
-  sh[threadIdx.x] = acc;
+// Fixed-order sum of at most 1024 partials by a block of 1024 threads, returned in warp 0; `wsum`: 32 words.
+__device__ __forceinline__ double sum_partials(const double* partial, int nparts, double* wsum) {
+  const int tid = threadIdx.x;
+  const double v = warp_sum(tid < nparts ? __ldcg(partial + tid) : 0.0);
+  if ((tid & 31) == 0) wsum[tid >> 5] = v;
   __syncthreads();
-  for (int o = blockDim.x / 2; o; o >>= 1) {
-    if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  return sh[0];
+  return tid < 32 ? warp_sum(wsum[tid]) : 0.0;
+}
+// The clipped matrix's sum of squares: `below` the clip's bin, the candidates' lo + hi 2^24 in units of the square of their last
+// place, and tau^2 for each of the n_clipped elements above it.
+__device__ __forceinline__ double clipped_squares(double below, unsigned long long lo, unsigned long long hi, uint32_t efield,
+                                                  double n_clipped, float tau) {
+  const int e2 = 2 * ((int)(efield ? efield : 1u) - 150);
+  const double cand = ldexp(__fma_rn((double)hi, 16777216.0, (double)lo), e2);
+  return __fma_rn(__dmul_rn(n_clipped, (double)tau), (double)tau, __dadd_rn(below, cand));
 }
 
 struct NormScalars { float nu, inv, amax0, sg; };
@@ -517,12 +557,10 @@ __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ Prep
   const double below = sum_partials(m.partial, g.stat_blocks, shd);
   if (tid == 0) {
     const float tau = __uint_as_float(tau_bits);
-    const int e2 = 2 * ((int)(efield ? efield : 1u) - 150);
-    const double cand_sq = ldexp((double)s_hi * 16777216.0 + (double)s_lo, e2);
     // clamped to tau: everything in the bins above the picked one, and the candidates above tau
     const double n_total = (double)g.n4 * 4.0;
     const double n_clipped = n_total - (double)hdr->count_below - (double)hdr->bin_count + (double)s_above;
-    const double total = below + cand_sq + n_clipped * (double)tau * (double)tau;
+    const double total = clipped_squares(below, s_lo, s_hi, efield, n_clipped, tau);
     m.scalars[g.ix.tau] = tau;
     write_norm_scalars(m.scalars, g.ix, norm_scalars(total, tau, g.eps, g.q.widen));
     hdr->overflow = 0;
@@ -965,7 +1003,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
 // histogram, compacts candidates and squares from them, and quantises them.  Between those phases the blocks
 // meet at (bounded) grid barriers; what a single block did between two launches - the bin of the rank, the select
 // among the candidates, the normalisation scalars - every block now computes for its own matrices, which costs less
-// than another exchange.  Same sums in another order: nu is a sum of FP64 partials per tile.
+// than another exchange.  The same sums in the same order (see kp_compact_stats).
 //
 // Bounds: latency - three barriers, 3200 cycles of shared-memory counting and 4500 of FP64 sums per tile, two radix rounds,
 // one tile's quantisation (18 us for one tile per SM, 42 us for three).  Whole 5-iteration calls, six launches before
@@ -1033,18 +1071,16 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       if (i != kBarrierWord) w[i] = 0;
   }
   __syncthreads();
-  // a thread's four 16-byte pieces of a tile: row tid / 8 of each 32-column box; f(values, in the caller's matrix)
+  // a thread's four 16-byte pieces of a tile: columns 4 lane .. 4 lane + 3 of rows warp, warp + 32, ...; f(value)
   auto pieces = [&](int it, auto&& f) {
     const PrepTileInfo ti = sh->info[it];
     const PrepMatrix& m = g.mat[ti.mi];
-    const int row = tid >> 3, c = ((tid & 7) ^ (row & 7)) * 4;
-    const bool row_in = ti.gr0 + row < (m.tall ? g.l0 : g.s0);
-    const int cols = (int)(m.tall ? g.s0 : g.l0) - ti.gc0;
-    const uint32_t at = smem_u32(smem + it * kPrepTile) + tid * 16;
+    const int rows = (int)(m.tall ? g.l0 : g.s0) - ti.gr0, cols = (int)(m.tall ? g.s0 : g.l0) - ti.gc0;
+    const uint32_t at = smem_u32(smem + it * kPrepTile);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const float4 v = lds128f(at + k * kPrepBox);
-      if (row_in && k * 32 + c < cols) { f(v.x); f(v.y); f(v.z); f(v.w); }
+      const float4 v = lds128f(prep_piece(at, warp + 32 * k, lane));
+      if (warp + 32 * k < rows && lane * 4 < cols) { f(v.x); f(v.y); f(v.z); f(v.w); }
     }
   };
   for (int it = 0; it < mine; ++it) wait_or_abort(&sh->full[it], 0, abort_flag);
@@ -1157,16 +1193,13 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
         }
       }
     });
-#pragma unroll
-    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    acc = warp_sum(acc);
     mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
     if (lane == 0) { sh->wsum[warp] = acc; sh->wmax[warp] = mx; }
     __syncthreads();
     const uint32_t nbuf = sh->cnt < kBuf ? sh->cnt : kBuf;
     if (warp == 0) {
-      acc = sh->wsum[lane];
-#pragma unroll
-      for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      acc = warp_sum(sh->wsum[lane]);
       mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sh->wmax[lane])));
       if (lane == 0) {
         m.partial[ti.pad] = acc;
@@ -1293,19 +1326,11 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       }
       if (lane == 0) { sh->wlo[warp] = lo; sh->whi[warp] = hi; sh->wabove[warp] = above; }
     }
-    // fixed-order sum of the tiles' partials
-    double acc = 0.0;
-    for (int i = tid; i < tiles_per_matrix; i += kPrepThreads) acc += __ldcg(m.partial + i);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) sh->wsum[warp] = acc;
-    __syncthreads();
+    double acc = sum_partials(m.partial, tiles_per_matrix, sh->wsum);
     if (warp == 0) {
-      acc = sh->wsum[lane];
       if (g.clip) { lo = sh->wlo[lane]; hi = sh->whi[lane]; above = sh->wabove[lane]; }
 #pragma unroll
       for (int o = 16; o; o >>= 1) {
-        acc += __shfl_xor_sync(0xffffffffu, acc, o);
         lo += __shfl_xor_sync(0xffffffffu, lo, o);
         hi += __shfl_xor_sync(0xffffffffu, hi, o);
         above += __shfl_xor_sync(0xffffffffu, above, o);
@@ -1315,11 +1340,9 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
         if (g.clip) {
           tau = __uint_as_float(tau_bits);
           maxabs = tau;
-          const int e2 = 2 * ((int)(efield ? efield : 1u) - 150);
-          const double cand_sq = ldexp((double)hi * 16777216.0 + (double)lo, e2);
           // clamped to tau: everything in the bins above the picked one, and the candidates above tau
           const double n_clipped = (double)g.n4 * 4.0 - (double)sh->below[it] - (double)sh->bin_count[it] + (double)above;
-          acc = acc + cand_sq + n_clipped * (double)tau * (double)tau;
+          acc = clipped_squares(acc, lo, hi, efield, n_clipped, tau);
         }
         const NormScalars ns = norm_scalars(acc, maxabs, g.eps, g.q.widen);
         sh->tau[it] = tau; sh->inv[it] = ns.inv; sh->sg[it] = ns.sg;
@@ -1380,7 +1403,6 @@ cudaError_t launch_prologue_group(const PrologueItem* items, int count, int writ
     const int64_t cap = pl.s0 * pl.l0 / 8 < region ? pl.s0 * pl.l0 / 8 : region;
     g.cand_cap = (uint32_t)cap;
     g.eps = pl.eps;
-    g.stat_blocks = pl.stat_blocks;
     g.write_q = write_q;
     g.zero_words = (int)(pl.zero_bytes / 4);
     g.ix = pl.ix;
@@ -1408,8 +1430,10 @@ cudaError_t launch_prologue_group(const PrologueItem* items, int count, int writ
       g.tmG[j] = *it.tmG;
     }
     const int sms = pl.sms;
-    const int64_t tiles = (pl.l / 128) * (pl.s / 128) * nn;
-    if (tiles <= (int64_t)kResTiles * sms) {
+    const int64_t matrix_tiles = (pl.l / 128) * (pl.s / 128), tiles = matrix_tiles * nn;
+    const bool tiled = matrix_tiles <= (int64_t)kResTiles * sms && matrix_tiles <= 1024;   // 1024 partials
+    g.stat_blocks = tiled ? (int)matrix_tiles : pl.stat_blocks;
+    if (tiled && tiles <= (int64_t)kResTiles * sms) {
       // everything fits the shared memories: one launch
       ProfScope ps(FP4_PROF_PREP, st);
       cudaError_t e = cudaMemsetAsync(&g.mat[0].hdr->barrier, 0, 4, st);
@@ -1441,7 +1465,7 @@ cudaError_t launch_prologue_group(const PrologueItem* items, int count, int writ
     }
     {
       ProfScope ps(FP4_PROF_STATS, st);
-      launch_chained(kp_compact_stats, gs, dim3(256), 0, st, g);
+      launch_chained(tiled ? kp_compact_stats<true> : kp_compact_stats<false>, gs, dim3(256), 0, st, g);
       // a block of the select per 4 M elements: some 10 k candidates of a Gaussian matrix
       const int64_t fb = g.n4 >> 20;
       launch_chained(kp_finalize, dim3((unsigned)(fb < 1 ? 1 : fb < 64 ? fb : 64), (unsigned)nn), dim3(1024), 0, st, g);

@@ -1,4 +1,6 @@
 """fp4_root_ns / fp4_root_ns_batched against the oracle, through the C ABI."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -812,4 +814,49 @@ def test_symmetric_products_in_one_launch_for_a_group():
     assert fp4.fp4_last_device_status(ws) == 0
     for g, o in zip(mats, outs):
         single, _ = run_gpu(g, steps=3)
+        assert np.array_equal(o.cpu().numpy(), single)
+
+
+def _norm_near_a_rounding_boundary(m, n, seed, clip):
+    """A matrix whose clipped Frobenius norm lies within 2^-50 of the midpoint of two floats: sums of its squares in two orders
+    round to either."""
+    rng = np.random.default_rng(seed)
+    g = rng.standard_normal(m * n).astype(np.float32)
+    g[:4] = 0
+    rank = -(-99 * g.size // 100)
+    tau = np.partition(np.abs(g), rank - 1)[rank - 1] if clip else np.float32(np.inf)
+    squares = np.square(np.minimum(np.abs(g), tau).astype(np.float64))
+    nu = np.float32(np.sqrt(squares.sum()))
+    up = np.nextafter(nu, np.float32(np.inf))
+    target = ((float(nu) + float(up)) / 2) ** 2                  # 25 bits squared: exact in FP64
+    if target <= squares.sum():
+        target = ((float(up) + float(np.nextafter(up, np.float32(np.inf)))) / 2) ** 2
+    for i in range(4):                                           # each takes the rest down by about 2^-23
+        rest = -math.fsum(np.append(squares, -target))
+        if rest <= 0:
+            break
+        g[i] = np.nextafter(np.float32(np.sqrt(rest)), np.float32(0))
+        assert g[i] < tau
+        squares[i] = float(g[i]) ** 2
+    return rng.permutation(g).reshape(m, n)
+
+
+@pytest.mark.parametrize("clip_quantile", [0.0, 0.99])
+@pytest.mark.parametrize("shape", [(640, 768), (752, 624)])
+def test_batched_norms_are_those_of_single_calls_to_the_last_bit(shape, clip_quantile):
+    """Sixteen matrices of 30 tiles take the passes over the matrix, one alone takes the resident prologue: the sums of squares
+    must be the same FP64 numbers, also where the last bit of the norm hangs on it."""
+    m, n = shape
+    mats = [_norm_near_a_rounding_boundary(m, n, seed, clip_quantile > 0) for seed in range(16)]
+    Gs = [torch.from_numpy(g).cuda() for g in mats]
+    outs = [torch.empty_like(g) for g in Gs]
+    ws = torch.empty(fp4.fp4_root_ns_batched_workspace_bytes([shape] * 16, 0), dtype=torch.uint8, device="cuda")
+    before = fp4.fp4_kernel_launches()
+    fp4.fp4_root_ns_batched(Gs, outs, 0, fp4.NsParams.make(clip_quantile=clip_quantile), ws)
+    assert fp4.fp4_kernel_launches() - before >= (6 if clip_quantile else 4)
+    assert fp4.fp4_last_device_status(ws) == 0
+    for g, o in zip(mats, outs):
+        before = fp4.fp4_kernel_launches()
+        single, _ = run_gpu(g, steps=0, clip_quantile=clip_quantile)
+        assert fp4.fp4_kernel_launches() - before == (2 if m > n else 1)
         assert np.array_equal(o.cpu().numpy(), single)
