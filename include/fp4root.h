@@ -185,6 +185,11 @@ fp4_status fp4_root_coeffs(int64_t m, int64_t n, int steps, float abc[3]);
  *   of equal shapes) chain their other kernels with programmatic dependent launch; the environment
  *   variable FP4ROOT_NO_PDL (any value) switches that off.  Kernels launched before or after
  *   the call on the same stream see ordinary stream order either way.
+ *   A cooperative launch starts when all its blocks - up to one per SM, each with most of an SM's shared
+ *   memory - can be resident at once: beside a long kernel on another stream it waits for
+ *   that kernel's SMs, where plain launches would have started on the free ones.  On a stream that owns only
+ *   a part of the device (a green context, a context with an SM limit) the sizes above shrink with
+ *   the part; results are the same.
  */
 size_t fp4_root_ns_workspace_bytes(int64_t m, int64_t n, int steps, uint32_t flags);
 fp4_status fp4_root_ns(const float* G, float* out, int64_t m, int64_t n, int steps,

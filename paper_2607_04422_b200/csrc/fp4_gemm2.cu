@@ -916,7 +916,7 @@ template <int MODE, bool PF, bool BH, bool UPD, bool DEEP>
 cudaError_t launch_pair_variant(const ProblemPack& pack, const GemmLaunch& L, int sms, cudaStream_t st) {
   const int tpp = L.symmetric ? L.tiles_n * (L.tiles_n + 1) / 2 : L.tiles_m * L.tiles_n;
   const int num_tiles = tpp * L.num_problems;
-  int pairs = sms / 2;
+  int pairs = sms > 1 ? sms / 2 : 1;
   if (pairs > num_tiles) pairs = num_tiles;
   count_launches(1);
   launch_chained(k_gemm_pair<MODE, PF, BH, UPD, DEEP>, dim3(2 * pairs), dim3(NTHREADS), Lay<MODE, DEEP>::SMEM_BYTES, st, pack, L);

@@ -50,7 +50,7 @@ struct NsPlan {
   size_t off_Xh;     // bf16: BF16 X in the workspace
   int64_t clip_rank;
   float eps;
-  int sms;
+  int sms;           // of the device
   int stat_blocks;
   size_t off_hist, off_partial;
   size_t zero_bytes;  // header + scalars + histogram, cleared at the start of a call
@@ -229,9 +229,9 @@ struct PrologueItem {
   uint32_t* hist_top;      // the caller's histogram of the top 13 magnitude bits of G, or null
   const CUtensorMap* tmG;  // G as an FP32 tensor: box = 32 columns x 128 rows, 128-byte swizzle
 };
-// count matrices that share the shape (s, l) and the clip / eps parameters
+// count matrices that share the shape (s, l) and the clip / eps parameters; sms: those the stream's kernels can occupy
 cudaError_t launch_prologue_group(const PrologueItem* items, int count, int write_q, const QuantOpts& q,
-                                  uint32_t* status, cudaStream_t st);
+                                  uint32_t* status, int sms, cudaStream_t st);
 // Root's parameter update on BF16 weights: decay = fl(1 - fl(lr * wd)), step = fl(lr * scale),
 // w <- BF16(fl(fl(w * decay) - fl(step * o))).
 struct ParamUpdate {

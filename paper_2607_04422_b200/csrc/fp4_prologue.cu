@@ -1383,7 +1383,7 @@ cudaError_t prologue_set_attributes() {
 
 // Enqueue the prologue for `count` matrices of one shape (s, l) and one parameter set.
 cudaError_t launch_prologue_group(const PrologueItem* items, int count, int write_q, const QuantOpts& q,
-                                  uint32_t* status, cudaStream_t st) {
+                                  uint32_t* status, int sms, cudaStream_t st) {
   for (int i0 = 0; i0 < count; i0 += kMaxPack) {
     const int nn = count - i0 < kMaxPack ? count - i0 : kMaxPack;
     const NsPlan& pl = *items[i0].pl;
@@ -1429,9 +1429,8 @@ cudaError_t launch_prologue_group(const PrologueItem* items, int count, int writ
       if (!it.hist_top) all_counted = false;
       g.tmG[j] = *it.tmG;
     }
-    const int sms = pl.sms;
     const int64_t matrix_tiles = (pl.l / 128) * (pl.s / 128), tiles = matrix_tiles * nn;
-    const bool tiled = matrix_tiles <= (int64_t)kResTiles * sms && matrix_tiles <= 1024;   // 1024 partials
+    const bool tiled = matrix_tiles <= (int64_t)kResTiles * pl.sms && matrix_tiles <= 1024;   // 1024 partials
     g.stat_blocks = tiled ? (int)matrix_tiles : pl.stat_blocks;
     if (tiled && tiles <= (int64_t)kResTiles * sms) {
       // everything fits the shared memories: one launch

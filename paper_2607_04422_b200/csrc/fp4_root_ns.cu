@@ -5,8 +5,11 @@
 #include <cmath>
 #include <mutex>
 #include <stdlib.h>
+#include <type_traits>
 #include <unordered_map>
 #include <vector>
+
+#include <cudaTypedefs.h>
 
 #include "fp4_gemm_common.cuh"
 
@@ -60,6 +63,10 @@ struct DeviceInfo {
   fp4_status status = FP4_OK;
   int sms = 0;
   EncodeTiledFn encode = nullptr;
+  // of drivers that know them (12.5): the context behind a stream, and what of the device it may use
+  PFN_cuStreamGetCtx_v12050 stream_context = nullptr;
+  PFN_cuCtxGetDevResource_v12040 context_resource = nullptr;
+  PFN_cuGreenCtxGetDevResource_v12040 green_resource = nullptr;
 };
 DeviceInfo g_dev[64];
 std::mutex g_mu;
@@ -82,12 +89,34 @@ const DeviceInfo* device_info() {
     d.status = FP4_ERR_CUDA; d.ready = true; return &d;
   }
   d.encode = reinterpret_cast<EncodeTiledFn>(fn);
+  auto optional = [&](const char* name, unsigned version, auto& entry) {
+    if (cudaGetDriverEntryPointByVersion(name, &fn, version, cudaEnableDefault, &qres) == cudaSuccess &&
+        qres == cudaDriverEntryPointSuccess && fn != nullptr)
+      entry = reinterpret_cast<std::decay_t<decltype(entry)>>(fn);
+    else
+      cudaGetLastError();
+  };
+  optional("cuStreamGetCtx", 12050, d.stream_context);
+  optional("cuCtxGetDevResource", 12040, d.context_resource);
+  optional("cuGreenCtxGetDevResource", 12040, d.green_resource);
   if (gemm_pair_set_attributes() != cudaSuccess ||
       chain_set_attributes() != cudaSuccess ||
       prologue_set_attributes() != cudaSuccess || quantize_set_attributes() != cudaSuccess)
     d.status = FP4_ERR_CUDA;
   d.ready = true;
   return &d;
+}
+
+// SMs that kernels on this stream can occupy: fewer than the device has where the stream belongs to a green context or to a
+// context with a limit of its own.  The cooperative launches need all their blocks resident there.
+int stream_sms(const DeviceInfo* d, cudaStream_t st) {
+  if (!d->stream_context || !d->context_resource || !d->green_resource) return d->sms;
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  CUdevResource r;
+  if (d->stream_context(st, &ctx, &green) != CUDA_SUCCESS) return d->sms;
+  const CUresult e = green ? d->green_resource(green, &r, CU_DEV_RESOURCE_TYPE_SM) : d->context_resource(ctx, &r, CU_DEV_RESOURCE_TYPE_SM);
+  return e == CUDA_SUCCESS && r.sm.smCount > 0 && (int)r.sm.smCount < d->sms ? (int)r.sm.smCount : d->sms;
 }
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -345,14 +374,14 @@ struct PairUs {
 // 4 x 512 x 512 106 / 170 / 179, 2 x 1024 x 2816 200 / 248 / 260.  (Not for inspection of BF16-stored intermediates: in
 // single launches A and X stay FP32 tensors with rounded values.)
 enum Route { kOneLaunch, kTwoLaunches, kThreeLaunches };
-Route route_of(const DeviceInfo* d, const NsPlan& pl, int count, const fp4_ns_params* p) {
+Route route_of(const NsPlan& pl, int count, const fp4_ns_params* p, int sms) {
   if (count > kChainMax || (pl.bf16 && (p->flags & FP4_FLAG_KEEP_OPERANDS))) return kThreeLaunches;
   const bool opts = (p->flags & (FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)) != 0;
-  const PairUs pair(pl.s, pl.l, count, opts, d->sms);
+  const PairUs pair(pl.s, pl.l, count, opts, sms);
   const double three = pair.g1 + pair.g2 + pair.g3;
-  const double sym = chain_symmetric_us(pl.s, pl.l, count, opts, d->sms);
+  const double sym = chain_symmetric_us(pl.s, pl.l, count, opts, sms);
   const double best = sym > 0.0 && sym + pair.g3 < three ? sym + pair.g3 : three;
-  const double one = chain_iteration_us(pl.s, pl.l, count, opts, d->sms);
+  const double one = chain_iteration_us(pl.s, pl.l, count, opts, sms);
   if (one > 0.0 && one <= best) return kOneLaunch;
   return best < three ? kTwoLaunches : kThreeLaunches;
 }
@@ -556,8 +585,9 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     if (steps > 0 && mats[i].pl.tall && !keep && !any_update) { direct_out[(size_t)i] = 1; any_direct = true; }
   const NsPlan& pl0 = mats[0].pl;
   const int64_t s = pl0.s, l = pl0.l;
+  const int sms = stream_sms(d, st);
   pdl_select(s * l * count);
-  const Route route = steps > 0 ? route_of(d, pl0, count, p) : kThreeLaunches;
+  const Route route = steps > 0 ? route_of(pl0, count, p, sms) : kThreeLaunches;
   {
     std::vector<PrologueItem> items((size_t)count);
     for (int i = 0; i < count; ++i) {
@@ -565,7 +595,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       items[(size_t)i] = PrologueItem{c.G, c.X, c.ws, &c.pl, clear_first_status && i == 0, c.store_x0, c.x_rows, c.x_cols,
                                       c.hist_top, &c.tm_G};
     }
-    if (launch_prologue_group(items.data(), count, steps > 0 || keep, quant_opts(p, 0), status, st) != cudaSuccess)
+    if (launch_prologue_group(items.data(), count, steps > 0 || keep, quant_opts(p, 0), status, sms, st) != cudaSuccess)
       return FP4_ERR_CUDA;
   }
   ChainPack pack;
@@ -592,7 +622,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       if (!keep) { direct_out[(size_t)j] = mats[j].pl.tall; fused_update[(size_t)j] = 1; }
     }
     ProfScope ps(FP4_PROF_G3, st);
-    if (launch_chain(pack, a, d->sms, st) != cudaSuccess) return FP4_ERR_CUDA;
+    if (launch_chain(pack, a, sms, st) != cudaSuccess) return FP4_ERR_CUDA;
   } else if (steps > 0) {
     // the problems of the five kinds of launches: G1, G2, G3 reading qXt[0] / qXt[1], the first G3
     std::vector<ProblemPack> packs(5);
@@ -632,10 +662,10 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       L1.out_h = bf16;
       if (route == kTwoLaunches) {
         ProfScope ps(FP4_PROF_G1, st);
-        if (launch_chain_symmetric(pack, a, k, d->sms, st) != cudaSuccess) return FP4_ERR_CUDA;
+        if (launch_chain_symmetric(pack, a, k, sms, st) != cudaSuccess) return FP4_ERR_CUDA;
       } else {
         ProfScope ps(FP4_PROF_G1, st);
-        if (launch_gemm_pair(kG1, packs[0], L1, d->sms, st) != cudaSuccess)
+        if (launch_gemm_pair(kG1, packs[0], L1, sms, st) != cudaSuccess)
           return FP4_ERR_CUDA;
       }
       GemmLaunch L2 = L1;
@@ -644,7 +674,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       L2.out_h = 0; L2.aux_h = bf16;
       if (route == kThreeLaunches) {
         ProfScope ps(FP4_PROF_G2, st);
-        if (launch_gemm_pair(kG2, packs[1], L2, d->sms, st) != cudaSuccess)
+        if (launch_gemm_pair(kG2, packs[1], L2, sms, st) != cudaSuccess)
           return FP4_ERR_CUDA;
       }
       GemmLaunch L3 = base;
@@ -675,7 +705,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       }
       {
         ProfScope ps(FP4_PROF_G3, st);
-        if (launch_gemm_pair(kG3, *pk, L3, d->sms, st) != cudaSuccess)
+        if (launch_gemm_pair(kG3, *pk, L3, sms, st) != cudaSuccess)
           return FP4_ERR_CUDA;
       }
     }
@@ -689,7 +719,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       if (launch_transpose_out(mats[i].X, s, l, mats[i].out, pl0.s0, pl0.l0, u, st) != cudaSuccess) return FP4_ERR_CUDA;
     } else if (u.W && !fused_update[(size_t)i]) {
       ProfScope ps(FP4_PROF_TRANSPOSE, st);
-      if (launch_param_update(mats[i].out, mats[i].pl.m * mats[i].pl.n, u, d->sms, st) != cudaSuccess) return FP4_ERR_CUDA;
+      if (launch_param_update(mats[i].out, mats[i].pl.m * mats[i].pl.n, u, sms, st) != cudaSuccess) return FP4_ERR_CUDA;
     }
   }
   return FP4_OK;
@@ -759,10 +789,11 @@ fp4_status fp4_quantize(const float* x, int64_t rows, int64_t cols, uint8_t* cod
   fp4_status rc = check_common(&d);
   if (rc != FP4_OK) return rc;
   CUtensorMap tm;
-  const bool small = quantize_fits_smem(rows * cols, d->sms);
+  const int sms = stream_sms(d, stream);
+  const bool small = quantize_fits_smem(rows * cols, sms);
   if (small && !make_blocks_map(d, &tm, x, rows * cols / 16)) return FP4_ERR_CUDA;
   ProfScope ps(FP4_PROF_QUANTIZE, stream);
-  return launch_quantize(small ? &tm : nullptr, x, rows, cols, codes, scales, tensor_scale, q, d->sms, stream) == cudaSuccess
+  return launch_quantize(small ? &tm : nullptr, x, rows, cols, codes, scales, tensor_scale, q, sms, stream) == cudaSuccess
              ? FP4_OK
              : FP4_ERR_CUDA;
 }
@@ -775,13 +806,14 @@ fp4_status fp4_selftest_quantize_wait(const float* x, int64_t rows, int64_t cols
   const DeviceInfo* d;
   fp4_status rc = check_common(&d);
   if (rc != FP4_OK) return rc;
-  if (!quantize_fits_smem(rows * cols, d->sms)) return FP4_ERR_SHAPE;
+  const int sms = stream_sms(d, stream);
+  if (!quantize_fits_smem(rows * cols, sms)) return FP4_ERR_SHAPE;
   QuantOpts q;
   memset(&q, 0, sizeof(q));
   q.widen = 1.0f;
   CUtensorMap tm;
   if (!make_blocks_map(d, &tm, x, rows * cols / 16)) return FP4_ERR_CUDA;
-  return launch_quantize(&tm, x, rows, cols, codes, scales, tensor_scale, q, d->sms, stream, (uint64_t)limit_us * 1000ull) ==
+  return launch_quantize(&tm, x, rows, cols, codes, scales, tensor_scale, q, sms, stream, (uint64_t)limit_us * 1000ull) ==
                  cudaSuccess
              ? FP4_OK
              : FP4_ERR_CUDA;
@@ -1033,7 +1065,7 @@ static fp4_status gemm_nt_impl(int dry, const uint8_t* a_codes, const uint8_t* a
   L.status = device_status;
   L.dry_operands = dry;
   if (dry && (M % 256 || N % 256 || K % 256)) return FP4_ERR_SHAPE;
-  return launch_gemm_pair(kPlain, pack, L, d->sms, stream) == cudaSuccess ? FP4_OK : FP4_ERR_CUDA;
+  return launch_gemm_pair(kPlain, pack, L, stream_sms(d, stream), stream) == cudaSuccess ? FP4_OK : FP4_ERR_CUDA;
 }
 
 fp4_status fp4_gemm_nt(const uint8_t* a_codes, const uint8_t* a_scales, float a_tensor_scale,

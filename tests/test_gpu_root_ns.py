@@ -860,3 +860,41 @@ def test_batched_norms_are_those_of_single_calls_to_the_last_bit(shape, clip_qua
         single, _ = run_gpu(g, steps=0, clip_quantile=clip_quantile)
         assert fp4.fp4_kernel_launches() - before == (2 if m > n else 1)
         assert np.array_equal(o.cpu().numpy(), single)
+
+
+def test_streams_that_own_a_part_of_the_device():
+    """On a stream of a green context the cooperative launches must fit its SMs; what does not takes the other launches and gives
+    the same bits.  24 SMs hold 72 tiles of a prologue, 24 tiles of G1 and 576 units of the quantiser."""
+    green = getattr(torch.cuda, "GreenContext", None)
+    if green is None or not torch.cuda.green_contexts.SUPPORTED:
+        pytest.skip("this PyTorch has no green contexts")
+    part = green.create(24, 0)
+    stream = torch.cuda.ExternalStream(part.Stream().native_handle)
+    for (m, n), flags, launches in [((256, 512), 0, 2), ((1040, 768), FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX, None),
+                                    ((2048, 2048), 0, 6 + 3 * 3), ((4096, 2048), FP4_FLAG_STORE_BF16, 6 + 3 * 3)]:
+        G = torch.from_numpy(workloads.gradient_like(m, n, seed=m)).cuda()
+        ws = torch.empty(fp4.fp4_root_ns_workspace_bytes(m, n, 3, flags), dtype=torch.uint8, device="cuda")
+        outs = [torch.empty_like(G) for _ in range(2)]
+        for out, st in zip(outs, (None, stream)):
+            torch.cuda.synchronize()
+            before = fp4.fp4_kernel_launches()
+            fp4.fp4_root_ns(G, out, 3, fp4.NsParams.make(flags=flags, seed=1), ws, st)
+            count = fp4.fp4_kernel_launches() - before
+            torch.cuda.synchronize()
+            assert fp4.fp4_last_device_status(ws) == 0
+        assert launches is None or count == launches
+        assert torch.equal(*outs)
+    for shape in ((512, 512), (1152, 2688)):
+        x = torch.from_numpy(workloads.gaussian(*shape, seed=1)).cuda()
+        got = []
+        for st in (None, stream):
+            codes = torch.empty((shape[0], shape[1] // 2), dtype=torch.uint8, device="cuda")
+            scales = torch.empty(fp4.fp4_scale_bytes(*shape), dtype=torch.uint8, device="cuda")
+            ts = torch.empty(1, device="cuda")
+            torch.cuda.synchronize()
+            before = fp4.fp4_kernel_launches()
+            fp4.fp4_quantize(x, codes, scales, ts, stream=st)
+            assert fp4.fp4_kernel_launches() - before == (3 if st is not None and shape[0] == 1152 else 1)
+            torch.cuda.synchronize()
+            got.append((codes, scales, ts))
+        assert all(torch.equal(a, b) for a, b in zip(*got))
