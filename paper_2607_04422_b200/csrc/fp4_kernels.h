@@ -200,6 +200,7 @@ struct AdamwConsts {
   uint64_t seed;
   float one;   // 1, kept from the compiler (fp4_adamw.cu)
   bool plain;  // rsb2 and eps leave sqrt(v) rsb2 + eps in the range of the unguarded square root and division
+  bool plain_zeros;  // also where v is 0
 };
 AdamwConsts adamw_consts(float lr, float beta1, float beta2, float eps, float weight_decay, int step, uint64_t seed);
 cudaError_t launch_adamw_update(uint16_t* W, const uint16_t* G, int64_t n, const AdamwConsts& k, bool sr,

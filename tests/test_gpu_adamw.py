@@ -154,3 +154,54 @@ def test_square_root_and_quotient_range_limits(exp):
         gpu.step(gb, t, sr=t == 2, seed=t, **hp)
         W, st, _, _ = oracle.adamw_update(W, gb, st, step=t, sr=t == 2, seed=t, **hp)
         _compare(gpu, W, st)
+
+
+@pytest.mark.parametrize("eps", [1e-8, 2.0 ** -41, 2.0 ** -42, 0.0])
+def test_zeros_among_in_range_values(eps):
+    # untouched tiles, rows and single parameters (gradients +0 and -0), touched ones whose gradient is zero later, and blocks that
+    # mix zeros with values out of range; from eps = 2^-41 on the zeros take the register-pair form of the update
+    n = 256 * 24
+    rng = np.random.default_rng(7)
+    W = _weights(n, seed=8)
+    W[rng.random(n) < 0.1] = 0
+    gpu, st = GpuAdam(W), None
+    for t in range(1, 5):
+        g = rng.standard_normal(n) * 1e-2
+        g[:256 * 4] = 0.0
+        g[256 * 4:256 * 8] *= t == 1                                         # (with signs: -0 among them)
+        g[256 * 8:256 * 12][rng.random(256 * 4) < 0.5] = 0.0
+        g[256 * 12:256 * 16] *= np.repeat(rng.random(64) < 0.5, 16)
+        g[256 * 16:256 * 18][rng.random(512) < 0.02] = 1e-18                 # v around 2^-120
+        g[256 * 16:256 * 18][rng.random(512) < 0.02] = 0.0
+        gb = oracle.bf16_bits(g.astype(np.float32))
+        hp = {**HP, "eps": eps if eps or t > 1 else 1e-8}
+        if eps == 0.0:
+            gb[gb << 1 & 0xFFFF == 0] = oracle.bf16_bits(np.array([1e-3], np.float32))[0] if t == 1 else 0
+        gpu.step(gb, t, sr=t % 2 == 0, seed=t, **hp)
+        W, st, _, _ = oracle.adamw_update(W, gb, st, step=t, sr=t % 2 == 0, seed=t, **hp)
+        _compare(gpu, W, st)
+
+
+def test_zeros_take_about_the_time_of_other_values():
+    # measured on 2^26 parameters: 182 us with every second gradient zero, 175 us with none; 340 us where zeros leave the fast path
+    n = 1 << 24
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    times = []
+    for share in (0.0, 0.5):
+        W = torch.randn(n, generator=gen, device="cuda").to(torch.bfloat16)
+        g = torch.randn(n, generator=gen, device="cuda") * 1e-2
+        G = torch.where(torch.rand(n, generator=gen, device="cuda") < share, torch.zeros_like(g), g).to(torch.bfloat16)
+        mc, vc = (torch.zeros(n // 2, dtype=torch.uint8, device="cuda") for _ in range(2))
+        ms, vs = (torch.zeros(n // 16, dtype=torch.int16, device="cuda") for _ in range(2))
+        vm = torch.zeros(n // 256, dtype=torch.int16, device="cuda")
+        runs = []
+        for t in range(1, 14):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(10):
+                fp4.fp4_adamw_update(W, G, mc, ms, vc, vs, vm, step=t, **HP)
+            e1.record()
+            torch.cuda.synchronize()
+            runs.append(e0.elapsed_time(e1))
+        times.append(np.median(runs[3:]))
+    assert times[1] < 1.4 * times[0], times
