@@ -420,6 +420,12 @@ fp4_status fp4_selftest_bounded_wait(uint32_t* device_status, uint32_t limit_us,
  * unspecified values.  Arguments as for fp4_quantize; a tensor too large for one launch: FP4_ERR_SHAPE. */
 fp4_status fp4_selftest_quantize_wait(const float* x, int64_t rows, int64_t cols, uint8_t* codes, uint8_t* scales,
                                       float* tensor_scale, uint32_t limit_us, cudaStream_t stream);
+/* The kernels' own square roots, reciprocals and quotients against the general operations (IEEE, to nearest even).
+ * counts: device, out, 8 uint32 - results that differ: [0] square root, every float of [2^-80, 2^30); [1] and [2] the two
+ *   reciprocals, every float of [2^-41, 2^36) and [2^-80, 2^80); [3] a sixth, every float of [2^-100, 2^100); [4] reciprocals of
+ *   BF16 values of [2^-110, 2^110] and of E4M3 scales; [5] and [6] the two quotients, every pair of significands whose
+ *   quotient lies within 3 2^-25 units in the last place of the midpoint of two floats; [7] the number of those pairs. */
+fp4_status fp4_selftest_rounding(uint32_t* counts, cudaStream_t stream);
 
 #ifdef __cplusplus
 }

@@ -32,7 +32,7 @@ EXPORTS = ("fp4_status_string", "fp4_scale_bytes", "fp4_quantize", "fp4_root_coe
            "fp4_root_ns_batched", "fp4_last_device_status", "fp4_root_ns_workspace_layout", "fp4_gemm_nt",
            "fp4_gemm_nt_resident",
            "fp4_profile_enable", "fp4_profile_collect", "fp4_kernel_launches", "fp4_root_ns_static",
-           "fp4_selftest_bounded_wait", "fp4_selftest_quantize_wait")
+           "fp4_selftest_bounded_wait", "fp4_selftest_quantize_wait", "fp4_selftest_rounding")
 PROF_CLASSES = ("clip", "stats", "prep", "G1", "G2", "G3", "transpose", "quantize", "momentum", "adamw")
 
 
@@ -148,6 +148,7 @@ def load_library():
     L.fp4_selftest_bounded_wait.argtypes = [vp, u32, vp]; L.fp4_selftest_bounded_wait.restype = C.c_int
     L.fp4_selftest_quantize_wait.argtypes = [vp, i64, i64, vp, vp, vp, u32, vp]
     L.fp4_selftest_quantize_wait.restype = C.c_int
+    L.fp4_selftest_rounding.argtypes = [vp, vp]; L.fp4_selftest_rounding.restype = C.c_int
     _lib = L
     return L
 
@@ -314,6 +315,11 @@ def fp4_selftest_quantize_wait(x: torch.Tensor, codes: torch.Tensor, scales: tor
     _check(load_library().fp4_selftest_quantize_wait(x.data_ptr(), rows, cols, codes.data_ptr(), scales.data_ptr(),
                                                      tensor_scale.data_ptr(), int(limit_us), _stream(stream)),
            "fp4_selftest_quantize_wait")
+
+
+def fp4_selftest_rounding(counts: torch.Tensor, stream=None) -> None:
+    """counts: 8 int32."""
+    _check(load_library().fp4_selftest_rounding(counts.data_ptr(), _stream(stream)), "fp4_selftest_rounding")
 
 
 def fp4_kernel_launches() -> int:

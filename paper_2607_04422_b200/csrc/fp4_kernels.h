@@ -214,6 +214,9 @@ struct ProfScope {
   ~ProfScope();
 };
 
+// counts: 8 device words (fp4_selftest_rounding)
+cudaError_t launch_selftest_rounding(uint32_t* counts, int sms, cudaStream_t st);
+
 cudaError_t quantize_set_attributes();
 bool quantize_fits_smem(int64_t elements, int sms);
 // tm: x as rows of 16 floats, box = 128 rows, 64-byte swizzle - given when the tensor fits the shared memories, else null

@@ -1116,6 +1116,15 @@ extern "C" fp4_status fp4_selftest_bounded_wait(uint32_t* device_status, uint32_
   return cudaGetLastError() == cudaSuccess ? FP4_OK : FP4_ERR_CUDA;
 }
 
+extern "C" fp4_status fp4_selftest_rounding(uint32_t* counts, cudaStream_t stream) {
+  if (!counts) return FP4_ERR_INVALID_ARG;
+  if (!fp4::aligned(counts, 4)) return FP4_ERR_ALIGNMENT;
+  const fp4::DeviceInfo* d;
+  fp4_status rc = fp4::check_common(&d);
+  if (rc != FP4_OK) return rc;
+  return fp4::launch_selftest_rounding(counts, d->sms, stream) == cudaSuccess ? FP4_OK : FP4_ERR_CUDA;
+}
+
 // ---- fp4_root_ns_static: the step with the workspace in a static device array ------------
 // For callers that cannot allocate device memory (no cudaMalloc allowed where they run, or
 // no pool to take a workspace from).  The array is part of the module image: every device

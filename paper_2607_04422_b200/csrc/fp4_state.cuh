@@ -218,10 +218,7 @@ __device__ __forceinline__ void state_encode(const float (&h)[16], uint64_t seed
   uint32_t lo, hi;
   float d, rcp;
   if (amax >= 0x1p-100f && amax <= 0x1p100f) {
-    const float sixth = 0.16666667163372039794921875f;  // RN(1/6)
-    float x = __fmul_rn(amax, sixth);
-    x = __fmaf_rn(__fmaf_rn(-x, 6.0f, amax), sixth, x);  // RN(amax / 6)
-    const uint32_t w = cvt_bf16x2(x, __fmul_rn(amax, 0.25f));
+    const uint32_t w = cvt_bf16x2(sixth_of(amax), __fmul_rn(amax, 0.25f));
     const float d6 = bf16_lo(w), d4 = bf16_hi(w);
     const float r6 = rcp_bf16(d6), r4 = rcp_bf16(d4);
     uint32_t lo4, hi4;
@@ -254,6 +251,46 @@ __device__ __forceinline__ void state_encode(const float (&h)[16], uint64_t seed
   c = make_uint2(lo, hi);
 }
 
+// Square root and quotient of register pairs for values in the normal range: an approximation, one Newton step and one residual (P.
+// Markstein, IBM J. Res. Dev. 34, 1990).  They round correctly while no intermediate leaves that range: the square root
+// agrees with __fsqrt_rn for every float in [2^-80, 2^30], the reciprocal with __frcp_rn for every float in [2^-41, 2^36];
+// before its last rounding the quotient is off by less than 3 2^-25 units in the last place, and every pair of significands
+// whose quotient lies that close to a midpoint of two floats agrees with __fdiv_rn (fp4_selftest_rounding repeats all three).
+__device__ __forceinline__ uint64_t rsqrt_neg2(uint64_t v) {
+  float a, b;
+  unpack2(v, a, b);
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(-a));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(b) : "f"(-b));
+  return pack2(a, b);
+}
+__device__ __forceinline__ uint64_t rcp_neg2(uint64_t v) {
+  float a, b;
+  unpack2(v, a, b);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(-a));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(b) : "f"(-b));
+  return pack2(a, b);
+}
+
+// -RN(sqrt(v)) from nv = -v.  ZEROS: nv may be -0 (any in-range reciprocal root will do; the result is a zero).
+template <bool ZEROS>
+__device__ __forceinline__ uint64_t neg_sqrt2(uint64_t nv) {
+  uint64_t at = nv;
+  if (ZEROS) {
+    float a, b;
+    unpack2(nv, a, b);
+    at = pack2(fminf(a, -0x1p-80f), fminf(b, -0x1p-80f));
+  }
+  const uint64_t r = rsqrt_neg2(at);
+  const uint64_t nt = mul2(nv, r);
+  return fma2(fma2(nt, nt, nv), mul2(r, pack2(0.5f, 0.5f)), nt);
+}
+// -RN(m / den)
+__device__ __forceinline__ uint64_t neg_quotient2(uint64_t m, uint64_t den) {
+  const uint64_t ny = rcp_neg2(den);
+  const uint64_t ny1 = fma2(fma2(den, ny, pack2(1.0f, 1.0f)), ny, ny);
+  const uint64_t nq = mul2(m, ny1);
+  return fma2(fma2(den, nq, m), ny1, nq);
+}
 // 256-bit global accesses (32-byte aligned): a thread moves its block of 16 floats as two full
 // 32-byte sectors, so no sector is touched by two instructions -- with 128-bit pieces at a
 // 64-byte lane stride every sector is looked up twice on loads and written as two partial

@@ -205,3 +205,12 @@ def test_zeros_take_about_the_time_of_other_values():
             runs.append(e0.elapsed_time(e1))
         times.append(np.median(runs[3:]))
     assert times[1] < 1.4 * times[0], times
+
+
+def test_own_square_roots_reciprocals_and_quotients_round_like_the_general_ones():
+    # nothing is sampled: all arguments, and for the quotients all pairs near enough to a midpoint to round differently
+    counts = torch.full((8,), -1, dtype=torch.int32, device="cuda")
+    fp4.fp4_selftest_rounding(counts)
+    got = counts.cpu().tolist()
+    assert got[:7] == [0] * 7, got
+    assert got[7] == 11630661      # pairs with 1 <= |a 2^e - M b| <= 2, counted with integers (numpy)
