@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
   const float4* src = reinterpret_cast<const float4*>(m.G);
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) s_cnt = 0;
+  for (int j = threadIdx.x; j < kSubBins; j += blockDim.x) s_sub[j] = 0;
   __syncthreads();
   double acc = 0.0;
   float mx = 0.0f;
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
       } else {
         const uint32_t gpos = atomicAdd(&m.hdr->cand_count, 1u);
         if (gpos < g.cand_cap) m.cand[gpos] = k;
-        atomicAdd(&m.hist[(k >> 9) & (kSubBins - 1)], 1u);
+        atomicAdd(&s_sub[(k >> 9) & (kSubBins - 1)], 1u);   // (in global memory: 14.1 ms for an all-zero 4096 x 4096)
       }
     }
   };
@@ -298,8 +299,6 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
   if (nbuf <= kSubBins) {
     for (uint32_t j = threadIdx.x; j < nbuf; j += blockDim.x) atomicAdd(&m.hist[(s_buf[j] >> 9) & (kSubBins - 1)], 1u);
   } else {   // fewer global atomics by way of shared counters
-    for (int j = threadIdx.x; j < kSubBins; j += blockDim.x) s_sub[j] = 0;
-    __syncthreads();
     for (uint32_t j = threadIdx.x; j < nbuf; j += blockDim.x) atomicAdd(&s_sub[(s_buf[j] >> 9) & (kSubBins - 1)], 1u);
     __syncthreads();
     for (int j = threadIdx.x; j < kSubBins; j += blockDim.x)
@@ -343,12 +342,22 @@ __device__ __forceinline__ void write_norm_scalars(float* scalars, const NsScala
 // ---- fallback when the candidate list overflowed (so many equal magnitudes that the picked bin holds more
 // than the list takes: constant matrices and the like).  One block finishes the job alone: two more
 // radix rounds over the whole matrix (bits 17..7, then 6..0) and the clamped sum of squares.  Slow
-// (three passes by 1024 threads) but rare, and it costs no launch when it is not needed.
+// (three passes by 1024 threads) but rare, and it costs no launch when it is not needed.  Bound by the latency of its loads and the
+// counters: all-zero 2560 x 2560, 2 iterations, 1606 us with one load in flight per thread, 1280 with four.
 // hist: 2048 counters; shd: 1024 doubles.
-__device__ void fallback_select_and_stats(const PrepGroup& g, const PrepMatrix& m, uint32_t* hist, double* shd) {
+__device__ __forceinline__ void fallback_select_and_stats(const PrepGroup& g, const PrepMatrix& m, uint32_t* hist, double* shd) {
   __shared__ uint32_t s_fb_prefix, s_fb_rank;
   NsHeader* hdr = m.hdr;
   const float4* src = reinterpret_cast<const float4*>(m.G);
+  auto each = [&](auto&& visit) {   // four loads in flight
+    const int64_t step = blockDim.x;
+    int64_t i = threadIdx.x;
+    for (; i + 3 * step < g.n4; i += 4 * step) {
+      const float4 v0 = __ldg(src + i), v1 = __ldg(src + i + step), v2 = __ldg(src + i + 2 * step), v3 = __ldg(src + i + 3 * step);
+      visit(v0); visit(v1); visit(v2); visit(v3);
+    }
+    for (; i < g.n4; i += step) visit(__ldg(src + i));
+  };
   if (threadIdx.x == 0) { s_fb_prefix = hdr->sel_prefix; s_fb_rank = hdr->sel_rank; }
   __syncthreads();
   for (int round = 0; round < 2; ++round) {
@@ -358,13 +367,12 @@ __device__ void fallback_select_and_stats(const PrepGroup& g, const PrepMatrix& 
     for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x) hist[i] = 0;
     __syncthreads();
     const uint32_t prefix = s_fb_prefix;
-    for (int64_t i = threadIdx.x; i < g.n4; i += blockDim.x) {
-      const float4 v = __ldg(src + i);
+    each([&](const float4& v) {
       const uint32_t k[4] = {mag_bits(v.x), mag_bits(v.y), mag_bits(v.z), mag_bits(v.w)};
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         if ((k[j] & high_mask) == prefix) atomicAdd(&hist[(k[j] >> shift) & (nb - 1)], 1u);
-    }
+    });
     __syncthreads();
     if (threadIdx.x == 0) {
       uint32_t run = 0;
@@ -378,12 +386,11 @@ __device__ void fallback_select_and_stats(const PrepGroup& g, const PrepMatrix& 
   }
   const float tau = __uint_as_float(s_fb_prefix);
   double acc = 0.0;
-  for (int64_t i = threadIdx.x; i < g.n4; i += blockDim.x) {
-    const float4 v = __ldg(src + i);
+  each([&](const float4& v) {
     const float c[4] = {fminf(fabsf(v.x), tau), fminf(fabsf(v.y), tau), fminf(fabsf(v.z), tau), fminf(fabsf(v.w), tau)};
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc += (double)c[j] * (double)c[j];
-  }
+  });
   shd[threadIdx.x] = acc;
   __syncthreads();
   for (int o = blockDim.x / 2; o; o >>= 1) {
@@ -1032,7 +1039,10 @@ static_assert(kResSmem + 64 <= 232448, "at most 227 KB of shared memory (64 byte
 template <bool PF>
 __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_constant__ PrepGroup g) {
   extern __shared__ uint8_t prep_smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(prep_smem_raw) + 1023) & ~(uintptr_t)1023);
+  // The offset is rounded up, not the pointer: through an integer the compiler loses that this is shared memory, and the
+  // counters' atomics on equal values, which the shared ones combine per warp, are done one by one (an all-zero
+  // matrix 1024 x 1024, 2 iterations: 292 us instead of 1620).
+  uint8_t* smem = prep_smem_raw + ((0u - smem_u32(prep_smem_raw)) & 1023u);
   uint8_t* uni = smem + kResTiles * kPrepTile;
   ResidentShared* sh = reinterpret_cast<ResidentShared*>(uni + kResUnion);
   volatile uint32_t* abort_flag = &sh->abort_flag;

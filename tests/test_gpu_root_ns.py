@@ -898,3 +898,56 @@ def test_streams_that_own_a_part_of_the_device():
             torch.cuda.synchronize()
             got.append((codes, scales, ts))
         assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+def _tau_and_nu(G):
+    a = np.abs(G).ravel()
+    rank = -(-99 * a.size // 100)
+    tau = np.partition(a, rank - 1)[rank - 1]
+    return tau, np.float32(np.sqrt(np.square(np.minimum(a, tau).astype(np.float64)).sum()))
+
+
+@pytest.mark.parametrize("shape,count", [((640, 768), 1), ((640, 768), 16), ((4096, 4096), 1)])
+def test_more_candidates_in_a_block_than_its_buffer_takes(shape, count):
+    """Candidates lie together, so that blocks of the prologue meet more of them than fit their shared-memory buffers (8192 where
+    tiles stay resident, 2048 in the passes by tiles and by elements) while the list itself does not overflow."""
+    m, n = shape
+    mats = []
+    for i in range(count):
+        rng = np.random.default_rng(i)
+        g = rng.standard_normal(shape).astype(np.float32) * np.float32(0.1)
+        rows, cols = (slice(128, 256), slice(256, 384)) if m < 4096 else (slice(0, m, 8), slice(0, 1024))
+        g[rows, cols] = np.float32(2.0) + np.float32(0.06) * rng.random(g[rows, cols].shape, dtype=np.float32)
+        mats.append(g)
+    Gs = [torch.from_numpy(g).cuda() for g in mats]
+    outs = [torch.empty_like(g) for g in Gs]
+    ws = torch.full((fp4.fp4_root_ns_batched_workspace_bytes([shape] * count, 1),), 0xFF, dtype=torch.uint8, device="cuda")
+    fp4.fp4_root_ns_batched(Gs, outs, 1, None, ws)
+    assert fp4.fp4_last_device_status(ws) == 0
+    lay = fp4_root_ns_workspace_layout(m, n, 1)
+    stride = (lay.total + 1023) // 1024 * 1024
+    for i in (0, count - 1):
+        sc = ws[i * stride + lay.scalars:i * stride + lay.scalars + 4096].cpu().numpy().view(np.float32)
+        assert (sc[lay.idx_tau], sc[lay.idx_nu]) == _tau_and_nu(mats[i])
+
+
+@pytest.mark.parametrize("shape", [(1024, 4096), (4096, 4096)])
+def test_all_zero_matrices_take_no_time_of_their_own(shape):
+    # every element in one bin: measured 8.8 and 14 times a Gaussian matrix's call (the passes of the finishing block), 69 and 51
+    # times where every element also takes an atomic of its own
+    times = []
+    for G in (torch.randn(shape, device="cuda"), torch.zeros(shape, device="cuda")):
+        out = torch.empty_like(G)
+        ws = torch.empty(fp4.fp4_root_ns_workspace_bytes(*shape, 2), dtype=torch.uint8, device="cuda")
+        runs = []
+        for _ in range(6):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(4):
+                fp4.fp4_root_ns(G, out, 2, None, ws)
+            e1.record()
+            torch.cuda.synchronize()
+            runs.append(e0.elapsed_time(e1))
+        times.append(np.median(runs[2:]))
+    assert not out.any()
+    assert times[1] < 25 * times[0], times
