@@ -89,7 +89,8 @@ typedef enum {
  * the caller's stream waits for it before the call returns, so callers see ordinary stream order and the
  * call can still be captured in a CUDA graph.  Off by default: with two large groups (the decoder-stack
  * benchmark) the gain or loss of about 1.5 % depends on the order in which the two groups' launches meet
- * on the device; the option is for batches of many small groups. */
+ * on the device; the option is for batches of many small groups, whose cooperative launches then take half
+ * of the SMs each. */
 #define FP4_FLAG_OVERLAP_GROUPS 32u
 #define FP4_QUANT_SIGNS(mask) ((uint32_t)(mask) << 16)
 

@@ -233,9 +233,10 @@ struct PrologueItem {
   uint32_t* hist_top;      // the caller's histogram of the top 13 magnitude bits of G, or null
   const CUtensorMap* tmG;  // G as an FP32 tensor: box = 32 columns x 128 rows, 128-byte swizzle
 };
-// count matrices that share the shape (s, l) and the clip / eps parameters; sms: those the stream's kernels can occupy
+// count matrices that share the shape (s, l) and the clip / eps parameters; sms: those the stream's kernels can occupy, coop_sms:
+// those a cooperative launch may count on
 cudaError_t launch_prologue_group(const PrologueItem* items, int count, int write_q, const QuantOpts& q,
-                                  uint32_t* status, int sms, cudaStream_t st);
+                                  uint32_t* status, int coop_sms, int sms, cudaStream_t st);
 // Root's parameter update on BF16 weights: decay = fl(1 - fl(lr * wd)), step = fl(lr * scale),
 // w <- BF16(fl(fl(w * decay) - fl(step * o))).
 struct ParamUpdate {

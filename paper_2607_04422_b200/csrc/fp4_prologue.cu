@@ -1393,7 +1393,7 @@ cudaError_t prologue_set_attributes() {
 
 // Enqueue the prologue for `count` matrices of one shape (s, l) and one parameter set.
 cudaError_t launch_prologue_group(const PrologueItem* items, int count, int write_q, const QuantOpts& q,
-                                  uint32_t* status, int sms, cudaStream_t st) {
+                                  uint32_t* status, int coop_sms, int sms, cudaStream_t st) {
   for (int i0 = 0; i0 < count; i0 += kMaxPack) {
     const int nn = count - i0 < kMaxPack ? count - i0 : kMaxPack;
     const NsPlan& pl = *items[i0].pl;
@@ -1442,13 +1442,13 @@ cudaError_t launch_prologue_group(const PrologueItem* items, int count, int writ
     const int64_t matrix_tiles = (pl.l / 128) * (pl.s / 128), tiles = matrix_tiles * nn;
     const bool tiled = matrix_tiles <= (int64_t)kResTiles * pl.sms && matrix_tiles <= 1024;   // 1024 partials
     g.stat_blocks = tiled ? (int)matrix_tiles : pl.stat_blocks;
-    if (tiled && tiles <= (int64_t)kResTiles * sms) {
+    if (tiled && tiles <= (int64_t)kResTiles * coop_sms) {
       // everything fits the shared memories: one launch
       ProfScope ps(FP4_PROF_PREP, st);
       cudaError_t e = cudaMemsetAsync(&g.mat[0].hdr->barrier, 0, 4, st);
       if (e != cudaSuccess) return e;
       cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)(tiles < sms ? tiles : sms)); cfg.blockDim = dim3(kPrepThreads);
+      cfg.gridDim = dim3((unsigned)(tiles < coop_sms ? tiles : coop_sms)); cfg.blockDim = dim3(kPrepThreads);
       cfg.dynamicSmemBytes = kResSmem; cfg.stream = st;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeCooperative;

@@ -560,7 +560,7 @@ fp4_status prepare_matrix(const DeviceInfo* d, const float* G, float* out, int64
 // then every Newton-Schulz stage as one launch over all matrices of the group.
 // count <= kPackMax: the problems of a launch travel as its parameter.
 fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps, const fp4_ns_params* p,
-                     uint32_t* status, bool clear_first_status, cudaStream_t st) {
+                     uint32_t* status, bool clear_first_status, bool two_streams, cudaStream_t st) {
   if (count < 1 || count > kPackMax) return FP4_ERR_INVALID_ARG;
   const bool keep = (p->flags & FP4_FLAG_KEEP_OPERANDS) != 0;
   ParamUpdate upd;
@@ -585,9 +585,14 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     if (steps > 0 && mats[i].pl.tall && !keep && !any_update) { direct_out[(size_t)i] = 1; any_direct = true; }
   const NsPlan& pl0 = mats[0].pl;
   const int64_t s = pl0.s, l = pl0.l;
-  const int sms = stream_sms(d, st);
+  // A cooperative launch that needs more than half of the SMs keeps the other stream's group waiting: the two take half each, and
+  // what does not fit is left to the plain launches, which share the SMs as they become free.
+  // Measured, 5 iterations, one stream / two with whole-device launches / with halves: six groups of one matrix (1536 x 1536 ..
+  // 2816) 1177 / 1160 / 834 us, eight of one (640 x 640 .. 1536) 885 / 680 / 490, six of two (1280 x 1280 .. 2560)
+  // 1197 / 1184 / 996, eight tiny ones 780 / 405 / 407; four groups of four with the quantiser options lose (1323 / 1447).
+  const int sms = stream_sms(d, st), coop_sms = two_streams && sms > 1 ? sms / 2 : sms;
   pdl_select(s * l * count);
-  const Route route = steps > 0 ? route_of(pl0, count, p, sms) : kThreeLaunches;
+  const Route route = steps > 0 ? route_of(pl0, count, p, coop_sms) : kThreeLaunches;
   {
     std::vector<PrologueItem> items((size_t)count);
     for (int i = 0; i < count; ++i) {
@@ -595,7 +600,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       items[(size_t)i] = PrologueItem{c.G, c.X, c.ws, &c.pl, clear_first_status && i == 0, c.store_x0, c.x_rows, c.x_cols,
                                       c.hist_top, &c.tm_G};
     }
-    if (launch_prologue_group(items.data(), count, steps > 0 || keep, quant_opts(p, 0), status, sms, st) != cudaSuccess)
+    if (launch_prologue_group(items.data(), count, steps > 0 || keep, quant_opts(p, 0), status, coop_sms, sms, st) != cudaSuccess)
       return FP4_ERR_CUDA;
   }
   ChainPack pack;
@@ -622,7 +627,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       if (!keep) { direct_out[(size_t)j] = mats[j].pl.tall; fused_update[(size_t)j] = 1; }
     }
     ProfScope ps(FP4_PROF_G3, st);
-    if (launch_chain(pack, a, sms, st) != cudaSuccess) return FP4_ERR_CUDA;
+    if (launch_chain(pack, a, coop_sms, st) != cudaSuccess) return FP4_ERR_CUDA;
   } else if (steps > 0) {
     // the problems of the five kinds of launches: G1, G2, G3 reading qXt[0] / qXt[1], the first G3
     std::vector<ProblemPack> packs(5);
@@ -662,7 +667,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       L1.out_h = bf16;
       if (route == kTwoLaunches) {
         ProfScope ps(FP4_PROF_G1, st);
-        if (launch_chain_symmetric(pack, a, k, sms, st) != cudaSuccess) return FP4_ERR_CUDA;
+        if (launch_chain_symmetric(pack, a, k, coop_sms, st) != cudaSuccess) return FP4_ERR_CUDA;
       } else {
         ProfScope ps(FP4_PROF_G1, st);
         if (launch_gemm_pair(kG1, packs[0], L1, sms, st) != cudaSuccess)
@@ -733,7 +738,7 @@ fp4_status run_one(const DeviceInfo* d, const float* G, float* out, int64_t m, i
   if (rc != FP4_OK) return rc;
   if (p->top_hist) c.hist_top = p->top_hist[0];
   if (p->weights) c.W = p->weights[0];
-  return run_group(d, &c, 1, steps, p, reinterpret_cast<uint32_t*>(ws + c.pl.lay.header), clear_status, st);
+  return run_group(d, &c, 1, steps, p, reinterpret_cast<uint32_t*>(ws + c.pl.lay.header), clear_status, false, st);
 }
 
 fp4_status check_common(const DeviceInfo** d) {
@@ -1017,7 +1022,7 @@ fp4_status fp4_root_ns_batched(int count, const float* const* G, float* const* o
   }
   for (size_t gi = 0; gi < groups.size(); ++gi) {
     cudaStream_t st = (side && (gi & 1)) ? side->stream : stream;
-    rc = run_group(d, groups[gi].data(), (int)groups[gi].size(), steps, p, status, !side && gi == 0, st);
+    rc = run_group(d, groups[gi].data(), (int)groups[gi].size(), steps, p, status, !side && gi == 0, side != nullptr, st);
     if (rc != FP4_OK) break;
   }
   if (side) {

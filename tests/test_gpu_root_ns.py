@@ -951,3 +951,29 @@ def test_all_zero_matrices_take_no_time_of_their_own(shape):
         times.append(np.median(runs[2:]))
     assert not out.any()
     assert times[1] < 25 * times[0], times
+
+
+def test_groups_on_two_streams_share_the_device():
+    """Six groups that a single launch each would spread over all SMs: with FP4_FLAG_OVERLAP_GROUPS two of them run side by side
+    (measured 834 us against 1177 one after the other; 1160 where a group's launch takes the whole device), same bits."""
+    shapes = [(1536, 1536 + 256 * i) for i in range(6)]
+    Gs = [torch.from_numpy(workloads.gradient_like(*s, seed=i)).cuda() for i, s in enumerate(shapes)]
+    results, times = [], []
+    for flags in (0, FP4_FLAG_OVERLAP_GROUPS):
+        outs = [torch.empty_like(g) for g in Gs]
+        ws = torch.empty(fp4.fp4_root_ns_batched_workspace_bytes(shapes, 5, flags), dtype=torch.uint8, device="cuda")
+        p = fp4.NsParams.make(flags=flags)
+        runs = []
+        for _ in range(8):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(5):
+                fp4.fp4_root_ns_batched(Gs, outs, 5, p, ws)
+            e1.record()
+            torch.cuda.synchronize()
+            runs.append(e0.elapsed_time(e1))
+        assert fp4.fp4_last_device_status(ws) == 0
+        results.append(outs)
+        times.append(np.median(runs[3:]))
+    assert all(torch.equal(a, b) for a, b in zip(*results))
+    assert times[1] < 0.9 * times[0], times
