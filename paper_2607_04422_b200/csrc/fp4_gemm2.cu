@@ -255,21 +255,6 @@ __device__ __forceinline__ void mbar_expect_tx_s(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive_s(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-#ifdef FP4_TRACE
-// Diagnostics build only: cycles each role spends waiting, summed per warp.
-__device__ unsigned long long g_trace[160 * 19 * 8];
-#define TR_DECL unsigned long long tr_[8] = {0, 0, 0, 0, 0, 0, 0, 0}; long long tr_t0_ = clock64(), tr_s_ = 0;
-#define TR_BEGIN tr_s_ = clock64();
-#define TR_END(k) tr_[k] += (unsigned long long)(clock64() - tr_s_);
-#define TR_COUNT(k) tr_[k] += 1;
-#define TR_FLUSH if ((threadIdx.x & 31) == 0) { tr_[7] = (unsigned long long)(clock64() - tr_t0_); for (int k_ = 0; k_ < 8; ++k_) g_trace[(blockIdx.x * 19 + (threadIdx.x >> 5)) * 8 + k_] = tr_[k_]; }
-#else
-#define TR_DECL
-#define TR_BEGIN
-#define TR_END(k)
-#define TR_COUNT(k)
-#define TR_FLUSH
-#endif
 
 // warp index, known to the compiler to be the same in all lanes
 __device__ __forceinline__ int uniform_warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
@@ -346,7 +331,6 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
     // ------------------------------------------------------------ operand producer (both CTAs)
     if (elect_one()) {
       int st = 0; uint32_t ph = 0;
-      TR_DECL
       // G3's operands (qB and the transposed copy of qX, some 20 MB per matrix) are re-read by every tile
       // while 200 MB of FP32 X stream through the L2 beside them: a stage completes when its last byte
       // has arrived, so even a small share of operand lines evicted to DRAM makes almost every stage wait
@@ -365,9 +349,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         const int arow = ti * PM + (int)rank * BM;   // this CTA's rows of the row operand
         const int brow = tj * PN + (int)rank * BM;   // this CTA's half of the column operand
         for (int kb = 0; kb < (dry ? min(num_kb, STAGES) : num_kb); ++kb) {
-          TR_BEGIN
           wait_or_abort(&bars->empty[st], ph ^ 1, abort_flag);
-          TR_END(0)
           const uint32_t full_leader = map_to_cta(&bars->full[st], 0);
           if (leader) mbar_expect_tx(&bars->full[st], 2 * STAGE_BYTES_CTA);
           TMA_OPERAND(smem + OFF_A + st * OPER_BYTES, &pr->tmA, kb * (BK / 2), arow, full_leader);
@@ -380,30 +362,21 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
           if (++st == STAGES) { st = 0; ph ^= 1; }
         }
       }
-      TR_FLUSH
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA only)
     if (leader && elect_one()) {
       int st = 0; uint32_t ph = 0, seq = 0;
-      TR_DECL
       for (int t = pair; t < num_tiles; t += num_pairs, ++seq) {
         const uint32_t par = seq & 1, buse = seq >> 1;
-        TR_COUNT(6)
-        TR_BEGIN
         // this buffer's previous tile is drained, and so are the columns it shares with the
         // buffer of the tile before this one
         wait_or_abort(&bars->acc_empty[par], (buse & 1) ^ 1, abort_flag);
-        TR_END(0)
-        TR_BEGIN
         if (seq > 0) wait_or_abort(&bars->ov_free, (seq - 1) & 1, abort_flag);
-        TR_END(1)
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + par * ACC1_COL;
         for (int kb = 0; kb < num_kb; ++kb) {
-          TR_BEGIN
           if (!dry || (seq == 0 && kb < STAGES)) wait_or_abort(&bars->full[st], ph, abort_flag);
-          TR_END(2)
           tc_fence_after();
           const uint32_t sf_t = tmem_base + TMEM_SF_COL;
           const uint8_t* sf = smem + OFF_SF + st * SF_BYTES;
@@ -423,7 +396,6 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         }
         tc_commit_pair(&bars->acc_full[par]);
       }
-      TR_FLUSH
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------ issuer of the half-tile stores
@@ -548,7 +520,6 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
     uint32_t seq = 0;
     int t = pair;
     Geo cur;
-    TR_DECL
     if (t < num_tiles) {
       cur = geometry(t, 0);
       if (HAS_AUX) {
@@ -605,10 +576,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
       const bool store_out = STORE_F32 && !(UPD && args.no_out && pr->W != nullptr);
       const bool stage = (store_out && !hout) || mirror;
       const bool rows_in = y32 < pr->out_rows;                          // else: zero padding of the work shape
-      TR_COUNT(6)
-      TR_BEGIN
       wait_or_abort(&bars->acc_full[par], (seq >> 1) & 1, abort_flag);
-      TR_END(0)
       tc_fence_after();
       const uint32_t acc_empty_leader = par ? acc_empty_leader1 : acc_empty_leader0;
 
@@ -670,9 +638,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         const int xcol = x64 + e * CHUNK;
         float v[16];
         if (HAS_AUX) {
-          TR_BEGIN
           wait_or_abort(xfull0 + b * 8, (uint32_t)(i / XBUF & 1), abort_flag);
-          TR_END(1)
         }
         tc_wait_ld16(acc);
         // ---- combine the accumulator block with the FP32 tile
@@ -837,9 +803,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         // scheduled after the fetch, and now and then the new block arrived first).
         if (HAS_AUX) fence_proxy_async_smem();
         __syncwarp();
-        TR_BEGIN
         if (lane == 0 && (STORE_F32 || i == 0)) bulk_wait_read<0>();
-        TR_END(3)
         if (XBUF == 1) __syncwarp();  // one buffer: the next chunk is staged over this one, after the store's read
         if (HAS_AUX) {
           if (i < TEAM_CHUNKS - XBUF) fetch(pr, x64, y32, (i + XBUF) ^ flip, false, b);
@@ -898,7 +862,6 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         atomicMax(reinterpret_cast<uint32_t*>(pr->scalars + slot), __float_as_uint(amax));
       }
     }
-    TR_FLUSH
     if (lane == 0) bulk_wait_all<0>();  // this warp's stores have left shared memory and are complete
   }
 
@@ -941,17 +904,6 @@ cudaError_t launch_pair_mode(const ProblemPack& pack, const GemmLaunch& L, int s
 }
 
 }  // namespace
-
-#ifdef FP4_TRACE
-extern "C" int fp4_trace_read(unsigned long long* dst, int clear) {
-  if (cudaMemcpyFromSymbol(dst, g_trace, sizeof(g_trace)) != cudaSuccess) return 1;
-  if (clear) {
-    static unsigned long long zero[160 * 19 * 8];
-    if (cudaMemcpyToSymbol(g_trace, zero, sizeof(zero)) != cudaSuccess) return 1;
-  }
-  return 0;
-}
-#endif
 
 template <int MODE, bool PF, bool BH, bool UPD, bool DEEP>
 static cudaError_t set_attribute() {
