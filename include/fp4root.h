@@ -76,8 +76,9 @@ typedef enum {
  * precision; FP32 is the default): A_k and X_k (k >= 1) are kept in BF16, round to nearest
  * even, which halves the FP32 traffic of the fused epilogues.  The NVFP4 operand copies and the
  * running maxima are still derived from the FP32 values in the epilogue, X_0 stays FP32 and
- * the result is FP32.  The copies are 2-byte tensors, except in a group small enough to run all
- * its iterations in one launch, where they are FP32 tensors that hold the rounded values. */
+ * the result is FP32.  The copies are 2-byte tensors, except in launches that hold several products, where
+ * they are FP32 tensors of the rounded values: both in a group small enough to run all its iterations in one launch, A in
+ * one that runs G1 and G2 in one (short sides up to 2048). */
 #define FP4_FLAG_STORE_BF16 8u
 /* With fp4_ns_params.weights: the FP32 result is not written (the parameter update is all the caller
  * wants).  `out` is still required - it is the working copy of X during the iterations of a wide matrix -

@@ -889,9 +889,11 @@ cudaError_t launch_pair_variant(const ProblemPack& pack, const GemmLaunch& L, in
 // G2 and G3 with a long contraction take the deep layout: there the main loop of a tile outlasts its epilogue, even one that
 // waits for every block of the FP32 tile.  Measured, G2 + G3 of 5 iterations, without / with: 16384 x 16384 20.1 / 18.0 ms,
 // 8192 x 8192 2.72 / 2.42, 4096 x 14336 1.10 / 0.99.  G2 (one tile read, none written) gains from shorter ones on: seven
-// matrices of a 3072-wide decoder block 525 / 495 us, one 2560 x 6912 105 / 104.  So does G3 in launches of many tiles, which
-// run under the power cap, where a clock cycle is longer and the latency of a fetch fewer of them: 28 such matrices
-// 5.29 / 5.05 ms, but seven 1.46 / 1.50 ms and one 0.325 / 0.330.  The quantiser options double the epilogue: G3 of
+// matrices of a 3072-wide decoder block 525 / 495 us, one 2560 x 6912 105 / 104.  So does G3 in launches of many tiles,
+// which run under the power cap, where a clock cycle is longer and the latency of a fetch fewer of them.  Stacks of decoder blocks
+// in sustained runs, without / with it in G3: 28 matrices 2816 wide 8.37 / 8.27 ms, 3072 10.09 / 9.93, 3328 12.36 / 11.97, 21 of
+// 3584 11.14 / 10.64, of 3840 13.34 / 12.79, two of 3072 x 32768 (3072 tiles) 4.20 / 3.95; but seven 3072-wide ones
+// (1152 tiles) 1.46 / 1.50 ms and one 0.325 / 0.330.  The quantiser options double the epilogue: G3 of
 // 8192 x 8192 1.71 / 1.47 ms, of 4096 x 16384 1.07 / 1.14, G2 of 4096 x 4096 186 / 182 us.
 template <int MODE, bool PF, bool BH, bool UPD = false>
 cudaError_t launch_pair_mode(const ProblemPack& pack, const GemmLaunch& L, int sms, cudaStream_t st) {

@@ -506,10 +506,10 @@ fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t
   return FP4_OK;
 }
 
-// Everything build_matrix derives (workspace plan, a dozen and a half TMA descriptors, the problem
+// Everything build_matrix derives (workspace plan, some forty TMA descriptors, the problem
 // descriptions) depends only on the pointers, the shape and a few parameters: an optimiser calls with
 // the same buffers every step, so the results are kept, keyed by exactly those inputs.  The library
-// keeps no other state between calls; a hit costs one hash lookup instead of ~20 driver calls.
+// keeps no other state between calls; a hit costs one hash lookup instead of some forty driver calls.
 struct CtxKey {
   int dev; int steps; uint32_t flags;
   const void* G; const void* out; const void* ws;
