@@ -157,20 +157,6 @@ __device__ __forceinline__ void mom_decode(uint2 c, uint32_t scale_bits, float (
   hadamard16_pairs(v);
 }
 
-// Two-candidate encoding of a transformed block by the plain operations of the definition.
-static __device__ __noinline__ uint3 encode_pair_exact(float h0, float h1, float h2, float h3, float h4, float h5, float h6,
-                                                       float h7, float h8, float h9, float h10, float h11, float h12,
-                                                       float h13, float h14, float h15, float amax) {
-  const float h[16] = {h0, h1, h2, h3, h4, h5, h6, h7, h8, h9, h10, h11, h12, h13, h14, h15};
-  const uint32_t w = cvt_bf16x2(__fdiv_rn(amax, 6.0f), __fdiv_rn(amax, 4.0f));
-  uint32_t lo, hi, lo4, hi4;
-  const float err6 = mom_encode_rtn(h, bf16_lo(w), lo, hi);
-  const float err4 = mom_encode_rtn(h, bf16_hi(w), lo4, hi4);
-  uint32_t scale_bits = w & 0xFFFFu;
-  if (err4 < err6) { scale_bits = w >> 16; lo = lo4; hi = hi4; }
-  return make_uint3(lo, hi, scale_bits);
-}
-
 // Nearest-rounding codes of one transformed block for a BF16 block scale d in the normal range, with rcp = RN(1 / d);
 // returns the sum of the squared FP32 errors in element order.  code * d has at most 2 + 8 significant bits, so one
 // fused operation gives the rounded difference that a product and a subtraction would.
@@ -198,6 +184,35 @@ __device__ __forceinline__ float mom_encode_fast(const float (&h)[16], float d, 
   return err;
 }
 
+// The same codes and another error: the squared differences between the scaled values and their codes, summed in any order.
+// A mixed-precision multiply-add on the FP16 value of a code and a fused square per pair take half of the instructions.
+__device__ __forceinline__ float mom_encode_scaled(const float (&h)[16], float rcp, uint32_t& lo, uint32_t& hi) {
+  const uint64_t rcp2 = pack2(rcp, rcp);
+  uint64_t sum[2];
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    float y[8];
+    uint32_t codes, q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) unpack2(mul2(pack2(h[8 * b + 2 * i], h[8 * b + 2 * i + 1]), rcp2), y[2 * i], y[2 * i + 1]);
+    cvt_e2m1x8_f16(y, codes, q);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float d0, d1;
+      asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\t"
+          "fma.rn.f32.f16 %0, a, %3, %4;\n\tfma.rn.f32.f16 %1, b, %3, %5;\n\t}"
+          : "=f"(d0), "=f"(d1)
+          : "r"(q[i]), "h"((uint16_t)0xBC00), "f"(y[2 * i]), "f"(y[2 * i + 1]));
+      const uint64_t dd = pack2(d0, d1);
+      sum[b] = i == 0 ? mul2(dd, dd) : fma2(dd, dd, sum[b]);
+    }
+    if (b == 0) lo = codes; else hi = codes;
+  }
+  float a, c;
+  unpack2(add2(sum[0], sum[1]), a, c);
+  return a + c;
+}
+
 // RN(1 / d) of a BF16 value in [2^-110, 2^110]: one Newton step on the approximation leaves a relative error near
 // 2^-46, and the reciprocals of 8-bit significands lie at least 2^-33 from the midpoint of two floats.
 __device__ __forceinline__ float rcp_bf16(float d) {
@@ -206,28 +221,58 @@ __device__ __forceinline__ float rcp_bf16(float d) {
   return __fmaf_rn(r, __fmaf_rn(-d, r, 1.0f), r);
 }
 
+// Two-candidate encoding of a transformed block with the errors of the definition: fused operations on pairs in a normal
+// range, else its plain operations.
+static __device__ __noinline__ uint3 encode_pair_exact(float h0, float h1, float h2, float h3, float h4, float h5, float h6,
+                                                       float h7, float h8, float h9, float h10, float h11, float h12,
+                                                       float h13, float h14, float h15, float amax) {
+  const float h[16] = {h0, h1, h2, h3, h4, h5, h6, h7, h8, h9, h10, h11, h12, h13, h14, h15};
+  uint32_t w, lo, hi, lo4, hi4;
+  float err6, err4;
+  if (amax >= 0x1p-100f && amax <= 0x1p100f) {
+    w = cvt_bf16x2(sixth_of(amax), __fmul_rn(amax, 0.25f));
+    err6 = mom_encode_fast(h, bf16_lo(w), rcp_bf16(bf16_lo(w)), lo, hi);
+    err4 = mom_encode_fast(h, bf16_hi(w), rcp_bf16(bf16_hi(w)), lo4, hi4);
+  } else {
+    w = cvt_bf16x2(__fdiv_rn(amax, 6.0f), __fdiv_rn(amax, 4.0f));
+    err6 = mom_encode_rtn(h, bf16_lo(w), lo, hi);
+    err4 = mom_encode_rtn(h, bf16_hi(w), lo4, hi4);
+  }
+  uint32_t scale_bits = w & 0xFFFFu;
+  if (err4 < err6) { scale_bits = w >> 16; lo = lo4; hi = hi4; }
+  return make_uint3(lo, hi, scale_bits);
+}
+
 // Encodes a transformed block: candidate scales BF16(amax / 6) and BF16(amax / 4), nearest rounding with each, the
 // smaller squared error (a tie keeps 6); SR: once more by stochastic rounding with the chosen scale, `first` =
-// the matrix index of the block's first element.  The kernels that call this are bound by the instructions they issue,
-// so the candidates' errors come from fused operations on pairs and the scales from multiplications: AdamW of 2^26
-// parameters 226 -> 208 us, momentum of 8192 x 4096 without other outputs 43.6 -> 39.5 us.  That needs a normal range:
-// blocks whose amax is zero or far from 1 take the plain operations.
+// the matrix index of the block's first element.  The kernels that call this are bound by the instructions they issue, so the
+// candidates are compared by the errors s6 and s4 of the scaled values, in units of the first scale d.  A scaled value is
+// at most 6.05 and off by 2^-23 of itself, which moves a sum S of sixteen squares by less than 2 sqrt(S) 4 2^-20.4 + 2^-36;
+// rounding the sums moves either form by less than 2^-19 of it, and the definition's loses another 32 2^-150 / d^2 < 2^-29
+// to underflow while amax >= 2^-55.  So the order is certain when the two differ by 2^-14 of the larger or of 1/16 (2 2^-17.4
+// sqrt(S) <= 2^-14.4 S for S >= 1/16, and 2^-18.4 below).  Closer ones, some 10^-4 of the blocks, and blocks out of range take
+// the errors of the definition; a block of zeros is all zeros.  AdamW of 2^26 parameters 174.2 -> 165.3 us.
 template <bool SR>
 __device__ __forceinline__ void state_encode(const float (&h)[16], uint64_t seed, uint64_t first, uint2& c, uint32_t& scale_bits) {
   const float amax = amax16(h);
-  uint32_t lo, hi;
-  float d, rcp;
-  if (amax >= 0x1p-100f && amax <= 0x1p100f) {
+  uint32_t lo = 0, hi = 0;
+  float d = 0.0f, rcp = 0.0f;
+  scale_bits = 0;
+  bool certain = amax == 0.0f;
+  if (amax >= 0x1p-55f && amax <= 0x1p55f) {
     const uint32_t w = cvt_bf16x2(sixth_of(amax), __fmul_rn(amax, 0.25f));
     const float d6 = bf16_lo(w), d4 = bf16_hi(w);
     const float r6 = rcp_bf16(d6), r4 = rcp_bf16(d4);
     uint32_t lo4, hi4;
-    const float err6 = mom_encode_fast(h, d6, r6, lo, hi);
-    const float err4 = mom_encode_fast(h, d4, r4, lo4, hi4);
+    const float s6 = mom_encode_scaled(h, r6, lo, hi);
+    const float ratio = d4 * r6;
+    const float s4 = mom_encode_scaled(h, r4, lo4, hi4) * (ratio * ratio);
+    certain = fabsf(s4 - s6) > 0x1p-14f * fmaxf(fmaxf(s4, s6), 0.0625f);
     d = d6; rcp = r6;
     scale_bits = w & 0xFFFFu;
-    if (err4 < err6) { d = d4; rcp = r4; scale_bits = w >> 16; lo = lo4; hi = hi4; }
-  } else {
+    if (s4 < s6) { d = d4; rcp = r4; scale_bits = w >> 16; lo = lo4; hi = hi4; }
+  }
+  if (!certain) {
     const uint3 e = encode_pair_exact(h[0], h[1], h[2], h[3], h[4], h[5], h[6], h[7], h[8], h[9], h[10], h[11], h[12], h[13],
                                       h[14], h[15], amax);
     lo = e.x; hi = e.y; scale_bits = e.z;

@@ -72,6 +72,56 @@ def test_ema_form_and_optional_outputs():
     assert np.array_equal(c, oc) and np.array_equal(s, os_)
 
 
+def _errors_of_both_scales(h):
+    """FP64 errors of the nearest-rounding codes of rows h for the scales BF16(amax / 6) and BF16(amax / 4)."""
+    grid = np.array([0, 0.5, 1, 1.5, 2, 3, 4, 6])
+    amax = np.abs(h).max(axis=1)
+    out = []
+    for div in (6, 4):
+        d = oracle.bf16_bits((amax / np.float32(div)).astype(np.float32)).astype(np.uint32)
+        d = (d << 16).view(np.float32).astype(np.float64)[:, None]
+        y = np.abs(h) / d
+        q = grid[np.abs(y[..., None] - grid).argmin(axis=-1)]
+        out.append((((y - q) * d) ** 2).sum(axis=1))
+    return out
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -90, 2.0 ** 95])
+def test_nearly_tied_candidate_scales_take_the_order_of_the_definition(scale):
+    """Blocks whose two candidate errors agree to a few parts per million, and neighbours of them on both sides of the tie:
+    what the kernel may decide from rounded sums and what it must leave to the definition."""
+    rng = np.random.default_rng(5)
+    H = np.array([[(-1) ** bin(i & j).count("1") for j in range(16)] for i in range(16)], np.float64) / 4
+    g = rng.standard_normal((1 << 17, 16)).astype(np.float32)
+    e6, e4 = _errors_of_both_scales((g.astype(np.float64) @ H).astype(np.float32))
+    close = np.abs(e4 - e6) / np.maximum(e4, e6)
+    g = g[np.argsort(close)[:256]]
+    assert close[np.argsort(close)[255]] < 2e-2 and close.min() < 1e-4
+    # a step along one element that moves the difference of the errors through zero
+    blocks = [g]
+    for i in (0, 7):
+        step = np.zeros_like(g)
+        step[:, i] = 2.0 ** -12
+        f = lambda x: (lambda a: a[1] - a[0])(_errors_of_both_scales((x.astype(np.float64) @ H).astype(np.float32)))
+        lo, hi = g - step * 64, g + step * 64
+        for _ in range(30):                            # bisection in FP32, where the signs differ
+            mid = ((lo.astype(np.float64) + hi) / 2).astype(np.float32)
+            same = (np.sign(f(mid)) == np.sign(f(lo)))[:, None]
+            lo, hi = np.where(same, mid, lo), np.where(same, hi, mid)
+        for ulps in (-3, -1, 0, 1, 3):
+            b = lo.copy()
+            b[:, i] = (b[:, i].view(np.int32) + ulps).view(np.float32)
+            blocks.append(b)
+    G = (np.concatenate(blocks).reshape(-1, 256) * np.float32(scale)).astype(np.float32)
+    st = GpuState(*G.shape)
+    _step(G, st, mu=0.0)
+    zero = np.zeros((G.shape[0], 128), np.uint8), np.zeros((G.shape[0], 16), np.uint16)
+    _, oc, os_, _ = oracle.momentum_update(G, *zero, 0.0, 1.0)
+    c, s = st.numpy()
+    assert np.array_equal(s, os_), mismatch_report(s, os_)
+    assert np.array_equal(c, oc), mismatch_report(c, oc)
+
+
 def test_ties_zero_blocks_and_extreme_magnitudes():
     f = np.float32
     H4 = oracle.hadamard16  # only to place chosen values in the transformed domain
