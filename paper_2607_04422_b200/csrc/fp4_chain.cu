@@ -12,18 +12,25 @@
 // b, b + grid, ... of every product.  Every dependency points to an earlier product and all blocks are
 // resident (cooperative launch), so the earliest unfinished tile can always run.  Since G1 and G2 list the
 // same tiles, and every G3 lists the same tiles, the FP32 values a tile combines with (A in G2, X in G3) were
-// written by the very thread that reads them: they need no ordering between blocks and are fetched
-// before the dependency is even looked at.
+// written by the very thread that reads them.  So they stay where they are: beside the accumulators the tensor memory has room
+// for 6 tiles of 64 columns or 2 of 128, and a block's first tiles of A and X live there from product to product
+// (place_resident); only the caller's matrix in the first G3, the result in the last, and tiles beyond that room
+// move through memory, fetched before the dependency is even looked at.
 //
 // Warp roles: 0-15 epilogue, 16 operand producer (TMA; also the only thread that polls the counter), 17 MMA
 // issuer and TMEM owner, 18 stores.  Epilogue warp w owns the TMEM lanes of quadrant w % 4 and the 16-column
-// (or two 16-column) pieces w / 4 of the tile; it moves its 32 x 16 FP32 blocks with its own TMA loads and
-// stores and shares nothing with the other epilogue warps but the staging area in which the tile's
+// (or two 16-column) pieces w / 4 of the tile; what moves through memory it moves with its own TMA loads and
+// stores, and it shares nothing with the other epilogue warps but the staging area in which the tile's
 // quantised outputs are collected.  The store warp sends that area off, waits until it has arrived, publishes
 // the running maximum and counts the tile.
 //
-// Bounds: latency.  A 5-iteration call is a chain of 15 dependent products.  At 256 x 512 a product takes about 5 us:
-// the counter's round trip and the release 1.5, operand copies and MMAs 1, the one tile's epilogue 2.
+// Bounds: latency.  A 5-iteration call is a chain of 15 dependent products.  At 256 x 512 a product takes about 4 us:
+// operand copies 0.75, MMAs 0.3, the one tile's epilogue 0.75-1.1, its stores and the release 1.1, the counter's way to the
+// slowest of the other blocks 0.8.  The epilogue has 96 registers per thread for 16 values in flight: with both passes' values
+// in registers at once it spilled, and every spill is a trip through the shared memory's pipe.  Resident tiles with
+// a path of their own that needs nothing else, and the second pass's values read after the first, whole calls: 256 x 512
+// 94.7 -> 83.0 us, 1024 x 1024 114.4 -> 101.7, 2048 x 2048 217 -> 201, with the signs of the transform in shared memory 640 x 768
+// with the quantiser options 137.6 -> 115.8, 1040 x 2896 212 -> 187; G1 and G2 of 2048 x 6144 with options 510 -> 470.
 // With the proxy fence on the reading side and one lane storing everything the iterations of 256 x 512 took 87 us
 // instead of 78, of 1408 x 2176 156 instead of 141.  Whole calls against three launches per iteration: 256 x 512
 // 175 -> 97 us, 1024 x 1024 190 -> 118, 1040 x 2896 with the paper's quantiser options 307 -> 223.
@@ -35,7 +42,7 @@ namespace {
 
 constexpr int BM = 128, BK = 256, KSTEPS = BK / 64;
 constexpr int CHUNK = 16;
-constexpr int NACC = 2;
+constexpr int NACC = 2;                       // accumulator buffers at most (ChainLaunch::nacc)
 constexpr int EPI_WARPS = 16;
 constexpr int W_LOAD = EPI_WARPS, W_MMA = EPI_WARPS + 1, W_STORE = EPI_WARPS + 2;
 constexpr int NTHREADS = (EPI_WARPS + 3) * 32;
@@ -44,6 +51,10 @@ constexpr int XBUF = 32 * 64;                 // a warp's 32 x 16 FP32 block: 64
 constexpr int MAX_STAGES = 5;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t SF_COLS = KSTEPS * 8;      // per stage: 4 columns per MMA for each operand
+constexpr uint32_t SF_RING = 2 * SF_COLS;     // copies and MMAs execute in issue order: two stages' columns in turn
+constexpr uint32_t ACC_COL = SF_RING;         // then the accumulators, then the resident tiles
+// Tiles of A and X that stay in the tensor memory beside nacc accumulators
+__host__ __device__ constexpr int resident_slots(int bn, int nacc) { return ((int)TMEM_COLS - (int)SF_RING - nacc * bn) / bn; }
 
 template <int BN>
 struct ChainLay {
@@ -59,9 +70,8 @@ struct ChainLay {
   static constexpr int OFF_OUT = OFF_X + EPI_WARPS * 2 * XBUF;  // two areas, used by alternate tiles
   static constexpr int OFF_BAR = OFF_OUT + 2 * OUT;
   static constexpr int SMEM = OFF_BAR + 2048 + 1024;
-  static constexpr uint32_t SF_COL = NACC * BN;
   static_assert(SMEM <= 232448 && STAGE_BYTES % 1024 == 0 && OFF_OUT % 1024 == 0 && OUT % 1024 == 0, "shared memory");
-  static_assert(STAGES <= MAX_STAGES && SF_COL + STAGES * SF_COLS <= TMEM_COLS, "tensor memory columns");
+  static_assert(STAGES <= MAX_STAGES && resident_slots(BN, NACC) >= 1, "tensor memory columns");
   // M = 128, N = BN, E2M1 x E2M1, UE4M3 scales, K-major operands
   static constexpr uint32_t IDESC = (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 };
@@ -73,6 +83,7 @@ struct ChainShared {
   uint64_t xfull[EPI_WARPS * 2];   // an FP32 block has landed
   uint64_t out_done[2], out_free[2];
   alignas(16) uint32_t amax[2][4]; // running maximum of the tile in a staging area (bit pattern), at its place among four slots
+  alignas(16) float signs[EPI_WARPS][16];   // of the product at hand, a copy per epilogue warp
   uint32_t tmem_base, abort_flag;
   uint32_t tiles[2][kChainTiles];  // this block's tiles of a symmetric product / of G3: p << 28 | ti << 16 | tj
 };
@@ -156,6 +167,31 @@ __device__ __forceinline__ void mbar_expect_s(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
+// A resident block of FP32 values -> 32 lanes x 16 columns of the tensor memory (lane = row), rounded to BF16 on request;
+// done when the warp's next tcgen05.wait::st returns.
+__device__ __forceinline__ void tc_st16(uint32_t taddr, const float (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+      "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]), "f"(r[8]), "f"(r[9]), "f"(r[10]),
+      "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15])
+      : "memory");
+}
+__device__ __forceinline__ void store_state(uint32_t taddr, const float (&v)[16], bool round) {
+  if (!round) {
+    tc_st16(taddr, v);
+    return;
+  }
+  float h[16];
+#pragma unroll
+  for (int i = 0; i < 16; i += 2) {
+    const uint32_t z = cvt_bf16x2(v[i], v[i + 1]);
+    h[i] = bf16_lo(z);
+    h[i + 1] = bf16_hi(z);
+  }
+  tc_st16(taddr, h);
+}
+__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 // Root's parameter update of a tall matrix: the parameter has the caller's orientation, so the 16 values of this
 // lane's row lie a row of the parameter apart.
 __device__ __noinline__ void chain_update_tall(uint16_t* w, int64_t ld, const float (&v)[16], float decay, float step) {
@@ -182,6 +218,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
   const int my_full = (nfull * a.count - (int)blockIdx.x + grid - 1) / grid;
   const int products = 3 * a.steps;
   const int first = SYM ? a.first : 0, end = SYM ? a.end : products;
+  const bool two_acc = a.nacc == 2;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < STAGES; ++i) { mbar_init(&sh->full[i], 1); mbar_init(&sh->empty[i], 1); }
@@ -278,14 +315,14 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
         for (int j = 0; j < mine; ++j, ++n) {
           // scale atoms cover 128 rows of the column operand: an odd 64-column tile uses their upper half
           const uint32_t sfb_shift = BN == 64 ? 2u * (sh->tiles[sym ? 0 : 1][j] & 1u) : 0u;
-          const uint32_t ab = n % NACC;
-          wait_or_abort(&sh->acc_empty[ab], ((n / NACC) & 1) ^ 1, abort_flag);
+          const uint32_t ab = two_acc ? n & 1u : 0u;
+          wait_or_abort(&sh->acc_empty[ab], ((two_acc ? n >> 1 : n) & 1) ^ 1, abort_flag);
           tc_fence_after();
-          const uint32_t d_tmem = tmem_base + ab * BN;
+          const uint32_t d_tmem = tmem_base + ACC_COL + ab * BN;
           for (int kb = 0; kb < num_kb; ++kb) {
             wait_or_abort(&sh->full[st], ph, abort_flag);
             tc_fence_after();
-            const uint32_t sf_t = tmem_base + L::SF_COL + st * SF_COLS;
+            const uint32_t sf_t = tmem_base + (uint32_t)(kb & 1) * SF_COLS;
             const uint32_t d = smem_u32(smem + st * L::STAGE_BYTES);
             const int ksteps = (K - kb * BK < BK ? K - kb * BK : BK) / 64;
             const uint64_t adesc = umma_desc(d, 1024, 2), bdesc = umma_desc(d + L::A_BYTES, 1024, 2);
@@ -294,13 +331,9 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
               if (i < ksteps) {
                 tc_cp_sf(sf_t + i * 4, umma_desc(d + L::A_BYTES + L::B_BYTES + i * 512, 128, 0));
                 tc_cp_sf(sf_t + KSTEPS * 4 + i * 4, umma_desc(d + L::A_BYTES + L::B_BYTES + L::SF_BYTES + i * 512, 128, 0));
-              }
-            }
-#pragma unroll
-            for (int i = 0; i < KSTEPS; ++i) {
-              if (i < ksteps)
                 tc_mma_nvf4(d_tmem, adesc + 2 * i, bdesc + 2 * i, L::IDESC, sf_t + i * 4, sf_t + KSTEPS * 4 + i * 4 + sfb_shift,
                             (kb | i) != 0 ? 1u : 0u);
+              }
             }
             tc_commit(&sh->empty[st]);
             if (++st == STAGES) { st = 0; ph ^= 1; }
@@ -381,9 +414,11 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
     const uint32_t col_base = area + g * (16 * 64);
     const uint32_t col_lane = (uint32_t)(g << 6 | cq << 2);
     const uint32_t tm_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
+    const uint32_t tm_state = tm_lane + ACC_COL + (two_acc ? 2u : 1u) * BN;   // resident tiles: X first, then A
     // staging offsets of this lane's outputs (chunk 0 of the warp)
     const uint32_t out0 = smem_u32(smem + L::OFF_OUT);
     const int row = quad * 32 + lane;
+    const uint32_t signs = smem_u32(&sh->signs[warp & (EPI_WARPS - 1)][0]);
 
     // Lane 0 starts the copy of the FP32 block a unit (tile, chunk) combines with.
     auto fetch = [&](int mode, int k, uint32_t tile, int c, int b) {
@@ -408,12 +443,13 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
       const bool do_q = !last || a.keep;
       const bool raw = mode == kG3 && k == 0;
       int cur_p = -1;
-      float scale = 0.0f, inv_sg = 1.0f, beta = 0.0f, gamma = 0.0f, tau = 0.0f, inv = 0.0f;
+      float scale = 0.0f, inv_sg = 1.0f, beta = 0.0f, gamma = 0.0f;
       bool fused = false;
-      QuantOpts qo = a.q;
       if (PF && a.q.rht) {
         const int j = mode == kG1 ? 2 * k + 1 : mode == kG2 ? 2 * k : 2 * k + 2;
-        qo.mask = rht_signs(a.seed, (uint64_t)j);
+        const uint32_t mask = rht_signs(a.seed, (uint64_t)j);
+        if (lane < 16) sh->signs[warp][lane] = (mask >> lane & 1u) ? -1.0f : 1.0f;
+        __syncwarp();
       }
       for (int j = 0; j < mine; ++j, ++n) {
         const uint32_t tile = sh->tiles[sym ? 0 : 1][j];
@@ -444,10 +480,6 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
             bound = __fmul_rn(__fmul_rn(4.0f, fabsf(pr.ca)), ax);
             beta = pr.ca;
             gamma = scale;
-            if (raw) {
-              tau = a.clip ? ld_scalar(sc + a.ix.tau) : __int_as_float(0x7f800000);
-              inv = ld_scalar(sc + a.ix.inv);
-            }
           }
           sg_out = scale_predicted(__fmul_rn(a.q.widen, bound));
           inv_sg = __frcp_rn(sg_out);
@@ -458,9 +490,110 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
           if (ti == 0 && tj == 0 && threadIdx.x == 0)
             pr.scalars[mode == kG1 ? a.ix.sg_A0 + k : mode == kG2 ? a.ix.sg_B0 + k : a.ix.sg_X0 + k + 1] = sg_out;
         }
-        const uint32_t ab = n % NACC;
+        const uint32_t ab = two_acc ? n & 1u : 0u;
+        // This tile's X (G3) or A (G1, G2) lies in the tensor memory; the first G3 reads the caller's matrix, the last
+        // one writes the caller's result.
+        const bool resident = mode == kG3 ? j < a.nx : j < a.na;
+        const bool from_tm = resident && (mode == kG2 || (mode == kG3 && !raw));
+        const bool to_tm = resident && (mode == kG1 || (mode == kG3 && !last));
+        const uint32_t state = tm_state + (uint32_t)(mode == kG3 ? j : a.nx + j) * BN;
         const uint32_t os = out0 + (n & 1) * L::OUT;
         float amax = 0.0f;
+        // ---- the common tile: nothing but its quantised outputs leaves the SM.  What it needs is in registers before the
+        // accumulator is waited for, and the FP32 block goes through shared memory for the pass down the columns only.
+        if (resident && !raw && !last && !(a.keep && mode == kG1)) {
+          wait_or_abort(&sh->out_free[n & 1], ((n >> 1) & 1) ^ 1, abort_flag);   // the stores of the tile two back
+          if (lane == 0) bulk_wait_read<0>();
+          const bool has_x = mode != kG1, round = a.bf16 && to_tm;
+          const float g1 = mode == kG1 ? scale : gamma;
+          const uint64_t b2 = pack2(beta, beta), g2 = pack2(g1, g1);
+          // The second 16 rows of the block are stored with neighbouring rows swapped: the half-warps, whose rows are 16 apart, then
+          // read down their columns in the same order and never meet in a bank.
+          const uint32_t put = area + (((uint32_t)lane ^ (uint32_t)g) << 6) + (((lane >> 1) & 3) << 4);
+          const uint32_t get = area + (uint32_t)(g << 10 | g << 6 | cq << 2);
+          // the next tile's block, when it comes from memory: into the warp's second buffer, this tile uses the first
+          have = has_x && j + 1 < mine && j + 1 >= (mode == kG3 ? a.nx : a.na);
+          if (have) fetch(mode, k, sh->tiles[sym ? 0 : 1][j + 1], 0, 1);
+          unit = 1;
+          __syncwarp();
+          wait_or_abort(&sh->acc_full[ab], (two_acc ? n >> 1 : n) & 1, abort_flag);
+          tc_fence_after();
+#pragma unroll 1
+          for (int c = 0; c < L::CHUNKS; ++c) {
+            const int ch = team * L::CHUNKS + c;
+            uint32_t acc[16];
+            float v[16];
+            tc_ld16_issue(tm_lane + ACC_COL + ab * BN + ch * CHUNK, acc);
+            if (has_x) {
+              uint32_t x[16];
+              tc_ld16_issue(state + ch * CHUNK, x);
+              tc_wait_ld16(acc);
+              tc_wait_ld16(x);
+#pragma unroll
+              for (int i = 0; i < 16; i += 2) {
+                const uint64_t ac2 = pack2(__uint_as_float(acc[i]), __uint_as_float(acc[i + 1]));
+                const uint64_t bx = mul2(b2, pack2(__uint_as_float(x[i]), __uint_as_float(x[i + 1])));
+                if (fused) {
+                  unpack2(fma2(ac2, g2, bx), v[i], v[i + 1]);
+                } else {
+                  float t0, t1, u0, u1;
+                  unpack2(bx, t0, t1);
+                  unpack2(mul2(ac2, g2), u0, u1);
+                  v[i] = __fadd_rn(t0, u0);
+                  v[i + 1] = __fadd_rn(t1, u1);
+                }
+              }
+            } else {
+              tc_wait_ld16(acc);
+#pragma unroll
+              for (int i = 0; i < 16; i += 2)
+                unpack2(mul2(pack2(__uint_as_float(acc[i]), __uint_as_float(acc[i + 1])), g2), v[i], v[i + 1]);
+            }
+            if (c == L::CHUNKS - 1) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&sh->acc_empty[ab]);
+            }
+            if (mirror) {
+              if (L::CHUNKS > 1) __syncwarp();   // every lane has read its column of the block before
+#pragma unroll
+              for (int i = 0; i < 4; ++i) sts_f4(put ^ (i << 4), v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+              __syncwarp();
+            }
+            if (to_tm) store_state(state + ch * CHUNK, v, round);
+            uint32_t lo, hi, sb;
+            float bmax;
+            if (PF) sb = quantize_block16_opts_p2<false>(v, a.q, inv_sg, lo, hi, bmax, signs);
+            else sb = quantize_block16_p2(v, inv_sg, lo, hi, bmax);
+            amax = fmaxf(amax, bmax);
+            sts_u2(os + (ch >> 2) * 4096 + row * 32 + (((ch & 3) * 8) ^ ((lane & 4) << 2)), lo, hi);
+            sts_b(os + L::RQ + L::CQ + (ch >> 2) * 512 + lane * 16 + quad * 4 + (ch & 3), sb);
+            if (mirror) {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) v[i] = lds_f1(get ^ (uint32_t)(i << 6 | ((i >> 1) & 3) << 4));
+              if (PF) sb = quantize_block16_opts_p2<false>(v, a.q, inv_sg, lo, hi, bmax, signs);
+              else sb = quantize_block16_p2(v, inv_sg, lo, hi, bmax);
+              const int col = ch * CHUNK + cq;
+              sts_u2(os + L::RQ + col * 64 + ((quad ^ ((col >> 1) & 3)) << 4) + g * 8, lo, hi);
+              sts_b(os + L::RQ + L::CQ + L::RSF + (quad >> 1) * (BN * 4) + (col & 31) * (BN / 8) + (col >> 5) * 4 + (quad & 1) * 2 + g, sb);
+            }
+          }
+          if (mode != kG2) {
+            const int slot = mode == kG1 ? a.ix.amax_A0 + k : a.ix.amax_X0 + k + 1;
+            const uint32_t wm = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
+            if (lane == 0) atomicMax(&sh->amax[n & 1][slot & 3], wm);
+          }
+          fence_proxy_async_smem();   // staged outputs and the block, before what the copies read and write there
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh->out_done[n & 1]);
+          if (to_tm) tc_wait_st();
+          continue;
+        }
+        float tau = 0.0f, inv = 0.0f;
+        if (raw) {
+          tau = a.clip ? ld_scalar(pr.scalars + a.ix.tau) : __int_as_float(0x7f800000);
+          inv = ld_scalar(pr.scalars + a.ix.inv);
+        }
 #pragma unroll 1
         for (int c = 0; c < L::CHUNKS; ++c, ++unit) {
           const int ch = team * L::CHUNKS + c;             // chunk of the tile
@@ -470,20 +603,22 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
           // both blocks' earlier stores have been read; the next unit of the same product is fetched now
           if (lane == 0) bulk_wait_read<0>();
           if (mode != kG1) {
-            if (!have) fetch(mode, k, tile, c, b);
-            const bool more = c + 1 < L::CHUNKS || j + 1 < mine;
+            if (!have && !from_tm) fetch(mode, k, tile, c, b);
+            const bool more = c + 1 < L::CHUNKS ? !from_tm : j + 1 < mine && (raw || j + 1 >= (mode == kG3 ? a.nx : a.na));
             if (more) fetch(mode, k, c + 1 < L::CHUNKS ? tile : sh->tiles[sym ? 0 : 1][j + 1], c + 1 < L::CHUNKS ? c + 1 : 0, b ^ 1);
             have = more;
           }
           __syncwarp();
           if (c == 0) {
-            wait_or_abort(&sh->acc_full[ab], (n / NACC) & 1, abort_flag);
+            wait_or_abort(&sh->acc_full[ab], (two_acc ? n >> 1 : n) & 1, abort_flag);
             tc_fence_after();
           }
           uint32_t acc[16];
-          tc_ld16_issue(tm_lane + ab * BN + ch * CHUNK, acc);
+          tc_ld16_issue(tm_lane + ACC_COL + ab * BN + ch * CHUNK, acc);
           float x[16];
-          if (mode != kG1) {
+          if (from_tm) {
+            tc_ld16(state + ch * CHUNK, x);
+          } else if (mode != kG1) {
             wait_or_abort(xfull + b * 8, (xph >> b) & 1, abort_flag);
             xph ^= 1u << b;
             if (xposed) {
@@ -529,20 +664,12 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
               }
             }
           }
-          // ---- stage the block (for the TMA store and for the pass down the columns) and send it off
-          if (out_t && !a.keep) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-              asm volatile("st.shared.f32 [%0], %1;" ::"r"(area + boff + i * 128 + lane * 4), "f"(v[i]) : "memory");
-          } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) sts_f4((row_addr + boff) ^ (i << 4), v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-          }
-          const bool round = a.bf16 && !last && mode != kG2;  // stored rounded to BF16, after the pass down the columns
-          bool send = mode != kG2;
+          const bool round = a.bf16 && !last && mode != kG2;  // stored rounded to BF16
+          if (to_tm) store_state(state + ch * CHUNK, v, round);
+          bool send = mode == kG1 && (!to_tm || a.keep);
           if (mode == kG3) {
             // the caller's matrix has no padding; X of a tall matrix lies in the workspace and has
-            send = (y < a.s0 && x0 < a.l0) || (pr.tall && !out_t);
+            send = !to_tm && ((y < a.s0 && x0 < a.l0) || (pr.tall && !out_t));
             if (last && a.update && pr.W) {
               const bool in = y + lane < a.s0 && x0 < a.l0;
               if (pr.tall) {
@@ -563,6 +690,15 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
               send = send && !a.no_out;
             }
           }
+          // ---- stage the block (for the TMA store and for the pass down the columns) and send it off
+          if (out_t && !a.keep) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              asm volatile("st.shared.f32 [%0], %1;" ::"r"(area + boff + i * 128 + lane * 4), "f"(v[i]) : "memory");
+          } else if (send || mirror) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sts_f4((row_addr + boff) ^ (i << 4), v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+          }
           // The FP32 block leaves by TMA; only this warp reads it back.  With several units per product (BN = 128) it
           // is sent now, so that its buffer is free in time; else after the outputs that other blocks wait for.
           auto send_block = [&]() {
@@ -575,38 +711,16 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
           if (send && early) fence_proxy_async_smem();
           __syncwarp();
           if (send && early && lane == 0) send_block();
-          float w[16];
-          if (mirror) {
+          uint32_t rounded[8];   // what is stored rounded to BF16 takes the block's place after the pass down the columns
+          if (round && send) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const uint32_t at = (col_base + boff) | (col_lane ^ (uint32_t)(i << 6 | ((i >> 1) & 3) << 4));
-              w[i] = lds_f1(at);
-              w[i + 8] = lds_f1(at + 512);
-            }
-            if (PF) {
-              // the transform and the error sums need the block in row order
-#pragma unroll
-              for (int i = 0; i < 16; i += 2) {
-                const float c0 = w[i], c1 = w[i + 1];
-                w[i] = g ? c1 : c0;
-                w[i + 1] = g ? c0 : c1;
-              }
-            }
-          }
-          if (round) {
-            // what is stored is rounded to BF16
-            __syncwarp();
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const uint32_t w0 = cvt_bf16x2(v[4 * i], v[4 * i + 1]), w1 = cvt_bf16x2(v[4 * i + 2], v[4 * i + 3]);
-              sts_f4((row_addr + boff) ^ (i << 4), bf16_lo(w0), bf16_hi(w0), bf16_lo(w1), bf16_hi(w1));
-            }
+            for (int i = 0; i < 8; ++i) rounded[i] = cvt_bf16x2(v[2 * i], v[2 * i + 1]);
           }
           if (do_q) {
             uint32_t lo, hi;
             float bmax;
             uint32_t sb;
-            if (PF) sb = quantize_block16_opts_p2<false>(v, qo, inv_sg, lo, hi, bmax);
+            if (PF) sb = quantize_block16_opts_p2<false>(v, a.q, inv_sg, lo, hi, bmax, signs);
             else sb = quantize_block16_p2(v, inv_sg, lo, hi, bmax);
             amax = fmaxf(amax, bmax);
             // the stores of the tile two back have read the staging area
@@ -614,14 +728,40 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
             sts_u2(os + (ch >> 2) * 4096 + row * 32 + (((ch & 3) * 8) ^ ((lane & 4) << 2)), lo, hi);
             sts_b(os + L::RQ + L::CQ + (ch >> 2) * 512 + lane * 16 + quad * 4 + (ch & 3), sb);
             if (mirror) {
-              if (PF) sb = quantize_block16_opts_p2<false>(w, qo, inv_sg, lo, hi, bmax);
-              else sb = quantize_block16_p2(w, inv_sg, lo, hi, bmax);
+              // the block again, down the columns (into the registers of the row pass: both at once would not fit)
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const uint32_t at = (col_base + boff) | (col_lane ^ (uint32_t)(i << 6 | ((i >> 1) & 3) << 4));
+                v[i] = lds_f1(at);
+                v[i + 8] = lds_f1(at + 512);
+              }
+            }
+            if (round && send) {
+              __syncwarp();
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                sts_f4((row_addr + boff) ^ (i << 4), bf16_lo(rounded[2 * i]), bf16_hi(rounded[2 * i]), bf16_lo(rounded[2 * i + 1]),
+                       bf16_hi(rounded[2 * i + 1]));
+            }
+            if (mirror) {
+              if (PF) {
+                // the transform and the error sums need the block in row order
+#pragma unroll
+                for (int i = 0; i < 16; i += 2) {
+                  const float c0 = v[i], c1 = v[i + 1];
+                  v[i] = g ? c1 : c0;
+                  v[i + 1] = g ? c0 : c1;
+                }
+              }
+              if (PF) sb = quantize_block16_opts_p2<false>(v, a.q, inv_sg, lo, hi, bmax, signs);
+              else sb = quantize_block16_p2(v, inv_sg, lo, hi, bmax);
               if (!PF && g) { lo = swap_nibbles(lo); hi = swap_nibbles(hi); }   // back into row order
               const int col = ch * CHUNK + cq;
               sts_u2(os + L::RQ + col * 64 + ((quad ^ ((col >> 1) & 3)) << 4) + g * 8, lo, hi);
               sts_b(os + L::RQ + L::CQ + L::RSF + (quad >> 1) * (BN * 4) + (col & 31) * (BN / 8) + (col >> 5) * 4 + (quad & 1) * 2 + g, sb);
             }
           }
+          if (to_tm) tc_wait_st();
           // The fence orders this lane's reads and writes of shared memory before what the copies (another proxy)
           // read and write there.
           fence_proxy_async_smem();
@@ -644,7 +784,8 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
         const int nk = np / 3, nmode = np - 3 * nk + kG1;
         const int nmine = nmode != kG3 ? my_sym : my_full;
         if (nmine == 0) continue;
-        if (nmode != kG1) {
+        const bool tm = nmode == kG3 ? nk > 0 && a.nx > 0 : a.na > 0;
+        if (nmode != kG1 && !tm) {
           if (lane == 0) bulk_wait_all<0>();
           fetch(nmode, nk, sh->tiles[nmode != kG3 ? 0 : 1][0], 0, (int)(unit & 1));
           have = true;
@@ -729,6 +870,16 @@ double chain_symmetric_us(int64_t s, int64_t l, int count, bool opts, int sms) {
   return 12.0 + t.g1() + t.g23();
 }
 
+// Which tiles stay in the tensor memory, when every block takes up to `full` tiles of G3 and `sym` of a symmetric product: A
+// first, which serves two products of an iteration (2048 x 2048 201 us, X first 215).  One accumulator instead of two where that lets
+// more of them stay: a tile's accumulator is read at the very start of its epilogue (201 us, with two accumulators 211).
+static void place_resident(ChainLaunch& a, int bn, int64_t full, int64_t sym) {
+  a.nacc = full + sym <= resident_slots(bn, 2) ? 2 : 1;
+  const int64_t slots = resident_slots(bn, a.nacc);
+  a.na = (int)(sym < slots ? sym : slots);
+  a.nx = (int)(full < slots - a.na ? full : slots - a.na);
+}
+
 cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st) {
   if (launch.count < 1 || launch.count > kChainMax || launch.steps < 1) return cudaErrorInvalidValue;
   ChainLaunch a = launch;
@@ -738,6 +889,7 @@ cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int s
   a.nsym = (int)sym_tiles(a.s, bn);
   const int64_t widest = (int64_t)(a.s / BM) * (a.l / bn) * a.count;
   const int grid = (int)(widest < sms ? widest : sms);
+  place_resident(a, bn, rounds(widest, grid), rounds((int64_t)a.nsym * a.count, grid));
   if (narrow) return pf ? launch_one<64, true>(pack, a, grid, st) : launch_one<64, false>(pack, a, grid, st);
   return pf ? launch_one<128, true>(pack, a, grid, st) : launch_one<128, false>(pack, a, grid, st);
 }
@@ -751,6 +903,7 @@ cudaError_t launch_chain_symmetric(const ChainPack& pack, const ChainLaunch& lau
   const int64_t widest = (int64_t)a.nsym * a.count;
   if (widest > sms) return cudaErrorInvalidValue;
   const int grid = (int)widest;
+  place_resident(a, 128, 0, 1);
   return a.q.rht || a.q.four_six ? launch_one<128, true, true>(pack, a, grid, st) : launch_one<128, false, true>(pack, a, grid, st);
 }
 

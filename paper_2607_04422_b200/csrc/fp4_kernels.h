@@ -143,6 +143,7 @@ struct ChainLaunch {
   int s, l, s0, l0;          // work shape, the caller's short and long side
   int first, end;            // launch_chain_symmetric: its products
   int nsym;                  // tiles per matrix of a symmetric product (set by the launch)
+  int nacc, nx, na;          // accumulator buffers; a block's first tiles of X and of A that stay in its tensor memory (set by the launch)
   int clip, keep, bf16;
   int update, no_out;
   float upd_decay, upd_step;

@@ -527,7 +527,7 @@ def test_clip_degenerate_inputs(kind):
         G[np.abs(G) > 2.0] = np.float32(2.25) * np.sign(G[np.abs(G) > 2.0])   # ~4.5 % of entries tie
     got, ws = run_gpu(G, steps=0)
     want, tr = oracle.root_ns(G, steps=0, trace_iter=0)
-    lay, sc, *_ = ws_view(ws, m, n, 0, 0)
+    lay, sc, *_ = ws_view(ws, m, n, 0)
     assert sc[lay.idx_tau] == np.float32(tr["tau"])
     assert abs(sc[lay.idx_nu] - tr["nu"]) <= 1.2e-7 * max(tr["nu"], 1e-30)
     assert rel(got, want) < 2e-7 or not want.any()
@@ -704,6 +704,27 @@ def test_iterations_in_one_launch_at_the_edges_of_its_tiles(shape, flags):
     before = fp4.fp4_kernel_launches()
     fp4.fp4_root_ns(Gd, out, 3, p, ws)
     assert fp4.fp4_kernel_launches() - before == 2      # prologue and iterations
+    assert fp4.fp4_last_device_status(ws) == 0
+    first = out.cpu().numpy()
+    pf = bool(flags & FP4_FLAG_RHT)
+    want = oracle.root_ns(G, steps=3, rht=pf, four_six=pf, seed=5, store_bf16=bool(flags & FP4_FLAG_STORE_BF16))
+    assert rel(first, want) <= TOL_OUT, rel(first, want)
+    fp4.fp4_root_ns(Gd, out, 3, p, ws)
+    assert np.array_equal(out.cpu().numpy(), first)
+
+
+@pytest.mark.parametrize("shape,flags", [((768, 8192), 0), ((8192, 768), FP4_FLAG_STORE_BF16), ((1536, 2816), 0),
+                                         ((1280, 2048), FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)])
+def test_iterations_in_one_launch_with_tiles_beyond_the_tensor_memory(shape, flags):
+    """More tiles per block than stay in the tensor memory: the first ones' A and X live there, the others' in the workspace,
+    next to one another in one product; the same bytes twice, also from a dirty workspace."""
+    m, n = shape
+    G = workloads.gradient_like(m, n, seed=m + n)
+    Gd = torch.from_numpy(G).cuda()
+    out = torch.empty_like(Gd)
+    ws = torch.full((fp4.fp4_root_ns_workspace_bytes(m, n, 3, flags),), 0xFF, dtype=torch.uint8, device="cuda")
+    p = fp4.NsParams.make(flags=flags, seed=5)
+    fp4.fp4_root_ns(Gd, out, 3, p, ws)
     assert fp4.fp4_last_device_status(ws) == 0
     first = out.cpu().numpy()
     pf = bool(flags & FP4_FLAG_RHT)
