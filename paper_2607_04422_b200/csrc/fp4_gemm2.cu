@@ -758,6 +758,16 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
           else tma_store_2d_s(&pr->tmOut, xcol, y32, area + boff);
           bulk_commit();
         }
+        // ---- quantise along the row
+        uint32_t rlo = 0, rhi = 0;
+        if (do_q) {
+          float bmax;
+          uint32_t sb;
+          if (PF) sb = quantize_block16_opts_p2<true>(v, args.q, inv_sg, rlo, rhi, bmax);
+          else sb = quantize_block16_p2(v, inv_sg, rlo, rhi, bmax);
+          if (MODE == kG1 || MODE == kG3) amax = fmaxf(amax, bmax);
+          sfw |= sb << (8 * e);
+        }
         // ---- blocks of 16 down the rows of this warp's own 32 x 16 block (the transposed operand
         // copy in G3, the mirrored triangle in G1/G2), read back from the buffer.
         float w[16];
@@ -784,16 +794,6 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
             tma_store_2d_s(&pr->tmH, xcol, y32, area + boff);
             bulk_commit();
           }
-        }
-        // ---- quantise along the row
-        uint32_t rlo = 0, rhi = 0;
-        if (do_q) {
-          float bmax;
-          uint32_t sb;
-          if (PF) sb = quantize_block16_opts_p2<true>(v, args.q, inv_sg, rlo, rhi, bmax);
-          else sb = quantize_block16_p2(v, inv_sg, rlo, rhi, bmax);
-          if (MODE == kG1 || MODE == kG3) amax = fmaxf(amax, bmax);
-          sfw |= sb << (8 * e);
         }
         // ---- the buffer is free once every lane has read its column and the store has read the
         // block; the block two chunks ahead is fetched into it.  (Waiting for the store's read here
