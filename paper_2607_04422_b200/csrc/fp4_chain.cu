@@ -852,7 +852,11 @@ static double width_us(int bn, int64_t s, int64_t l, int count, bool opts, int s
   const int64_t rs = rounds(sym_tiles(s, bn) * count, sms), rf = rounds(s / BM * (l / bn) * count, sms);
   if (rf > kChainTiles) return 0.0;
   const TileUs t(bn, s, l, opts);
-  return 3 * 4.0 + (double)rs * t.g1() + (double)(rs + rf) * t.g23();
+  // narrow tiles beyond the tensor memory: their X moves through the shared memory and back.  (With the quantiser options the
+  // arithmetic covers that.)  5 iterations in one launch / two launches each: 1280 x 7168 297 / 285 us, 1408 x 6144 300 / 289, 1280 x 8192
+  // 332 / 327, 1152 x 8192 312 / 327, 1024 x 8192 264 / 266; with options 1152 x 8192 370 / 416.
+  const int64_t beyond = bn == 64 && !opts ? rs + rf - resident_slots(64, 1) : 0;
+  return 3 * 4.0 + (double)rs * t.g1() + (double)(rs + rf) * t.g23() + (beyond > 0 ? 1.2 * (double)beyond : 0.0);
 }
 // The width of a single launch's tiles.  Measured, 5 iterations, 64 / 128 columns: 256 x 512 95 / 126 us, 1024 x 4096
 // 185 / 212 (with the quantiser options 240 / 293), 8 x 768 x 768 176 / 211, 1536 x 4096 264 / 261, 2048 x 2048 228 / 224.
