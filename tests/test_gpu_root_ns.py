@@ -527,7 +527,7 @@ def test_clip_degenerate_inputs(kind):
         G[np.abs(G) > 2.0] = np.float32(2.25) * np.sign(G[np.abs(G) > 2.0])   # ~4.5 % of entries tie
     got, ws = run_gpu(G, steps=0)
     want, tr = oracle.root_ns(G, steps=0, trace_iter=0)
-    lay, sc, *_ = ws_view(ws, m, n, 0)
+    lay, sc, *_ = ws_view(ws, m, n, 0, 0)
     assert sc[lay.idx_tau] == np.float32(tr["tau"])
     assert abs(sc[lay.idx_nu] - tr["nu"]) <= 1.2e-7 * max(tr["nu"], 1e-30)
     assert rel(got, want) < 2e-7 or not want.any()
