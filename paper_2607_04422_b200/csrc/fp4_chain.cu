@@ -858,7 +858,7 @@ static double width_us(int bn, int64_t s, int64_t l, int count, bool opts, int s
   const int64_t beyond = bn == 64 && !opts ? rs + rf - resident_slots(64, 1) : 0;
   return 3 * 4.0 + (double)rs * t.g1() + (double)(rs + rf) * t.g23() + (beyond > 0 ? 1.2 * (double)beyond : 0.0);
 }
-// The width of a single launch's tiles.  Measured, 5 iterations, 64 / 128 columns: 256 x 512 95 / 126 us, 1024 x 4096
+// The width of a single launch's tiles.  Measured before tiles stayed in the tensor memory, 5 iterations, 64 / 128 columns: 256 x 512 95 / 126 us, 1024 x 4096
 // 185 / 212 (with the quantiser options 240 / 293), 8 x 768 x 768 176 / 211, 1536 x 4096 264 / 261, 2048 x 2048 228 / 224.
 static bool narrow_tiles(int64_t s, int64_t l, int count, bool opts, int sms) {
   const double n = width_us(64, s, l, count, opts, sms), w = width_us(128, s, l, count, opts, sms);

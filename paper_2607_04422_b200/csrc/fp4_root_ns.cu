@@ -368,7 +368,9 @@ struct PairUs {
 
 // How a group runs its iterations: all of them in one launch (fp4_chain.cu), three launches of the CTA-pair kernel per
 // iteration, or two - G1 and G2 as one launch with a 128 x 128 tile per SM where their 256 x 256 tiles would leave half of
-// the SM pairs idle, and the pairs' G3.  What is estimated to be fastest.  Measured, 5 iterations, one launch / two / three
+// the SM pairs idle, and the pairs' G3.  What is estimated to be fastest.  Since A and X stay in the tensor memory single launches
+// take 5 to 14 % and the two of a pair's G1 and G2 3 to 7 % less than here, which moves the line little (estimates 12 % lower sent
+// 2304 x 2304, 261 us, and 1792 x 4096, 252 us, to single launches of 309 and 295 us).  Before that, 5 iterations, one launch / two / three
 // per iteration: 1024 x 1024 119 / 174 / 179 us, 2048 x 2048 224 / 221 / 231, 2048 x 4096 318 / 287 / 307, 1536 x 6144
 // 339 / 305 / 330, 2048 x 8192 492 / 446 / 450 (with the quantiser options 669 / 604 / 619), 2304 x 2304 295 / - / 264,
 // 4 x 512 x 512 106 / 170 / 179, 2 x 1024 x 2816 200 / 248 / 260.  (Not for inspection of BF16-stored intermediates: in
