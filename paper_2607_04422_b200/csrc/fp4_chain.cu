@@ -15,7 +15,9 @@
 // written by the very thread that reads them.  So they stay where they are: beside the accumulators the tensor memory has room
 // for 6 tiles of 64 columns or 2 of 128, and a block's first tiles of A and X live there from product to product
 // (place_resident); only the caller's matrix in the first G3, the result in the last, and tiles beyond that room
-// move through memory, fetched before the dependency is even looked at.
+// move through memory.  A block of those is fetched while the tile before it is worked on, the first one of a product that
+// has no resident tile before its dependency is even looked at; the copies that wrote them have arrived by then, because the
+// warp waits for all its own at the end of the product before.
 //
 // Warp roles: 0-15 epilogue, 16 operand producer (TMA; also the only thread that polls the counter), 17 MMA
 // issuer and TMEM owner, 18 stores.  Epilogue warp w owns the TMEM lanes of quadrant w % 4 and the 16-column
@@ -779,16 +781,20 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
           if (send && !early && lane == 0) send_block();
         }
       }
-      // The next product's first block: once this warp's own stores (its A, its X) have arrived.
+      // What the next product reads from memory: blocks this warp has stored itself (A in G1, X in the G3 before), so every store
+      // of the warp has to have arrived - also when the product begins with resident tiles and fetches later.  A product
+      // that begins beyond them has its first block fetched here.
       if (mine > 0) for (int np = pi + 1; np < end && np <= pi + 3; ++np) {
         const int nk = np / 3, nmode = np - 3 * nk + kG1;
         const int nmine = nmode != kG3 ? my_sym : my_full;
         if (nmine == 0) continue;
-        const bool tm = nmode == kG3 ? nk > 0 && a.nx > 0 : a.na > 0;
-        if (nmode != kG1 && !tm) {
+        const int in_tm = nmode == kG1 ? nmine : nmode == kG2 ? a.na : nk > 0 ? a.nx : 0;
+        if (nmine > in_tm) {
           if (lane == 0) bulk_wait_all<0>();
-          fetch(nmode, nk, sh->tiles[nmode != kG3 ? 0 : 1][0], 0, (int)(unit & 1));
-          have = true;
+          if (in_tm == 0) {
+            fetch(nmode, nk, sh->tiles[nmode != kG3 ? 0 : 1][0], 0, (int)(unit & 1));
+            have = true;
+          }
         }
         break;
       }

@@ -734,6 +734,36 @@ def test_iterations_in_one_launch_with_tiles_beyond_the_tensor_memory(shape, fla
     assert np.array_equal(out.cpu().numpy(), first)
 
 
+@pytest.mark.parametrize("count,side,flags", [(12, 896, 0), (12, 896, FP4_FLAG_STORE_BF16), (9, 1152, 0),
+                                              (10, 1152, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)])
+def test_iterations_in_one_launch_for_a_group_with_a_and_x_in_memory(count, side, flags):
+    """On 148 SMs a block takes 3 (7 narrow ones with the options) tiles of A and 4 to 11 of X, of which the tensor memory holds 2
+    (6) of A: the other A go through the workspace from G1 to G2 of one iteration, and all X from one G3 to the next."""
+    mats = [workloads.gradient_like(side, side, seed=60 + i) for i in range(count)]
+    Gs = [torch.from_numpy(g).cuda() for g in mats]
+    outs = [torch.empty_like(g) for g in Gs]
+    p = fp4.NsParams.make(flags=flags, seed=5)
+    ws = torch.full((fp4.fp4_root_ns_batched_workspace_bytes([g.shape for g in mats], 3, flags),), 0xFF, dtype=torch.uint8,
+                    device="cuda")
+    launches = []
+    for steps in (1, 3):
+        before = fp4.fp4_kernel_launches()
+        fp4.fp4_root_ns_batched(Gs, outs, steps, p, ws)
+        launches.append(fp4.fp4_kernel_launches() - before)
+        assert fp4.fp4_last_device_status(ws) == 0
+    assert launches[0] == launches[1]                   # one launch however many iterations
+    first = [o.cpu().numpy() for o in outs]
+    pf = bool(flags & FP4_FLAG_RHT)
+    want = oracle.root_ns(mats[-1], steps=3, rht=pf, four_six=pf, seed=5, store_bf16=bool(flags & FP4_FLAG_STORE_BF16))
+    assert rel(first[-1], want) <= TOL_OUT, rel(first[-1], want)
+    for g, o in zip(mats, first):
+        single, _ = run_gpu(g, steps=3, flags=flags, seed=5)
+        assert np.array_equal(o, single)
+    for _ in range(5):
+        fp4.fp4_root_ns_batched(Gs, outs, 3, p, ws)
+        assert all(np.array_equal(o.cpu().numpy(), f) for o, f in zip(outs, first))
+
+
 def test_iterations_in_one_launch_for_a_group_are_those_of_single_calls():
     """Fourteen equal shapes, wide and tall, share one launch; a fifteenth makes the group take the other route."""
     for count in (14, 15):
