@@ -54,9 +54,8 @@ typedef enum {
 
 /* flags of fp4_ns_params */
 #define FP4_FLAG_KEEP_OPERANDS 1u /* the last iteration also writes the NVFP4 copies of
-                                     its result, and small matrices A (otherwise
-                                     skipped as dead work); for inspection through
-                                     fp4_root_ns_workspace_layout */
+                                     its result (otherwise skipped as dead work); for
+                                     inspection through fp4_root_ns_workspace_layout */
 /* Paper-faithful quantiser options (Section 3.4: operands are rotated by a random Hadamard
  * transform along the contraction axis, and every quantisation uses adaptive 4/6 scaling).
  * Off by default; each costs epilogue arithmetic.

@@ -15,9 +15,9 @@
 // written by the very thread that reads them.  So they stay where they are: beside the accumulators the tensor memory has room
 // for 6 tiles of 64 columns or 2 of 128, and a block's first tiles of A and X live there from product to product
 // (place_resident); only the caller's matrix in the first G3, the result in the last, and tiles beyond that room
-// move through memory.  A block of those is fetched while the tile before it is worked on, the first one of a product that
-// has no resident tile before its dependency is even looked at; the copies that wrote them have arrived by then, because the
-// warp waits for all its own at the end of the product before.
+// move through memory (and, stored only, what the workspace keeps of the last iteration).  A block of those is fetched while
+// the tile before it is worked on, the first one of a product that has no resident tile before its dependency is even looked
+// at; the copies that wrote them have arrived by then, because the warp waits for all its own at the end of the product before.
 //
 // Warp roles: 0-15 epilogue, 16 operand producer (TMA; also the only thread that polls the counter), 17 MMA
 // issuer and TMEM owner, 18 stores.  Epilogue warp w owns the TMEM lanes of quadrant w % 4 and the 16-column
@@ -438,6 +438,36 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
     uint32_t n = 0, unit = 0, xph = 0;   // tiles, units, phases of the two block barriers
     bool have = false;                   // the copy of the unit at hand is under way
     for (int pi = first; pi < end; ++pi) {
+      // The workspace keeps A of the last iteration and, of a tall matrix whose result leaves transposed, the X before that.  While
+      // the other blocks finish the product before the last one (SYM: before the last G2), the resident tiles of both are copied
+      // out, through the buffer that holds no fetched block.  (X of a wide matrix lies in `out`, where nothing would order such
+      // a copy and the result.  With a.keep the tiles of G1 store A themselves, and the last G3 X.)  Had the tiles stored them in
+      // the last iteration, 256 x 512 would take 1.4 us more instead of 0.4, 2048 x 2048 5 instead of 0.3.
+      if (!a.keep && pi == products - (SYM ? 2 : 1)) {
+        const int tiles_a = min(my_sym, a.na), tiles_x = !SYM && a.tall && a.steps > 1 ? min(my_full, a.nx) : 0;
+        const uint32_t dst = (unit & 1) ? 0u : (uint32_t)XBUF;
+#pragma unroll 1
+        for (int i = 0; i < (tiles_a + tiles_x) * L::CHUNKS; ++i) {
+          const int j = i / L::CHUNKS, ch = team * L::CHUNKS + i % L::CHUNKS;
+          const bool is_a = j < tiles_a;
+          const uint32_t tile = sh->tiles[is_a ? 0 : 1][is_a ? j : j - tiles_a];
+          const ChainProblem& pr = pack.p[tile >> 28];
+          if (!is_a && !pr.tall) continue;
+          float v[16];
+          tc_ld16(tm_state + (uint32_t)(is_a ? a.nx + j : j - tiles_a) * BN + ch * CHUNK, v);
+          if (lane == 0) bulk_wait_read<0>();
+          __syncwarp();
+#pragma unroll
+          for (int q = 0; q < 4; ++q) sts_f4((row_addr + dst) ^ (q << 4), v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            tma_store_s(is_a ? &pr.tm_A : &pr.tm_X, (int)(tile & 0xFFFF) * BN + ch * CHUNK,
+                        ((int)(tile >> 16) & 0xFFF) * BM + quad * 32, area + dst);
+            bulk_commit();
+          }
+        }
+      }
       const int k = pi / 3, mode = pi - 3 * k + kG1;
       const bool sym = mode != kG3;
       const int mine = sym ? my_sym : my_full;

@@ -145,6 +145,7 @@ struct ChainLaunch {
   int nsym;                  // tiles per matrix of a symmetric product (set by the launch)
   int nacc, nx, na;          // accumulator buffers; a block's first tiles of X and of A that stay in its tensor memory (set by the launch)
   int clip, keep, bf16;
+  int tall;                  // one of the matrices at least is tall
   int update, no_out;
   float upd_decay, upd_step;
   float l_cols;

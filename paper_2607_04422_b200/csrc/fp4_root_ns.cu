@@ -616,6 +616,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     a.count = count; a.steps = steps;
     a.s = (int)s; a.l = (int)l; a.s0 = (int)pl0.s0; a.l0 = (int)pl0.l0;
     a.clip = pl0.clip; a.keep = keep; a.bf16 = pl0.bf16;
+    for (int j = 0; j < count; ++j) a.tall |= mats[j].pl.tall;
     a.update = any_update && !keep; a.no_out = upd.no_out; a.upd_decay = upd.decay; a.upd_step = upd.step;
     a.l_cols = (float)l;
     a.q = quant_opts(p, 0);

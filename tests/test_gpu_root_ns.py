@@ -764,6 +764,28 @@ def test_iterations_in_one_launch_for_a_group_with_a_and_x_in_memory(count, side
         assert all(np.array_equal(o.cpu().numpy(), f) for o, f in zip(outs, first))
 
 
+@pytest.mark.parametrize("shape,steps", [((256, 512), 3), ((512, 256), 1), ((1152, 384), 3), ((2048, 2048), 2), ((8192, 768), 3),
+                                         ((1536, 4096), 3), ((6144, 1536), 2), ((2304, 2304), 2)])
+def test_intermediates_are_left_without_the_inspection_flag(shape, steps):
+    """A of the last iteration, and of a tall matrix the X it started from, lie in a dirty workspace after a plain call, also of
+    the tiles that stay in the tensor memory: single launches, and the two and three per iteration of the largest shapes."""
+    m, n = shape
+    G = workloads.gradient_like(m, n, seed=m + 2 * n)
+    _, kept = run_gpu(G, steps=steps, flags=FP4_FLAG_KEEP_OPERANDS)
+    ws = torch.full_like(kept, 0xFF)
+    Gd = torch.from_numpy(G).cuda()
+    out = torch.empty_like(Gd)
+    fp4.fp4_root_ns(Gd, out, steps, None, ws)
+    assert fp4.fp4_last_device_status(ws) == 0
+    lay, _, f32, _, s, l = ws_view(ws, m, n, steps, 0)
+    _, _, f32_kept, _, _, _ = ws_view(kept, m, n, steps, FP4_FLAG_KEEP_OPERANDS)
+    upper = np.kron(np.triu(np.ones((s // 128, s // 128))), np.ones((128, 128))).astype(bool)
+    assert np.array_equal(f32(lay.A, s, s)[upper], f32_kept(lay.A, s, s)[upper])
+    if m > n and steps > 1:
+        before, _ = run_gpu(G, steps=steps - 1)
+        assert np.array_equal(f32(lay.X, s, l), before.T)
+
+
 def test_iterations_in_one_launch_for_a_group_are_those_of_single_calls():
     """Fourteen equal shapes, wide and tall, share one launch; a fifteenth makes the group take the other route."""
     for count in (14, 15):
