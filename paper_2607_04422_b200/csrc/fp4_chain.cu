@@ -86,6 +86,7 @@ struct ChainShared {
   uint64_t out_done[2], out_free[2];
   alignas(16) uint32_t amax[2][4]; // running maximum of the tile in a staging area (bit pattern), at its place among four slots
   alignas(16) float signs[EPI_WARPS][16];   // of the product at hand, a copy per epilogue warp
+  float clip[EPI_WARPS][2];                 // threshold and reciprocal norm of the matrix at hand, a copy per epilogue warp
   uint32_t tmem_base, abort_flag;
   uint32_t tiles[2][kChainTiles];  // this block's tiles of a symmetric product / of G3: p << 28 | ti << 16 | tj
 };
@@ -512,6 +513,14 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
             bound = __fmul_rn(__fmul_rn(4.0f, fabsf(pr.ca)), ax);
             beta = pr.ca;
             gamma = scale;
+            // Fetched with the matrix, not with every tile of the first G3, where nothing covers the two loads: one launch of
+            // 1280 x 8192 318 -> 305 us, 8192 x 1280 with BF16 storage 323 -> 311, 1024 x 10240 316 -> 302.  In shared memory:
+            // registers for the one product that needs them would be spilled in all (309, 313, 306).
+            if (raw && lane == 0) {
+              sh->clip[warp & (EPI_WARPS - 1)][0] = a.clip ? ld_scalar(sc + a.ix.tau) : __int_as_float(0x7f800000);
+              sh->clip[warp & (EPI_WARPS - 1)][1] = ld_scalar(sc + a.ix.inv);
+            }
+            __syncwarp();
           }
           sg_out = scale_predicted(__fmul_rn(a.q.widen, bound));
           inv_sg = __frcp_rn(sg_out);
@@ -621,11 +630,6 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
           if (to_tm) tc_wait_st();
           continue;
         }
-        float tau = 0.0f, inv = 0.0f;
-        if (raw) {
-          tau = a.clip ? ld_scalar(pr.scalars + a.ix.tau) : __int_as_float(0x7f800000);
-          inv = ld_scalar(pr.scalars + a.ix.inv);
-        }
 #pragma unroll 1
         for (int c = 0; c < L::CHUNKS; ++c, ++unit) {
           const int ch = team * L::CHUNKS + c;             // chunk of the tile
@@ -665,6 +669,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
               }
             }
             if (raw) {
+              const float tau = sh->clip[warp & (EPI_WARPS - 1)][0], inv = sh->clip[warp & (EPI_WARPS - 1)][1];
 #pragma unroll
               for (int i = 0; i < 16; ++i) x[i] = __fmul_rn(fminf(fmaxf(x[i], -tau), tau), inv);
             }
