@@ -122,6 +122,53 @@ def test_nearly_tied_candidate_scales_take_the_order_of_the_definition(scale):
     assert np.array_equal(c, oc), mismatch_report(c, oc)
 
 
+@pytest.mark.parametrize("sr", [False, True])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -54, 2.0 ** -57, 2.0 ** 53, 2.0 ** 56])
+def test_blocks_of_one_magnitude_and_their_exact_ties(scale, sr):
+    """Constant blocks and blocks of one element: in the transformed domain one value beside zeros, and sixteen equal magnitudes.
+    A third of them have the same values with both scales, some lie midway between the values of both: exact ties, which keep 6
+    without the sums of the definition.  Their neighbours on both sides are not ties.  Also around the ends of the range in
+    which the kernel compares scaled errors (2^-55, 2^55)."""
+    amax = 1 + np.arange(2048) / 2048
+    amax = np.concatenate([amax, np.nextafter(amax.astype(np.float32), np.float32(2)), np.nextafter(amax.astype(np.float32), np.float32(0))])
+    amax = amax.astype(np.float32)
+    d6, d4 = ((oracle.bf16_bits((amax / np.float32(k)).astype(np.float32)).astype(np.uint32) << 16).view(np.float32).astype(np.float64)
+              for k in (6, 4))
+    e6, e4 = np.abs(amax - 6 * d6), np.abs(amax - 4 * d4)
+    assert (d4 == 1.5 * d6).sum() > 500 and ((d4 != 1.5 * d6) & (e6 == e4)).sum() > 20
+    assert (e6 < e4).sum() > 1000 and (e4 < e6).sum() > 1000
+    amax = amax * np.float32(scale)
+    G = np.zeros((2, amax.size, 16), np.float32)
+    G[0] = amax[:, None] / 4                                    # h = amax, 0, 0, ...
+    G[1, np.arange(amax.size), np.arange(amax.size) % 16] = 4 * amax   # |h| = amax
+    G = G.reshape(-1, 256)
+    st = GpuState(*G.shape)
+    _step(G, st, mu=0.0, sr=sr, seed=9)
+    zero = np.zeros((G.shape[0], 128), np.uint8), np.zeros((G.shape[0], 16), np.uint16)
+    _, oc, os_, _ = oracle.momentum_update(G, *zero, 0.0, 1.0, sr=sr, seed=9)
+    c, s = st.numpy()
+    assert np.array_equal(s, os_), mismatch_report(s, os_)
+    assert np.array_equal(c, oc), mismatch_report(c, oc)
+
+
+@pytest.mark.parametrize("nonzeros", [2, 3, 4])
+def test_blocks_of_few_magnitudes(nonzeros):
+    """Sparse blocks, five steps of the same gradient: states that settle on few magnitudes and tie often."""
+    rng = np.random.default_rng(nonzeros)
+    G = np.zeros((4096, 16), np.float32)
+    for _ in range(nonzeros):
+        G[np.arange(4096), rng.integers(0, 16, 4096)] = rng.integers(-64, 65, 4096)
+    G = G.reshape(-1, 256)
+    st = GpuState(*G.shape)
+    oc, os_ = np.zeros((256, 128), np.uint8), np.zeros((256, 16), np.uint16)
+    for _ in range(5):
+        _step(G, st, mu=0.875, g_scale=0.125)
+        _, oc, os_, _ = oracle.momentum_update(G, oc, os_, 0.875, 0.125)
+        c, s = st.numpy()
+        assert np.array_equal(s, os_), mismatch_report(s, os_)
+        assert np.array_equal(c, oc), mismatch_report(c, oc)
+
+
 def test_ties_zero_blocks_and_extreme_magnitudes():
     f = np.float32
     H4 = oracle.hadamard16  # only to place chosen values in the transformed domain
