@@ -14,7 +14,7 @@
 // same tiles, and every G3 lists the same tiles, the FP32 values a tile combines with (A in G2, X in G3) were
 // written by the very thread that reads them.  So they stay where they are: beside the accumulators the tensor memory has room
 // for 6 tiles of 64 columns or 2 of 128, and a block's first tiles of A and X live there from product to product
-// (place_resident); only the caller's matrix in the first G3, the result in the last, and tiles beyond that room
+// (residents); only the caller's matrix in the first G3, the result in the last, and tiles beyond that room
 // move through memory (and, stored only, what the workspace keeps of the last iteration).  A block of those is fetched while
 // the tile before it is worked on, the first one of a product that has no resident tile before its dependency is even looked
 // at; the copies that wrote them have arrived by then, because the warp waits for all its own at the end of the product before.
@@ -877,30 +877,42 @@ cudaError_t chain_set_attributes() {
   return cudaSuccess;
 }
 
-// Estimated times in us.  A product costs a dependency round trip and rounds of tiles that take an epilogue or a main
-// loop each, whichever is longer.  The constants here and of the CTA-pair kernel's estimate beside the caller are fitted to
-// the times of all routes at 54 shapes and groups, 128 to 2560 wide, plain and with the quantiser options; choosing by
-// them loses 0.5 % on average against always knowing the fastest, 4 % at worst.
+// Which tiles stay in the tensor memory, when every block takes up to `full` tiles of G3 and `sym` of a symmetric product: A
+// first, which serves two products of an iteration (2048 x 2048 201 us, X first 215).  One accumulator instead of two where that lets
+// more of them stay: a tile's accumulator is read at the very start of its epilogue (201 us, with two accumulators 211).
+struct Residents { int nacc, na, nx; };
+static Residents residents(int bn, int64_t full, int64_t sym) {
+  const int nacc = full + sym <= resident_slots(bn, 2) ? 2 : 1;
+  const int64_t slots = resident_slots(bn, nacc), na = sym < slots ? sym : slots;
+  return {nacc, (int)na, (int)(full < slots - na ? full : slots - na)};
+}
+
+// Estimated times in us.  A product costs a dependency round trip and a block's tiles, each an epilogue - short where its FP32 values
+// stay in the tensor memory, long where they move through memory - or a main loop, whichever is longer.  The constants here
+// and of the CTA-pair kernel's estimate beside the caller are fitted to the times of all routes and both widths at 213 shapes and
+// groups (short sides 128 to 2304, long sides to 32768, 1 to 14 matrices, plain and with the quantiser options): choosing by them
+// loses 0.1 % on average against always knowing the fastest, 3.5 % at worst, and 0.7 % (9 %) at 100 others drawn at random.
 struct TileUs {
-  double epi, k1, k2;   // epilogue; main loop of G1; of G2 and G3
+  double product, resident, memory, k1, k2;   // k1, k2: main loop of G1; of G2 and G3
   TileUs(int bn, int64_t s, int64_t l, bool opts)
-      : epi(2.5 * (bn / 64) * (opts ? 1.6 : 1.0)), k1(0.4 * (double)((l + 255) / 256)), k2(0.4 * (double)((s + 255) / 256)) {}
-  double g1() const { return epi > k1 ? epi : k1; }
-  double g23() const { return epi > k2 ? epi : k2; }
+      : product(bn == 64 ? 4.0 : 5.0), resident((bn == 64 ? 0.65 : 1.0) * (opts ? 1.45 : 1.0)),
+        memory((bn == 64 ? 1.7 : 4.75) * (opts ? 1.45 : 1.0)), k1(0.22 * (double)((l + 255) / 256)), k2(0.26 * (double)((s + 255) / 256)) {}
+  static double tiles(int64_t n, int in_tm, double resident, double memory, double k) {
+    return in_tm * (resident > k ? resident : k) + (double)(n - in_tm) * (memory > k ? memory : k);
+  }
 };
 // one iteration of a single launch with tiles of bn columns; 0 when a block would take more tiles than its list holds
 static double width_us(int bn, int64_t s, int64_t l, int count, bool opts, int sms) {
   const int64_t rs = rounds(sym_tiles(s, bn) * count, sms), rf = rounds(s / BM * (l / bn) * count, sms);
   if (rf > kChainTiles) return 0.0;
+  const Residents r = residents(bn, rf, rs);
   const TileUs t(bn, s, l, opts);
-  // narrow tiles beyond the tensor memory: their X moves through the shared memory and back.  (With the quantiser options the
-  // arithmetic covers that.)  5 iterations in one launch / two launches each: 1280 x 7168 297 / 285 us, 1408 x 6144 300 / 289, 1280 x 8192
-  // 332 / 327, 1152 x 8192 312 / 327, 1024 x 8192 264 / 266; with options 1152 x 8192 370 / 416.
-  const int64_t beyond = bn == 64 && !opts ? rs + rf - resident_slots(64, 1) : 0;
-  return 3 * 4.0 + (double)rs * t.g1() + (double)(rs + rf) * t.g23() + (beyond > 0 ? 1.2 * (double)beyond : 0.0);
+  return 3 * t.product + t.tiles(rs, r.na, t.resident, t.memory, t.k1) + t.tiles(rs, r.na, t.resident, t.memory, t.k2) +
+         t.tiles(rf, r.nx, t.resident, t.memory, t.k2);
 }
-// The width of a single launch's tiles.  Measured before tiles stayed in the tensor memory, 5 iterations, 64 / 128 columns: 256 x 512 95 / 126 us, 1024 x 4096
-// 185 / 212 (with the quantiser options 240 / 293), 8 x 768 x 768 176 / 211, 1536 x 4096 264 / 261, 2048 x 2048 228 / 224.
+// The width of a single launch's tiles.  Measured, 5 iterations, 64 / 128 columns: 256 x 512 83 / 101 us, 1024 x 4096 159 / 185 (with the
+// quantiser options 200 / 243), 8 x 768 x 768 155 / 179, 1152 x 8192 290 / 324, 1536 x 1536 148 / 139, 1536 x 2816 196 / 188,
+// 2048 x 2048 210 / 196 (250 / 249).
 static bool narrow_tiles(int64_t s, int64_t l, int count, bool opts, int sms) {
   const double n = width_us(64, s, l, count, opts, sms), w = width_us(128, s, l, count, opts, sms);
   return n > 0.0 && n <= w;
@@ -912,17 +924,7 @@ double chain_iteration_us(int64_t s, int64_t l, int count, bool opts, int sms) {
 double chain_symmetric_us(int64_t s, int64_t l, int count, bool opts, int sms) {
   if (sym_tiles(s, 128) * count > sms) return 0.0;
   const TileUs t(128, s, l, opts);
-  return 12.0 + t.g1() + t.g23();
-}
-
-// Which tiles stay in the tensor memory, when every block takes up to `full` tiles of G3 and `sym` of a symmetric product: A
-// first, which serves two products of an iteration (2048 x 2048 201 us, X first 215).  One accumulator instead of two where that lets
-// more of them stay: a tile's accumulator is read at the very start of its epilogue (201 us, with two accumulators 211).
-static void place_resident(ChainLaunch& a, int bn, int64_t full, int64_t sym) {
-  a.nacc = full + sym <= resident_slots(bn, 2) ? 2 : 1;
-  const int64_t slots = resident_slots(bn, a.nacc);
-  a.na = (int)(sym < slots ? sym : slots);
-  a.nx = (int)(full < slots - a.na ? full : slots - a.na);
+  return 12.5 + t.tiles(1, 1, t.resident, t.memory, t.k1) + t.tiles(1, 1, t.resident, t.memory, t.k2);
 }
 
 cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st) {
@@ -934,7 +936,8 @@ cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int s
   a.nsym = (int)sym_tiles(a.s, bn);
   const int64_t widest = (int64_t)(a.s / BM) * (a.l / bn) * a.count;
   const int grid = (int)(widest < sms ? widest : sms);
-  place_resident(a, bn, rounds(widest, grid), rounds((int64_t)a.nsym * a.count, grid));
+  const Residents r = residents(bn, rounds(widest, grid), rounds((int64_t)a.nsym * a.count, grid));
+  a.nacc = r.nacc; a.na = r.na; a.nx = r.nx;
   if (narrow) return pf ? launch_one<64, true>(pack, a, grid, st) : launch_one<64, false>(pack, a, grid, st);
   return pf ? launch_one<128, true>(pack, a, grid, st) : launch_one<128, false>(pack, a, grid, st);
 }
@@ -948,7 +951,8 @@ cudaError_t launch_chain_symmetric(const ChainPack& pack, const ChainLaunch& lau
   const int64_t widest = (int64_t)a.nsym * a.count;
   if (widest > sms) return cudaErrorInvalidValue;
   const int grid = (int)widest;
-  place_resident(a, 128, 0, 1);
+  const Residents r = residents(128, 0, 1);
+  a.nacc = r.nacc; a.na = r.na; a.nx = r.nx;
   return a.q.rht || a.q.four_six ? launch_one<128, true, true>(pack, a, grid, st) : launch_one<128, false, true>(pack, a, grid, st);
 }
 

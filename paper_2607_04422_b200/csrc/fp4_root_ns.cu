@@ -357,28 +357,29 @@ struct PairUs {
   PairUs(int64_t s, int64_t l, int count, bool opts, int sms) {
     const double ts = (double)((s + 255) / 256), tl = (double)((l + 255) / 256), pairs = (double)(sms / 2);
     auto rounds = [](double r) { return (std::ceil(r) + (r > 1.0 ? r : 1.0)) / 2; };
-    const double epi = 6.0 * (opts ? 1.7 : 1.0), kb = 0.3;
+    const double epi = 3.95 * (opts ? 1.5 : 1.0), kb = 0.22;
     const double k1 = kb * tl, k2 = kb * ts;
     const double rs = rounds(ts * (ts + 1) / 2 * count / pairs), rf = rounds(ts * tl * count / pairs);
-    g1 = 8.0 + rs * (epi > k1 ? epi : k1);
-    g2 = 8.0 + rs * (epi > k2 ? epi : k2);
-    g3 = 8.0 + rf * (epi > k2 ? epi : k2);
+    g1 = 6.25 + rs * (epi > k1 ? epi : k1);
+    g2 = 6.25 + rs * (epi > k2 ? epi : k2);
+    g3 = 6.25 + rf * (epi > k2 ? epi : k2);
   }
 };
 
 // How a group runs its iterations: all of them in one launch (fp4_chain.cu), three launches of the CTA-pair kernel per
 // iteration, or two - G1 and G2 as one launch with a 128 x 128 tile per SM where their 256 x 256 tiles would leave half of
-// the SM pairs idle, and the pairs' G3.  What is estimated to be fastest.  Since A and X stay in the tensor memory single launches
-// take 5 to 14 % and the two of a pair's G1 and G2 3 to 7 % less than here, which moves the line little (estimates 12 % lower sent
-// 2304 x 2304, 261 us, and 1792 x 4096, 252 us, to single launches of 309 and 295 us).  Before that, 5 iterations, one launch / two / three
-// per iteration: 1024 x 1024 119 / 174 / 179 us, 2048 x 2048 224 / 221 / 231, 2048 x 4096 318 / 287 / 307, 1536 x 6144
-// 339 / 305 / 330, 2048 x 8192 492 / 446 / 450 (with the quantiser options 669 / 604 / 619), 2304 x 2304 295 / - / 264,
-// 4 x 512 x 512 106 / 170 / 179, 2 x 1024 x 2816 200 / 248 / 260.  (Not for inspection of BF16-stored intermediates: in
-// single launches A and X stay FP32 tensors with rounded values.)
+// the SM pairs idle, and the pairs' G3.  What is estimated to be fastest.  Measured, 5 iterations, one launch (width of its tiles) / two /
+// three per iteration: 1024 x 1024 102 (64) / 159 / 178 us, 1280 x 8192 304 (64) / 324 / 358, 1280 x 10240 353 (64) / 347 / 380,
+// 1536 x 4096 241 (128) / 232 / 254, 2048 x 2048 196 (128) / 200 / 223, 2048 x 8192 502 (128) / 422 / 450, 2304 x 2304 277 (64) / - / 262
+// (with the quantiser options 332 / - / 370), 12 x 896 x 896 308 (64) / - / 373, 7 x 1040 x 1040 326 (64) / - / 377, 2 x 1792 x 1792
+// 242 (64) / - / 273, 8 x 1280 x 1280 415 (64) / - / 413.  (Not for inspection of BF16-stored intermediates: in single launches A and
+// X stay FP32 tensors with rounded values.  Nor, without the options, for long sides beyond 32768, where one launch would be the
+// faster, 458 (64) / 559 / 545 at 128 x 56784: these keep the route that they have been tested on.)
+constexpr int64_t kChainLong = 32768;
 enum Route { kOneLaunch, kTwoLaunches, kThreeLaunches };
 Route route_of(const NsPlan& pl, int count, const fp4_ns_params* p, int sms) {
-  if (count > kChainMax || (pl.bf16 && (p->flags & FP4_FLAG_KEEP_OPERANDS))) return kThreeLaunches;
   const bool opts = (p->flags & (FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)) != 0;
+  if (count > kChainMax || (pl.l > kChainLong && !opts) || (pl.bf16 && (p->flags & FP4_FLAG_KEEP_OPERANDS))) return kThreeLaunches;
   const PairUs pair(pl.s, pl.l, count, opts, sms);
   const double three = pair.g1 + pair.g2 + pair.g3;
   const double sym = chain_symmetric_us(pl.s, pl.l, count, opts, sms);
