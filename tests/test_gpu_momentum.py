@@ -86,10 +86,11 @@ def _errors_of_both_scales(h):
     return out
 
 
-@pytest.mark.parametrize("scale", [1.0, 2.0 ** -90, 2.0 ** 95])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -56, 2.0 ** 54, 2.0 ** -90, 2.0 ** 95])
 def test_nearly_tied_candidate_scales_take_the_order_of_the_definition(scale):
     """Blocks whose two candidate errors agree to a few parts per million, and neighbours of them on both sides of the tie:
-    what the kernel may decide from rounded sums and what it must leave to the definition."""
+    what the kernel may decide from rounded sums and what it must leave to the definition, in the middle and around both
+    ends of the range in which it uses rounded sums.  Far outside all squares underflow or overflow: ties, which keep 6."""
     rng = np.random.default_rng(5)
     H = np.array([[(-1) ** bin(i & j).count("1") for j in range(16)] for i in range(16)], np.float64) / 4
     g = rng.standard_normal((1 << 17, 16)).astype(np.float32)
@@ -104,6 +105,7 @@ def test_nearly_tied_candidate_scales_take_the_order_of_the_definition(scale):
         step[:, i] = 2.0 ** -12
         f = lambda x: (lambda a: a[1] - a[0])(_errors_of_both_scales((x.astype(np.float64) @ H).astype(np.float32)))
         lo, hi = g - step * 64, g + step * 64
+        assert (np.sign(f(lo)) != np.sign(f(hi))).sum() > 50
         for _ in range(30):                            # bisection in FP32, where the signs differ
             mid = ((lo.astype(np.float64) + hi) / 2).astype(np.float32)
             same = (np.sign(f(mid)) == np.sign(f(lo)))[:, None]
@@ -117,6 +119,13 @@ def test_nearly_tied_candidate_scales_take_the_order_of_the_definition(scale):
     _step(G, st, mu=0.0)
     zero = np.zeros((G.shape[0], 128), np.uint8), np.zeros((G.shape[0], 16), np.uint16)
     _, oc, os_, _ = oracle.momentum_update(G, *zero, 0.0, 1.0)
+    amax = np.abs((G.reshape(-1, 16).astype(np.float64) @ H).astype(np.float32)).max(axis=1)
+    six, four = ((os_.ravel() == oracle.bf16_bits((amax / np.float32(k)).astype(np.float32))).sum() for k in (6, 4))
+    if 2.0 ** -60 < scale < 2.0 ** 60:
+        assert min(six, four) > 0.2 * amax.size         # both candidates are chosen
+        assert scale == 1.0 or amax.min() < 2.0 ** (-55 if scale < 1 else 55) < amax.max()
+    else:
+        assert six > 0.95 * amax.size
     c, s = st.numpy()
     assert np.array_equal(s, os_), mismatch_report(s, os_)
     assert np.array_equal(c, oc), mismatch_report(c, oc)

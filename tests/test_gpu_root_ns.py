@@ -690,11 +690,12 @@ def test_bf16_storage_of_shapes_that_pad_to_multiples_of_256(shape):
 
 
 @pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX, FP4_FLAG_STORE_BF16])
-@pytest.mark.parametrize("shape", [(16, 16), (128, 128), (144, 112), (128, 1040), (1040, 256), (1168, 1072), (1280, 1536)])
+@pytest.mark.parametrize("shape", [(16, 16), (128, 128), (144, 112), (128, 1040), (1040, 256), (1168, 1072), (1280, 1536), (1280, 2048),
+                                   (1536, 1536)])
 def test_iterations_in_one_launch_at_the_edges_of_its_tiles(shape, flags):
     """Small matrices run all iterations in one cooperative launch with 128 x 64 or 128 x 128 tiles: one tile, one
-    block per 128 rows, partial last tiles, more tiles than SMs (the last two; 1280 x 1536 takes the wide
-    tiles).  The result on a dirty workspace is the oracle's, twice the same."""
+    block per 128 rows, partial last tiles, more tiles than SMs (from 1168 x 1072 on), wide tiles (1536 x 1536).  The
+    result on a dirty workspace is the oracle's, twice the same."""
     m, n = shape
     G = workloads.gradient_like(m, n, seed=m + n)
     Gd = torch.from_numpy(G).cuda()
@@ -714,18 +715,24 @@ def test_iterations_in_one_launch_at_the_edges_of_its_tiles(shape, flags):
 
 
 @pytest.mark.parametrize("shape,flags", [((768, 8192), 0), ((8192, 768), FP4_FLAG_STORE_BF16), ((1536, 2816), 0),
-                                         ((1280, 2048), FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)])
+                                         ((768, 8192), FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)])
 def test_iterations_in_one_launch_with_tiles_beyond_the_tensor_memory(shape, flags):
-    """More tiles per block than stay in the tensor memory: the first ones' A and X live there, the others' in the workspace,
-    next to one another in one product; the same bytes twice, also from a dirty workspace."""
+    """More tiles of X per block than stay in the tensor memory (6 of which 5, the third 2 of which 1): the first ones' X lives
+    there, the others' in the workspace, next to one another in one product; A, a tile per block, is always resident.  The
+    same bytes twice, also from a dirty workspace."""
     m, n = shape
     G = workloads.gradient_like(m, n, seed=m + n)
     Gd = torch.from_numpy(G).cuda()
     out = torch.empty_like(Gd)
     ws = torch.full((fp4.fp4_root_ns_workspace_bytes(m, n, 3, flags),), 0xFF, dtype=torch.uint8, device="cuda")
     p = fp4.NsParams.make(flags=flags, seed=5)
-    fp4.fp4_root_ns(Gd, out, 3, p, ws)
-    assert fp4.fp4_last_device_status(ws) == 0
+    launches = []
+    for steps in (1, 3):
+        before = fp4.fp4_kernel_launches()
+        fp4.fp4_root_ns(Gd, out, steps, p, ws)
+        launches.append(fp4.fp4_kernel_launches() - before)
+        assert fp4.fp4_last_device_status(ws) == 0
+    assert launches[0] == launches[1]                   # one launch however many iterations
     first = out.cpu().numpy()
     pf = bool(flags & FP4_FLAG_RHT)
     want = oracle.root_ns(G, steps=3, rht=pf, four_six=pf, seed=5, store_bf16=bool(flags & FP4_FLAG_STORE_BF16))
