@@ -29,13 +29,13 @@
 // Bounds: latency.  A 5-iteration call is a chain of 15 dependent products.  At 256 x 512 a product takes about 4 us:
 // operand copies 0.75, MMAs 0.3, the one tile's epilogue 0.75-1.1, its stores and the release 1.1, the counter's way to the
 // slowest of the other blocks 0.8.  The epilogue has 96 registers per thread for 16 values in flight: with both passes' values
-// in registers at once it spilled, and every spill is a trip through the shared memory's pipe.  Resident tiles with
+// in registers at once it spilled, and the spill area of 608 threads does not fit the L1 that the shared memory leaves.  Resident tiles with
 // a path of their own that needs nothing else, and the second pass's values read after the first, whole calls: 256 x 512
-// 94.7 -> 83.0 us, 1024 x 1024 114.4 -> 101.7, 2048 x 2048 217 -> 201, with the signs of the transform in shared memory 640 x 768
+// 94.7 -> 82.2 us, 1024 x 1024 114.4 -> 101.6, 2048 x 2048 217 -> 198, with the signs of the transform in shared memory 640 x 768
 // with the quantiser options 137.6 -> 115.8, 1040 x 2896 212 -> 187; G1 and G2 of 2048 x 6144 with options 510 -> 470.
 // With the proxy fence on the reading side and one lane storing everything the iterations of 256 x 512 took 87 us
 // instead of 78, of 1408 x 2176 156 instead of 141.  Whole calls against three launches per iteration: 256 x 512
-// 175 -> 97 us, 1024 x 1024 190 -> 118, 1040 x 2896 with the paper's quantiser options 307 -> 223.
+// 152 -> 83 us, 1024 x 1024 178 -> 102, 1040 x 2896 with the paper's quantiser options 300 -> 186.
 #include "fp4_gemm_common.cuh"
 
 namespace fp4 {
