@@ -818,13 +818,14 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
       }
       // What the next product reads from memory: blocks this warp has stored itself (A in G1, X in the G3 before), so every store
       // of the warp has to have arrived - also when the product begins with resident tiles and fetches later.  A product
-      // that begins beyond them has its first block fetched here.
+      // that begins beyond them has its first block fetched here.  (a.keep: resident tiles of A are stored in every
+      // iteration, to the same place.)
       if (mine > 0) for (int np = pi + 1; np < end && np <= pi + 3; ++np) {
         const int nk = np / 3, nmode = np - 3 * nk + kG1;
         const int nmine = nmode != kG3 ? my_sym : my_full;
         if (nmine == 0) continue;
         const int in_tm = nmode == kG1 ? nmine : nmode == kG2 ? a.na : nk > 0 ? a.nx : 0;
-        if (nmine > in_tm) {
+        if (nmine > in_tm || a.keep) {
           if (lane == 0) bulk_wait_all<0>();
           if (in_tm == 0) {
             fetch(nmode, nk, sh->tiles[nmode != kG3 ? 0 : 1][0], 0, (int)(unit & 1));
