@@ -1,6 +1,7 @@
 // fp4_quantize: standalone NVFP4 block quantiser (Section 2, "NVFP4 format"), and the
 // transposing copy that returns the result of a tall input.
 #include "fp4_gemm_common.cuh"
+#include "fp4_state.cuh"
 
 namespace fp4 {
 
@@ -37,35 +38,47 @@ __global__ void __launch_bounds__(256) k_amax(const float4* __restrict__ x, int6
   }
 }
 
+// 8 values by one 256-bit load where the tensor lies on a 32-byte boundary, else by two 128-bit ones
+__device__ __forceinline__ void load8(const float* p, bool wide, float* v) {
+  if (wide) {
+    ldg_f32x8(p, v);
+  } else {
+    const float4 s = __ldg(reinterpret_cast<const float4*>(p)), t = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    v[0] = s.x; v[1] = s.y; v[2] = s.z; v[3] = s.w;
+    v[4] = t.x; v[5] = t.y; v[6] = t.z; v[7] = t.w;
+  }
+}
+__device__ __forceinline__ void load_block16(const float* p, bool wide, float (&v)[16]) {
+  load8(p, wide, v);
+  load8(p + 8, wide, v + 8);
+}
+
 // ----------------------------------------------------------------------------------
-// Row quantiser: one thread per block of 16 (four 128-bit loads = 64 contiguous bytes, a warp
-// covers 512 consecutive elements of a row), so the two IEEE divisions of a block are done
-// once; 8-byte code store and 1-byte scale store per thread.  Thread blocks walk the tensor
-// from its end: the amax pass has just read it front to back, so the end is what L2 still
-// holds.  grid: rows x ceil(cols / 4096) thread blocks.
-// amax_bits holds the tensor amax on entry (bit pattern).
+// Row quantiser: one thread per block of 16 (64 contiguous bytes, a warp covers 512 consecutive elements of a row); 8-byte code
+// store and 1-byte scale store per thread.  Thread blocks walk the tensor from its end: the amax pass has just read it
+// front to back, so the end is what L2 still holds (74 of 268 MB at most: with 128-bit loads and another block order 37).
+// grid: rows x ceil(cols / 4096) thread blocks.  amax_bits holds the tensor amax on entry (bit pattern).
+//
+// Bounds: HBM with reads and writes mixed, 5.5 TB/s of it.  With 256-bit loads (every sector looked up once), no 64-bit division for the
+// place and none of the two IEEE divisions per block, whole calls, before / after: 8192 x 8192 92.9 / 91.4 us, 16384 x 8192
+// 179 / 173, 4096 x 4096 29.4 / 28.3, 2048 x 4352 20.5 / 19.1, 8192 x 8192 with the options 116 / 111.  (One cooperative launch in
+// which every block walks the same units in both passes finds 74 MB of 8192 x 8192 in the L2, and is slower all the same:
+// 93.3 us, prefetched a unit ahead or not.)
 // ----------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_quantize_rows(const float* __restrict__ x, int64_t rows, int64_t cols,
                                                        uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                                                       const uint32_t* __restrict__ amax_bits) {
+                                                       const uint32_t* __restrict__ amax_bits, const bool wide) {
   pdl_launch_dependents();
   pdl_wait();
   const float sg = scale_exact(__uint_as_float(*amax_bits));
-  const float six_sg = __fmul_rn(6.0f, sg);
-  const int64_t groups = ((cols >> 4) + 255) / 256;  // thread blocks per row
-  const int64_t bid = (int64_t)gridDim.x - 1 - blockIdx.x;
-  const int64_t r = bid / groups;
-  const int64_t kb = (bid % groups) * 256 + threadIdx.x;
-  if (r >= rows || kb >= (cols >> 4)) return;
-  const float4* src = reinterpret_cast<const float4*>(x + r * cols + kb * 16);
+  const float six_sg = __fmul_rn(6.0f, sg), rcp_six_sg = __frcp_rn(six_sg);
+  const int64_t r = (int64_t)gridDim.x - 1 - blockIdx.x;
+  const int64_t kb = (int64_t)(gridDim.y - 1 - blockIdx.y) * 256 + threadIdx.x;
+  if (kb >= (cols >> 4)) return;
   float v[16];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float4 t = __ldg(src + j);
-    v[4 * j] = t.x; v[4 * j + 1] = t.y; v[4 * j + 2] = t.z; v[4 * j + 3] = t.w;
-  }
+  load_block16(x + r * cols + kb * 16, wide, v);
   uint32_t lo, hi;
-  const uint32_t sb = quantize_block16(v, six_sg, sg, lo, hi);
+  const uint32_t sb = quantize_block16_fast(v, sg, six_sg, rcp_six_sg, lo, hi);
   *reinterpret_cast<uint2*>(codes + r * (cols / 2) + kb * 8) = make_uint2(lo, hi);
   scales[sf_offset(r, kb, cols >> 4)] = (uint8_t)sb;
 }
@@ -80,23 +93,16 @@ __global__ void k_finish_tensor_scale(float* ts, float widen) {
 // consecutive elements of a row.  grid: rows x ceil(cols / 4096) thread blocks, row-major.
 __global__ void __launch_bounds__(256) k_quantize_rows_opts(const float* __restrict__ x, int64_t rows, int64_t cols,
                                                             uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                                                            const uint32_t* __restrict__ amax_bits,
+                                                            const uint32_t* __restrict__ amax_bits, const bool wide,
                                                             const QuantOpts q) {
   pdl_launch_dependents();
   pdl_wait();
   const float sg = scale_exact(__fmul_rn(q.widen, __uint_as_float(*amax_bits)));
-  const int64_t groups = ((cols >> 4) + 255) / 256;  // thread blocks per row
-  const int64_t bid = (int64_t)gridDim.x - 1 - blockIdx.x;  // from the end, as k_quantize_rows
-  const int64_t r = bid / groups;
-  const int64_t kb = (bid % groups) * 256 + threadIdx.x;
-  if (r >= rows || kb >= (cols >> 4)) return;
-  const float4* src = reinterpret_cast<const float4*>(x + r * cols + kb * 16);
+  const int64_t r = (int64_t)gridDim.x - 1 - blockIdx.x;   // from the end, as k_quantize_rows
+  const int64_t kb = (int64_t)(gridDim.y - 1 - blockIdx.y) * 256 + threadIdx.x;
+  if (kb >= (cols >> 4)) return;
   float v[16];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float4 t = __ldg(src + j);
-    v[4 * j] = t.x; v[4 * j + 1] = t.y; v[4 * j + 2] = t.z; v[4 * j + 3] = t.w;
-  }
+  load_block16(x + r * cols + kb * 16, wide, v);
   uint32_t lo, hi;
   const uint32_t sb = quantize_block16_opts(v, q, sg, lo, hi);
   *reinterpret_cast<uint2*>(codes + r * (cols / 2) + kb * 8) = make_uint2(lo, hi);
@@ -194,7 +200,7 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
   }
   bits = __reduce_max_sync(0xffffffffu, bits);
   const float sg = scale_exact(__fmul_rn(q.widen, __uint_as_float(bits)));
-  const float six_sg = __fmul_rn(6.0f, sg);
+  const float six_sg = __fmul_rn(6.0f, sg), rcp_six_sg = __frcp_rn(six_sg);
   grid_barrier(counter, 2 * blocks, abort_flag, limit_ns);   // everyone has read the maxima: scales may be written
   const uint32_t kblocks = (uint32_t)(cols >> 4);
   for (int i = 0; i < m; ++i) {
@@ -203,7 +209,7 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
     const uint32_t b = (uint32_t)(first + i * step) * 128 + row;   // block of the tensor
     uint32_t lo, hi, sb;
     if (PF) sb = quantize_block16_opts(v, q, sg, lo, hi);
-    else sb = quantize_block16(v, six_sg, sg, lo, hi);
+    else sb = quantize_block16_fast(v, sg, six_sg, rcp_six_sg, lo, hi);
     *reinterpret_cast<uint2*>(codes + (int64_t)b * 8) = make_uint2(lo, hi);
     const uint32_t r = b / kblocks;
     scales[sf_offset(r, b - r * kblocks, kblocks)] = (uint8_t)sb;
@@ -310,15 +316,16 @@ cudaError_t launch_quantize(const CUtensorMap* tm, const float* x, int64_t rows,
                               tensor_scale, q, (uint32_t)grid + (give_up_ns ? 1u : 0u), give_up_ns ? give_up_ns : kWaitLimitNs);
   }
   const int64_t n4 = rows * cols / 4;
+  const bool wide = (reinterpret_cast<uintptr_t>(x) & 31) == 0;
   cudaError_t e = cudaMemsetAsync(tensor_scale, 0, 4, st);
   if (e != cudaSuccess) return e;
   // chained: a kernel's blocks become resident while the one before drains (8192 x 8192: 96 -> 92.5 us)
   pdl_select(0);
   uint32_t* amax = reinterpret_cast<uint32_t*>(tensor_scale);
   launch_chained(k_amax, dim3(grid_for(n4, 256 * 8, sms)), dim3(256), 0, st, reinterpret_cast<const float4*>(x), n4, amax);
-  const dim3 qgrid((unsigned)(((cols / 16 + 255) / 256) * rows));
-  if (pf) launch_chained(k_quantize_rows_opts, qgrid, dim3(256), 0, st, x, rows, cols, codes, scales, amax, q);
-  else launch_chained(k_quantize_rows, qgrid, dim3(256), 0, st, x, rows, cols, codes, scales, amax);
+  const dim3 qgrid((unsigned)rows, (unsigned)((cols / 16 + 255) / 256));
+  if (pf) launch_chained(k_quantize_rows_opts, qgrid, dim3(256), 0, st, x, rows, cols, codes, scales, amax, wide, q);
+  else launch_chained(k_quantize_rows, qgrid, dim3(256), 0, st, x, rows, cols, codes, scales, amax, wide);
   launch_chained(k_finish_tensor_scale, dim3(1), dim3(1), 0, st, tensor_scale, q.widen);
   count_launches(3);
   return cudaGetLastError();

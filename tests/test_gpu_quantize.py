@@ -159,6 +159,30 @@ def test_single_launch_quantiser_at_its_limits(shape, flags):
         assert np.array_equal(codes.cpu().numpy(), oc), mismatch_report(codes.cpu().numpy(), oc)
 
 
+@pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX])
+@pytest.mark.parametrize("offset", [0, 4, 8])
+@pytest.mark.parametrize("shape,scale", [((1792, 4224), 1.0), ((57088, 128), 1.0), ((1792, 4224), 2.0 ** -75)])
+def test_two_pass_quantiser_on_every_alignment(shape, scale, offset, flags):
+    """Tensors beyond the single launch: on 32-byte boundaries (256-bit loads) and only on 16-byte ones, a row of one and a bit
+    thread blocks and of half a warp, a tensor scale below 2^-60 (plain operations)."""
+    rows, cols = shape
+    x_np = workloads.row_lognormal(rows, cols, seed=rows) * np.float32(scale)
+    mask = 0xA5C3 if flags else 0
+    store = torch.empty(rows * cols + 8, device="cuda")
+    x = store[offset:offset + rows * cols].view(rows, cols)
+    assert x.data_ptr() % 32 == offset * 4 % 32
+    x.copy_(torch.from_numpy(x_np))
+    oc, os_, osg = oracle.quantize(x_np, rht=True, mask=mask, four_six=True) if flags else oracle.quantize(x_np)
+    codes = torch.full((rows, cols // 2), 0xEE, dtype=torch.uint8, device="cuda")
+    scales = torch.full((fp4.fp4_scale_bytes(rows, cols),), 0xEE, dtype=torch.uint8, device="cuda")
+    ts = torch.full((1,), float("nan"), device="cuda")
+    fp4.fp4_quantize(x, codes, scales, ts, flags=flags | mask << 16)
+    assert np.float32(ts.item()) == np.float32(osg)
+    got = sf_from_atoms(scales.cpu().numpy(), rows, cols // 16)
+    assert np.array_equal(got, os_), mismatch_report(got, os_)
+    assert np.array_equal(codes.cpu().numpy(), oc), mismatch_report(codes.cpu().numpy(), oc)
+
+
 @pytest.mark.parametrize("scale", [1.0, 1e-41])    # the second: a tensor scale of a few units of 2^-149
 @pytest.mark.parametrize("shape", [(128, 128), (1024, 1152), (1152, 2688)])
 def test_single_launch_quantiser_waits_for_no_word_that_it_overwrites(shape, scale):
