@@ -184,35 +184,6 @@ __device__ __forceinline__ float mom_encode_fast(const float (&h)[16], float d, 
   return err;
 }
 
-// The same codes and another error: the squared differences between the scaled values and their codes, summed in any order.
-// A mixed-precision multiply-add on the FP16 value of a code and a fused square per pair take half of the instructions.
-__device__ __forceinline__ float mom_encode_scaled(const float (&h)[16], float rcp, uint32_t& lo, uint32_t& hi) {
-  const uint64_t rcp2 = pack2(rcp, rcp);
-  uint64_t sum[2];
-#pragma unroll
-  for (int b = 0; b < 2; ++b) {
-    float y[8];
-    uint32_t codes, q[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) unpack2(mul2(pack2(h[8 * b + 2 * i], h[8 * b + 2 * i + 1]), rcp2), y[2 * i], y[2 * i + 1]);
-    cvt_e2m1x8_f16(y, codes, q);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float d0, d1;
-      asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\t"
-          "fma.rn.f32.f16 %0, a, %3, %4;\n\tfma.rn.f32.f16 %1, b, %3, %5;\n\t}"
-          : "=f"(d0), "=f"(d1)
-          : "r"(q[i]), "h"((uint16_t)0xBC00), "f"(y[2 * i]), "f"(y[2 * i + 1]));
-      const uint64_t dd = pack2(d0, d1);
-      sum[b] = i == 0 ? mul2(dd, dd) : fma2(dd, dd, sum[b]);
-    }
-    if (b == 0) lo = codes; else hi = codes;
-  }
-  float a, c;
-  unpack2(add2(sum[0], sum[1]), a, c);
-  return a + c;
-}
-
 // RN(1 / d) of a BF16 value in [2^-110, 2^110]: one Newton step on the approximation leaves a relative error near
 // 2^-46, and the reciprocals of 8-bit significands lie at least 2^-33 from the midpoint of two floats.
 __device__ __forceinline__ float rcp_bf16(float d) {
@@ -244,11 +215,7 @@ static __device__ __noinline__ uint3 encode_pair_exact(float h0, float h1, float
 }
 
 // Does every element have the same error with both scales, so that the definition's sums are equal?  What makes blocks tie:
-// equal values (d4 = 1.5 d6, and the second codes times 1.5 are the first; of the grid only 0, 1, 2 and 4 have a multiple by
-// 1.5 on it, the even codes with the next odd one), or a single magnitude amax beside zeros, midway between 6 d6 and 4 d4.
-__device__ __forceinline__ bool codes_match(uint32_t six, uint32_t four) {
-  return ((four | (((four >> 1) | (four >> 2)) & 0x11111111u)) ^ six | (four & 0x11111111u)) == 0u;
-}
+// equal values (d4 = 1.5 d6, see codes_match), or a single magnitude amax beside zeros, midway between 6 d6 and 4 d4.
 __device__ __forceinline__ bool same_errors(const float (&h)[16], float amax, float d6, float d4, uint32_t lo, uint32_t hi, uint32_t lo4,
                                             uint32_t hi4) {
   if (d4 == 1.5f * d6) return codes_match(lo, lo4) && codes_match(hi, hi4);
@@ -283,9 +250,9 @@ __device__ __forceinline__ void state_encode(const float (&h)[16], uint64_t seed
     const float d6 = bf16_lo(w), d4 = bf16_hi(w);
     const float r6 = rcp_bf16(d6), r4 = rcp_bf16(d4);
     uint32_t lo4, hi4;
-    const float s6 = mom_encode_scaled(h, r6, lo, hi);
+    const float s6 = encode_block16_scaled(h, r6, lo, hi);
     const float ratio = d4 * r6;
-    const float s4 = mom_encode_scaled(h, r4, lo4, hi4) * (ratio * ratio);
+    const float s4 = encode_block16_scaled(h, r4, lo4, hi4) * (ratio * ratio);
     const float diff = s4 - s6, S = fmaxf(s4, s6);
     certain = diff * diff > fmaf(S, fmaf(S, 0x1p-32f, 0x1p-32f), 0x1p-53f);
     bool four = diff < 0.0f;

@@ -135,6 +135,60 @@ def test_argument_errors():
     assert e.value.code == 1
 
 
+def _errors_of_both_scales(x, sg):
+    """FP64 errors of the nearest-rounding codes of blocks x for the scales E4M3(amax / 6 sg) and E4M3(amax / 4 sg)."""
+    grid = np.array([0, 0.5, 1, 1.5, 2, 3, 4, 6])
+    amax = np.abs(x).max(axis=1).astype(np.float64)
+    out = []
+    for div in (6, 4):
+        t = amax / (div * float(sg))
+        ulp = 2.0 ** (np.floor(np.log2(np.maximum(t, 2.0 ** -6))) - 3)
+        d = (np.rint(t / ulp) * ulp * float(sg))[:, None]
+        y = np.abs(x) / d
+        q = grid[np.abs(y[..., None] - grid).argmin(axis=-1)]
+        out.append((((y - q) * d) ** 2).sum(axis=1))
+    return out
+
+
+@pytest.mark.parametrize("sg", [1.0, 1.37, 1.37 * 2.0 ** -47, 1.37 * 2.0 ** -49, 1.37 * 2.0 ** 59, 1.37 * 2.0 ** 61])
+def test_nearly_tied_scales_take_the_order_of_the_definition(sg):
+    """4/6 without the transform: blocks whose two errors agree to a few units in the last place, and exact ties (equal magnitudes,
+    scales with a ratio of 1.5), inside and on both sides of the range in which the kernel decides from rounded sums."""
+    rng = np.random.default_rng(3)
+    sg = np.float32(sg)
+    g = (rng.standard_normal((1 << 16, 16)) * np.exp2(rng.uniform(-2, 9, (1 << 16, 1)))).astype(np.float32) * sg
+    e6, e4 = _errors_of_both_scales(g, sg)
+    close = np.abs(e4 - e6) / np.maximum(e4, e6)
+    g = g[np.argsort(close + (close == 0))[:256]]
+    blocks = [g]
+    for i in (0, 7):
+        step = np.zeros_like(g)
+        step[:, i] = np.abs(g).max(axis=1) * 2.0 ** -6
+        f = lambda x: (lambda a: a[1] - a[0])(_errors_of_both_scales(x, sg))
+        lo, hi = g - step, g + step
+        assert (np.sign(f(lo)) != np.sign(f(hi))).sum() > 50
+        for _ in range(30):                            # bisection in FP32, where the signs differ
+            mid = ((lo.astype(np.float64) + hi) / 2).astype(np.float32)
+            same = (np.sign(f(mid)) == np.sign(f(lo)))[:, None]
+            lo, hi = np.where(same, mid, lo), np.where(same, hi, mid)
+        for ulps in (-3, -1, 0, 1, 3):
+            b = lo.copy()
+            b[:, i] = (b[:, i].view(np.int32) + ulps).view(np.float32)
+            blocks.append(b)
+    one = np.where(rng.random((512, 16)) < 0.5, 0, rng.choice([-1.0, 1.0], (512, 16)))
+    blocks.append((one * rng.uniform(1, 16, (512, 1))).astype(np.float32) * sg)
+    tiny = rng.standard_normal((512, 16)) * np.exp2(rng.uniform(-12, -6, (512, 1)))   # scale bytes in the subnormals, and zero
+    blocks.append(tiny.astype(np.float32) * sg)
+    x = np.concatenate(blocks)
+    x = np.concatenate([x, np.zeros((-len(x) % 1024, 16), np.float32)]).reshape(-1, 128)
+    x[-1, -1] = np.float32(2688.0) * sg                # makes sg the tensor scale
+    c, s, got = _run(x, FP4_FLAG_FOUR_SIX)
+    oc, os_, osg = oracle.quantize(x, four_six=True)
+    assert np.float32(got) == np.float32(osg) == sg
+    assert np.array_equal(s, os_), mismatch_report(s, os_)
+    assert np.array_equal(c, oc), mismatch_report(c, oc)
+
+
 @pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX])
 @pytest.mark.parametrize("shape", [(128, 128), (128, 384), (640, 2432), (128, 56832), (128, 56960)])
 def test_single_launch_quantiser_at_its_limits(shape, flags):
