@@ -104,7 +104,7 @@ typedef struct {
                           per million.  Default 0.99; <= 0 or >= 1 disables the clip.      */
   float eps;           /* X0 = G_c / (||G_c||_F + eps).  Default 1e-7.                     */
   uint32_t flags;      /* FP4_FLAG_*; default 0; unknown bits: FP4_ERR_INVALID_ARG             */
-  uint32_t max_group;  /* fp4_root_ns_batched: at most this many equal-shape matrices run their
+  uint32_t max_group;  /* fp4_root_ns_batched: at most this many matrices run their
                           stages in lockstep as single launches; 0 or more than 16 = 16        */
   uint64_t seed;       /* FP4_FLAG_RHT: seed of the sign draws; default 0                    */
   uint32_t* const* top_hist; /* NULL (default), or a host array with one entry per matrix of the call
@@ -202,9 +202,9 @@ fp4_status fp4_root_ns(const float* G, float* out, int64_t m, int64_t n, int ste
  * One parameter block applies to all (coefficients per matrix when p->a is NaN).
  * ws: device, at least fp4_root_ns_batched_workspace_bytes(...) bytes, 256-byte aligned: one
  *   single-matrix workspace per matrix plus the tables of the grouped launches.
- * Matrices of equal shape (after orientation) are grouped: each Newton-Schulz stage of a
- * group is one launch whose tile list spans all its matrices.  Results are bit-identical to
- * calling fp4_root_ns on each matrix.
+ * Matrices are grouped, those of equal shape (after orientation) first, then groups of different shapes
+ * where they are estimated to be the faster together: each Newton-Schulz stage of a group is one launch whose tile
+ * list spans all its matrices.  Results are bit-identical to calling fp4_root_ns on each matrix.
  * All launches go to `stream` unless FP4_FLAG_OVERLAP_GROUPS is set (see there).
  */
 size_t fp4_root_ns_batched_workspace_bytes(int count, const int64_t* m, const int64_t* n,

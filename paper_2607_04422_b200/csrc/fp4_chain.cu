@@ -51,6 +51,7 @@ constexpr int NTHREADS = (EPI_WARPS + 3) * 32;
 constexpr int DEP_RING = 16;
 constexpr int XBUF = 32 * 64;                 // a warp's 32 x 16 FP32 block: 64-byte rows, 64-byte swizzle
 constexpr int MAX_STAGES = 5;
+constexpr int SHARED_BYTES = 2304;            // of ChainShared
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t SF_COLS = KSTEPS * 8;      // per stage: 4 columns per MMA for each operand
 constexpr uint32_t SF_RING = 2 * SF_COLS;     // copies and MMAs execute in issue order: two stages' columns in turn
@@ -71,7 +72,7 @@ struct ChainLay {
   static constexpr int OFF_X = STAGES * STAGE_BYTES;         // two blocks per epilogue warp
   static constexpr int OFF_OUT = OFF_X + EPI_WARPS * 2 * XBUF;  // two areas, used by alternate tiles
   static constexpr int OFF_BAR = OFF_OUT + 2 * OUT;
-  static constexpr int SMEM = OFF_BAR + 2048 + 1024;
+  static constexpr int SMEM = OFF_BAR + SHARED_BYTES + 1024;
   static_assert(SMEM <= 232448 && STAGE_BYTES % 1024 == 0 && OFF_OUT % 1024 == 0 && OUT % 1024 == 0, "shared memory");
   static_assert(STAGES <= MAX_STAGES && resident_slots(BN, NACC) >= 1, "tensor memory columns");
   // M = 128, N = BN, E2M1 x E2M1, UE4M3 scales, K-major operands
@@ -89,14 +90,17 @@ struct ChainShared {
   float clip[EPI_WARPS][2];                 // threshold and reciprocal norm of the matrix at hand, a copy per epilogue warp
   uint32_t tmem_base, abort_flag;
   uint32_t tiles[2][kChainTiles];  // this block's tiles of a symmetric product / of G3: p << 28 | ti << 16 | tj
+  uint16_t depth[3][kChainTiles];  // their contraction lengths in G1, G2, G3, in blocks of 128
 };
-static_assert(sizeof(ChainShared) <= 2048, "shared block");
+static_assert(sizeof(ChainShared) <= SHARED_BYTES, "shared block");
 
-// Tile t of a product; the symmetric products list the tiles whose 128-column block is on or above the diagonal.
+// Tile t of a product of all matrices; the symmetric products list the tiles whose 128-column block is on or above the diagonal.
 template <int BN>
-__device__ __forceinline__ uint32_t chain_tile(int t, bool sym, int per_problem, int cols) {
-  const int p = t / per_problem;
-  t -= p * per_problem;
+__device__ __forceinline__ uint32_t chain_tile(int t, bool sym, const ChainProblem* probs, int count) {
+  int p = 0;
+  while (p + 1 < count && t >= (sym ? probs[p + 1].first_sym : probs[p + 1].first_full)) ++p;
+  t -= sym ? probs[p].first_sym : probs[p].first_full;
+  const int cols = (sym ? probs[p].s : probs[p].l) / BN;
   int ti, tj;
   if (!sym) {
     ti = t / cols;
@@ -214,11 +218,10 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
   ChainShared* sh = reinterpret_cast<ChainShared*>(smem + L::OFF_BAR);
   volatile uint32_t* abort_flag = &sh->abort_flag;
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  const int nsym = a.nsym, nfull = (a.s / BM) * (a.l / BN);   // tiles per matrix of a symmetric product / of G3
   const int grid = (int)gridDim.x;
   // tiles of this block
-  const int my_sym = (nsym * a.count - (int)blockIdx.x + grid - 1) / grid;
-  const int my_full = (nfull * a.count - (int)blockIdx.x + grid - 1) / grid;
+  const int my_sym = (a.sym_tiles - (int)blockIdx.x + grid - 1) / grid;
+  const int my_full = (a.full_tiles - (int)blockIdx.x + grid - 1) / grid;
   const int products = 3 * a.steps;
   const int first = SYM ? a.first : 0, end = SYM ? a.end : products;
   const bool two_acc = a.nacc == 2;
@@ -234,8 +237,13 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
   }
   for (int i = (int)threadIdx.x - 64; i >= 0 && i < 2 * kChainTiles; i += NTHREADS) {
     const int list = i / kChainTiles, j = i % kChainTiles;
-    if (j < (list ? my_full : my_sym))
-      sh->tiles[list][j] = chain_tile<BN>((int)blockIdx.x + j * grid, list == 0, list ? nfull : nsym, (list ? a.l : a.s) / BN);
+    if (j < (list ? my_full : my_sym)) {
+      const uint32_t tile = chain_tile<BN>((int)blockIdx.x + j * grid, list == 0, pack.p, a.count);
+      const ChainProblem& pr = pack.p[tile >> 28];
+      sh->tiles[list][j] = tile;
+      sh->depth[list ? 2 : 1][j] = (uint16_t)(pr.s / 128);
+      if (!list) sh->depth[0][j] = (uint16_t)(pr.l / 128);
+    }
   }
   for (int i = (int)threadIdx.x; i < a.count * kChainMaps; i += NTHREADS)   // descriptors come first in a problem
     tma_prefetch_desc(reinterpret_cast<const CUtensorMap*>(&pack.p[i / kChainMaps]) + i % kChainMaps);
@@ -256,16 +264,16 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
         const int k = pi / 3, mode = pi - 3 * k + kG1;
         const bool sym = mode != kG3;
         const int mine = sym ? my_sym : my_full;
-        const int K = mode == kG1 ? a.l : a.s;
-        const int num_kb = (K + BK - 1) / BK;
-        // tiles of the matrix's earlier products (SYM: what the launches before have left is complete)
-        const uint32_t need = SYM ? (mode == kG1 ? 0u : (uint32_t)((2 * k + 1) * nsym))
-                                  : (uint32_t)(k * (2 * nsym + nfull) + (mode - kG1) * nsym);
         int seen = -1;
         for (int j = 0; j < mine; ++j, ++n) {
           const uint32_t tile = sh->tiles[sym ? 0 : 1][j];
           const int p = (int)(tile >> 28), ti = (int)(tile >> 16) & 0xFFF, tj = (int)(tile & 0xFFFF);
           const ChainProblem& pr = pack.p[p];
+          const int K = sh->depth[mode - kG1][j] * 128;
+          const int num_kb = (K + BK - 1) / BK;
+          // tiles of the matrix's earlier products (SYM: what the launches before have left is complete)
+          const uint32_t need = SYM ? (mode == kG1 ? 0u : (uint32_t)((2 * k + 1) * pr.nsym))
+                                    : (uint32_t)(k * (2 * pr.nsym + (pr.s / BM) * (pr.l / BN)) + (mode - kG1) * pr.nsym);
           if (p != seen && need != 0) {
             // all tiles of the matrix's earlier products are stored
             bool met = ld_acquire(pr.done) >= need;
@@ -313,9 +321,13 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
         const int mode = pi % 3 + kG1;
         const bool sym = mode != kG3;
         const int mine = sym ? my_sym : my_full;
-        const int K = mode == kG1 ? a.l : a.s;
-        const int num_kb = (K + BK - 1) / BK;
+        int p = 0;
         for (int j = 0; j < mine; ++j, ++n) {
+          // from the block's index and the parameters, which the compiler knows to be uniform, as the descriptors have to be
+          const int t = (int)blockIdx.x + j * grid;
+          while (p + 1 < a.count && t >= (sym ? pack.p[p + 1].first_sym : pack.p[p + 1].first_full)) ++p;
+          const int K = mode == kG1 ? pack.p[p].l : pack.p[p].s;
+          const int num_kb = (K + BK - 1) / BK;
           // scale atoms cover 128 rows of the column operand: an odd 64-column tile uses their upper half
           const uint32_t sfb_shift = BN == 64 ? 2u * (sh->tiles[sym ? 0 : 1][j] & 1u) : 0u;
           const uint32_t ab = two_acc ? n & 1u : 0u;
@@ -353,7 +365,6 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
       const bool sym = mode != kG3;
       const int mine = sym ? my_sym : my_full;
       if (pi == products - 1 && !a.keep) break;
-      const int rq_k = sym ? a.s : a.l;
       for (int j = 0; j < mine; ++j, ++n) {
         const uint32_t tile = sh->tiles[sym ? 0 : 1][j];
         const int p = (int)(tile >> 28), ti = (int)(tile >> 16) & 0xFFF, tj = (int)(tile & 0xFFFF);
@@ -364,8 +375,8 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
         const CUtensorMap* mr = mode == kG1 ? &pr.st_qA : mode == kG2 ? &pr.st_qB : &pr.st_qX;
         const CUtensorMap* mc = mode == kG1 ? &pr.st_qAc : mode == kG2 ? &pr.st_qBc : &pr.st_qXt[(k & 1) ^ 1];
         uint8_t* sym_sf = mode == kG1 ? pr.qa_sf : pr.qb_sf;
-        uint8_t* rsf = (sym ? sym_sf : pr.qx_sf) + ((int64_t)ti * (rq_k / 64) + tj * (BN / 64)) * 512;
-        uint8_t* csf = (sym ? sym_sf : pr.qt_sf[(k & 1) ^ 1]) + ((int64_t)(tj * BN / 128) * (a.s / 64) + ti * 2) * 512;
+        uint8_t* rsf = (sym ? sym_sf : pr.qx_sf) + ((int64_t)ti * ((sym ? pr.s : pr.l) / 64) + tj * (BN / 64)) * 512;
+        uint8_t* csf = (sym ? sym_sf : pr.qt_sf[(k & 1) ^ 1]) + ((int64_t)(tj * BN / 128) * (pr.s / 64) + ti * 2) * 512;
         const int slot = mode == kG1 ? a.ix.amax_A0 + k : a.ix.amax_X0 + k + 1;
         float* maxima = pr.scalars + (slot & ~3);
         uint32_t* done = pr.done;
@@ -499,7 +510,7 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
           if (mode == kG1) {
             const float sgx = ld_scalar(sc + a.ix.sg_X0 + k), ax = ld_scalar(sc + a.ix.amax_X0 + k);
             scale = __fmul_rn(sgx, sgx);
-            bound = fminf(__fmul_rn(__fmul_rn(__fmul_rn(2.0f, a.l_cols), ax), ax), 4.0f);
+            bound = fminf(__fmul_rn(__fmul_rn(__fmul_rn(2.0f, pr.l_cols), ax), ax), 4.0f);
           } else if (mode == kG2) {
             const float sga = ld_scalar(sc + a.ix.sg_A0 + k), aa = ld_scalar(sc + a.ix.amax_A0 + k);
             scale = __fmul_rn(sga, sga);
@@ -706,13 +717,13 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
           bool send = mode == kG1 && (!to_tm || a.keep);
           if (mode == kG3) {
             // the caller's matrix has no padding; X of a tall matrix lies in the workspace and has
-            send = !to_tm && ((y < a.s0 && x0 < a.l0) || (pr.tall && !out_t));
+            send = !to_tm && ((y < pr.s0 && x0 < pr.l0) || (pr.tall && !out_t));
             if (last && a.update && pr.W) {
-              const bool in = y + lane < a.s0 && x0 < a.l0;
+              const bool in = y + lane < pr.s0 && x0 < pr.l0;
               if (pr.tall) {
-                if (in) chain_update_tall(pr.W + (int64_t)x0 * a.s0 + y + lane, a.s0, v, a.upd_decay, a.upd_step);
+                if (in) chain_update_tall(pr.W + (int64_t)x0 * pr.s0 + y + lane, pr.s0, v, a.upd_decay, a.upd_step);
               } else if (in) {
-                uint4* w = reinterpret_cast<uint4*>(pr.W + ((int64_t)y + lane) * a.l0 + x0);
+                uint4* w = reinterpret_cast<uint4*>(pr.W + ((int64_t)y + lane) * pr.l0 + x0);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                   uint4 o = w[h];
@@ -894,64 +905,100 @@ static Residents residents(int bn, int64_t full, int64_t sym) {
 // groups (short sides 128 to 2304, long sides to 32768, 1 to 14 matrices, plain and with the quantiser options): choosing by them
 // loses 0.1 % on average against always knowing the fastest, 3.5 % at worst, and 0.7 % (9 %) at 100 others drawn at random.
 struct TileUs {
-  double product, resident, memory, k1, k2;   // k1, k2: main loop of G1; of G2 and G3
-  TileUs(int bn, int64_t s, int64_t l, bool opts)
+  double product, resident, memory;
+  TileUs(int bn, bool opts)
       : product(bn == 64 ? 4.0 : 5.0), resident((bn == 64 ? 0.65 : 1.0) * (opts ? 1.45 : 1.0)),
-        memory((bn == 64 ? 1.7 : 4.75) * (opts ? 1.45 : 1.0)), k1(0.22 * (double)((l + 255) / 256)), k2(0.26 * (double)((s + 255) / 256)) {}
-  static double tiles(int64_t n, int in_tm, double resident, double memory, double k) {
-    return in_tm * (resident > k ? resident : k) + (double)(n - in_tm) * (memory > k ? memory : k);
+        memory((bn == 64 ? 1.7 : 4.75) * (opts ? 1.45 : 1.0)) {}
+  static double k1(int64_t l) { return 0.22 * (double)((l + 255) / 256); }   // main loop of G1
+  static double k2(int64_t s) { return 0.26 * (double)((s + 255) / 256); }   // of G2 and G3
+};
+// Mean times of a tile of one product, resident or not
+struct MeanTile {
+  double resident = 0.0, memory = 0.0;
+  void add(double share, const TileUs& t, double k) {
+    resident += share * (t.resident > k ? t.resident : k);
+    memory += share * (t.memory > k ? t.memory : k);
   }
+  double tiles(int64_t n, int in_tm) const { return in_tm * resident + (double)(n - in_tm) * memory; }
 };
 // one iteration of a single launch with tiles of bn columns; 0 when a block would take more tiles than its list holds
-static double width_us(int bn, int64_t s, int64_t l, int count, bool opts, int sms) {
-  const int64_t rs = rounds(sym_tiles(s, bn) * count, sms), rf = rounds(s / BM * (l / bn) * count, sms);
+static double width_us(int bn, const WorkShape* w, int count, bool opts, int sms) {
+  int64_t sym = 0, full = 0;
+  for (int j = 0; j < count; ++j) { sym += sym_tiles(w[j].s, bn); full += w[j].s / BM * (w[j].l / bn); }
+  const int64_t rs = rounds(sym, sms), rf = rounds(full, sms);
   if (rf > kChainTiles) return 0.0;
   const Residents r = residents(bn, rf, rs);
-  const TileUs t(bn, s, l, opts);
-  return 3 * t.product + t.tiles(rs, r.na, t.resident, t.memory, t.k1) + t.tiles(rs, r.na, t.resident, t.memory, t.k2) +
-         t.tiles(rf, r.nx, t.resident, t.memory, t.k2);
+  const TileUs t(bn, opts);
+  MeanTile g1, g2, g3;
+  for (int j = 0; j < count; ++j) {
+    const double share = (double)sym_tiles(w[j].s, bn) / (double)sym;
+    g1.add(share, t, TileUs::k1(w[j].l));
+    g2.add(share, t, TileUs::k2(w[j].s));
+    g3.add((double)(w[j].s / BM * (w[j].l / bn)) / (double)full, t, TileUs::k2(w[j].s));
+  }
+  return 3 * t.product + g1.tiles(rs, r.na) + g2.tiles(rs, r.na) + g3.tiles(rf, r.nx);
 }
 // The width of a single launch's tiles.  Measured, 5 iterations, 64 / 128 columns: 256 x 512 83 / 101 us, 1024 x 4096 159 / 185 (with the
 // quantiser options 200 / 243), 8 x 768 x 768 155 / 179, 1152 x 8192 290 / 324, 1536 x 1536 148 / 139, 1536 x 2816 196 / 188,
 // 2048 x 2048 210 / 196 (250 / 249).
-static bool narrow_tiles(int64_t s, int64_t l, int count, bool opts, int sms) {
-  const double n = width_us(64, s, l, count, opts, sms), w = width_us(128, s, l, count, opts, sms);
-  return n > 0.0 && n <= w;
+static bool narrow_tiles(const WorkShape* w, int count, bool opts, int sms) {
+  const double narrow = width_us(64, w, count, opts, sms), wide = width_us(128, w, count, opts, sms);
+  return narrow > 0.0 && narrow <= wide;
 }
-double chain_iteration_us(int64_t s, int64_t l, int count, bool opts, int sms) {
-  return width_us(narrow_tiles(s, l, count, opts, sms) ? 64 : 128, s, l, count, opts, sms);
+double chain_iteration_us(const WorkShape* w, int count, bool opts, int sms) {
+  return width_us(narrow_tiles(w, count, opts, sms) ? 64 : 128, w, count, opts, sms);
 }
 // G1 and G2 of an iteration in a launch of their own, where every SM has at most one tile (else 0)
-double chain_symmetric_us(int64_t s, int64_t l, int count, bool opts, int sms) {
-  if (sym_tiles(s, 128) * count > sms) return 0.0;
-  const TileUs t(128, s, l, opts);
-  return 12.5 + t.tiles(1, 1, t.resident, t.memory, t.k1) + t.tiles(1, 1, t.resident, t.memory, t.k2);
+double chain_symmetric_us(const WorkShape* w, int count, bool opts, int sms) {
+  int64_t sym = 0, s = 0, l = 0;
+  for (int j = 0; j < count; ++j) {
+    sym += sym_tiles(w[j].s, 128);
+    s = w[j].s > s ? w[j].s : s;
+    l = w[j].l > l ? w[j].l : l;
+  }
+  if (sym > sms) return 0.0;
+  const TileUs t(128, opts);
+  const double k1 = TileUs::k1(l), k2 = TileUs::k2(s);
+  return 12.5 + (t.resident > k1 ? t.resident : k1) + (t.resident > k2 ? t.resident : k2);
 }
 
-cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st) {
+// Places of the matrices in the launch's tile lists
+static void place_tiles(ChainPack& pack, ChainLaunch& a, int bn) {
+  a.sym_tiles = a.full_tiles = 0;
+  for (int j = 0; j < a.count; ++j) {
+    ChainProblem& pr = pack.p[j];
+    pr.nsym = (int)sym_tiles(pr.s, bn);
+    pr.first_sym = a.sym_tiles;
+    pr.first_full = a.full_tiles;
+    a.sym_tiles += pr.nsym;
+    a.full_tiles += pr.s / BM * (pr.l / bn);
+  }
+}
+
+cudaError_t launch_chain(ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st) {
   if (launch.count < 1 || launch.count > kChainMax || launch.steps < 1) return cudaErrorInvalidValue;
   ChainLaunch a = launch;
   const bool pf = a.q.rht || a.q.four_six;
-  const bool narrow = narrow_tiles(a.s, a.l, a.count, pf, sms);
+  WorkShape w[kChainMax];
+  for (int j = 0; j < a.count; ++j) w[j] = {pack.p[j].s, pack.p[j].l};
+  const bool narrow = narrow_tiles(w, a.count, pf, sms);
   const int bn = narrow ? 64 : 128;
-  a.nsym = (int)sym_tiles(a.s, bn);
-  const int64_t widest = (int64_t)(a.s / BM) * (a.l / bn) * a.count;
-  const int grid = (int)(widest < sms ? widest : sms);
-  const Residents r = residents(bn, rounds(widest, grid), rounds((int64_t)a.nsym * a.count, grid));
+  place_tiles(pack, a, bn);
+  const int grid = a.full_tiles < sms ? a.full_tiles : sms;
+  const Residents r = residents(bn, rounds(a.full_tiles, grid), rounds(a.sym_tiles, grid));
   a.nacc = r.nacc; a.na = r.na; a.nx = r.nx;
   if (narrow) return pf ? launch_one<64, true>(pack, a, grid, st) : launch_one<64, false>(pack, a, grid, st);
   return pf ? launch_one<128, true>(pack, a, grid, st) : launch_one<128, false>(pack, a, grid, st);
 }
 
 // G1 and G2 of iteration `step` in one launch with a 128 x 128 tile per SM.
-cudaError_t launch_chain_symmetric(const ChainPack& pack, const ChainLaunch& launch, int step, int sms, cudaStream_t st) {
+cudaError_t launch_chain_symmetric(ChainPack& pack, const ChainLaunch& launch, int step, int sms, cudaStream_t st) {
   if (launch.count < 1 || launch.count > kChainMax || launch.steps < 1) return cudaErrorInvalidValue;
   ChainLaunch a = launch;
-  a.nsym = (int)sym_tiles(a.s, 128);
+  place_tiles(pack, a, 128);
   a.first = 3 * step; a.end = a.first + 2;
-  const int64_t widest = (int64_t)a.nsym * a.count;
-  if (widest > sms) return cudaErrorInvalidValue;
-  const int grid = (int)widest;
+  if (a.sym_tiles > sms) return cudaErrorInvalidValue;
+  const int grid = a.sym_tiles;
   const Residents r = residents(128, 0, 1);
   a.nacc = r.nacc; a.na = r.na; a.nx = r.nx;
   return a.q.rht || a.q.four_six ? launch_one<128, true, true>(pack, a, grid, st) : launch_one<128, false, true>(pack, a, grid, st);

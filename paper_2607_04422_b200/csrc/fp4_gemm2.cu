@@ -292,12 +292,9 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
   const bool leader = (rank == 0);
   const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
   const GemmProblem* probs = pack.p;
-  // args.tiles_m / tiles_n count 256 x 256 tiles here
   // only the two symmetric products are ever launched with triangle tiles: a compile-time fact for the others
   const bool sym = (MODE == kG1 || MODE == kG2) && args.symmetric != 0;
-  const int tiles_per_problem = sym ? args.tiles_n * (args.tiles_n + 1) / 2 : args.tiles_m * args.tiles_n;
-  const int num_tiles = tiles_per_problem * args.num_problems;
-  const int num_kb = (args.K + BK - 1) / BK;
+  const int num_tiles = args.num_tiles;
   constexpr bool HAS_AUX = (MODE == kG2 || MODE == kG3);
   constexpr bool STORE_F32 = (MODE == kPlain || MODE == kG1 || MODE == kG3);
   const bool do_q = (MODE != kPlain) && !UPD && args.write_q;  // the update variant is launched without quantised outputs
@@ -342,10 +339,11 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
     if (MODE == kG3) tma_load_2d_pair_hint(dst, map, x, y, bar, keep);            \
     else tma_load_2d_pair(dst, map, x, y, bar);                                   \
   } while (0)
+      int p = 0, ti, tj;
       for (int t = pair; t < (dry ? min(num_tiles, pair + 1) : num_tiles); t += num_pairs) {
-        int p, ti, tj;
-        decode_tile(t, args, tiles_per_problem, p, ti, tj, sym);
+        decode_tile(t, probs, args.num_problems, p, ti, tj, sym);
         const GemmProblem* pr = probs + p;
+        const int num_kb = (pr->K + BK - 1) / BK;
         const int arow = ti * PM + (int)rank * BM;   // this CTA's rows of the row operand
         const int brow = tj * PN + (int)rank * BM;   // this CTA's half of the column operand
         for (int kb = 0; kb < (dry ? min(num_kb, STAGES) : num_kb); ++kb) {
@@ -366,8 +364,10 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA only)
     if (leader && elect_one()) {
-      int st = 0; uint32_t ph = 0, seq = 0;
+      int st = 0, p = 0; uint32_t ph = 0, seq = 0;
       for (int t = pair; t < num_tiles; t += num_pairs, ++seq) {
+        while (p + 1 < args.num_problems && t >= probs[p + 1].first_tile) ++p;
+        const int K = probs[p].K, num_kb = (K + BK - 1) / BK;
         const uint32_t par = seq & 1, buse = seq >> 1;
         // this buffer's previous tile is drained, and so are the columns it shares with the
         // buffer of the tile before this one
@@ -382,7 +382,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
           const uint8_t* sf = smem + OFF_SF + st * SF_BYTES;
           const uint64_t adesc = umma_desc(smem_u32(smem + OFF_A + st * OPER_BYTES), OPER_SBO, OPER_SWIZZLE);
           const uint64_t bdesc = umma_desc(smem_u32(smem + OFF_B + st * OPER_BYTES), OPER_SBO, OPER_SWIZZLE);
-          const bool half_stage = (kb + 1) * BK > args.K;   // K is a multiple of 128
+          const bool half_stage = (kb + 1) * BK > K;   // K is a multiple of 128
 #pragma unroll
           for (int k = 0; k < KSTEPS; ++k) {
             if (k == KSTEPS / 2 && half_stage) break;
@@ -403,25 +403,25 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
     // off: column-quantised codes by TMA (64-byte rows), the two kinds of scale bytes as whole atoms.
     if (do_q && elect_one()) {
       uint32_t seq = 0;
+      int p = 0, ti, tj;
       for (int t = pair; t < num_tiles; t += num_pairs, ++seq) {
-        int p, ti, tj;
-        decode_tile(t, args, tiles_per_problem, p, ti, tj, sym);
+        decode_tile(t, probs, args.num_problems, p, ti, tj, sym);
         const GemmProblem* pr = probs + p;
         const int bi = ti * 2 + (int)rank;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int hcol = (seq & 1) ? h : 1 - h;          // which 128 columns of the tile this half holds
           const int bj = tj * 2 + hcol;
-          const bool below = (sym && bj < bi) || bi >= args.blocks_m || bj >= args.blocks_n;
+          const bool below = (sym && bj < bi) || bi >= pr->blocks_m || bj >= pr->blocks_n;
           const bool mirror = !below && (MODE == kG3 || (sym && bi != bj));
           wait_or_abort(&bars->half_done[h], seq & 1, abort_flag);
           if (!below) {
             const uint32_t st = smem_u32(smem + OFF_HALF + h * HALF_AREA);
-            bulk_store_s(pr->rq_sf + ((int64_t)bi * (args.rq_K >> 6) + bj * 2) * 512, st + HALF_CQ_BYTES + HALF_SF_BYTES,
+            bulk_store_s(pr->rq_sf + ((int64_t)bi * (pr->blocks_n * 2) + bj * 2) * 512, st + HALF_CQ_BYTES + HALF_SF_BYTES,
                          HALF_SF_BYTES);
             if (mirror) {
               tma_store_2d_s(&pr->tmCq, bi * (BM / 2), bj * 128, st);
-              bulk_store_s(pr->cq_sf + ((int64_t)bj * (args.cq_K >> 6) + bi * 2) * 512, st + HALF_CQ_BYTES, HALF_SF_BYTES);
+              bulk_store_s(pr->cq_sf + ((int64_t)bj * (pr->blocks_m * 2) + bi * 2) * 512, st + HALF_CQ_BYTES, HALF_SF_BYTES);
             }
           }
         }
@@ -502,9 +502,10 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
     };
     // geometry of a tile for this warp
     struct Geo { int p, ti, tj, x64, y32; bool below; };
-    auto geometry = [&](int t, uint32_t seq_) {
+    auto geometry = [&](int t, int p_, uint32_t seq_) {
       Geo q;
-      decode_tile(t, args, tiles_per_problem, q.p, q.ti, q.tj, sym);
+      q.p = p_;
+      decode_tile(t, probs, args.num_problems, q.p, q.ti, q.tj, sym);
       const int cgx = (seq_ & 1) ? team : TEAMS - 1 - team;       // column group: mirrored on buffer 0
       const int bi_ = q.ti * 2 + (int)rank;
       q.x64 = q.tj * PN + cgx * (TEAM_CHUNKS * CHUNK);
@@ -513,7 +514,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
       // A redundant block of a diagonal tile, or one outside the matrix.  (Blocks outside run through G3's epilogue as
       // zeros and TMA drops what they store: the path that skips a block costs G3 registers, 9 % of its time with
       // BF16 storage.)
-      q.below = sym && (bj_ < bi_ || bi_ >= args.blocks_m || bj_ >= args.blocks_n);
+      q.below = sym && (bj_ < bi_ || bi_ >= probs[q.p].blocks_m || bj_ >= probs[q.p].blocks_n);
       return q;
     };
 
@@ -521,7 +522,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
     int t = pair;
     Geo cur;
     if (t < num_tiles) {
-      cur = geometry(t, 0);
+      cur = geometry(t, 0, 0);
       if (HAS_AUX) {
         // chunk position e of slot i: i on buffer 1, 3 - i on buffer 0 (seq = 0 uses buffer 0)
         fetch(probs + cur.p, cur.x64, cur.y32, 3, cur.below, 0);
@@ -535,7 +536,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
       // the next tile of this pair: its first two blocks are fetched during this tile's last two chunks
       const bool has_next = t + num_pairs < num_tiles;
       Geo nxt = cur;
-      if (has_next) nxt = geometry(t + num_pairs, seq + 1);
+      if (has_next) nxt = geometry(t + num_pairs, p, seq + 1);
       if (p != cur_p) {
         if ((MODE == kG1 || MODE == kG3) && cur_p >= 0) {
 #pragma unroll
@@ -549,7 +550,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
         cur_p = p;
         pr = probs + p;
         epilogue_scalars<MODE>(*pr, args, scale, sg_out,
-                               leader && t == p * tiles_per_problem && threadIdx.x == ROLE_WARPS * 32);
+                               leader && t == pr->first_tile && threadIdx.x == ROLE_WARPS * 32);
         inv_sg = __frcp_rn(sg_out);  // exact: the predicted scales are powers of two
         ca = pr->ca; cb = pr->cb; cc = pr->cc;
         // a power-of-two scale (every tensor scale produced inside the loop is one) multiplies exactly
@@ -877,10 +878,8 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
 
 template <int MODE, bool PF, bool BH, bool UPD, bool DEEP>
 cudaError_t launch_pair_variant(const ProblemPack& pack, const GemmLaunch& L, int sms, cudaStream_t st) {
-  const int tpp = L.symmetric ? L.tiles_n * (L.tiles_n + 1) / 2 : L.tiles_m * L.tiles_n;
-  const int num_tiles = tpp * L.num_problems;
   int pairs = sms > 1 ? sms / 2 : 1;
-  if (pairs > num_tiles) pairs = num_tiles;
+  if (pairs > L.num_tiles) pairs = L.num_tiles;
   count_launches(1);
   launch_chained(k_gemm_pair<MODE, PF, BH, UPD, DEEP>, dim3(2 * pairs), dim3(NTHREADS), Lay<MODE, DEEP>::SMEM_BYTES, st, pack, L);
   return cudaGetLastError();
@@ -898,9 +897,11 @@ cudaError_t launch_pair_variant(const ProblemPack& pack, const GemmLaunch& L, in
 template <int MODE, bool PF, bool BH, bool UPD = false>
 cudaError_t launch_pair_mode(const ProblemPack& pack, const GemmLaunch& L, int sms, cudaStream_t st) {
   if constexpr (MODE == kG2 || MODE == kG3) {
-    const int tiles = (L.symmetric ? L.tiles_n * (L.tiles_n + 1) / 2 : L.tiles_m * L.tiles_n) * L.num_problems;
-    const int from = MODE == kG2 ? (PF ? 4096 : 2816) : PF ? 5120 : tiles >= 1536 ? 2816 : 4096;
-    if (L.K >= from) return launch_pair_variant<MODE, PF, BH, UPD, true>(pack, L, sms, st);
+    const int from = MODE == kG2 ? (PF ? 4096 : 2816) : PF ? 5120 : L.num_tiles >= 1536 ? 2816 : 4096;
+    int deep = 0;   // tiles of matrices that gain
+    for (int j = 0; j < L.num_problems; ++j)
+      if (pack.p[j].K >= from) deep += (j + 1 < L.num_problems ? pack.p[j + 1].first_tile : L.num_tiles) - pack.p[j].first_tile;
+    if (2 * deep >= L.num_tiles) return launch_pair_variant<MODE, PF, BH, UPD, true>(pack, L, sms, st);
   }
   return launch_pair_variant<MODE, PF, BH, UPD, false>(pack, L, sms, st);
 }
@@ -945,21 +946,22 @@ int gemm_pair_stage_k(GemmMode mode) {
   }
 }
 
-// `launch` carries tile counts in 128-blocks; M, N and K are multiples of 128.
-cudaError_t launch_gemm_pair(GemmMode mode, const ProblemPack& pack, const GemmLaunch& launch, int sms,
-                             cudaStream_t st) {
-  if (launch.K % 128) return cudaErrorInvalidValue;
+cudaError_t launch_gemm_pair(GemmMode mode, ProblemPack& pack, const GemmLaunch& launch, int sms, cudaStream_t st) {
   if (launch.num_problems < 1 || launch.num_problems > kPackMax) return cudaErrorInvalidValue;
   GemmLaunch L = launch;
-  L.blocks_m = launch.tiles_m;
-  L.blocks_n = launch.tiles_n;
-  L.tiles_m = (launch.tiles_m + 1) / 2;
-  L.tiles_n = (launch.tiles_n + 1) / 2;
-  // Row order reads the whole column operand once per row of tiles, which is cheap as long as it stays in the L2 (126 MB, shared
-  // with the streaming FP32 tile); beyond that, bands of 8 rows keep the 74 tiles in flight near a square.  Measured, 5
-  // iterations, row order / bands: 16384 x 16384 24.9 / 21.1 ms, 12288 x 12288 10.9 / 10.0, 8192 x 16384 6.3 / 5.75, 8192 x 8192
-  // (a column operand of 32 MB) 3.45 / 3.36, 6144 x 6144 (18 MB) 1.68 / 1.73.  Bands of 6 and 12 rows: +1 %.
-  L.band = (int64_t)L.blocks_n * 128 * L.K / 2 >= (int64_t)32 << 20 ? 8 : 1;
+  L.num_tiles = 0;
+  for (int j = 0; j < launch.num_problems; ++j) {
+    GemmProblem& pr = pack.p[j];
+    if (pr.K % 128) return cudaErrorInvalidValue;
+    const int tiles_m = (pr.blocks_m + 1) / 2, tiles_n = (pr.blocks_n + 1) / 2;
+    pr.first_tile = L.num_tiles;
+    L.num_tiles += L.symmetric ? tiles_n * (tiles_n + 1) / 2 : tiles_m * tiles_n;
+    // Row order reads the whole column operand once per row of tiles, which is cheap as long as it stays in the L2 (126 MB, shared
+    // with the streaming FP32 tile); beyond that, bands of 8 rows keep the 74 tiles in flight near a square.  Measured, 5
+    // iterations, row order / bands: 16384 x 16384 24.9 / 21.1 ms, 12288 x 12288 10.9 / 10.0, 8192 x 16384 6.3 / 5.75, 8192 x 8192
+    // (a column operand of 32 MB) 3.45 / 3.36, 6144 x 6144 (18 MB) 1.68 / 1.73.  Bands of 6 and 12 rows: +1 %.
+    pr.band = (int64_t)pr.blocks_n * 128 * pr.K / 2 >= (int64_t)32 << 20 ? 8 : 1;
+  }
   const bool pf = launch.q.rht || launch.q.four_six;
   const bool bh = launch.aux_h != 0 || launch.out_h != 0;
 #define FP4_PAIR_CASE(M)                                                                \

@@ -73,17 +73,17 @@ __device__ __forceinline__ void grid_barrier(uint32_t* counter, uint32_t want, v
   __syncthreads();
 }
 
-// tile index of a launch -> (problem, tile row, tile column): bands of L.band tile rows, each walked column by column
-// (only the tiles on and above the diagonal of a symmetric product); a band of one row is plain row order
-__device__ __forceinline__ void decode_tile(int t, const GemmLaunch& L, int tiles_per_problem, int& p, int& ti,
-                                            int& tj, bool sym) {
-  p = t / tiles_per_problem;
-  t -= p * tiles_per_problem;
-  const int tiles_n = L.tiles_n, band = L.band;
+// tile index of a launch -> (problem, tile row, tile column): bands of `band` tile rows, each walked column by column
+// (only the tiles on and above the diagonal of a symmetric product); a band of one row is plain row order.  p comes in as a
+// problem at or before the tile's (a thread's tiles are in ascending order).
+__device__ __forceinline__ void decode_tile(int t, const GemmProblem* probs, int num_problems, int& p, int& ti, int& tj, bool sym) {
+  while (p + 1 < num_problems && t >= probs[p + 1].first_tile) ++p;
+  t -= probs[p].first_tile;
+  const int tiles_n = (probs[p].blocks_n + 1) >> 1, band = probs[p].band;
   if (!sym) {
     const int b = t / (band * tiles_n);
     t -= b * band * tiles_n;
-    const int h = min(band, L.tiles_m - b * band);   // the last band may be lower
+    const int h = min(band, ((probs[p].blocks_m + 1) >> 1) - b * band);   // the last band may be lower
     tj = t / h;
     ti = b * band + (t - tj * h);
   } else {
@@ -123,7 +123,7 @@ __device__ __forceinline__ void epilogue_scalars(const GemmProblem& pr, const Ge
     const float sgx = sc[args.ix.sg_X0 + args.iter];
     const float ax = sc[args.ix.amax_X0 + args.iter];
     scale = __fmul_rn(sgx, sgx);
-    float bound = __fmul_rn(__fmul_rn(__fmul_rn(2.0f, args.l_cols), ax), ax);
+    float bound = __fmul_rn(__fmul_rn(__fmul_rn(2.0f, pr.l_cols), ax), ax);
     sg_out = scale_predicted(__fmul_rn(args.q.widen, fminf(bound, 4.0f)));
     if (publish) sc[args.ix.sg_A0 + args.iter] = sg_out;
   } else if (MODE == kG2) {

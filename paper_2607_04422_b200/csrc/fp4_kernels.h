@@ -64,8 +64,7 @@ enum GemmMode : int {
   kG3 = 3      // P = qB qXt^T; X+ = aX + P; store X+, emit qX+, qXt+, track amax(X+)
 };
 
-// One matrix product of a launch.  A launch runs the same stage for a group of matrices
-// of one shape.
+// One matrix product of a launch.  A launch runs the same stage for a group of matrices.
 struct alignas(64) GemmProblem {
   CUtensorMap tmA, tmB;      // NVFP4 codes of the row and the column operand
   CUtensorMap tmAux, tmOut;  // FP32 tile combined in the epilogue / FP32 result (box: 16 columns x 32 rows, one
@@ -85,8 +84,12 @@ struct alignas(64) GemmProblem {
   int aux_tr;                // kG3: tmAux maps a matrix stored as the transpose of the tile grid (box = 32 x 16)
   int out_tr;                // kG3: so does tmOut (the caller's result of a tall input)
   int out_rows, out_cols;    // extent of the matrix behind tmOut (chunks that start outside it are not stored)
+  int K;                     // contraction length in elements (multiple of 128)
   uint16_t* W;               // kG3 with launch.update: the BF16 parameter (same shape and orientation as the
   int64_t W_ld;              //   result, row-major, leading dimension in elements) updated with the result; or null
+  int blocks_m, blocks_n;    // extent of the product in blocks of 128 (row lengths of the two quantised outputs: blocks_n, blocks_m)
+  float l_cols;              // (float) l, for the bound on amax(A)
+  int first_tile, band;      // set by launch_gemm_pair: place in the launch's tile list, tile rows per band of the tile order
 };
 
 // The problems of one launch travel as a kernel parameter (descriptors in parameter space need no
@@ -98,15 +101,10 @@ static_assert(sizeof(ProblemPack) + 256 <= 32764, "kernel parameter space");
 // What all problems of a launch share.
 struct GemmLaunch {
   int num_problems;
-  int K;               // contraction length in elements (multiple of 128)
-  int tiles_m, tiles_n;        // callers: in blocks of 128; inside the kernel: 256 x 256 tiles, rounded up
-  int blocks_m, blocks_n;      // extent in blocks of 128 (set by launch_gemm_pair)
-  int band;            // tile rows per band of the tile order (set by launch_gemm_pair)
+  int num_tiles;       // 256 x 256 tiles of all problems (set by launch_gemm_pair)
   int symmetric;       // only tiles with tile_n >= tile_m; mirrored quantised output
   int iter;            // Newton-Schulz iteration index k
   int write_q;         // emit the quantised outputs
-  int rq_K, cq_K;      // row lengths (elements) of the two quantised outputs
-  float l_cols;        // (float) l, for the bound on amax(A)
   QuantOpts q;         // how this stage's output is quantised (q.widen = 1 in the base mode)
   int clip;            // kG3 on a problem with aux_raw: whether tau applies
   int aux_h;           // the combined tile is read from tmH (BF16)
@@ -133,6 +131,9 @@ struct alignas(64) ChainProblem {
   uint8_t *qx_sf, *qt_sf[2], *qa_sf, *qb_sf;
   float ca, cb, cc;
   int tall;
+  int s, l, s0, l0;          // work shape, the caller's short and long side
+  float l_cols;              // (float) l
+  int nsym, first_sym, first_full;   // set by the launch: tiles of a symmetric product, places in the launch's tile lists
 };
 constexpr int kChainMaps = 16;   // tensor maps at the start of a ChainProblem
 constexpr int kChainMax = 14;    // matrices of a launch
@@ -140,15 +141,13 @@ constexpr int kChainTiles = 32;  // tiles of one product that a block takes at m
 struct ChainPack { ChainProblem p[kChainMax]; };
 struct ChainLaunch {
   int count, steps;
-  int s, l, s0, l0;          // work shape, the caller's short and long side
   int first, end;            // launch_chain_symmetric: its products
-  int nsym;                  // tiles per matrix of a symmetric product (set by the launch)
+  int sym_tiles, full_tiles; // of all matrices, of a symmetric product and of G3 (set by the launch)
   int nacc, nx, na;          // accumulator buffers; a block's first tiles of X and of A that stay in its tensor memory (set by the launch)
   int clip, keep, bf16;
   int tall;                  // one of the matrices at least is tall
   int update, no_out;
   float upd_decay, upd_step;
-  float l_cols;
   QuantOpts q;               // mask unused: drawn per product from seed
   uint64_t seed;
   NsScalarIdx ix;
@@ -164,10 +163,13 @@ __host__ __device__ inline uint32_t rht_signs(uint64_t seed, uint64_t j) {
   return (uint32_t)(z & 0xFFFFu);
 }
 cudaError_t chain_set_attributes();
-double chain_iteration_us(int64_t s, int64_t l, int count, bool opts, int sms);
-double chain_symmetric_us(int64_t s, int64_t l, int count, bool opts, int sms);
-cudaError_t launch_chain(const ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st);
-cudaError_t launch_chain_symmetric(const ChainPack& pack, const ChainLaunch& launch, int step, int sms, cudaStream_t st);
+// Work shapes of the matrices of a launch
+struct WorkShape { int64_t s, l; };
+double chain_iteration_us(const WorkShape* shapes, int count, bool opts, int sms);
+double prologue_us(const WorkShape* shapes, int count, int device_sms, int coop_sms);
+double chain_symmetric_us(const WorkShape* shapes, int count, bool opts, int sms);
+cudaError_t launch_chain(ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st);
+cudaError_t launch_chain_symmetric(ChainPack& pack, const ChainLaunch& launch, int step, int sms, cudaStream_t st);
 
 // Measurement support: counts kernel launches and, when profiling is on, brackets a group of
 // launches with events.
@@ -235,7 +237,7 @@ struct PrologueItem {
   uint32_t* hist_top;      // the caller's histogram of the top 13 magnitude bits of G, or null
   const CUtensorMap* tmG;  // G as an FP32 tensor: box = 32 columns x 128 rows, 128-byte swizzle
 };
-// count matrices that share the shape (s, l) and the clip / eps parameters; sms: those the stream's kernels can occupy, coop_sms:
+// count matrices that share the clip / eps parameters; sms: those the stream's kernels can occupy, coop_sms:
 // those a cooperative launch may count on
 cudaError_t launch_prologue_group(const PrologueItem* items, int count, int write_q, const QuantOpts& q,
                                   uint32_t* status, int coop_sms, int sms, cudaStream_t st);
@@ -258,9 +260,8 @@ cudaError_t launch_param_update(const float* O, int64_t n, const ParamUpdate& up
 cudaError_t prologue_set_attributes();
 
 cudaError_t gemm_pair_set_attributes();
-// pack: the launch.num_problems (<= kPackMax) problems of the launch
-cudaError_t launch_gemm_pair(GemmMode mode, const ProblemPack& pack, const GemmLaunch& launch, int sms,
-                             cudaStream_t st);
+// pack: the launch.num_problems (<= kPackMax) problems of the launch; their places in its tile list are filled in
+cudaError_t launch_gemm_pair(GemmMode mode, ProblemPack& pack, const GemmLaunch& launch, int sms, cudaStream_t st);
 int gemm_pair_stage_k(GemmMode mode);  // the same for a mode of the CTA-pair kernel
 
 }  // namespace fp4

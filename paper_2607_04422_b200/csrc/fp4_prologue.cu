@@ -1,4 +1,4 @@
-// Prologue of the Root step for a group of equal-size matrices (Section 3.4: "p99 outlier
+// Prologue of the Root step for a group of matrices (Section 3.4: "p99 outlier
 // clipping"; normalisation; the first operand copies qX = Q_1x16(X), qX^{16x1} = Q_16x1(X)).
 // Every kernel covers the whole group (gridDim.y = matrix, or a tile list over all matrices), so a
 // group needs six launches instead of six per matrix; a group that fits the shared memories of all SMs
@@ -41,20 +41,23 @@ struct PrepMatrix {
   int tall;
   int clear_status;
   int store_x;
-  int64_t x_rows, x_cols;  // extent and row pitch of X
+  int x_rows, x_cols;  // extent and row pitch of X
+  int s, l;            // work shape (multiples of 128)
+  int s0, l0;          // the caller's short and long side; the rest of the work shape is zero padding
+  int64_t n4;          // elements of the caller's matrix / 4
+  uint32_t clip_rank;
+  uint32_t cand_cap;
+  int tiles, first_tile;   // 128 x 128 tiles, place in the launch's tile list
+  int tiled;           // the sum of squares is taken tile by tile (see kp_compact_stats)
+  int hist_blocks, stat_blocks, select_blocks;   // thread blocks of the passes
 };
 
 struct PrepGroup {
   PrepMatrix mat[kMaxPack];
   int count;
-  int64_t n4;          // elements of the caller's matrix / 4
-  int64_t s, l;        // work shape (multiples of 128)
-  int64_t s0, l0;      // the caller's short and long side; the rest of the work shape is zero padding
+  int tiles;           // of all matrices
   int clip;
-  uint32_t clip_rank;
-  uint32_t cand_cap;
   float eps;
-  int stat_blocks;
   int write_q;
   int zero_words;      // 32-bit words of header + scalars + histogram to clear
   QuantOpts q;         // quantiser options of X0's operand copies
@@ -76,7 +79,7 @@ __global__ void __launch_bounds__(256) kp_init(const __grid_constant__ PrepGroup
   // the select starts with an empty prefix and the wanted rank (written instead of the zero)
   const int rank_word = (int)(offsetof(NsHeader, sel_rank) / 4);
   for (int i = first + blockIdx.x * blockDim.x + threadIdx.x; i < g.zero_words; i += gridDim.x * blockDim.x)
-    w[i] = (i == rank_word) ? g.clip_rank : 0u;
+    w[i] = (i == rank_word) ? m.clip_rank : 0u;
 }
 
 constexpr int kTopBits = 13;                 // bits of the first radix pass
@@ -158,13 +161,13 @@ __global__ void __launch_bounds__(512) kp_hist_top(const __grid_constant__ PrepG
   pdl_wait();
   __shared__ uint32_t sh[kTopBins];
   const PrepMatrix& m = g.mat[blockIdx.y];
-  if (m.hist_top) return;  // the caller counted this matrix already
+  if (m.hist_top || (int)blockIdx.x >= m.hist_blocks) return;  // the caller counted this matrix already; a smaller matrix
   for (int i = threadIdx.x; i < kTopBins; i += blockDim.x) sh[i] = 0;
   __syncthreads();
   const float4* src = reinterpret_cast<const float4*>(m.G);
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t stride = (int64_t)m.hist_blocks * blockDim.x;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  for (; i + stride < g.n4; i += 2 * stride) {
+  for (; i + stride < m.n4; i += 2 * stride) {
     const float4 v = __ldg(src + i), w = __ldg(src + i + stride);
     atomicAdd(&sh[mag_bits(v.x) >> kTopShift], 1u);
     atomicAdd(&sh[mag_bits(v.y) >> kTopShift], 1u);
@@ -175,7 +178,7 @@ __global__ void __launch_bounds__(512) kp_hist_top(const __grid_constant__ PrepG
     atomicAdd(&sh[mag_bits(w.z) >> kTopShift], 1u);
     atomicAdd(&sh[mag_bits(w.w) >> kTopShift], 1u);
   }
-  for (; i < g.n4; i += stride) {
+  for (; i < m.n4; i += stride) {
     const float4 v = __ldg(src + i);
     atomicAdd(&sh[mag_bits(v.x) >> kTopShift], 1u);
     atomicAdd(&sh[mag_bits(v.y) >> kTopShift], 1u);
@@ -216,6 +219,7 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
   __shared__ uint32_t s_sub[kSubBins];
   __shared__ uint32_t s_cnt, s_base;
   const PrepMatrix& m = g.mat[blockIdx.y];
+  if ((m.tiled != 0) != TILED || (int)blockIdx.x >= m.stat_blocks) return;
   const uint32_t bin = g.clip ? (m.hdr->sel_prefix >> kTopShift) : 0xFFFFFFFFu;
   const float4* src = reinterpret_cast<const float4*>(m.G);
   const int lane = threadIdx.x & 31;
@@ -236,7 +240,7 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
         s_buf[pos] = k;
       } else {
         const uint32_t gpos = atomicAdd(&m.hdr->cand_count, 1u);
-        if (gpos < g.cand_cap) m.cand[gpos] = k;
+        if (gpos < m.cand_cap) m.cand[gpos] = k;
         atomicAdd(&s_sub[(k >> 9) & (kSubBins - 1)], 1u);   // (in global memory: 14.1 ms for an all-zero 4096 x 4096)
       }
     }
@@ -245,8 +249,8 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
   __shared__ float wm[8];
   const int warp = threadIdx.x >> 5;
   if (TILED) {
-    const int rows = (int)(m.tall ? g.l0 : g.s0), cols = (int)(m.tall ? g.s0 : g.l0);
-    const int tiles_x = (int)((m.tall ? g.s : g.l) >> 7), ty = (int)blockIdx.x / tiles_x;
+    const int rows = (m.tall ? m.l0 : m.s0), cols = (m.tall ? m.s0 : m.l0);
+    const int tiles_x = (m.tall ? m.s : m.l) >> 7, ty = (int)blockIdx.x / tiles_x;
     const int row0 = ty * 128, col = ((int)blockIdx.x - ty * tiles_x) * 128 + lane * 4;
 #pragma unroll 1
     for (int r = warp; r < 32; r += 8) {
@@ -266,14 +270,14 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
       if (lane == 0) wa[r] = acc;
     }
   } else {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t stride = (int64_t)m.stat_blocks * blockDim.x;
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    for (; i + stride < g.n4; i += 2 * stride) {
+    for (; i + stride < m.n4; i += 2 * stride) {
       const float4 v = __ldg(src + i), w = __ldg(src + i + stride);
       visit(v.x); visit(v.y); visit(v.z); visit(v.w);
       visit(w.x); visit(w.y); visit(w.z); visit(w.w);
     }
-    for (; i < g.n4; i += stride) {
+    for (; i < m.n4; i += stride) {
       const float4 v = __ldg(src + i);
       visit(v.x); visit(v.y); visit(v.z); visit(v.w);
     }
@@ -294,7 +298,7 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
   __syncthreads();
   for (uint32_t j = threadIdx.x; j < nbuf; j += blockDim.x) {
     const uint32_t gpos = s_base + j;
-    if (gpos < g.cand_cap) m.cand[gpos] = s_buf[j];
+    if (gpos < m.cand_cap) m.cand[gpos] = s_buf[j];
   }
   if (nbuf <= kSubBins) {
     for (uint32_t j = threadIdx.x; j < nbuf; j += blockDim.x) atomicAdd(&m.hist[(s_buf[j] >> 9) & (kSubBins - 1)], 1u);
@@ -352,11 +356,11 @@ __device__ __forceinline__ void fallback_select_and_stats(const PrepGroup& g, co
   auto each = [&](auto&& visit) {   // four loads in flight
     const int64_t step = blockDim.x;
     int64_t i = threadIdx.x;
-    for (; i + 3 * step < g.n4; i += 4 * step) {
+    for (; i + 3 * step < m.n4; i += 4 * step) {
       const float4 v0 = __ldg(src + i), v1 = __ldg(src + i + step), v2 = __ldg(src + i + 2 * step), v3 = __ldg(src + i + 3 * step);
       visit(v0); visit(v1); visit(v2); visit(v3);
     }
-    for (; i < g.n4; i += step) visit(__ldg(src + i));
+    for (; i < m.n4; i += step) visit(__ldg(src + i));
   };
   if (threadIdx.x == 0) { s_fb_prefix = hdr->sel_prefix; s_fb_rank = hdr->sel_rank; }
   __syncthreads();
@@ -443,6 +447,7 @@ __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ Prep
   pdl_launch_dependents();
   pdl_wait();
   const PrepMatrix& m = g.mat[blockIdx.y];
+  if ((int)blockIdx.x >= m.select_blocks) return;
   __shared__ double shd[1024];
   __shared__ uint32_t hist[kSubBins];
   __shared__ uint32_t wtot[32];
@@ -453,13 +458,13 @@ __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ Prep
   const int tid = threadIdx.x;
   if (!g.clip) {
     if (blockIdx.x) return;
-    const double total = sum_partials(m.partial, g.stat_blocks, shd);
+    const double total = sum_partials(m.partial, m.stat_blocks, shd);
     if (tid == 0)
       write_norm_scalars(m.scalars, g.ix, norm_scalars(total, __uint_as_float(hdr->maxabs_bits), g.eps, g.q.widen));
     return;
   }
   const uint32_t count = hdr->cand_count;
-  if (count > g.cand_cap) {
+  if (count > m.cand_cap) {
     if (blockIdx.x) return;
     if (tid == 0) hdr->overflow = 1;
     __shared__ uint32_t fb_hist[2048];
@@ -484,7 +489,7 @@ __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ Prep
   const uint32_t prefix = s_prefix, rank = s_rank;
   unsigned long long lo = 0, hi = 0;
   uint32_t above = 0;
-  const uint32_t stride = gridDim.x * blockDim.x;
+  const uint32_t stride = m.select_blocks * blockDim.x;
   for (uint32_t i0 = blockIdx.x * blockDim.x + tid; i0 < count; i0 += 8 * stride) {
     uint32_t k[8];
 #pragma unroll
@@ -517,14 +522,14 @@ __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ Prep
     atomicAdd(&s_above, above);
   }
   __syncthreads();
-  if (gridDim.x > 1) {
+  if (m.select_blocks > 1) {
     if (tid < kSubBins && hist[tid]) atomicAdd(&sums->low[tid], hist[tid]);
     if (tid == 0) {
       atomicAdd(&sums->lo, s_lo);
       atomicAdd(&sums->hi, s_hi);
       atomicAdd(&sums->above, s_above);
     }
-    if (!last_block(&hdr->ticket, gridDim.x)) return;
+    if (!last_block(&hdr->ticket, m.select_blocks)) return;
     if (tid < kSubBins) hist[tid] = __ldcg(&sums->low[tid]);
     if (tid == 0) { s_lo = __ldcg(&sums->lo); s_hi = __ldcg(&sums->hi); s_above = __ldcg(&sums->above); }
     __syncthreads();
@@ -561,11 +566,11 @@ __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ Prep
     atomicAdd(&s_above, above);
   }
   __syncthreads();
-  const double below = sum_partials(m.partial, g.stat_blocks, shd);
+  const double below = sum_partials(m.partial, m.stat_blocks, shd);
   if (tid == 0) {
     const float tau = __uint_as_float(tau_bits);
     // clamped to tau: everything in the bins above the picked one, and the candidates above tau
-    const double n_total = (double)g.n4 * 4.0;
+    const double n_total = (double)m.n4 * 4.0;
     const double n_clipped = n_total - (double)hdr->count_below - (double)hdr->bin_count + (double)s_above;
     const double total = clipped_squares(below, s_lo, s_hi, efield, n_clipped, tau);
     m.scalars[g.ix.tau] = tau;
@@ -597,7 +602,26 @@ constexpr int kPrepStage = 8 * kQtSlot + 2 * 1024;  // + two scale atoms per pas
 constexpr int kPrepWarps = 32;
 constexpr int kPrepThreads = kPrepWarps * 32;
 
-struct PrepTileInfo { int mi, gr0, gc0, pad; };  // matrix, origin of the tile in G
+struct PrepTileInfo {
+  int mi, gr0, gc0, index;   // matrix, origin of the tile in G, its index in the matrix
+  uint32_t row_k, col_k;     // contraction lengths of what is quantised along the rows and along the columns of G (for a wide G
+                             // qX and qX^T, for a tall one qX^T and qX)
+};
+// Tile t of the launch; mi: a matrix at or before its own.
+__device__ __forceinline__ PrepTileInfo place_tile(const PrepGroup& g, int t, int mi) {
+  PrepTileInfo ti;
+  ti.mi = mi;
+  while (ti.mi + 1 < g.count && t >= g.mat[ti.mi + 1].first_tile) ++ti.mi;
+  const PrepMatrix& m = g.mat[ti.mi];
+  ti.index = t - m.first_tile;
+  ti.row_k = (uint32_t)(m.tall ? m.s : m.l);
+  ti.col_k = (uint32_t)(m.tall ? m.l : m.s);
+  const int tiles_x = (int)(ti.row_k >> 7);  // tiles along a row of G
+  const int ty = ti.index / tiles_x;
+  ti.gr0 = ty * 128;
+  ti.gc0 = (ti.index - ty * tiles_x) * 128;
+  return ti;
+}
 struct PrepShared {
   uint64_t full[kPrepBufs];
   uint32_t abort_flag;
@@ -767,7 +791,8 @@ __device__ __forceinline__ PrepScalars prep_scalars(float tau, float inv, float 
 // column codes and scale bytes are staged.
 template <bool PF>
 __device__ __forceinline__ void prep_tile(const PrepGroup& g, const PrepMatrix& m, const PrepScalars& ps, const PrepLane& pl,
-                                          uint32_t tile, uint8_t* stage, int gr0, int gc0) {
+                                          uint32_t tile, uint8_t* stage, const PrepTileInfo& at) {
+  const int gr0 = at.gr0, gc0 = at.gc0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool row_warp = pl.row_warp;
   const int rr = pl.rr, box = pl.box, band = pl.band, cp = pl.cp;
@@ -799,7 +824,6 @@ __device__ __forceinline__ void prep_tile(const PrepGroup& g, const PrepMatrix& 
     }
   }
 
-  const int64_t rp_k = tall ? g.s : g.l;  // blocks along the rows of G are qX for a wide G, qX^T for a tall one
   if (g.write_q) {
     uint8_t* sf_stage = stage + 8 * kQtSlot;
     const uint32_t tb = tile + base_off;
@@ -848,7 +872,7 @@ __device__ __forceinline__ void prep_tile(const PrepGroup& g, const PrepMatrix& 
       }
       // the four lanes of a row write 64 contiguous bytes
       uint8_t* rp_codes = tall ? m.qt_codes : m.qx_codes;
-      *reinterpret_cast<uint4*>(rp_codes + (int64_t)(gr0 + rr) * (rp_k / 2) + gc0 / 2 + box * 16) =
+      *reinterpret_cast<uint4*>(rp_codes + (uint64_t)(uint32_t)(gr0 + rr) * (at.row_k / 2) + gc0 / 2 + box * 16) =
           make_uint4(code[0], code[1], code[2], code[3]);
       *reinterpret_cast<uint16_t*>(sf_stage + (box >> 1) * 512 + (rr & 31) * 16 + (rr >> 5) * 4 + (box & 1) * 2) =
           (uint16_t)sfw;
@@ -901,9 +925,9 @@ __device__ __forceinline__ void prep_tile(const PrepGroup& g, const PrepMatrix& 
 
 }
 // The staged bytes of a tile go out (after a block-wide barrier).
-__device__ __forceinline__ void prep_copy_out(const PrepGroup& g, const PrepMatrix& m, const uint8_t* stage, int gr0, int gc0) {
+__device__ __forceinline__ void prep_copy_out(const PrepGroup& g, const PrepMatrix& m, const uint8_t* stage, const PrepTileInfo& at) {
+  const int gr0 = at.gr0, gc0 = at.gc0;
   const int tall = m.tall;
-  const int64_t rp_k = tall ? g.s : g.l, cp_k = tall ? g.l : g.s;  // contraction length of the passes' destinations
   if (g.write_q) {
     const int tid = threadIdx.x;
     if (tid < 512) {
@@ -913,12 +937,12 @@ __device__ __forceinline__ void prep_copy_out(const PrepGroup& g, const PrepMatr
       const uint8_t* src = stage + c * 8;
       const uint2 a = *reinterpret_cast<const uint2*>(src + (2 * h) * kQtSlot);
       const uint2 d = *reinterpret_cast<const uint2*>(src + (2 * h + 1) * kQtSlot);
-      *reinterpret_cast<uint4*>(cp_codes + (int64_t)(gc0 + c) * (cp_k / 2) + gr0 / 2 + h * 16) = make_uint4(a.x, a.y, d.x, d.y);
+      *reinterpret_cast<uint4*>(cp_codes + (uint64_t)(uint32_t)(gc0 + c) * (at.col_k / 2) + gr0 / 2 + h * 16) = make_uint4(a.x, a.y, d.x, d.y);
     } else if (tid < 640) {
       // scale atoms: two adjacent 512-byte atoms per pass
       const bool rowpass = tid < 576;
       uint8_t* sf_base = rowpass ? (tall ? m.qt_sf : m.qx_sf) : (tall ? m.qx_sf : m.qt_sf);
-      const int64_t row0 = rowpass ? gr0 : gc0, k0 = rowpass ? gc0 : gr0, kk = rowpass ? rp_k : cp_k;
+      const int64_t row0 = rowpass ? gr0 : gc0, k0 = rowpass ? gc0 : gr0, kk = rowpass ? at.row_k : at.col_k;
       const int j = tid & 63;
       const uint4 w = *reinterpret_cast<const uint4*>(stage + 8 * kQtSlot + (rowpass ? 0 : 1024) + j * 16);
       *reinterpret_cast<uint4*>(sf_base + sf_offset(row0, k0 / 16, kk / 16) + j * 16) = w;
@@ -933,9 +957,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
   uint8_t* stage_base = smem + kPrepBufs * kPrepTile;
   PrepShared* sh = reinterpret_cast<PrepShared*>(stage_base + kPrepBufs * kPrepStage);
   volatile uint32_t* abort_flag = &sh->abort_flag;
-  const int tiles_per_matrix = (int)((g.s >> 7) * (g.l >> 7));
-  const int total = tiles_per_matrix * g.count;
-  const int my_tiles = (total - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // tiles of this block
+  const int my_tiles = (g.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // tiles of this block
   pdl_launch_dependents();
 
   // Tile `it` of this block: work out where it lies, publish that in the ring and start its copy.  Called by
@@ -944,14 +966,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
     if (it_ >= my_tiles) return;
     const int t_ = (int)blockIdx.x + it_ * (int)gridDim.x;
     const int b_ = it_ % kPrepBufs;
-    PrepTileInfo ti;
-    ti.pad = 0;
-    ti.mi = t_ / tiles_per_matrix;
-    const int r_ = t_ - ti.mi * tiles_per_matrix;
-    const int tiles_x = (int)((g.mat[ti.mi].tall ? g.s : g.l) >> 7);  // tiles along a row of G
-    const int ty = r_ / tiles_x;
-    ti.gr0 = ty * 128;
-    ti.gc0 = (r_ - ty * tiles_x) * 128;
+    const PrepTileInfo ti = place_tile(g, t_, it_ > 0 ? sh->info[(it_ - 1) & 3].mi : 0);
     sh->info[it_ & 3] = ti;
     mbar_expect_tx(&sh->full[b_], kPrepTile);
 #pragma unroll
@@ -980,9 +995,9 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
   ps.tau = ps.inv = ps.tinv = ps.six_sg = ps.rcp_six_sg = ps.sg = 0.0f; ps.rcp_tab = 0; ps.near_limit = 0;
   for (int it = 0; it < my_tiles; ++it) {
     const int b = it % kPrepBufs, use = it / kPrepBufs;
-    const PrepTileInfo ti = sh->info[it & 3];   // written before an earlier barrier
+    const PrepTileInfo& ti = sh->info[it & 3];   // written before an earlier barrier
     wait_or_abort(&sh->full[b], (uint32_t)use & 1u, abort_flag);
-    const int mi = ti.mi, gr0 = ti.gr0, gc0 = ti.gc0;
+    const int mi = ti.mi;
     const PrepMatrix& m = g.mat[mi];
     if (mi != cur) {
       cur = mi;
@@ -990,7 +1005,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
                         smem_u32(&sh->rcp_tab[mi][0]));
     }
     uint8_t* stage = stage_base + b * kPrepStage;
-    prep_tile<PF>(g, m, ps, pl, smem_u32(smem + b * kPrepTile), stage, gr0, gc0);
+    prep_tile<PF>(g, m, ps, pl, smem_u32(smem + b * kPrepTile), stage, ti);
 
     // Every warp has read the tile and staged its output: the buffer takes the tile three ahead, the
     // staged bytes go out.
@@ -999,7 +1014,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_prep_operands(const __grid
       fence_proxy_async_smem();
       fetch(it + kPrepBufs);
     }
-    if (g.write_q) prep_copy_out(g, m, stage, gr0, gc0);
+    if (g.write_q) prep_copy_out(g, m, stage, ti);
   }
   if (threadIdx.x == 0 && sh->abort_flag) report_timeout(g.status);
 }
@@ -1021,7 +1036,7 @@ constexpr int kResUnion = kTopBins * 4;     // histogram / candidate buffer / se
 static_assert(kResUnion >= kPrepStage && kResUnion >= 4096 + 1024 * 8, "union area");
 struct ResidentShared {
   uint64_t full[kResTiles];
-  PrepTileInfo info[kResTiles];              // pad: index of the tile within its matrix
+  PrepTileInfo info[kResTiles];
   uint32_t prefix[kResTiles], rank[kResTiles], bin_count[kResTiles], below[kResTiles];   // of the tile's matrix
   float tau[kResTiles], inv[kResTiles], sg[kResTiles];
   float rcp_tab[8];
@@ -1047,9 +1062,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
   ResidentShared* sh = reinterpret_cast<ResidentShared*>(uni + kResUnion);
   volatile uint32_t* abort_flag = &sh->abort_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tiles_per_matrix = (int)((g.s >> 7) * (g.l >> 7));
-  const int total = tiles_per_matrix * g.count;
-  const int mine = (total - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // 1 .. kResTiles
+  const int mine = (g.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // 1 .. kResTiles
   uint32_t* counter = &g.mat[0].hdr->barrier;
   uint32_t round = 0;
   if (tid == 0) {
@@ -1057,14 +1070,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
     sh->abort_flag = 0;
     mbar_fence_init();
     for (int it = 0; it < mine; ++it) {
-      const int t = (int)blockIdx.x + it * (int)gridDim.x;
-      PrepTileInfo ti;
-      ti.mi = t / tiles_per_matrix;
-      ti.pad = t - ti.mi * tiles_per_matrix;
-      const int tiles_x = (int)((g.mat[ti.mi].tall ? g.s : g.l) >> 7);
-      const int ty = ti.pad / tiles_x;
-      ti.gr0 = ty * 128;
-      ti.gc0 = (ti.pad - ty * tiles_x) * 128;
+      const PrepTileInfo ti = place_tile(g, (int)blockIdx.x + it * (int)gridDim.x, 0);
       sh->info[it] = ti;
       mbar_expect_tx(&sh->full[it], kPrepTile);
 #pragma unroll
@@ -1085,7 +1091,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
   auto pieces = [&](int it, auto&& f) {
     const PrepTileInfo ti = sh->info[it];
     const PrepMatrix& m = g.mat[ti.mi];
-    const int rows = (int)(m.tall ? g.l0 : g.s0) - ti.gr0, cols = (int)(m.tall ? g.s0 : g.l0) - ti.gc0;
+    const int rows = (m.tall ? m.l0 : m.s0) - ti.gr0, cols = (m.tall ? m.s0 : m.l0) - ti.gc0;
     const uint32_t at = smem_u32(smem + it * kPrepTile);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -1143,7 +1149,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       if (lane == 0) sh->wtot[warp] = all;
       __syncthreads();
       const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? sh->wtot[lane] : 0u);
-      if (g.clip_rank > before && g.clip_rank <= before + all) {
+      if (g.mat[mi].clip_rank > before && g.mat[mi].clip_rank <= before + all) {
         uint32_t run = before;
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
@@ -1155,13 +1161,13 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
             if (lane >= o) incl += t;
           }
           uint32_t at = run + incl - v;
-          if (g.clip_rank > at && g.clip_rank <= at + v) {
+          if (g.mat[mi].clip_rank > at && g.mat[mi].clip_rank <= at + v) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               const uint32_t n = c[half * 4 + q];
-              if (g.clip_rank > at && g.clip_rank <= at + n) {
+              if (g.mat[mi].clip_rank > at && g.mat[mi].clip_rank <= at + n) {
                 sh->prefix[it] = (uint32_t)(warp * 256 + half * 128 + lane * 4 + q) << kTopShift;
-                sh->rank[it] = g.clip_rank - at;
+                sh->rank[it] = g.mat[mi].clip_rank - at;
                 sh->bin_count[it] = n;
                 sh->below[it] = at;
               }
@@ -1199,7 +1205,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
           buf[pos] = k;
         } else {
           const uint32_t gpos = atomicAdd(&m.hdr->cand_count, 1u);
-          if (gpos < g.cand_cap) m.cand[gpos] = k;
+          if (gpos < m.cand_cap) m.cand[gpos] = k;
         }
       }
     });
@@ -1212,7 +1218,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       acc = warp_sum(sh->wsum[lane]);
       mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sh->wmax[lane])));
       if (lane == 0) {
-        m.partial[ti.pad] = acc;
+        m.partial[ti.index] = acc;
         atomicMax(&m.hdr->maxabs_bits, __float_as_uint(mx));
         sh->base = nbuf ? atomicAdd(&m.hdr->cand_count, nbuf) : 0u;
       }
@@ -1220,7 +1226,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
     __syncthreads();
     for (uint32_t j = tid; j < nbuf; j += kPrepThreads) {
       const uint32_t gpos = sh->base + j;
-      if (gpos < g.cand_cap) m.cand[gpos] = buf[j];
+      if (gpos < m.cand_cap) m.cand[gpos] = buf[j];
     }
     __syncthreads();
   }
@@ -1237,11 +1243,11 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       __syncthreads();
       continue;
     }
-    const bool owner = sh->info[it].pad == 0;
+    const bool owner = sh->info[it].index == 0;
     if (owner && g.clip && m.hist_top)   // the caller's counters are consumed, whichever way tau is found: every block has read them
       for (int i = tid; i < kTopBins; i += kPrepThreads) m.hist_top[i] = 0;
     const uint32_t count = g.clip ? __ldcg(&hdr->cand_count) : 0u;
-    if (count > g.cand_cap) {
+    if (count > m.cand_cap) {
       // so many equal magnitudes that the list overflowed: the owner finishes alone, the others wait for it
       if (owner) {
         if (tid == 0) { hdr->sel_prefix = sh->prefix[it]; hdr->sel_rank = sh->rank[it]; }
@@ -1336,7 +1342,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       }
       if (lane == 0) { sh->wlo[warp] = lo; sh->whi[warp] = hi; sh->wabove[warp] = above; }
     }
-    double acc = sum_partials(m.partial, tiles_per_matrix, sh->wsum);
+    double acc = sum_partials(m.partial, m.tiles, sh->wsum);
     if (warp == 0) {
       if (g.clip) { lo = sh->wlo[lane]; hi = sh->whi[lane]; above = sh->wabove[lane]; }
 #pragma unroll
@@ -1351,7 +1357,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
           tau = __uint_as_float(tau_bits);
           maxabs = tau;
           // clamped to tau: everything in the bins above the picked one, and the candidates above tau
-          const double n_clipped = (double)g.n4 * 4.0 - (double)sh->below[it] - (double)sh->bin_count[it] + (double)above;
+          const double n_clipped = (double)m.n4 * 4.0 - (double)sh->below[it] - (double)sh->bin_count[it] + (double)above;
           acc = clipped_squares(acc, lo, hi, efield, n_clipped, tau);
         }
         const NormScalars ns = norm_scalars(acc, maxabs, g.eps, g.q.widen);
@@ -1368,20 +1374,39 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
   // ---- operand copies of X0 from the resident tiles
   const PrepLane pl = prep_lane();
   for (int it = 0; it < mine; ++it) {
-    const PrepTileInfo ti = sh->info[it];
+    const PrepTileInfo& ti = sh->info[it];
     const PrepMatrix& m = g.mat[ti.mi];
     if (tid < 8) sh->rcp_tab[tid] = __frcp_rn(__fmul_rn((float)(8 + tid), sh->sg[it]));
     __syncthreads();
     const PrepScalars ps = prep_scalars(sh->tau[it], sh->inv[it], sh->sg[it], smem_u32(&sh->rcp_tab[0]));
-    prep_tile<PF>(g, m, ps, pl, smem_u32(smem + it * kPrepTile), uni, ti.gr0, ti.gc0);
+    prep_tile<PF>(g, m, ps, pl, smem_u32(smem + it * kPrepTile), uni, ti);
     __syncthreads();
-    if (g.write_q) prep_copy_out(g, m, uni, ti.gr0, ti.gc0);
+    if (g.write_q) prep_copy_out(g, m, uni, ti);
     __syncthreads();
   }
   if (tid == 0 && sh->abort_flag) report_timeout(g.status);
 }
 
 }  // namespace
+
+// Whether a matrix of this many tiles is summed tile by tile, as the single launch does it (at most 1024 partials), and whether
+// matrices of `tiles` in all fit that launch.
+static bool tiled_sum(int64_t matrix_tiles, int device_sms) { return matrix_tiles <= (int64_t)kResTiles * device_sms && matrix_tiles <= 1024; }
+static bool fits_resident(int64_t tiles, int coop_sms) { return tiles <= (int64_t)kResTiles * coop_sms; }
+
+// Estimated time in us: one launch, per tile that a block takes; or six launches, bound by HBM and by their instructions.
+// Measured: 8 / 256 / 405 tiles 18 / 29 / 40 us; 8192 x 2048 71 us, sixteen 3072 x 3072 437.
+double prologue_us(const WorkShape* w, int count, int device_sms, int coop_sms) {
+  int64_t tiles = 0;
+  bool tiled = true;
+  for (int j = 0; j < count; ++j) {
+    const int64_t n = w[j].s / 128 * (w[j].l / 128);
+    tiled = tiled && tiled_sum(n, device_sms);
+    tiles += n;
+  }
+  if (tiled && fits_resident(tiles, coop_sms)) return 7.0 + 11.0 * (double)((tiles + coop_sms - 1) / coop_sms);
+  return 28.0 + 2.7e-6 * 16384.0 * (double)tiles;
+}
 
 cudaError_t prologue_set_attributes() {
   cudaError_t e = cudaFuncSetAttribute(kp_prep_operands<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepSmem);
@@ -1391,64 +1416,79 @@ cudaError_t prologue_set_attributes() {
   return cudaFuncSetAttribute(kp_resident<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
 }
 
-// Enqueue the prologue for `count` matrices of one shape (s, l) and one parameter set.
+// Enqueue the prologue for `count` matrices that share clip, eps and options.
 cudaError_t launch_prologue_group(const PrologueItem* items, int count, int write_q, const QuantOpts& q,
                                   uint32_t* status, int coop_sms, int sms, cudaStream_t st) {
   for (int i0 = 0; i0 < count; i0 += kMaxPack) {
     const int nn = count - i0 < kMaxPack ? count - i0 : kMaxPack;
-    const NsPlan& pl = *items[i0].pl;
     PrepGroup g;
     memset(&g, 0, sizeof(g));
     g.count = nn;
-    g.n4 = pl.s0 * pl.l0 / 4;
-    g.s = pl.s; g.l = pl.l;
-    g.s0 = pl.s0; g.l0 = pl.l0;
-    g.clip = pl.clip;
-    g.clip_rank = (uint32_t)pl.clip_rank;
-    // The candidate list lives in workspace that nothing else uses before the first product: the A buffer
-    // (s x s words) or, for a matrix much longer than high, the second set of transposed operand codes
-    // (s x l / 8 words).  An eighth of the elements is more than any bin of a spread-out distribution holds.
-    const bool cand_in_qxt = pl.s * pl.l / 8 > pl.s * pl.s;
-    const int64_t region = cand_in_qxt ? pl.s * pl.l / 8 : pl.s * pl.s;
-    const int64_t cap = pl.s0 * pl.l0 / 8 < region ? pl.s0 * pl.l0 / 8 : region;
-    g.cand_cap = (uint32_t)cap;
-    g.eps = pl.eps;
+    g.clip = items[i0].pl->clip;
+    g.eps = items[i0].pl->eps;
     g.write_q = write_q;
-    g.zero_words = (int)(pl.zero_bytes / 4);
-    g.ix = pl.ix;
+    g.zero_words = (int)(items[i0].pl->zero_bytes / 4);
+    g.ix = items[i0].pl->ix;
     g.q = q;
     g.status = status;
-    bool all_counted = true;
+    bool all_counted = true, all_tiled = true, none_tiled = true;
+    int hist_blocks = 1, stat_tiled = 1, stat_other = 1, select_blocks = 1;
     for (int j = 0; j < nn; ++j) {
       const PrologueItem& it = items[i0 + j];
-      const fp4_ws_layout& L = it.pl->lay;
+      const NsPlan& pl = *it.pl;
+      const fp4_ws_layout& L = pl.lay;
       PrepMatrix& m = g.mat[j];
+      // The candidate list lives in workspace that nothing else uses before the first product: the A buffer
+      // (s x s words) or, for a matrix much longer than high, the second set of transposed operand codes
+      // (s x l / 8 words).  An eighth of the elements is more than any bin of a spread-out distribution holds.
+      const bool cand_in_qxt = pl.s * pl.l / 8 > pl.s * pl.s;
+      const int64_t region = cand_in_qxt ? pl.s * pl.l / 8 : pl.s * pl.s;
+      m.cand_cap = (uint32_t)(pl.s0 * pl.l0 / 8 < region ? pl.s0 * pl.l0 / 8 : region);
       m.G = it.G; m.X = it.X;
       m.hdr = reinterpret_cast<NsHeader*>(it.ws + L.header);
       m.scalars = reinterpret_cast<float*>(it.ws + L.scalars);
-      m.hist = reinterpret_cast<uint32_t*>(it.ws + it.pl->off_hist);
-      m.partial = reinterpret_cast<double*>(it.ws + it.pl->off_partial);
+      m.hist = reinterpret_cast<uint32_t*>(it.ws + pl.off_hist);
+      m.partial = reinterpret_cast<double*>(it.ws + pl.off_partial);
       m.cand = reinterpret_cast<uint32_t*>(it.ws + (cand_in_qxt ? L.qXt_codes[1] : L.A));
       m.qx_codes = it.ws + L.qX_codes; m.qx_sf = it.ws + L.qX_scales;
       m.qt_codes = it.ws + L.qXt_codes[0]; m.qt_sf = it.ws + L.qXt_scales[0];
-      m.tall = it.pl->tall;
+      m.tall = pl.tall;
       m.clear_status = it.clear_status ? 1 : 0;
       m.store_x = it.store_x ? 1 : 0;
-      m.x_rows = it.x_rows; m.x_cols = it.x_cols;
+      m.x_rows = (int)it.x_rows; m.x_cols = (int)it.x_cols;
       m.hist_top = it.hist_top;
-      if (!it.hist_top) all_counted = false;
+      m.n4 = pl.s0 * pl.l0 / 4;
+      m.s = (int)pl.s; m.l = (int)pl.l;
+      m.s0 = (int)pl.s0; m.l0 = (int)pl.l0;
+      m.clip_rank = (uint32_t)pl.clip_rank;
+      const int64_t tiles = (pl.l / 128) * (pl.s / 128);
+      m.tiled = tiled_sum(tiles, pl.sms);
+      m.tiles = (int)tiles;
+      m.first_tile = g.tiles;
+      g.tiles += m.tiles;
+      const int64_t hb = (m.n4 + 512 * 4 - 1) / (512 * 4);
+      m.hist_blocks = (int)(hb < (int64_t)sms * 4 ? (hb < 1 ? 1 : hb) : (int64_t)sms * 4);
+      m.stat_blocks = m.tiled ? m.tiles : pl.stat_blocks;
+      // a block of the select per 4 M elements: some 10 k candidates of a Gaussian matrix
+      const int64_t fb = m.n4 >> 20;
+      m.select_blocks = (int)(fb < 1 ? 1 : fb < 64 ? fb : 64);
+      if (!it.hist_top) {
+        all_counted = false;
+        hist_blocks = hist_blocks > m.hist_blocks ? hist_blocks : m.hist_blocks;
+      }
+      int& stat = m.tiled ? stat_tiled : stat_other;
+      stat = stat > m.stat_blocks ? stat : m.stat_blocks;
+      (m.tiled ? none_tiled : all_tiled) = false;
+      select_blocks = select_blocks > m.select_blocks ? select_blocks : m.select_blocks;
       g.tmG[j] = *it.tmG;
     }
-    const int64_t matrix_tiles = (pl.l / 128) * (pl.s / 128), tiles = matrix_tiles * nn;
-    const bool tiled = matrix_tiles <= (int64_t)kResTiles * pl.sms && matrix_tiles <= 1024;   // 1024 partials
-    g.stat_blocks = tiled ? (int)matrix_tiles : pl.stat_blocks;
-    if (tiled && tiles <= (int64_t)kResTiles * coop_sms) {
+    if (all_tiled && fits_resident(g.tiles, coop_sms)) {
       // everything fits the shared memories: one launch
       ProfScope ps(FP4_PROF_PREP, st);
       cudaError_t e = cudaMemsetAsync(&g.mat[0].hdr->barrier, 0, 4, st);
       if (e != cudaSuccess) return e;
       cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)(tiles < coop_sms ? tiles : coop_sms)); cfg.blockDim = dim3(kPrepThreads);
+      cfg.gridDim = dim3((unsigned)(g.tiles < coop_sms ? g.tiles : coop_sms)); cfg.blockDim = dim3(kPrepThreads);
       cfg.dynamicSmemBytes = kResSmem; cfg.stream = st;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeCooperative;
@@ -1459,9 +1499,7 @@ cudaError_t launch_prologue_group(const PrologueItem* items, int count, int writ
       if (e != cudaSuccess) return e;
       continue;
     }
-    int64_t hb = (g.n4 + 512 * 4 - 1) / (512 * 4);
-    const int hist_blocks = (int)(hb < (int64_t)sms * 4 ? (hb < 1 ? 1 : hb) : (int64_t)sms * 4);
-    const dim3 gy1(1, (unsigned)nn), gh((unsigned)hist_blocks, (unsigned)nn), gs((unsigned)g.stat_blocks, (unsigned)nn);
+    const dim3 gy1(1, (unsigned)nn), gh((unsigned)hist_blocks, (unsigned)nn);
     {
       ProfScope ps(FP4_PROF_CLIP, st);
       launch_chained(kp_init, dim3(4, (unsigned)nn), dim3(256), 0, st, g);
@@ -1474,15 +1512,15 @@ cudaError_t launch_prologue_group(const PrologueItem* items, int count, int writ
     }
     {
       ProfScope ps(FP4_PROF_STATS, st);
-      launch_chained(tiled ? kp_compact_stats<true> : kp_compact_stats<false>, gs, dim3(256), 0, st, g);
-      // a block of the select per 4 M elements: some 10 k candidates of a Gaussian matrix
-      const int64_t fb = g.n4 >> 20;
-      launch_chained(kp_finalize, dim3((unsigned)(fb < 1 ? 1 : fb < 64 ? fb : 64), (unsigned)nn), dim3(1024), 0, st, g);
-      count_launches(2);
+      // a pass for each kind of sum
+      if (!none_tiled) launch_chained(kp_compact_stats<true>, dim3((unsigned)stat_tiled, (unsigned)nn), dim3(256), 0, st, g);
+      if (!all_tiled) launch_chained(kp_compact_stats<false>, dim3((unsigned)stat_other, (unsigned)nn), dim3(256), 0, st, g);
+      launch_chained(kp_finalize, dim3((unsigned)select_blocks, (unsigned)nn), dim3(1024), 0, st, g);
+      count_launches(none_tiled || all_tiled ? 2 : 3);
     }
     {
       ProfScope ps(FP4_PROF_PREP, st);
-      const unsigned gp = (unsigned)(tiles < sms ? tiles : sms);
+      const unsigned gp = (unsigned)(g.tiles < sms ? g.tiles : sms);
       if (q.rht || q.four_six) launch_chained(kp_prep_operands<true>, dim3(gp), dim3(kPrepThreads), kPrepSmem, st, g);
       else launch_chained(kp_prep_operands<false>, dim3(gp), dim3(kPrepThreads), kPrepSmem, st, g);
       count_launches(1);

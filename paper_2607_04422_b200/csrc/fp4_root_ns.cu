@@ -1,6 +1,7 @@
 // Host side of the library: argument checks, workspace layout, TMA descriptors, and the
 // sequence of launches of the Root Newton-Schulz step (Section 3.4).  Everything here
 // only enqueues work on the caller's stream.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <mutex>
@@ -354,15 +355,24 @@ struct MatrixCtx {
 // tiles over the SM pairs, an epilogue or a main loop; a partly filled last round costs half of what it lacks.
 struct PairUs {
   double g1, g2, g3;
-  PairUs(int64_t s, int64_t l, int count, bool opts, int sms) {
-    const double ts = (double)((s + 255) / 256), tl = (double)((l + 255) / 256), pairs = (double)(sms / 2);
+  PairUs(const WorkShape* w, int count, bool opts, int sms) {
+    const double pairs = (double)(sms / 2);
     auto rounds = [](double r) { return (std::ceil(r) + (r > 1.0 ? r : 1.0)) / 2; };
     const double epi = 3.95 * (opts ? 1.5 : 1.0), kb = 0.22;
-    const double k1 = kb * tl, k2 = kb * ts;
-    const double rs = rounds(ts * (ts + 1) / 2 * count / pairs), rf = rounds(ts * tl * count / pairs);
-    g1 = 6.25 + rs * (epi > k1 ? epi : k1);
-    g2 = 6.25 + rs * (epi > k2 ? epi : k2);
-    g3 = 6.25 + rf * (epi > k2 ? epi : k2);
+    double sym = 0.0, full = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;   // tiles, and their times in all
+    for (int j = 0; j < count; ++j) {
+      const double ts = (double)((w[j].s + 255) / 256), tl = (double)((w[j].l + 255) / 256);
+      const double k1 = kb * tl, k2 = kb * ts, n = ts * (ts + 1) / 2;
+      sym += n;
+      full += ts * tl;
+      t1 += n * (epi > k1 ? epi : k1);
+      t2 += n * (epi > k2 ? epi : k2);
+      t3 += ts * tl * (epi > k2 ? epi : k2);
+    }
+    const double rs = rounds(sym / pairs), rf = rounds(full / pairs);
+    g1 = 6.25 + rs * (t1 / sym);
+    g2 = 6.25 + rs * (t2 / sym);
+    g3 = 6.25 + rf * (t3 / full);
   }
 };
 
@@ -377,16 +387,21 @@ struct PairUs {
 // faster, 458 (64) / 559 / 545 at 128 x 56784: these keep the route that they have been tested on.)
 constexpr int64_t kChainLong = 32768;
 enum Route { kOneLaunch, kTwoLaunches, kThreeLaunches };
-Route route_of(const NsPlan& pl, int count, const fp4_ns_params* p, int sms) {
+struct Plan { Route route; double iteration_us; };
+Plan plan_of(const WorkShape* w, int count, const fp4_ns_params* p, int sms) {
   const bool opts = (p->flags & (FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)) != 0;
-  if (count > kChainMax || (pl.l > kChainLong && !opts) || (pl.bf16 && (p->flags & FP4_FLAG_KEEP_OPERANDS))) return kThreeLaunches;
-  const PairUs pair(pl.s, pl.l, count, opts, sms);
-  const double three = pair.g1 + pair.g2 + pair.g3;
-  const double sym = chain_symmetric_us(pl.s, pl.l, count, opts, sms);
-  const double best = sym > 0.0 && sym + pair.g3 < three ? sym + pair.g3 : three;
-  const double one = chain_iteration_us(pl.s, pl.l, count, opts, sms);
-  if (one > 0.0 && one <= best) return kOneLaunch;
-  return best < three ? kTwoLaunches : kThreeLaunches;
+  const PairUs pair(w, count, opts, sms);
+  Plan plan{kThreeLaunches, pair.g1 + pair.g2 + pair.g3};
+  int64_t longest = 0;
+  for (int j = 0; j < count; ++j) longest = w[j].l > longest ? w[j].l : longest;
+  if (count > kChainMax || (longest > kChainLong && !opts) ||
+      ((p->flags & FP4_FLAG_STORE_BF16) && (p->flags & FP4_FLAG_KEEP_OPERANDS)))
+    return plan;
+  const double sym = chain_symmetric_us(w, count, opts, sms);
+  if (sym > 0.0 && sym + pair.g3 < plan.iteration_us) plan = {kTwoLaunches, sym + pair.g3};
+  const double one = chain_iteration_us(w, count, opts, sms);
+  if (one > 0.0 && one <= plan.iteration_us) plan = {kOneLaunch, one};
+  return plan;
 }
 
 fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t m, int64_t n, int steps,
@@ -437,12 +452,16 @@ fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t
   base.scalars = reinterpret_cast<float*>(ws + L.scalars);
   base.ca = abc[0]; base.cb = abc[1]; base.cc = abc[2];
   base.out_rows = (int)s; base.out_cols = (int)s;
+  base.K = (int)s;
+  base.blocks_m = base.blocks_n = (int)(s / 128);
+  base.l_cols = (float)l;
   const bool bf16 = c->pl.bf16 != 0;
   CUtensorMap tm_Ah, tm_Xh;
   uint8_t* Xh = bf16 ? ws + c->pl.off_Xh : nullptr;
   if (bf16 && (!make_bf16_map(d, &tm_Ah, ws + L.A, s, s) || !make_bf16_map(d, &tm_Xh, Xh, s, l))) return FP4_ERR_CUDA;
   // G1: A = qX qX^T (upper-triangle tiles), qA in both triangles
   c->g1 = base;
+  c->g1.K = (int)l;
   c->g1.tmA = c->g1.tmB = tm_qX; c->g1.tmAux = c->g1.tmOut = tm_A;
   c->g1.tmRq = st_qA_r; c->g1.tmCq = st_qA_c;
   c->g1.tmSfa = c->g1.tmSfb = sf_qX;
@@ -459,6 +478,7 @@ fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t
   for (int cur = 0; cur < 2; ++cur) {
     GemmProblem& g = c->g3[cur];
     g = base;
+    g.blocks_n = (int)(l / 128);
     g.tmA = tm_qB; g.tmB = tm_qXt[cur]; g.tmAux = g.tmOut = tm_X;
     g.out_rows = (int)xr; g.out_cols = (int)xc;
     if (bf16) g.tmH = tm_Xh;
@@ -490,6 +510,8 @@ fp4_status build_matrix(const DeviceInfo* d, const float* G, float* out, int64_t
     h.qa_sf = ws + L.qA_scales; h.qb_sf = ws + L.qB_scales;
     h.ca = abc[0]; h.cb = abc[1]; h.cc = abc[2];
     h.tall = tall;
+    h.s = (int)s; h.l = (int)l; h.s0 = (int)c->pl.s0; h.l0 = (int)c->pl.l0;
+    h.l_cols = (float)l;
   }
   c->g3_first = c->g3[0];
   if (c->pl.tall) {
@@ -559,11 +581,11 @@ fp4_status prepare_matrix(const DeviceInfo* d, const float* G, float* out, int64
   return FP4_OK;
 }
 
-// Enqueue the whole step for a group of matrices of one shape (s, l): the prologue per matrix,
-// then every Newton-Schulz stage as one launch over all matrices of the group.
+// Enqueue the whole step for a group of matrices: the prologue, then every Newton-Schulz stage as one launch over all
+// matrices of the group.
 // count <= kPackMax: the problems of a launch travel as its parameter.
 fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps, const fp4_ns_params* p,
-                     uint32_t* status, bool clear_first_status, bool two_streams, cudaStream_t st) {
+                     uint32_t* status, bool clear_status, bool two_streams, cudaStream_t st) {
   if (count < 1 || count > kPackMax) return FP4_ERR_INVALID_ARG;
   const bool keep = (p->flags & FP4_FLAG_KEEP_OPERANDS) != 0;
   ParamUpdate upd;
@@ -586,21 +608,26 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
   bool any_direct = false;
   for (int i = 0; i < count; ++i)
     if (steps > 0 && mats[i].pl.tall && !keep && !any_update) { direct_out[(size_t)i] = 1; any_direct = true; }
-  const NsPlan& pl0 = mats[0].pl;
-  const int64_t s = pl0.s, l = pl0.l;
+  const NsPlan& pl0 = mats[0].pl;   // for what does not depend on the shape
+  WorkShape shapes[kPackMax];
+  int64_t elements = 0;
+  for (int i = 0; i < count; ++i) {
+    shapes[i] = {mats[i].pl.s, mats[i].pl.l};
+    elements += mats[i].pl.s * mats[i].pl.l;
+  }
   // A cooperative launch that needs more than half of the SMs keeps the other stream's group waiting: the two take half each, and
   // what does not fit is left to the plain launches, which share the SMs as they become free.
   // Measured, 5 iterations, one stream / two with whole-device launches / with halves: six groups of one matrix (1536 x 1536 ..
   // 2816) 1177 / 1160 / 834 us, eight of one (640 x 640 .. 1536) 885 / 680 / 490, six of two (1280 x 1280 .. 2560)
   // 1197 / 1184 / 996, eight tiny ones 780 / 405 / 407; four groups of four with the quantiser options lose (1323 / 1447).
   const int sms = stream_sms(d, st), coop_sms = two_streams && sms > 1 ? sms / 2 : sms;
-  pdl_select(s * l * count);
-  const Route route = steps > 0 ? route_of(pl0, count, p, coop_sms) : kThreeLaunches;
+  pdl_select(elements);
+  const Route route = steps > 0 ? plan_of(shapes, count, p, coop_sms).route : kThreeLaunches;
   {
     std::vector<PrologueItem> items((size_t)count);
     for (int i = 0; i < count; ++i) {
       MatrixCtx& c = mats[i];
-      items[(size_t)i] = PrologueItem{c.G, c.X, c.ws, &c.pl, clear_first_status && i == 0, c.store_x0, c.x_rows, c.x_cols,
+      items[(size_t)i] = PrologueItem{c.G, c.X, c.ws, &c.pl, clear_status && reinterpret_cast<uint32_t*>(c.ws + c.pl.lay.header) == status, c.store_x0, c.x_rows, c.x_cols,
                                       c.hist_top, &c.tm_G};
     }
     if (launch_prologue_group(items.data(), count, steps > 0 || keep, quant_opts(p, 0), status, coop_sms, sms, st) != cudaSuccess)
@@ -615,11 +642,9 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     }
     memset(&a, 0, sizeof(a));
     a.count = count; a.steps = steps;
-    a.s = (int)s; a.l = (int)l; a.s0 = (int)pl0.s0; a.l0 = (int)pl0.l0;
     a.clip = pl0.clip; a.keep = keep; a.bf16 = pl0.bf16;
     for (int j = 0; j < count; ++j) a.tall |= mats[j].pl.tall;
     a.update = any_update && !keep; a.no_out = upd.no_out; a.upd_decay = upd.decay; a.upd_step = upd.step;
-    a.l_cols = (float)l;
     a.q = quant_opts(p, 0);
     a.seed = p->seed;
     a.ix = pl0.ix;
@@ -657,7 +682,6 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     memset(&base, 0, sizeof(base));
     base.num_problems = count;
     base.ix = pl0.ix;
-    base.l_cols = (float)l;
     base.status = status;
     base.clip = pl0.clip;
     const int bf16 = pl0.bf16;
@@ -665,8 +689,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       const int cur = k & 1;
       const bool last = (k == steps - 1);
       GemmLaunch L1 = base;
-      L1.iter = k; L1.K = (int)l; L1.tiles_m = L1.tiles_n = (int)(s / 128); L1.symmetric = 1;
-      L1.rq_K = L1.cq_K = (int)s; L1.write_q = 1;
+      L1.iter = k; L1.symmetric = 1; L1.write_q = 1;
       L1.q = quant_opts(p, 2 * (uint64_t)k + 1);  // qA_k
       L1.out_h = bf16;
       if (route == kTwoLaunches) {
@@ -678,7 +701,6 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
           return FP4_ERR_CUDA;
       }
       GemmLaunch L2 = L1;
-      L2.K = (int)s;
       L2.q = quant_opts(p, 2 * (uint64_t)k);      // qB_k meets qX_k^{16x1}
       L2.out_h = 0; L2.aux_h = bf16;
       if (route == kThreeLaunches) {
@@ -687,8 +709,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
           return FP4_ERR_CUDA;
       }
       GemmLaunch L3 = base;
-      L3.iter = k; L3.K = (int)s; L3.tiles_m = (int)(s / 128); L3.tiles_n = (int)(l / 128); L3.symmetric = 0;
-      L3.rq_K = (int)l; L3.cq_K = (int)s;
+      L3.iter = k; L3.symmetric = 0;
       L3.write_q = (!last || keep) ? 1 : 0;
       L3.q = quant_opts(p, 2 * (uint64_t)k + 2);  // both copies of X_{k+1}
       L3.aux_h = k > 0 ? bf16 : 0;   // X_0 is FP32 (or the raw input)
@@ -698,7 +719,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
         L3.upd_decay = upd.decay; L3.upd_step = upd.step;
         L3.no_out = upd.no_out;
       }
-      const ProblemPack* pk = &packs[k == 0 ? 4 : 2 + cur];
+      ProblemPack* pk = &packs[k == 0 ? 4 : 2 + cur];
       ProblemPack last_pack;
       if (last && any_direct) {
         // tall inputs whose result goes straight to the caller's matrix, transposed on the way out
@@ -708,7 +729,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
             GemmProblem& g = last_pack.p[j];
             g.tmOut = mats[j].tm_outT;
             g.out_tr = 1;
-            g.out_rows = (int)pl0.s0; g.out_cols = (int)pl0.l0;
+            g.out_rows = (int)mats[j].pl.s0; g.out_cols = (int)mats[j].pl.l0;
           }
         pk = &last_pack;
       }
@@ -725,13 +746,90 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
     if (direct_out[(size_t)i]) continue;
     if (mats[i].pl.tall) {
       ProfScope ps(FP4_PROF_TRANSPOSE, st);
-      if (launch_transpose_out(mats[i].X, s, l, mats[i].out, pl0.s0, pl0.l0, u, st) != cudaSuccess) return FP4_ERR_CUDA;
+      if (launch_transpose_out(mats[i].X, mats[i].pl.s, mats[i].pl.l, mats[i].out, mats[i].pl.s0, mats[i].pl.l0, u, st) != cudaSuccess) return FP4_ERR_CUDA;
     } else if (u.W && !fused_update[(size_t)i]) {
       ProfScope ps(FP4_PROF_TRANSPOSE, st);
       if (launch_param_update(mats[i].out, mats[i].pl.m * mats[i].pl.n, u, sms, st) != cudaSuccess) return FP4_ERR_CUDA;
     }
   }
   return FP4_OK;
+}
+
+// Matrices of one shape form a group whose stages run as single launches over all of them (many tiles per launch: no idle SMs
+// in a last partial wave, the two CTAs of an SM fall out of step so that main loops and epilogues overlap).  A group has at most
+// `cap` matrices, which bounds the working set competing for L2.
+std::vector<std::vector<MatrixCtx>> group_by_shape(const std::vector<MatrixCtx>& ctx, int cap) {
+  const size_t count = ctx.size();
+  std::vector<char> done(count, 0);
+  std::vector<std::vector<MatrixCtx>> groups;
+  for (size_t i = 0; i < count; ++i) {
+    if (done[i]) continue;
+    groups.emplace_back();
+    std::vector<MatrixCtx>& group = groups.back();
+    for (size_t j = i; j < count && (int)group.size() < cap; ++j) {
+      if (!done[j] && ctx[j].pl.s0 == ctx[i].pl.s0 && ctx[j].pl.l0 == ctx[i].pl.l0) {
+        group.push_back(ctx[j]);
+        done[j] = 1;
+      }
+    }
+  }
+  return groups;
+}
+
+// Groups of different shapes run together where one set of launches over all their tiles is estimated to be the faster: a launch
+// has a start, a last partial wave and, in a prologue, passes of one block that all matrices share.  The groups are ordered by their
+// short side, then the long one, descending (the longest main loops first in a launch's tile list), and neighbours
+// merge, the best pair first.  Measured, the groups one after the other / together: the 14 matrices of two decoder blocks 512 wide (four each of
+// 512 x 512 and 128 x 512, six of 512 x 1536) 310 / 172 us, of one 1024 wide (1024, 256, 2816) 470 / 323, of two 1600 wide (400,
+// 4304) 1425 / 1220, of one 4096 wide (1024, 11008) with the quantiser options 5600 / 5420, the optimiser step around one
+// 3072 wide (8192) 3240 / 3095.  (Single matrices only join a group, they do not form one: for a call of single matrices of many
+// shapes FP4_FLAG_OVERLAP_GROUPS is the faster way, as it has been tested to be.  Six of 1536 x 1536 .. 2816 1177 us, with the
+// option 823; together they would take 540.)  The group of the call's first matrix, whose prologue clears the status word, comes first.
+void merge_groups(std::vector<std::vector<MatrixCtx>>& groups, int cap, int steps, const fp4_ns_params* p, int device_sms, int sms) {
+  if (groups.size() < 2) return;
+  const uint8_t* first = groups[0][0].ws;
+  std::vector<std::vector<WorkShape>> shapes;
+  auto estimate = [&](const std::vector<WorkShape>& w) {
+    const double prologue = prologue_us(w.data(), (int)w.size(), device_sms, sms);
+    return steps > 0 ? prologue + steps * plan_of(w.data(), (int)w.size(), p, sms).iteration_us : prologue;
+  };
+  std::sort(groups.begin(), groups.end(), [](const std::vector<MatrixCtx>& a, const std::vector<MatrixCtx>& b) {
+    return a[0].pl.s != b[0].pl.s ? a[0].pl.s > b[0].pl.s : a[0].pl.l > b[0].pl.l;
+  });
+  std::vector<double> alone, together;   // of every group; of it and the next one
+  for (const auto& g : groups) {
+    shapes.emplace_back();
+    for (const MatrixCtx& c : g) shapes.back().push_back({c.pl.s, c.pl.l});
+    alone.push_back(estimate(shapes.back()));
+  }
+  auto pair_us = [&](size_t i) {
+    if (shapes[i].size() + shapes[i + 1].size() > (size_t)cap || (shapes[i].size() == 1 && shapes[i + 1].size() == 1)) return 1e30;
+    std::vector<WorkShape> w = shapes[i];
+    w.insert(w.end(), shapes[i + 1].begin(), shapes[i + 1].end());
+    return estimate(w);
+  };
+  for (size_t i = 0; i + 1 < groups.size(); ++i) together.push_back(pair_us(i));
+  for (;;) {
+    size_t best = 0;
+    double gain = 0.0;
+    for (size_t i = 0; i + 1 < groups.size(); ++i) {
+      const double saved = alone[i] + alone[i + 1] - together[i];
+      if (saved > gain) { gain = saved; best = i; }
+    }
+    if (gain <= 0.0) break;
+    groups[best].insert(groups[best].end(), groups[best + 1].begin(), groups[best + 1].end());
+    shapes[best].insert(shapes[best].end(), shapes[best + 1].begin(), shapes[best + 1].end());
+    alone[best] = together[best];
+    groups.erase(groups.begin() + best + 1);
+    shapes.erase(shapes.begin() + best + 1);
+    alone.erase(alone.begin() + best + 1);
+    together.erase(together.begin() + best);
+    if (best > 0) together[best - 1] = pair_us(best - 1);
+    if (best + 1 < groups.size()) together[best] = pair_us(best);
+  }
+  for (size_t i = 1; i < groups.size(); ++i)
+    for (const MatrixCtx& c : groups[i])
+      if (c.ws == first) { std::swap(groups[0], groups[i]); return; }
 }
 
 // Enqueue the whole step for one matrix.
@@ -991,25 +1089,8 @@ fp4_status fp4_root_ns_batched(int count, const float* const* G, float* const* o
   }
   uint32_t* status = reinterpret_cast<uint32_t*>(base);  // header of the first matrix
 
-  // Matrices of one shape form a group whose stages run as single launches over all of
-  // them (many tiles per launch: no idle SMs in a last partial wave, the two CTAs of an SM
-  // fall out of step so that main loops and epilogues overlap).  A group is split when it
-  // exceeds max_group matrices, which bounds the working set competing for L2.
   const int cap = p->max_group > 0 && (int)p->max_group < kPackMax ? (int)p->max_group : kDefaultMaxGroup;
-  std::vector<char> done((size_t)count, 0);
-  std::vector<std::vector<MatrixCtx>> groups;
-  for (int i = 0; i < count; ++i) {
-    if (done[(size_t)i]) continue;
-    groups.emplace_back();
-    std::vector<MatrixCtx>& group = groups.back();
-    for (int j = i; j < count && (int)group.size() < cap; ++j) {
-      if (done[(size_t)j]) continue;
-      if (ctx[(size_t)j].pl.s0 == ctx[(size_t)i].pl.s0 && ctx[(size_t)j].pl.l0 == ctx[(size_t)i].pl.l0) {
-        group.push_back(ctx[(size_t)j]);
-        done[(size_t)j] = 1;
-      }
-    }
-  }
+  std::vector<std::vector<MatrixCtx>> groups = group_by_shape(ctx, cap);
   // Groups do not depend on one another.  On request (FP4_FLAG_OVERLAP_GROUPS) they alternate between the
   // caller's stream and a second one that forks from it and joins it again before the call returns: every
   // launch is a persistent grid that ends in a partial wave of tiles, and the next launch of the same
@@ -1017,6 +1098,7 @@ fp4_status fp4_root_ns_batched(int count, const float* const* G, float* const* o
   // are being collected: the event pairs of the two streams would overlap.)
   SideStream* side = (p->flags & FP4_FLAG_OVERLAP_GROUPS) && groups.size() >= 2 && g_prof_on.load() == 0
                          ? side_stream((int)(d - g_dev)) : nullptr;
+  if (!side) merge_groups(groups, cap, steps, p, d->sms, stream_sms(d, stream));
   if (side) {
     // the status word is cleared once, before the fork (a group's own clearing kernel could wipe what
     // a kernel of the other group has just reported)
@@ -1026,7 +1108,7 @@ fp4_status fp4_root_ns_batched(int count, const float* const* G, float* const* o
   }
   for (size_t gi = 0; gi < groups.size(); ++gi) {
     cudaStream_t st = (side && (gi & 1)) ? side->stream : stream;
-    rc = run_group(d, groups[gi].data(), (int)groups[gi].size(), steps, p, status, !side && gi == 0, side != nullptr, st);
+    rc = run_group(d, groups[gi].data(), (int)groups[gi].size(), steps, p, status, !side, side != nullptr, st);
     if (rc != FP4_OK) break;
   }
   if (side) {
@@ -1067,10 +1149,11 @@ static fp4_status gemm_nt_impl(int dry, const uint8_t* a_codes, const uint8_t* a
   pr.tmAux = pr.tmOut;
   pr.sg_a = a_tensor_scale; pr.sg_b = b_tensor_scale;
   pr.out_rows = (int)M; pr.out_cols = (int)N;
+  pr.K = (int)K;
+  pr.blocks_m = (int)(M / 128); pr.blocks_n = (int)(N / 128);
   GemmLaunch L;
   memset(&L, 0, sizeof(L));
   L.num_problems = 1;
-  L.K = (int)K; L.tiles_m = (int)(M / 128); L.tiles_n = (int)(N / 128);
   L.status = device_status;
   L.dry_operands = dry;
   if (dry && (M % 256 || N % 256 || K % 256)) return FP4_ERR_SHAPE;

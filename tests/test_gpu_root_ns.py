@@ -1078,3 +1078,53 @@ def test_groups_on_two_streams_share_the_device():
         times.append(np.median(runs[3:]))
     assert all(torch.equal(a, b) for a, b in zip(*results))
     assert times[1] < 0.9 * times[0], times
+
+
+# matrices of a call, and the launches they take together (prologue, and per iteration 1, 2 or 3 of one or of several shapes)
+MIXED = [
+    ([(256, 512)] * 2 + [(512, 256), (128, 1024), (384, 400), (384, 400)], lambda k: 2),                    # one launch of all iterations
+    ([(400, 1600)] * 2 + [(1600, 1600)] * 2 + [(4304, 1600), (1600, 4304)], lambda k: 6 + 3 * k),          # CTA pairs
+    ([(2048, 4096)] * 2 + [(640, 1024), (1040, 1040), (2304, 1024)], lambda k: 7 + 3 * k),                  # sums of both kinds
+]
+
+
+@pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX, FP4_FLAG_STORE_BF16, FP4_FLAG_KEEP_OPERANDS])
+@pytest.mark.parametrize("shapes,launches", MIXED, ids=["one-launch", "pairs", "both-sums"])
+def test_matrices_of_several_shapes_share_their_launches(shapes, launches, flags):
+    """Groups of different shapes in one set of launches: the bits of single calls, wide and tall, ragged, with what the workspace
+    keeps; no further launches than a call of one shape takes (but a transpose per tall matrix where operands are kept)."""
+    steps = 3
+    Gs = [torch.from_numpy(workloads.gradient_like(*s, seed=i)).cuda() for i, s in enumerate(shapes)]
+    outs = [torch.empty_like(g) for g in Gs]
+    ws = torch.full((fp4.fp4_root_ns_batched_workspace_bytes(shapes, steps, flags),), 0xCD, dtype=torch.uint8, device="cuda")
+    p = fp4.NsParams.make(flags=flags, seed=5)
+    for _ in range(2):
+        before = fp4.fp4_kernel_launches()
+        fp4.fp4_root_ns_batched(Gs, outs, steps, p, ws)
+        count = fp4.fp4_kernel_launches() - before
+        torch.cuda.synchronize()
+        assert fp4.fp4_last_device_status(ws) == 0
+    transposes = sum(m > n for m, n in shapes) if flags & FP4_FLAG_KEEP_OPERANDS else 0
+    assert flags or count == launches(steps)
+    assert count <= launches(steps) + transposes or flags & (FP4_FLAG_STORE_BF16 | FP4_FLAG_RHT)
+    for g, out in zip(Gs, outs):
+        one = torch.empty_like(g)
+        ws1 = torch.empty(fp4.fp4_root_ns_workspace_bytes(*g.shape, steps, flags), dtype=torch.uint8, device="cuda")
+        fp4.fp4_root_ns(g, one, steps, p, ws1)
+        assert torch.equal(one, out), g.shape
+
+
+def test_max_group_bounds_what_runs_together():
+    shapes = [(256, 512)] * 2 + [(384, 512)] * 2
+    Gs = [torch.from_numpy(workloads.gaussian(*s, seed=i)).cuda() for i, s in enumerate(shapes)]
+    outs = [torch.empty_like(g) for g in Gs]
+    ws = torch.empty(fp4.fp4_root_ns_batched_workspace_bytes(shapes, 2, 0), dtype=torch.uint8, device="cuda")
+    counts, results = [], []
+    for cap in (0, 3, 2, 1):
+        before = fp4.fp4_kernel_launches()
+        fp4.fp4_root_ns_batched(Gs, outs, 2, fp4.NsParams.make(max_group=cap), ws)
+        counts.append(fp4.fp4_kernel_launches() - before)
+        results.append([o.clone() for o in outs])
+    assert counts == [2, 4, 4, 8]
+    for r in results[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(r, results[0]))
