@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(256, SR ? 4 : 5) k_momentum_update(const float
     }
     uint2 c_out;
     uint32_t s_out;
-    hadamard16_pairs(m);
+    hadamard16_pairs<false>(m);
     state_encode<SR>(m, seed, (uint64_t)b * 16, c_out, s_out);
     *reinterpret_cast<uint2*>(codes + b * 8) = c_out;
     scales[b] = (uint16_t)s_out;

@@ -14,9 +14,10 @@ __device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t idx) {
   return z ^ (z >> 31);
 }
 
-// v <- v H_16 / 4, the natural-order butterfly of hadamard16 with no signs: the stride-1 stage on
+// v <- v H_16 / 4 (QUARTER; else without the factor), the natural-order butterfly of hadamard16 with no signs: the stride-1 stage on
 // scalars, the strides 2, 4, 8 and the factor 1/4 on packed pairs (v[2k], v[2k+1]); every lane
 // is the same single rounded operation as in the scalar form.
+template <bool QUARTER = true>
 __device__ __forceinline__ void hadamard16_pairs(float (&v)[16]) {
   uint64_t p[8];
 #pragma unroll
@@ -37,7 +38,7 @@ __device__ __forceinline__ void hadamard16_pairs(float (&v)[16]) {
   }
   const uint64_t q = pack2(0.25f, 0.25f);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) unpack2(mul2(p[k], q), v[2 * k], v[2 * k + 1]);
+  for (int k = 0; k < 8; ++k) unpack2(QUARTER ? mul2(p[k], q) : p[k], v[2 * k], v[2 * k + 1]);
 }
 
 // Nearest-rounding codes of one transformed block for the block scale d; returns the sum of the
@@ -102,8 +103,10 @@ __device__ __forceinline__ uint32_t hsub2(uint32_t a, uint32_t b) {
 // [2^-100, 2^100] (zero, negative, gradual underflow, overflow) take the butterfly of the FP32 products.
 // HALF off takes the FP32 butterfly always.  AdamW of 2^26 parameters: 175 us against 181 without; momentum with the histogram
 // of 8192 x 4096, where the counters and not the arithmetic bind: 58 us with, 56 without.
-template <bool HALF>
-__device__ __forceinline__ void mom_decode(uint2 c, uint32_t scale_bits, float (&v)[16]) {
+// ADD: plus `add`, a fused operation with that product, and so rounded once like the sum (`one`: 1, unknown to the compiler, which
+// could fuse a plain sum with a product before it).
+template <bool HALF, bool ADD = false>
+__device__ __forceinline__ void mom_decode(uint2 c, uint32_t scale_bits, float (&v)[16], float add = 0.0f, float one = 1.0f) {
   const float d = __uint_as_float(scale_bits << 16);
   if (HALF && d >= 0x1p-100f && d <= 0x1p100f) {
     uint32_t p[8];
@@ -138,12 +141,12 @@ __device__ __forceinline__ void mom_decode(uint2 c, uint32_t scale_bits, float (
       }
     }
     const float dq = __fmul_rn(d, 0.25f);
-    const uint64_t d2 = pack2(dq, dq);
+    const uint64_t d2 = pack2(dq, dq), add2s = pack2(add, add);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       float a, b;
       half2_to_float2(p[k], a, b);
-      unpack2(mul2(pack2(a, b), d2), v[2 * k], v[2 * k + 1]);
+      unpack2(ADD ? fma2(pack2(a, b), d2, add2s) : mul2(pack2(a, b), d2), v[2 * k], v[2 * k + 1]);
     }
     return;
   }
@@ -155,6 +158,10 @@ __device__ __forceinline__ void mom_decode(uint2 c, uint32_t scale_bits, float (
     unpack2(mul2(pack2(q.x, q.y), d2), v[2 * i], v[2 * i + 1]);
   }
   hadamard16_pairs(v);
+  if (ADD) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __fmaf_rn(v[i], one, add);
+  }
 }
 
 // Nearest-rounding codes of one transformed block for a BF16 block scale d in the normal range, with rcp = RN(1 / d);
@@ -216,16 +223,17 @@ static __device__ __noinline__ uint3 encode_pair_exact(float h0, float h1, float
 
 // Does every element have the same error with both scales, so that the definition's sums are equal?  What makes blocks tie:
 // equal values (d4 = 1.5 d6, see codes_match), or a single magnitude amax beside zeros, midway between 6 d6 and 4 d4.
-__device__ __forceinline__ bool same_errors(const float (&h)[16], float amax, float d6, float d4, uint32_t lo, uint32_t hi, uint32_t lo4,
+__device__ __forceinline__ bool same_errors(const float (&h4)[16], float amax4, float d6, float d4, uint32_t lo, uint32_t hi, uint32_t lo4,
                                             uint32_t hi4) {
   if (d4 == 1.5f * d6) return codes_match(lo, lo4) && codes_match(hi, hi4);
-  bool one = __fmaf_rn(6.0f, d6, 4.0f * d4) == 2.0f * amax;   // exact: sums of 10-bit numbers
+  bool one = __fmaf_rn(6.0f, d6, 4.0f * d4) == 0.5f * amax4;   // exact: sums of 10-bit numbers
 #pragma unroll
-  for (int i = 0; i < 16; ++i) one = one && (h[i] == 0.0f || fabsf(h[i]) == amax);
+  for (int i = 0; i < 16; ++i) one = one && (h4[i] == 0.0f || fabsf(h4[i]) == amax4);
   return one;
 }
 
-// Encodes a transformed block: candidate scales BF16(amax / 6) and BF16(amax / 4), nearest rounding with each, the
+// Encodes a transformed block h = h4 / 4 (the quarter is taken by the reciprocals: a power of two changes no rounding in the
+// normal range): candidate scales BF16(amax / 6) and BF16(amax / 4), nearest rounding with each, the
 // smaller squared error (a tie keeps 6); SR: once more by stochastic rounding with the chosen scale, `first` =
 // the matrix index of the block's first element.  The kernels that call this are bound by the instructions they issue, so the
 // candidates are compared by the errors s6 and s4 of the scaled values, in units of the first scale d.  A scaled value is
@@ -235,14 +243,14 @@ __device__ __forceinline__ bool same_errors(const float (&h)[16], float amax, fl
 // sqrt(S) 2^-16.4 + S 2^-17 + 2^-28.9, whose square is below S (2^-32 + S 2^-32) + 2^-53.  Closer ones, 10^-4 of the blocks,
 // and blocks out of range take the errors of the definition; blocks of few different magnitudes, of which a third can
 // tie exactly because both scales give the same values, keep 6 at once; a block of zeros is all zeros.
-// AdamW of 2^26 parameters, errors of the definition for all blocks / now: 174.3 / 161.9 us; the same gradient every step with one
+// AdamW of 2^26 parameters, errors of the definition for all blocks / as here: 174.3 / 161.9 us; the same gradient every step with one
 // non-zero per block 180 / 180 (without the look at ties 202, with a margin of 2^-14 of max(S, 1/16) 227), constant
 // blocks 174 / 169 (195, 219), new constants every step 174 / 177 (184, 219); blocks out of range 252 / 246.
 template <bool SR>
-__device__ __forceinline__ void state_encode(const float (&h)[16], uint64_t seed, uint64_t first, uint2& c, uint32_t& scale_bits) {
-  const float amax = amax16(h);
+__device__ __forceinline__ void state_encode(const float (&h4)[16], uint64_t seed, uint64_t first, uint2& c, uint32_t& scale_bits) {
+  const float amax4 = amax16(h4), amax = __fmul_rn(amax4, 0.25f);
   uint32_t lo = 0, hi = 0;
-  float d = 0.0f, rcp = 0.0f;
+  float rcp = 0.0f;
   scale_bits = 0;
   bool certain = amax == 0.0f;
   if (amax >= 0x1p-55f && amax <= 0x1p55f) {
@@ -250,40 +258,46 @@ __device__ __forceinline__ void state_encode(const float (&h)[16], uint64_t seed
     const float d6 = bf16_lo(w), d4 = bf16_hi(w);
     const float r6 = rcp_bf16(d6), r4 = rcp_bf16(d4);
     uint32_t lo4, hi4;
-    const float s6 = encode_block16_scaled(h, r6, lo, hi);
+    const float s6 = encode_block16_scaled(h4, 0.25f * r6, lo, hi);
     const float ratio = d4 * r6;
-    const float s4 = encode_block16_scaled(h, r4, lo4, hi4) * (ratio * ratio);
+    const float s4 = encode_block16_scaled(h4, 0.25f * r4, lo4, hi4) * (ratio * ratio);
     const float diff = s4 - s6, S = fmaxf(s4, s6);
     certain = diff * diff > fmaf(S, fmaf(S, 0x1p-32f, 0x1p-32f), 0x1p-53f);
     bool four = diff < 0.0f;
-    if (!certain && same_errors(h, amax, d6, d4, lo, hi, lo4, hi4)) {
+    if (!certain && same_errors(h4, amax4, d6, d4, lo, hi, lo4, hi4)) {
       certain = true;
       four = false;
     }
-    d = d6; rcp = r6;
+    rcp = r6;
     scale_bits = w & 0xFFFFu;
-    if (four) { d = d4; rcp = r4; scale_bits = w >> 16; lo = lo4; hi = hi4; }
+    if (four) { rcp = r4; scale_bits = w >> 16; lo = lo4; hi = hi4; }
   }
-  if (!certain) {
+  // one generator output per 8 elements of the matrix: its low word for the first four
+  auto stochastic = [&](auto&& y) {
+    const uint64_t z0 = splitmix64_at(seed, first >> 3), z1 = splitmix64_at(seed, (first >> 3) + 1);
+    const uint32_t c0 = cvt_rs_e2m1x4(y(0), y(1), y(2), y(3), (uint32_t)z0), c1 = cvt_rs_e2m1x4(y(4), y(5), y(6), y(7), (uint32_t)(z0 >> 32));
+    const uint32_t c2 = cvt_rs_e2m1x4(y(8), y(9), y(10), y(11), (uint32_t)z1);
+    const uint32_t c3 = cvt_rs_e2m1x4(y(12), y(13), y(14), y(15), (uint32_t)(z1 >> 32));
+    lo = c0 | (c1 << 16);
+    hi = c2 | (c3 << 16);
+  };
+  if (certain) {
+    if (SR && scale_bits != 0) {
+      const float r = 0.25f * rcp;
+      stochastic([&](int i) { return __fmul_rn(h4[i], r); });
+    }
+  } else {
+    float h[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) h[i] = __fmul_rn(h4[i], 0.25f);
     const uint3 e = encode_pair_exact(h[0], h[1], h[2], h[3], h[4], h[5], h[6], h[7], h[8], h[9], h[10], h[11], h[12], h[13],
                                       h[14], h[15], amax);
     lo = e.x; hi = e.y; scale_bits = e.z;
-    d = __uint_as_float(scale_bits << 16);
-    rcp = d != 0.0f ? __frcp_rn(d) : 0.0f;
-  }
-  if (SR && d != 0.0f) {
-    // one generator output per 8 elements of the matrix: its low word for the first four
-    const uint64_t z0 = splitmix64_at(seed, first >> 3), z1 = splitmix64_at(seed, (first >> 3) + 1);
-    const uint32_t c0 = cvt_rs_e2m1x4(__fmul_rn(h[0], rcp), __fmul_rn(h[1], rcp), __fmul_rn(h[2], rcp),
-                                      __fmul_rn(h[3], rcp), (uint32_t)z0);
-    const uint32_t c1 = cvt_rs_e2m1x4(__fmul_rn(h[4], rcp), __fmul_rn(h[5], rcp), __fmul_rn(h[6], rcp),
-                                      __fmul_rn(h[7], rcp), (uint32_t)(z0 >> 32));
-    const uint32_t c2 = cvt_rs_e2m1x4(__fmul_rn(h[8], rcp), __fmul_rn(h[9], rcp), __fmul_rn(h[10], rcp),
-                                      __fmul_rn(h[11], rcp), (uint32_t)z1);
-    const uint32_t c3 = cvt_rs_e2m1x4(__fmul_rn(h[12], rcp), __fmul_rn(h[13], rcp), __fmul_rn(h[14], rcp),
-                                      __fmul_rn(h[15], rcp), (uint32_t)(z1 >> 32));
-    lo = c0 | (c1 << 16);
-    hi = c2 | (c3 << 16);
+    const float d = __uint_as_float(scale_bits << 16);
+    if (SR && d != 0.0f) {
+      rcp = __frcp_rn(d);
+      stochastic([&](int i) { return __fmul_rn(h[i], rcp); });
+    }
   }
   c = make_uint2(lo, hi);
 }
