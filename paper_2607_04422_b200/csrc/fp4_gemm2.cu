@@ -272,7 +272,9 @@ __device__ __forceinline__ void stg256(void* p, const uint32_t (&r)[8]) {
 // BH: instantiation with BF16 storage of the FP32 tiles (args.aux_h / args.out_h may be set)
 // UPD: the last G3 stage of a call that also applies Root's parameter update (args.update): every lane
 //   loads the 16 BF16 weights under its row of a chunk (one 32-byte sector, fetched a chunk ahead),
-//   forms W * decay - step * X+ from the values it holds and stores the sector back.
+//   forms W * decay - step * X+ from the values it holds and stores the sector back.  The weights of a tall matrix lie the other way
+//   round, 16 rows of 32 under a chunk: half a warp takes a row, a lane two weights of it, and the values come from the chunk as it
+//   is staged for its transposed store.  (In a transpose pass of its own the update of two 8192 x 3072 took 76 us.)
 template <int MODE, bool PF, bool BH, bool UPD, bool DEEP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ GemmLaunch args) {
@@ -626,9 +628,25 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
       // parameter update: this lane's row of the weight under the tile, one 32-byte piece per chunk
       uint16_t* wrow = nullptr;
       uint32_t wnext[8];
+      // the weights under chunk position e, or their new values
+      auto load_weights = [&](int e) {
+        if (!wrow || x64 + e * CHUNK >= pr->out_cols) return;
+        if (out_tr) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) wnext[q] = *reinterpret_cast<const uint32_t*>(wrow + (int64_t)(e * CHUNK + 2 * q) * pr->W_ld);
+        } else {
+          ldg256(wrow + e * CHUNK, wnext);
+        }
+      };
       if (UPD) {
-        if (pr->W && rows_in && y32 + lane < pr->out_rows) wrow = pr->W + ((int64_t)y32 + lane) * pr->W_ld + x64;
-        if (wrow && x64 + flip * CHUNK < pr->out_cols) ldg256(wrow + flip * CHUNK, wnext);
+        if (pr->W && rows_in) {
+          if (out_tr) {
+            if (y32 + 2 * cq < pr->out_rows) wrow = pr->W + ((int64_t)x64 + g) * pr->W_ld + y32 + 2 * cq;
+          } else if (y32 + lane < pr->out_rows) {
+            wrow = pr->W + ((int64_t)y32 + lane) * pr->W_ld + x64;
+          }
+        }
+        load_weights(flip);
       }
       tc_ld16_issue(tm_acc + flip * CHUNK, acc);
 #pragma unroll
@@ -718,16 +736,13 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(acc_empty_leader);  // done with the buffer
         }
+        uint32_t wcur[8];
+        const bool upd_here = UPD && wrow && xcol < pr->out_cols;
         if (UPD) {
-          uint32_t wcur[8];
 #pragma unroll
           for (int q = 0; q < 8; ++q) wcur[q] = wnext[q];
-          const bool upd_here = wrow && xcol < pr->out_cols;
-          if (i + 1 < TEAM_CHUNKS) {
-            const int e1 = (i + 1) ^ flip;
-            if (wrow && x64 + e1 * CHUNK < pr->out_cols) ldg256(wrow + e1 * CHUNK, wnext);
-          }
-          if (upd_here) {
+          if (i + 1 < TEAM_CHUNKS) load_weights((i + 1) ^ flip);
+          if (upd_here && !out_tr) {
 #pragma unroll
             for (int q = 0; q < 8; ++q)
               wcur[q] = cvt_bf16x2(param_update_value(bf16_lo(wcur[q]), v[2 * q], args.upd_decay, args.upd_step),
@@ -758,6 +773,17 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
           if (TR && out_tr) tma_store_2d_s(&pr->tmOut, y32, xcol, area + boff);
           else tma_store_2d_s(&pr->tmOut, xcol, y32, area + boff);
           bulk_commit();
+        }
+        if (UPD && out_tr && upd_here) {
+          // this lane's two columns of rows g, g + 2, ... of the staged block
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            float a, b;
+            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(a), "=f"(b) : "r"(area + boff + (2 * q + g) * 128 + cq * 8));
+            *reinterpret_cast<uint32_t*>(wrow + (int64_t)(e * CHUNK + 2 * q) * pr->W_ld) =
+                cvt_bf16x2(param_update_value(bf16_lo(wcur[q]), a, args.upd_decay, args.upd_step),
+                           param_update_value(bf16_hi(wcur[q]), b, args.upd_decay, args.upd_step));
+          }
         }
         // ---- quantise along the row
         uint32_t rlo = 0, rhi = 0;

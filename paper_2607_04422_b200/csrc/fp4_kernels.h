@@ -86,7 +86,7 @@ struct alignas(64) GemmProblem {
   int out_rows, out_cols;    // extent of the matrix behind tmOut (chunks that start outside it are not stored)
   int K;                     // contraction length in elements (multiple of 128)
   uint16_t* W;               // kG3 with launch.update: the BF16 parameter (same shape and orientation as the
-  int64_t W_ld;              //   result, row-major, leading dimension in elements) updated with the result; or null
+  int64_t W_ld;              //   caller's result, row-major, leading dimension in elements) updated with it; or null
   int blocks_m, blocks_n;    // extent of the product in blocks of 128 (row lengths of the two quantised outputs: blocks_n, blocks_m)
   float l_cols;              // (float) l, for the bound on amax(A)
   int first_tile, band;      // set by launch_gemm_pair: place in the launch's tile list, tile rows per band of the tile order

@@ -603,11 +603,11 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
   for (int i = 0; i < count; ++i) any_update = any_update || mats[i].W != nullptr;
   std::vector<char> fused_update((size_t)count, 0);
   // a tall input's result leaves the last G3 stage transposed (no transpose pass) unless that stage also has to
-  // write operand copies, or the call updates parameters (the update of a tall matrix rides on the transpose)
+  // write operand copies
   std::vector<char> direct_out((size_t)count, 0);
   bool any_direct = false;
   for (int i = 0; i < count; ++i)
-    if (steps > 0 && mats[i].pl.tall && !keep && !any_update) { direct_out[(size_t)i] = 1; any_direct = true; }
+    if (steps > 0 && mats[i].pl.tall && !keep) { direct_out[(size_t)i] = 1; any_direct = true; }
   const NsPlan& pl0 = mats[0].pl;   // for what does not depend on the shape
   WorkShape shapes[kPackMax];
   int64_t elements = 0;
@@ -652,8 +652,8 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
   }
   if (route == kOneLaunch) {
     for (int j = 0; j < count; ++j) {
-      // the results of tall matrices and the parameter updates are written there, too, unless operand copies are kept
-      if (!keep) { direct_out[(size_t)j] = mats[j].pl.tall; fused_update[(size_t)j] = 1; }
+      // the parameter updates are written there, too, unless operand copies are kept
+      if (!keep) fused_update[(size_t)j] = 1;
     }
     ProfScope ps(FP4_PROF_G3, st);
     if (launch_chain(pack, a, coop_sms, st) != cudaSuccess) return FP4_ERR_CUDA;
@@ -666,13 +666,12 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
         packs[(size_t)kind].p[j] = kind == 0 ? c.g1 : kind == 1 ? c.g2 : kind == 4 ? c.g3_first : c.g3[kind - 2];
       }
     }
-    // Root's parameter update: fused into the last G3 stage of a matrix in the caller's orientation when no
-    // operand copies are wanted from that stage; into the final transpose for a tall matrix; a separate
-    // elementwise pass otherwise (below).
+    // Root's parameter update: fused into the last G3 stage when no operand copies are wanted from that stage; else into the final
+    // transpose for a tall matrix, and a separate elementwise pass otherwise (below).
     if (!keep) {
       for (int kind = 2; kind < 5; ++kind)
         for (int j = 0; j < count; ++j)
-          if (mats[j].W && !mats[j].pl.tall) {
+          if (mats[j].W) {
             packs[(size_t)kind].p[j].W = mats[j].W;
             packs[(size_t)kind].p[j].W_ld = mats[j].pl.n;
             fused_update[(size_t)j] = 1;

@@ -1,7 +1,6 @@
 """Root's parameter update fused into the step (fp4_ns_params.weights): the BF16 parameter is updated from
-the orthogonalised matrix in the epilogue of the last product (CTA-pair kernel, wide or square matrix),
-in the final transpose (tall matrix), or by a separate pass (single-CTA kernel shapes, no iterations,
-FP4_FLAG_KEEP_OPERANDS).  All routes compute W <- BF16(fl(W*fl(1-fl(lr*wd))) - fl(fl(lr*scale)*X_k));
+the orthogonalised matrix in the epilogue of the last product, in the final transpose (tall matrix with
+FP4_FLAG_KEEP_OPERANDS), or by a separate pass (no iterations, FP4_FLAG_KEEP_OPERANDS).  All routes compute W <- BF16(fl(W*fl(1-fl(lr*wd))) - fl(fl(lr*scale)*X_k));
 the oracle applies the same rule to the X_k the GPU returned, so W must agree bit for bit."""
 import numpy as np
 import pytest
@@ -114,3 +113,31 @@ def test_two_chained_optimiser_steps_momentum_root_update(shape):
         assert np.linalg.norm(X - ref) / np.linalg.norm(ref) <= 2e-3
         w_or = oracle.root_param_update(w_or, X, LR, WD, SCALE)
         assert np.array_equal(bits(W), w_or), t
+
+
+@pytest.mark.parametrize("flags", [0, FP4_FLAG_NO_OUT, FP4_FLAG_STORE_BF16, FP4_FLAG_STORE_BF16 | FP4_FLAG_NO_OUT])
+def test_update_of_tall_matrices_in_the_last_product_of_the_cta_pairs(flags):
+    """Tall matrices too large for single launches: tiles that stick out of the matrix on either side (3088 and 4304 rows, 2576 and 2064
+    columns), beside wide ones and one without weights; contractions that take the layout with three stages and the one with four."""
+    shapes = [(3088, 2576), (2576, 3088), (4304, 2064), (4304, 2064), (4240, 4224)]
+    steps = 2
+    Gs = [torch.from_numpy(workloads.gradient_like(m, n, seed=i)).cuda() for i, (m, n) in enumerate(shapes)]
+    for parts in ([0, 1, 2, 3], [4]):
+        sub = [shapes[i] for i in parts]
+        ws = torch.empty(fp4.fp4_root_ns_batched_workspace_bytes(sub, steps, flags), dtype=torch.uint8, device="cuda")
+        plain = [torch.empty_like(Gs[i]) for i in parts]
+        start = fp4.fp4_kernel_launches()
+        fp4.fp4_root_ns_batched([Gs[i] for i in parts], plain, steps, fp4.NsParams.make(flags=flags & FP4_FLAG_STORE_BF16), ws)
+        Ws = [None if i == 3 else make_weight(*shapes[i], 20 + i) for i in parts]
+        w0 = [None if w is None else bits(w).copy() for w in Ws]
+        outs = [torch.full_like(Gs[i], float("nan")) for i in parts]
+        before = fp4.fp4_kernel_launches()
+        fp4.fp4_root_ns_batched([Gs[i] for i in parts], outs, steps,
+                                fp4.NsParams.make(flags=flags, weights=Ws, lr=LR, weight_decay=WD, update_scale=SCALE), ws)
+        assert fp4.fp4_kernel_launches() - before == before - start     # no pass of its own
+        assert fp4.fp4_last_device_status(ws) == 0
+        for w, b, out, ref in zip(Ws, w0, outs, plain):
+            if w is None or not flags & FP4_FLAG_NO_OUT:
+                assert torch.equal(out, ref)
+            if w is not None:
+                assert np.array_equal(bits(w), oracle.root_param_update(b, ref.cpu().numpy(), LR, WD, SCALE))
