@@ -259,6 +259,17 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
   if (warp == W_LOAD) {
     // ------------------------------------------------------------ operand producer
     if (elect_one()) {
+      // until `need` tiles of a matrix are stored
+      auto wait_tiles = [&](const uint32_t* done, uint32_t need) {
+        bool met = ld_acquire(done) >= need;
+        if (met) return;
+        const uint64_t t0 = globaltimer_ns();
+        for (;;) {
+          for (int i = 0; i < 64 && !met; ++i) met = ld_acquire(done) >= need;
+          if (met) break;
+          if (*abort_flag || globaltimer_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; break; }
+        }
+      };
       int st = 0; uint32_t ph = 0, n = 0;
       for (int pi = first; pi < end; ++pi) {
         const int k = pi / 3, mode = pi - 3 * k + kG1;
@@ -271,43 +282,55 @@ k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLau
           const ChainProblem& pr = pack.p[p];
           const int K = sh->depth[mode - kG1][j] * 128;
           const int num_kb = (K + BK - 1) / BK;
-          // tiles of the matrix's earlier products (SYM: what the launches before have left is complete)
-          const uint32_t need = SYM ? (mode == kG1 ? 0u : (uint32_t)((2 * k + 1) * pr.nsym))
-                                    : (uint32_t)(k * (2 * pr.nsym + (pr.s / BM) * (pr.l / BN)) + (mode - kG1) * pr.nsym);
-          if (p != seen && need != 0) {
-            // all tiles of the matrix's earlier products are stored
-            bool met = ld_acquire(pr.done) >= need;
-            if (!met) {
-              const uint64_t t0 = globaltimer_ns();
-              for (;;) {
-                for (int i = 0; i < 64 && !met; ++i) met = ld_acquire(pr.done) >= need;
-                if (met) break;
-                if (*abort_flag || globaltimer_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; break; }
-              }
-            }
-          }
-          seen = p;
-          mbar_arrive(&sh->dep[n % DEP_RING]);
           const CUtensorMap* ma = mode == kG1 ? &pr.tm_qX : mode == kG2 ? &pr.tm_qA : &pr.tm_qB;
           const CUtensorMap* mb = mode == kG1 ? &pr.tm_qX : mode == kG2 ? &pr.tm_qA : &pr.tm_qXt[k & 1];
           const uint8_t* sfa = (mode == kG1 ? pr.qx_sf : mode == kG2 ? pr.qa_sf : pr.qb_sf) + (size_t)ti * (K / 64) * 512;
           const uint8_t* sfb = (mode == kG1 ? pr.qx_sf : mode == kG2 ? pr.qa_sf : pr.qt_sf[k & 1]) +
                                (size_t)(tj * BN / 128) * (K / 64) * 512;
-          for (int kb = 0; kb < num_kb; ++kb) {
-            wait_or_abort(&sh->empty[st], ph ^ 1, abort_flag);
-            // a half-full last stage: the operand boxes are zero-filled beyond K (and still credit their full
-            // size), only the scale atoms that exist are fetched
-            const int kvalid = K - kb * BK < BK ? K - kb * BK : BK;
-            const uint32_t sf_bytes = (uint32_t)(kvalid / 64) * 512;
-            uint8_t* d = smem + st * L::STAGE_BYTES;
-            mbar_expect_tx(&sh->full[st], L::A_BYTES + L::B_BYTES + 2 * sf_bytes);
-            tma_load_2d(d, ma, kb * (BK / 2), ti * BM, &sh->full[st]);
-            tma_load_2d(d + L::A_BYTES / 2, ma, kb * (BK / 2), ti * BM + 64, &sh->full[st]);
+          // A half-full last stage: the operand boxes are zero-filled beyond K (and still credit their full
+          // size), only the scale atoms that exist are fetched.
+          auto sf_bytes = [&](int kb) { return (uint32_t)((K - kb * BK < BK ? K - kb * BK : BK) / 64) * 512; };
+          auto load_rows = [&](int s_, int kb) {
+            uint8_t* d = smem + s_ * L::STAGE_BYTES;
+            tma_load_2d(d, ma, kb * (BK / 2), ti * BM, &sh->full[s_]);
+            tma_load_2d(d + L::A_BYTES / 2, ma, kb * (BK / 2), ti * BM + 64, &sh->full[s_]);
+            bulk_load_1d(d + L::A_BYTES + L::B_BYTES, sfa + (size_t)kb * L::SF_BYTES, sf_bytes(kb), &sh->full[s_]);
+          };
+          auto load_cols = [&](int s_, int kb) {
+            uint8_t* d = smem + s_ * L::STAGE_BYTES;
+            mbar_expect_tx(&sh->full[s_], L::A_BYTES + L::B_BYTES + 2 * sf_bytes(kb));
 #pragma unroll
             for (int h = 0; h < BN / 64; ++h)
-              tma_load_2d(d + L::A_BYTES + h * (64 * BK / 2), mb, kb * (BK / 2), tj * BN + h * 64, &sh->full[st]);
-            bulk_load_1d(d + L::A_BYTES + L::B_BYTES, sfa + (size_t)kb * L::SF_BYTES, sf_bytes, &sh->full[st]);
-            bulk_load_1d(d + L::A_BYTES + L::B_BYTES + L::SF_BYTES, sfb + (size_t)kb * L::SF_BYTES, sf_bytes, &sh->full[st]);
+              tma_load_2d(d + L::A_BYTES + h * (64 * BK / 2), mb, kb * (BK / 2), tj * BN + h * 64, &sh->full[s_]);
+            bulk_load_1d(d + L::A_BYTES + L::B_BYTES + L::SF_BYTES, sfb + (size_t)kb * L::SF_BYTES, sf_bytes(kb), &sh->full[s_]);
+          };
+          // tiles of the matrix's earlier products (SYM: what the launches before have left is complete)
+          const uint32_t before = (uint32_t)(k * (2 * pr.nsym + (pr.s / BM) * (pr.l / BN)));
+          const uint32_t need = SYM ? (mode == kG1 ? 0u : (uint32_t)((2 * k + 1) * pr.nsym)) : before + (uint32_t)((mode - kG1) * pr.nsym);
+          int ahead = 0;
+          if (p != seen && need != 0) {
+            if (!SYM && mode == kG3) {
+              // The column operand of G3 comes from the iteration before: its first stages are fetched while B is still under way.
+              // 1024 x 1024 101.7 -> 99.8 us, 256 x 512 82.9 -> 82.2, 1040 x 2896 with options 186.2 -> 184.4, 2048 x 2048 196.4 -> 195.9.
+              if (before != 0) wait_tiles(pr.done, before);
+              ahead = num_kb < STAGES ? num_kb : STAGES;
+              int s_ = st; uint32_t ph_ = ph;
+              for (int kb = 0; kb < ahead; ++kb) {
+                wait_or_abort(&sh->empty[s_], ph_ ^ 1, abort_flag);
+                load_cols(s_, kb);
+                if (++s_ == STAGES) { s_ = 0; ph_ ^= 1; }
+              }
+            }
+            wait_tiles(pr.done, need);
+          }
+          seen = p;
+          mbar_arrive(&sh->dep[n % DEP_RING]);
+          for (int kb = 0; kb < num_kb; ++kb) {
+            if (kb >= ahead) {
+              wait_or_abort(&sh->empty[st], ph ^ 1, abort_flag);
+              load_cols(st, kb);
+            }
+            load_rows(st, kb);
             if (++st == STAGES) { st = 0; ph ^= 1; }
           }
         }
