@@ -305,7 +305,7 @@ k_gemm_pair(const __grid_constant__ ProblemPack pack, const __grid_constant__ Ge
   // instruction stream, same epilogue.
   const bool dry = (MODE == kPlain) && args.dry_operands != 0;
 
-  pdl_launch_dependents();
+  if (!UPD) pdl_launch_dependents();   // (the last of a call: what comes next would take the SMs that drain first)
   if (threadIdx.x == 0) {
     for (int i = 0; i < STAGES; ++i) { mbar_init(&bars->full[i], 1); mbar_init(&bars->empty[i], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&bars->acc_full[i], 1); mbar_init(&bars->acc_empty[i], 2 * EPI_WARPS); }

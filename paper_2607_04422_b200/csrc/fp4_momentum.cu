@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(256, SR ? 4 : 5) k_momentum_update(const float
     for (int i = threadIdx.x; i < kMomBins; i += blockDim.x) sh[i] = 0;
     __syncthreads();
   }
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const uint64_t mu2 = pack2(mu, mu), gs2 = pack2(g_scale, g_scale);
   for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nblocks; b += stride) {
@@ -111,8 +112,13 @@ cudaError_t launch_update(const float* G, int64_t nblocks, float mu, float g_sca
     const int64_t iters = (units + slots - 1) / slots;
     grid = (units + iters - 1) / iters;
   }
-  k_momentum_update<SR, HIST><<<(unsigned)grid, 256, 0, st>>>(G, nblocks, mu, g_scale, seed, codes, scales, M_out,
-                                                              hist);
+  // Chained: the launch and the clearing of the counters overlap with the kernel before.  The kernel itself lets none start early:
+  // the successor's blocks would fill what room is left on some SMs and be spread unevenly.  With histogram and stochastic rounding,
+  // plain / chained / with early successors: 2048 x 2048 12.6 / 11.3 / 11.1 us, 8192 x 4096 55.7 / 53.2 / 56.5 (to nearest 54.0 / 51.6 / 61);
+  // the optimiser step on a decoder block 768 wide 283 / 265 / 264, 1024 wide 420 / 403 / 405, 1600 wide 996 / 982 / 1003.
+  pdl_select(0);
+  launch_chained(k_momentum_update<SR, HIST>, dim3((unsigned)grid), dim3(256), 0, st, G, nblocks, mu, g_scale, seed, codes, scales, M_out,
+                 hist);
   count_launches(1);
   return cudaGetLastError();
 }
