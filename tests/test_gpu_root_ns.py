@@ -1128,3 +1128,32 @@ def test_max_group_bounds_what_runs_together():
     assert counts == [2, 4, 4, 8]
     for r in results[1:]:
         assert all(torch.equal(a, b) for a, b in zip(r, results[0]))
+
+
+@pytest.mark.parametrize("clip_quantile", [0.99, 0.0])
+@pytest.mark.parametrize("shape", [(16, 16), (128, 256), (256, 272), (640, 128), (1152, 128), (400, 512), (512, 512)])
+def test_prologue_of_one_cluster_is_that_of_the_cooperative_launch(shape, clip_quantile):
+    """1, 2, 6, 5, 9 and 16 tiles of 128 x 128 (clusters of 1 to 16 blocks, some without a tile) on their own, and beside enough others
+    for the cooperative launch: same bits, with a zero matrix and one of equal magnitudes (the list of candidates overflows) among
+    them; several matrices in one cluster."""
+    tiles = -(-shape[0] // 128) * -(-shape[1] // 128)
+    gen = torch.Generator(device="cuda").manual_seed(sum(shape))
+    Gs = [torch.randn(shape, device="cuda", generator=gen) for _ in range(max(3, 17 // tiles + 1))]
+    Gs[1] = torch.zeros_like(Gs[1])
+    Gs[2] = torch.sign(Gs[2]) * 0.5
+    for steps, flags in ((0, FP4_FLAG_KEEP_OPERANDS), (2, 0), (2, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)):
+        p = fp4.NsParams.make(flags=flags, seed=2, clip_quantile=clip_quantile)
+        results = []
+        for parts in ([[i] for i in range(len(Gs))], [list(range(16 // tiles))], [list(range(len(Gs)))]):
+            outs = {}
+            for part in parts:
+                ws = torch.full((fp4.fp4_root_ns_batched_workspace_bytes([shape] * len(part), steps, flags),), 0xAB, dtype=torch.uint8,
+                                device="cuda")
+                out = [torch.full_like(Gs[i], float("nan")) for i in part]
+                fp4.fp4_root_ns_batched([Gs[i] for i in part], out, steps, p, ws)
+                assert fp4.fp4_last_device_status(ws) == 0
+                outs.update(zip(part, out))
+            results.append(outs)
+        for outs in results:
+            for i, out in outs.items():
+                assert torch.equal(out, results[2][i]), (i, steps, flags)
