@@ -168,8 +168,9 @@ struct WorkShape { int64_t s, l; };
 double chain_iteration_us(const WorkShape* shapes, int count, bool opts, int sms);
 double prologue_us(const WorkShape* shapes, int count, int device_sms, int coop_sms);
 double chain_symmetric_us(const WorkShape* shapes, int count, bool opts, int sms);
-cudaError_t launch_chain(ChainPack& pack, const ChainLaunch& launch, int sms, cudaStream_t st);
-cudaError_t launch_chain_symmetric(ChainPack& pack, const ChainLaunch& launch, int step, int sms, cudaStream_t st);
+// sms: those to count on; whole_device: the stream's kernels can occupy all of the device's
+cudaError_t launch_chain(ChainPack& pack, const ChainLaunch& launch, int sms, bool whole_device, cudaStream_t st);
+cudaError_t launch_chain_symmetric(ChainPack& pack, const ChainLaunch& launch, int step, int sms, bool whole_device, cudaStream_t st);
 
 // Measurement support: counts kernel launches and, when profiling is on, brackets a group of
 // launches with events.

@@ -1080,6 +1080,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
     }
   };
   if (CLUSTER) {
+    pdl_launch_dependents();
     pdl_wait();
     if (mine == 0) {   // a cluster has a power of two of blocks
       for (int i = 0; i < (g.clip ? 3 : 2); ++i) all_blocks();

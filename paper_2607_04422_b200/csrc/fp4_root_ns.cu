@@ -656,7 +656,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       if (!keep) fused_update[(size_t)j] = 1;
     }
     ProfScope ps(FP4_PROF_G3, st);
-    if (launch_chain(pack, a, coop_sms, st) != cudaSuccess) return FP4_ERR_CUDA;
+    if (launch_chain(pack, a, coop_sms, sms == d->sms, st) != cudaSuccess) return FP4_ERR_CUDA;
   } else if (steps > 0) {
     // the problems of the five kinds of launches: G1, G2, G3 reading qXt[0] / qXt[1], the first G3
     std::vector<ProblemPack> packs(5);
@@ -693,7 +693,7 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       L1.out_h = bf16;
       if (route == kTwoLaunches) {
         ProfScope ps(FP4_PROF_G1, st);
-        if (launch_chain_symmetric(pack, a, k, coop_sms, st) != cudaSuccess) return FP4_ERR_CUDA;
+        if (launch_chain_symmetric(pack, a, k, coop_sms, sms == d->sms, st) != cudaSuccess) return FP4_ERR_CUDA;
       } else {
         ProfScope ps(FP4_PROF_G1, st);
         if (launch_gemm_pair(kG1, packs[0], L1, sms, st) != cudaSuccess)
