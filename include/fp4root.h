@@ -183,9 +183,8 @@ fp4_status fp4_root_coeffs(int64_t m, int64_t n, int steps, float abc[3]);
  *   transposed from the last product).  Groups of up to a few million elements run all
  *   iterations in one cooperative launch instead, whose blocks wait on one another (bounded
  *   waits); somewhat larger ones (short sides up to 2048) run two of the three products of an
- *   iteration in such a launch.  Calls on small matrices (up to 8 M elements per group
- *   of equal shapes) chain their other kernels with programmatic dependent launch; the environment
- *   variable FP4ROOT_NO_PDL (any value) switches that off.  Kernels launched before or after
+ *   iteration in such a launch.  Short kernels are chained with programmatic dependent launch;
+ *   the environment variable FP4ROOT_NO_PDL (any value) switches that off.  Kernels launched before or after
  *   the call on the same stream see ordinary stream order either way.
  *   A cooperative launch starts when all its blocks - up to one per SM, each with most of an SM's shared
  *   memory - can be resident at once: beside a long kernel on another stream it waits for

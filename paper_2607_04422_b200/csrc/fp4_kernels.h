@@ -178,10 +178,10 @@ void count_launches(int n);
 
 // Launch of a kernel of the Newton-Schulz chain: with the programmatic-stream-serialisation attribute (the
 // kernel's blocks may become resident before the previous launch has completed; the kernel itself waits,
-// see pdl_wait) for the groups of a call that are bound by launch latency (pdl_select, called per group),
+// see pdl_wait) where pdl_select has switched that on,
 // unless the environment variable FP4ROOT_NO_PDL is set.
 bool pdl_enabled();
-void pdl_select(int64_t group_elements);
+void pdl_select(bool on);
 template <typename... KArgs, typename... Args>
 cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};

@@ -116,7 +116,7 @@ cudaError_t launch_update(const float* G, int64_t nblocks, float mu, float g_sca
   // the successor's blocks would fill what room is left on some SMs and be spread unevenly.  With histogram and stochastic rounding,
   // plain / chained / with early successors: 2048 x 2048 12.6 / 11.3 / 11.1 us, 8192 x 4096 55.7 / 53.2 / 56.5 (to nearest 54.0 / 51.6 / 61);
   // the optimiser step on a decoder block 768 wide 283 / 265 / 264, 1024 wide 420 / 403 / 405, 1600 wide 996 / 982 / 1003.
-  pdl_select(0);
+  pdl_select(true);
   launch_chained(k_momentum_update<SR, HIST>, dim3((unsigned)grid), dim3(256), 0, st, G, nblocks, mu, g_scale, seed, codes, scales, M_out,
                  hist);
   count_launches(1);

@@ -320,7 +320,7 @@ cudaError_t launch_quantize(const CUtensorMap* tm, const float* x, int64_t rows,
   cudaError_t e = cudaMemsetAsync(tensor_scale, 0, 4, st);
   if (e != cudaSuccess) return e;
   // chained: a kernel's blocks become resident while the one before drains (8192 x 8192: 96 -> 92.5 us)
-  pdl_select(0);
+  pdl_select(true);
   uint32_t* amax = reinterpret_cast<uint32_t*>(tensor_scale);
   launch_chained(k_amax, dim3(grid_for(n4, 256 * 8, sms)), dim3(256), 0, st, reinterpret_cast<const float4*>(x), n4, amax);
   const dim3 qgrid((unsigned)rows, (unsigned)((cols / 16 + 255) / 256));

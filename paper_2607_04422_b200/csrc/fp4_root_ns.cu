@@ -26,9 +26,9 @@ std::mutex g_prof_mu;
 
 void count_launches(int n) { g_launches.fetch_add((uint64_t)n, std::memory_order_relaxed); }
 
-// Programmatic dependent launch pays where a call is bound by launch latency (a 5-iteration call on one
-// 512 x 512 .. 2048 x 2048 matrix: 0.22 -> 0.19, 0.25 -> 0.21, 0.28 -> 0.25 ms) and measured 2 % slower on
-// groups that fill the machine for milliseconds, so each group of a call decides by its size.
+// Programmatic dependent launch hides a launch behind the kernel before, but a successor's blocks take the SMs as they drain: where
+// launches fill the machine for long, the CTA pairs of the next one then lie less favourably.  So each part of a call decides
+// (run_group).
 namespace {
 thread_local bool t_pdl_group = false;
 }
@@ -36,7 +36,7 @@ bool pdl_enabled() {
   static const bool allowed = getenv("FP4ROOT_NO_PDL") == nullptr;
   return allowed && t_pdl_group;
 }
-void pdl_select(int64_t group_elements) { t_pdl_group = group_elements <= (int64_t)8 << 20; }
+void pdl_select(bool on) { t_pdl_group = on; }
 
 ProfScope::ProfScope(int cls_, cudaStream_t st_) : cls(cls_), st(st_), e0(nullptr), on(g_prof_on.load() != 0) {
   if (on) {
@@ -621,7 +621,6 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
   // 2816) 1177 / 1160 / 834 us, eight of one (640 x 640 .. 1536) 885 / 680 / 490, six of two (1280 x 1280 .. 2560)
   // 1197 / 1184 / 996, eight tiny ones 780 / 405 / 407; four groups of four with the quantiser options lose (1323 / 1447).
   const int sms = stream_sms(d, st), coop_sms = two_streams && sms > 1 ? sms / 2 : sms;
-  pdl_select(elements);
   const Route route = steps > 0 ? plan_of(shapes, count, p, coop_sms).route : kThreeLaunches;
   {
     std::vector<PrologueItem> items((size_t)count);
@@ -630,9 +629,17 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       items[(size_t)i] = PrologueItem{c.G, c.X, c.ws, &c.pl, clear_status && reinterpret_cast<uint32_t*>(c.ws + c.pl.lay.header) == status, c.store_x0, c.x_rows, c.x_cols,
                                       c.hist_top, &c.tm_G};
     }
+    pdl_select(true);   // its launches are short: 8192 x 2048 413 -> 406 us, 1536 x 8192 345 -> 334, two blocks of a stack none
     if (launch_prologue_group(items.data(), count, steps > 0 || keep, quant_opts(p, 0), status, coop_sms, sms, st) != cudaSuccess)
       return FP4_ERR_CUDA;
   }
+  // The stages: always where two short launches make an iteration (2048 x 8192, chained / plain, 396 / 406 us, with options 548 / 560,
+  // 2048 x 16384 681 / 690, 1024 x 30720 720 / 729); with three up to some 13 M elements (2304 x 4096 312 / 324, 3072 x 3072 373 / 391,
+  // 3072 x 4096 444 / 454, 3584 x 3584 466 / 475, 2560 x 5120 394 / 394; but 2304 x 6144 408 / 389, 2560 x 8192 545 / 526, 4096 x 4096
+  // 610 / 600, one decoder block 1536 wide 581 / 566), with the quantiser options 8 M (2560 x 3200 438 / 438, 3072 x 4096
+  // 654 / 622, 4096 x 4096 814 / 738).
+  const bool opts = (p->flags & (FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX)) != 0;
+  pdl_select(route != kThreeLaunches || elements <= (opts ? (int64_t)8 << 20 : (int64_t)25 << 19));
   ChainPack pack;
   ChainLaunch a;
   if (route != kThreeLaunches) {
@@ -1128,7 +1135,7 @@ fp4_status fp4_last_device_status(const void* ws, cudaStream_t stream) {
 static fp4_status gemm_nt_impl(int dry, const uint8_t* a_codes, const uint8_t* a_scales, float a_tensor_scale,
                        const uint8_t* b_codes, const uint8_t* b_scales, float b_tensor_scale, int64_t M, int64_t N,
                        int64_t K, float* D, uint32_t* device_status, cudaStream_t stream) {
-  pdl_select(INT64_MAX);  // a single product: plain launch
+  pdl_select(false);  // a single product: plain launch
   if (!a_codes || !a_scales || !b_codes || !b_scales || !D) return FP4_ERR_INVALID_ARG;
   if (!shape_ok(M) || !shape_ok(N) || !shape_ok(K)) return FP4_ERR_SHAPE;
   if (!aligned(a_codes, 16) || !aligned(a_scales, 16) || !aligned(b_codes, 16) || !aligned(b_scales, 16) ||
