@@ -208,9 +208,9 @@ __device__ __noinline__ void chain_update_tall(uint16_t* w, int64_t ld, const fl
 }
 
 // SYM: the products [a.first, a.end) only, G1 and G2 of an iteration (loop bounds the compiler cannot unroll by); else all products of all iterations
-template <int BN, bool PF, bool SYM>
+template <int BN, bool PF, bool SYM, int MAX>
 __global__ void __launch_bounds__(NTHREADS, 1)
-k_chain(const __grid_constant__ ChainPack pack, const __grid_constant__ ChainLaunch a) {
+k_chain(const __grid_constant__ ChainPackOf<MAX> pack, const __grid_constant__ ChainLaunch a) {
   using L = ChainLay<BN>;
   constexpr int STAGES = L::STAGES;
   extern __shared__ uint8_t smem_raw[];
@@ -911,7 +911,8 @@ cudaError_t launch_one(const ChainPack& pack, const ChainLaunch& a, int grid, bo
     cfg.numAttrs = 1;
   }
   count_launches(1);
-  return cudaLaunchKernelEx(&cfg, k_chain<BN, PF, SYM>, pack, a);
+  if (a.count == 1) return cudaLaunchKernelEx(&cfg, k_chain<BN, PF, SYM, 1>, ChainPackOf<1>{{pack.p[0]}}, a);
+  return cudaLaunchKernelEx(&cfg, k_chain<BN, PF, SYM, kChainMax>, pack, a);
 }
 
 int64_t sym_tiles(int64_t s, int bn) {
@@ -922,9 +923,9 @@ int64_t sym_tiles(int64_t s, int bn) {
 int64_t rounds(int64_t tiles, int sms) { return (tiles + sms - 1) / sms; }
 }  // namespace
 
-template <int BN, bool PF, bool SYM>
+template <int BN, bool PF, bool SYM, int MAX>
 static cudaError_t chain_set_attribute(int dev) {
-  const auto kernel = k_chain<BN, PF, SYM>;
+  const auto kernel = k_chain<BN, PF, SYM, MAX>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainLay<BN>::SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
@@ -944,6 +945,11 @@ static cudaError_t chain_set_attribute(int dev) {
   if (blocks < 8) blocks = 0;
   if (blocks < g_cluster_blocks[dev]) g_cluster_blocks[dev] = blocks;
   return cudaSuccess;
+}
+template <int BN, bool PF, bool SYM>
+static cudaError_t chain_set_attribute(int dev) {
+  const cudaError_t e = chain_set_attribute<BN, PF, SYM, 1>(dev);
+  return e != cudaSuccess ? e : chain_set_attribute<BN, PF, SYM, kChainMax>(dev);
 }
 cudaError_t chain_set_attributes() {
   int dev = 0;
