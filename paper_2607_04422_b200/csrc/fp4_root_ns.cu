@@ -629,7 +629,9 @@ fp4_status run_group(const DeviceInfo* d, MatrixCtx* mats, int count, int steps,
       items[(size_t)i] = PrologueItem{c.G, c.X, c.ws, &c.pl, clear_status && reinterpret_cast<uint32_t*>(c.ws + c.pl.lay.header) == status, c.store_x0, c.x_rows, c.x_cols,
                                       c.hist_top, &c.tm_G};
     }
-    pdl_select(true);   // its launches are short: 8192 x 2048 413 -> 406 us, 1536 x 8192 345 -> 334, two blocks of a stack none
+    // Up to 64 M elements the launches of the prologue are short: 8192 x 2048 413 -> 406 us, 1536 x 8192 345 -> 334, a decoder block
+    // 2048 wide (44 M) 1009 -> 995; the 28 matrices of four blocks 3072 wide 10.22 -> 10.24 ms.
+    pdl_select(elements <= (int64_t)64 << 20);
     if (launch_prologue_group(items.data(), count, steps > 0 || keep, quant_opts(p, 0), status, coop_sms, sms, st) != cudaSuccess)
       return FP4_ERR_CUDA;
   }
