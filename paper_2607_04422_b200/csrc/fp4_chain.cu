@@ -1,5 +1,5 @@
-// All iterations of the Newton-Schulz step (Section 3.4, display equations) for a small group of equal-shape
-// matrices in ONE cooperative launch.
+// All iterations of the Newton-Schulz step (Section 3.4, display equations) for a small group of
+// matrices, of one or of several shapes, in ONE launch (cooperative, or a single cluster).
 //
 // A matrix of up to a few million elements has fewer 256 x 256 tiles than the GPU has SM pairs, and with a
 // launch per product its time is launch latency, cold instruction fetches and the epilogue of one large tile.
@@ -35,7 +35,7 @@
 // with the quantiser options 137.6 -> 115.8, 1040 x 2896 212 -> 187; G1 and G2 of 2048 x 6144 with options 510 -> 470.
 // With the proxy fence on the reading side and one lane storing everything the iterations of 256 x 512 took 87 us
 // instead of 78, of 1408 x 2176 156 instead of 141.  Whole calls against three launches per iteration: 256 x 512
-// 152 -> 83 us, 1024 x 1024 178 -> 102, 1040 x 2896 with the paper's quantiser options 300 -> 186.
+// 152 -> 74 us, 1024 x 1024 178 -> 101, 1040 x 2896 with the paper's quantiser options 300 -> 186.
 #include "fp4_gemm_common.cuh"
 
 namespace fp4 {
