@@ -1068,7 +1068,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
   ResidentShared* sh = reinterpret_cast<ResidentShared*>(uni + kResUnion);
   volatile uint32_t* abort_flag = &sh->abort_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int mine = (g.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // 1 .. kResTiles
+  const int mine = (g.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // 1 .. kResTiles (CLUSTER: 0 or 1)
   uint32_t* counter = &g.mat[0].hdr->barrier;
   uint32_t round = 0;
   auto all_blocks = [&]() {
@@ -1082,10 +1082,6 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
   if (CLUSTER) {
     pdl_launch_dependents();
     pdl_wait();
-    if (mine == 0) {   // a cluster has a power of two of blocks
-      for (int i = 0; i < (g.clip ? 3 : 2); ++i) all_blocks();
-      return;
-    }
   }
   if (tid == 0) {
     for (int i = 0; i < kResTiles; ++i) mbar_init(&sh->full[i], 1);
@@ -1107,6 +1103,10 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
     for (int i = (g.mat[j].clear_status ? 0 : 4) + (int)blockIdx.x * kPrepThreads + tid; i < g.zero_words;
          i += (int)gridDim.x * kPrepThreads)
       if (i != kBarrierWord) w[i] = 0;
+  }
+  if (CLUSTER && mine == 0) {   // a cluster has a power of two of blocks: one without a tile clears its share, too
+    for (int i = 0; i < (g.clip ? 3 : 2); ++i) all_blocks();
+    return;
   }
   __syncthreads();
   // a thread's four 16-byte pieces of a tile: columns 4 lane .. 4 lane + 3 of rows warp, warp + 32, ...; f(value)

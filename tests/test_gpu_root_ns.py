@@ -1157,3 +1157,43 @@ def test_prologue_of_one_cluster_is_that_of_the_cooperative_launch(shape, clip_q
         for outs in results:
             for i, out in outs.items():
                 assert torch.equal(out, results[2][i]), (i, steps, flags)
+
+
+@pytest.mark.parametrize("tiles", range(1, 17))
+def test_prologue_of_one_cluster_counts_from_zero(tiles):
+    """Every number of tiles of 128 x 128 that one cluster takes (blocks without a tile wherever it is no power of two), as one wide,
+    tall or ragged matrix and as several matrices; magnitudes whose counters lie all over the histogram; workspaces full of garbage,
+    used twice, and the library's own.  tau is the oracle's, the bits are those of the cooperative launch over several such matrices."""
+    cases = [[(128, 128 * tiles)], [(128 * tiles, 128)], [(112, 128 * tiles - 48)], [(128, 128)] * tiles]
+    for shapes in cases if tiles > 1 else cases[:3]:
+        for scale in (2.0 ** -60, 2.0 ** -26, 1.0, 2.0 ** 12, 2.0 ** 50):
+            rng = np.random.default_rng(tiles)
+            calls = []
+            for _ in range(2):
+                mats = [(scale * rng.standard_normal(s)).astype(np.float32) for s in shapes]
+                calls.append((mats, [oracle.root_ns(g, steps=0, trace_iter=0)[1] for g in mats]))
+            for fill in (0xAB, 0xFF):
+                ws = torch.full((fp4.fp4_root_ns_batched_workspace_bytes(shapes, 0),), fill, dtype=torch.uint8, device="cuda")
+                for mats, traces in calls:
+                    Gs = [torch.from_numpy(g).cuda() for g in mats]
+                    outs = [torch.full_like(g, float("nan")) for g in Gs]
+                    before = fp4.fp4_kernel_launches()
+                    fp4.fp4_root_ns_batched(Gs, outs, 0, None, ws)
+                    assert fp4.fp4_kernel_launches() - before == 1 + sum(m > n for m, n in shapes)
+                    assert fp4.fp4_last_device_status(ws) == 0
+                    off = 0
+                    for g, tr in zip(mats, traces):
+                        lay = fp4_root_ns_workspace_layout(*g.shape, 0, 0)
+                        sc = ws[off + lay.scalars:off + lay.scalars + 4096].cpu().numpy().view(np.float32)
+                        assert sc[lay.idx_tau] == np.float32(tr["tau"]), (shapes, scale, fill)
+                        assert abs(sc[lay.idx_nu] - tr["nu"]) <= 1.2e-7 * tr["nu"]
+                        off += -(-lay.total // 1024) * 1024
+                    if len(shapes) > 1 or tiles == 1:
+                        continue
+                    own = torch.full_like(Gs[0], float("nan"))
+                    fp4.fp4_root_ns_static(Gs[0], own, 0)
+                    count = 16 // tiles + 1
+                    many = [torch.full_like(own, float("nan")) for _ in range(count)]
+                    ws_many = torch.full((count * ws.numel(),), fill, dtype=torch.uint8, device="cuda")
+                    fp4.fp4_root_ns_batched(Gs * count, many, 0, None, ws_many)
+                    assert torch.equal(own, outs[0]) and all(torch.equal(o, outs[0]) for o in many), (shapes, scale, fill)
