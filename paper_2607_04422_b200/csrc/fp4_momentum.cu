@@ -33,7 +33,7 @@ constexpr int kMomBins = 8192;
 // grid: any number of thread blocks; threads stride over the 16-blocks of the matrix.  48 registers without stochastic rounding:
 // five thread blocks per SM instead of four, 34.9 -> 32.0 us for the state alone of 8192 x 4096.
 template <bool SR, bool HIST>
-__global__ void __launch_bounds__(256, SR ? 4 : 5) k_momentum_update(const float* __restrict__ G, int64_t nblocks, float mu,
+__global__ void __launch_bounds__(256, SR ? 4 : 5) k_momentum_update(const float* G, int64_t nblocks, float mu,
                                                          float g_scale, uint64_t seed, uint8_t* codes,
                                                          uint16_t* scales, float* __restrict__ M_out,
                                                          uint32_t* __restrict__ hist) {
@@ -49,8 +49,8 @@ __global__ void __launch_bounds__(256, SR ? 4 : 5) k_momentum_update(const float
     const uint2 c_in = *reinterpret_cast<const uint2*>(codes + b * 8);
     const uint32_t s_in = scales[b];
     float g[16], m[16];
-    ldg_f32x8(G + b * 16, g);
-    ldg_f32x8(G + b * 16 + 8, g + 8);
+    ld_f32x8(G + b * 16, g);
+    ld_f32x8(G + b * 16 + 8, g + 8);
     mom_decode<!HIST>(c_in, s_in, m);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {

@@ -109,12 +109,12 @@ __device__ __forceinline__ void pick_top_bin(NsHeader* hdr, uint32_t* hist) {
   if ((reinterpret_cast<uintptr_t>(hist) & 15) == 0) {
 #pragma unroll
     for (int j = 0; j < PER; j += 4) {
-      const uint4 v = __ldcg(reinterpret_cast<const uint4*>(hist + threadIdx.x * PER + j));
+      const uint4 v = ld_cg(reinterpret_cast<const uint4*>(hist + threadIdx.x * PER + j));
       local[j] = v.x; local[j + 1] = v.y; local[j + 2] = v.z; local[j + 3] = v.w;
     }
   } else {   // a caller's histogram need only be 4-byte aligned
 #pragma unroll
-    for (int j = 0; j < PER; ++j) local[j] = __ldcg(hist + threadIdx.x * PER + j);
+    for (int j = 0; j < PER; ++j) local[j] = ld_cg(hist + threadIdx.x * PER + j);
   }
 #pragma unroll
   for (int j = 0; j < PER; ++j) sum += local[j];
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(512) kp_hist_top(const __grid_constant__ PrepG
   const int64_t stride = (int64_t)m.hist_blocks * blockDim.x;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   for (; i + stride < m.n4; i += 2 * stride) {
-    const float4 v = __ldg(src + i), w = __ldg(src + i + stride);
+    const float4 v = ld_f32x4(src + i), w = ld_f32x4(src + i + stride);
     atomicAdd(&sh[mag_bits(v.x) >> kTopShift], 1u);
     atomicAdd(&sh[mag_bits(v.y) >> kTopShift], 1u);
     atomicAdd(&sh[mag_bits(v.z) >> kTopShift], 1u);
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(512) kp_hist_top(const __grid_constant__ PrepG
     atomicAdd(&sh[mag_bits(w.w) >> kTopShift], 1u);
   }
   for (; i < m.n4; i += stride) {
-    const float4 v = __ldg(src + i);
+    const float4 v = ld_f32x4(src + i);
     atomicAdd(&sh[mag_bits(v.x) >> kTopShift], 1u);
     atomicAdd(&sh[mag_bits(v.y) >> kTopShift], 1u);
     atomicAdd(&sh[mag_bits(v.z) >> kTopShift], 1u);
@@ -260,8 +260,8 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
         for (int k = 0; k < 128; k += 64) {
           const int ra = row0 + r + k, rb = ra + 32;
           const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-          const float4 v = ra < rows ? __ldg(src + ((int64_t)ra * cols + col) / 4) : zero;
-          const float4 w = rb < rows ? __ldg(src + ((int64_t)rb * cols + col) / 4) : zero;
+          const float4 v = ra < rows ? ld_f32x4(src + ((int64_t)ra * cols + col) / 4) : zero;
+          const float4 w = rb < rows ? ld_f32x4(src + ((int64_t)rb * cols + col) / 4) : zero;
           if (ra < rows) { visit(v.x); visit(v.y); visit(v.z); visit(v.w); }
           if (rb < rows) { visit(w.x); visit(w.y); visit(w.z); visit(w.w); }
         }
@@ -273,12 +273,12 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
     const int64_t stride = (int64_t)m.stat_blocks * blockDim.x;
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     for (; i + stride < m.n4; i += 2 * stride) {
-      const float4 v = __ldg(src + i), w = __ldg(src + i + stride);
+      const float4 v = ld_f32x4(src + i), w = ld_f32x4(src + i + stride);
       visit(v.x); visit(v.y); visit(v.z); visit(v.w);
       visit(w.x); visit(w.y); visit(w.z); visit(w.w);
     }
     for (; i < m.n4; i += stride) {
-      const float4 v = __ldg(src + i);
+      const float4 v = ld_f32x4(src + i);
       visit(v.x); visit(v.y); visit(v.z); visit(v.w);
     }
     acc = warp_sum(acc);
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(256, 8) kp_compact_stats(const __grid_constant
 // Fixed-order sum of at most 1024 partials by a block of 1024 threads, returned in warp 0; `wsum`: 32 words.
 __device__ __forceinline__ double sum_partials(const double* partial, int nparts, double* wsum) {
   const int tid = threadIdx.x;
-  const double v = warp_sum(tid < nparts ? __ldcg(partial + tid) : 0.0);
+  const double v = warp_sum(tid < nparts ? ld_cg(partial + tid) : 0.0);
   if ((tid & 31) == 0) wsum[tid >> 5] = v;
   __syncthreads();
   return tid < 32 ? warp_sum(wsum[tid]) : 0.0;
@@ -357,10 +357,10 @@ __device__ __forceinline__ void fallback_select_and_stats(const PrepGroup& g, co
     const int64_t step = blockDim.x;
     int64_t i = threadIdx.x;
     for (; i + 3 * step < m.n4; i += 4 * step) {
-      const float4 v0 = __ldg(src + i), v1 = __ldg(src + i + step), v2 = __ldg(src + i + 2 * step), v3 = __ldg(src + i + 3 * step);
+      const float4 v0 = ld_f32x4(src + i), v1 = ld_f32x4(src + i + step), v2 = ld_f32x4(src + i + 2 * step), v3 = ld_f32x4(src + i + 3 * step);
       visit(v0); visit(v1); visit(v2); visit(v3);
     }
-    for (; i < m.n4; i += step) visit(__ldg(src + i));
+    for (; i < m.n4; i += step) visit(ld_f32x4(src + i));
   };
   if (threadIdx.x == 0) { s_fb_prefix = hdr->sel_prefix; s_fb_rank = hdr->sel_rank; }
   __syncthreads();
@@ -530,8 +530,8 @@ __global__ void __launch_bounds__(1024) kp_finalize(const __grid_constant__ Prep
       atomicAdd(&sums->above, s_above);
     }
     if (!last_block(&hdr->ticket, m.select_blocks)) return;
-    if (tid < kSubBins) hist[tid] = __ldcg(&sums->low[tid]);
-    if (tid == 0) { s_lo = __ldcg(&sums->lo); s_hi = __ldcg(&sums->hi); s_above = __ldcg(&sums->above); }
+    if (tid < kSubBins) hist[tid] = ld_cg(&sums->low[tid]);
+    if (tid == 0) { s_lo = ld_cg(&sums->lo); s_hi = ld_cg(&sums->hi); s_above = ld_cg(&sums->above); }
     __syncthreads();
   }
   const uint32_t cnt = tid < kSubBins ? hist[tid] : 0u;
@@ -1161,11 +1161,11 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       const uint32_t* h = (g.mat[mi].hist_top ? g.mat[mi].hist_top : g.mat[mi].hist) + warp * 256 + lane * 4;
       uint32_t c[8];
       if ((reinterpret_cast<uintptr_t>(h) & 15) == 0) {
-        const uint4 a = __ldcg(reinterpret_cast<const uint4*>(h)), b = __ldcg(reinterpret_cast<const uint4*>(h + 128));
+        const uint4 a = ld_cg(reinterpret_cast<const uint4*>(h)), b = ld_cg(reinterpret_cast<const uint4*>(h + 128));
         c[0] = a.x; c[1] = a.y; c[2] = a.z; c[3] = a.w; c[4] = b.x; c[5] = b.y; c[6] = b.z; c[7] = b.w;
       } else {   // a caller's histogram need only be 4-byte aligned
 #pragma unroll
-        for (int q = 0; q < 8; ++q) c[q] = __ldcg(h + (q >> 2) * 128 + (q & 3));
+        for (int q = 0; q < 8; ++q) c[q] = ld_cg(h + (q >> 2) * 128 + (q & 3));
       }
       const uint32_t s0 = c[0] + c[1] + c[2] + c[3], s1 = c[4] + c[5] + c[6] + c[7];
       const uint32_t all = __reduce_add_sync(0xffffffffu, s0 + s1);
@@ -1269,7 +1269,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
     const bool owner = sh->info[it].index == 0;
     if (owner && g.clip && m.hist_top)   // the caller's counters are consumed, whichever way tau is found: every block has read them
       for (int i = tid; i < kTopBins; i += kPrepThreads) m.hist_top[i] = 0;
-    const uint32_t count = g.clip ? __ldcg(&hdr->cand_count) : 0u;
+    const uint32_t count = g.clip ? ld_cg(&hdr->cand_count) : 0u;
     if (count > m.cand_cap) {
       // so many equal magnitudes that the list overflowed: the owner finishes alone, the others wait for it
       if (owner) {
@@ -1292,9 +1292,9 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
       }
       __syncthreads();
       if (tid == 0) {
-        sh->tau[it] = __ldcg(m.scalars + g.ix.tau);
-        sh->inv[it] = __ldcg(m.scalars + g.ix.inv);
-        sh->sg[it] = __ldcg(m.scalars + g.ix.sg_X0);
+        sh->tau[it] = ld_cg(m.scalars + g.ix.tau);
+        sh->inv[it] = ld_cg(m.scalars + g.ix.inv);
+        sh->sg[it] = ld_cg(m.scalars + g.ix.sg_X0);
       }
       __syncthreads();
       continue;
@@ -1319,7 +1319,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
         for (uint32_t i0 = tid; i0 < count; i0 += 8 * kPrepThreads) {
           uint32_t k[8];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) k[u] = i0 + u * kPrepThreads < count ? __ldcg(m.cand + i0 + u * kPrepThreads) : 0xFFFFFFFFu;
+          for (int u = 0; u < 8; ++u) k[u] = i0 + u * kPrepThreads < count ? ld_cg(m.cand + i0 + u * kPrepThreads) : 0xFFFFFFFFu;
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
             if (k[u] == 0xFFFFFFFFu) continue;
@@ -1375,7 +1375,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) kp_resident(const __grid_cons
         above += __shfl_xor_sync(0xffffffffu, above, o);
       }
       if (lane == 0) {
-        float maxabs = __uint_as_float(__ldcg(&hdr->maxabs_bits)), tau = __int_as_float(0x7f800000);
+        float maxabs = __uint_as_float(ld_cg(&hdr->maxabs_bits)), tau = __int_as_float(0x7f800000);
         if (g.clip) {
           tau = __uint_as_float(tau_bits);
           maxabs = tau;

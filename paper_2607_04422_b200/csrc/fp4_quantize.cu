@@ -14,18 +14,18 @@ __device__ __forceinline__ float amax4(float4 v) {
   return fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
 }
 
-__global__ void __launch_bounds__(256) k_amax(const float4* __restrict__ x, int64_t n4, uint32_t* amax_bits) {
+__global__ void __launch_bounds__(256) k_amax(const float4* x, int64_t n4, uint32_t* amax_bits) {
   pdl_launch_dependents();
   pdl_wait();
   float m = 0.0f;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   for (; i + 3 * stride < n4; i += 4 * stride) {
-    const float4 a = __ldg(x + i), b = __ldg(x + i + stride), c = __ldg(x + i + 2 * stride),
-                 d = __ldg(x + i + 3 * stride);
+    const float4 a = ld_f32x4(x + i), b = ld_f32x4(x + i + stride), c = ld_f32x4(x + i + 2 * stride),
+                 d = ld_f32x4(x + i + 3 * stride);
     m = fmaxf(m, fmaxf(fmaxf(amax4(a), amax4(b)), fmaxf(amax4(c), amax4(d))));
   }
-  for (; i < n4; i += stride) m = fmaxf(m, amax4(__ldg(x + i)));
+  for (; i < n4; i += stride) m = fmaxf(m, amax4(ld_f32x4(x + i)));
 #pragma unroll
   for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   __shared__ float wm[8];
@@ -41,9 +41,9 @@ __global__ void __launch_bounds__(256) k_amax(const float4* __restrict__ x, int6
 // 8 values by one 256-bit load where the tensor lies on a 32-byte boundary, else by two 128-bit ones
 __device__ __forceinline__ void load8(const float* p, bool wide, float* v) {
   if (wide) {
-    ldg_f32x8(p, v);
+    ld_f32x8(p, v);
   } else {
-    const float4 s = __ldg(reinterpret_cast<const float4*>(p)), t = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    const float4 s = ld_f32x4(reinterpret_cast<const float4*>(p)), t = ld_f32x4(reinterpret_cast<const float4*>(p) + 1);
     v[0] = s.x; v[1] = s.y; v[2] = s.z; v[3] = s.w;
     v[4] = t.x; v[5] = t.y; v[6] = t.z; v[7] = t.w;
   }
@@ -65,12 +65,12 @@ __device__ __forceinline__ void load_block16(const float* p, bool wide, float (&
 // which every block walks the same units in both passes finds 74 MB of 8192 x 8192 in the L2, and is slower all the same:
 // 93.3 us, prefetched a unit ahead or not.)
 // ----------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_quantize_rows(const float* __restrict__ x, int64_t rows, int64_t cols,
+__global__ void __launch_bounds__(256) k_quantize_rows(const float* x, int64_t rows, int64_t cols,
                                                        uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                                                       const uint32_t* __restrict__ amax_bits, const bool wide) {
+                                                       const uint32_t* amax_bits, const bool wide) {
   pdl_launch_dependents();
   pdl_wait();
-  const float sg = scale_exact(__uint_as_float(*amax_bits));
+  const float sg = scale_exact(__uint_as_float(ld_u32(amax_bits)));
   const float six_sg = __fmul_rn(6.0f, sg), rcp_six_sg = __frcp_rn(six_sg);
   const int64_t r = (int64_t)gridDim.x - 1 - blockIdx.x;
   const int64_t kb = (int64_t)(gridDim.y - 1 - blockIdx.y) * 256 + threadIdx.x;
@@ -91,13 +91,13 @@ __global__ void k_finish_tensor_scale(float* ts, float widen) {
 // Row quantiser with the paper-faithful options (Section 3.4): one thread per block of 16
 // (the transform and the two candidate encodings are local to a block), a warp covers 512
 // consecutive elements of a row.  grid: rows x ceil(cols / 4096) thread blocks, row-major.
-__global__ void __launch_bounds__(256) k_quantize_rows_opts(const float* __restrict__ x, int64_t rows, int64_t cols,
+__global__ void __launch_bounds__(256) k_quantize_rows_opts(const float* x, int64_t rows, int64_t cols,
                                                             uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                                                            const uint32_t* __restrict__ amax_bits, const bool wide,
+                                                            const uint32_t* amax_bits, const bool wide,
                                                             const QuantOpts q) {
   pdl_launch_dependents();
   pdl_wait();
-  const float sg = scale_exact(__fmul_rn(q.widen, __uint_as_float(*amax_bits)));
+  const float sg = scale_exact(__fmul_rn(q.widen, __uint_as_float(ld_u32(amax_bits))));
   const int64_t r = (int64_t)gridDim.x - 1 - blockIdx.x;   // from the end, as k_quantize_rows
   const int64_t kb = (int64_t)(gridDim.y - 1 - blockIdx.y) * 256 + threadIdx.x;
   if (kb >= (cols >> 4)) return;
@@ -225,7 +225,7 @@ k_quantize_small(const __grid_constant__ CUtensorMap tm, int units, int64_t cols
 // out (l0 x s0) = the leading s0 x l0 part of X^T, X being s x l (row pitch l): 64 x 64 tiles through
 // shared memory, 128-bit loads along the rows of X and 128-bit stores along the rows of out
 // (s0 and l0 are multiples of 16, so a 16-byte piece is all inside or all outside).
-__global__ void __launch_bounds__(256) k_transpose_out(const float* __restrict__ X, int64_t l, float* __restrict__ out,
+__global__ void __launch_bounds__(256) k_transpose_out(const float* X, int64_t l, float* __restrict__ out,
                                                        int64_t s0, int64_t l0, const ParamUpdate upd) {
   __shared__ float t[64][65];
   pdl_launch_dependents();
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(256) k_transpose_out(const float* __restrict__
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int r = row + 16 * j;
-    const float4 v = __ldg(reinterpret_cast<const float4*>(X + (r0 + r) * l + c0) + q);  // inside the padded work matrix
+    const float4 v = ld_f32x4(reinterpret_cast<const float4*>(X + (r0 + r) * l + c0) + q);  // inside the padded work matrix
     t[r][4 * q] = v.x; t[r][4 * q + 1] = v.y; t[r][4 * q + 2] = v.z; t[r][4 * q + 3] = v.w;
   }
   __syncthreads();
@@ -261,11 +261,11 @@ __global__ void __launch_bounds__(256) k_transpose_out(const float* __restrict__
 }
 
 // W <- update(W, O) elementwise, 8 elements per thread
-__global__ void __launch_bounds__(256) k_param_update(const float* __restrict__ O, int64_t n8, const ParamUpdate upd) {
+__global__ void __launch_bounds__(256) k_param_update(const float* O, int64_t n8, const ParamUpdate upd) {
   pdl_launch_dependents();
   pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(O) + 2 * i), b = __ldg(reinterpret_cast<const float4*>(O) + 2 * i + 1);
+    const float4 a = ld_f32x4(reinterpret_cast<const float4*>(O) + 2 * i), b = ld_f32x4(reinterpret_cast<const float4*>(O) + 2 * i + 1);
     uint4* wp = reinterpret_cast<uint4*>(upd.W) + i;
     const uint4 w = *wp;
     *wp = make_uint4(cvt_bf16x2(param_update_value(bf16_lo(w.x), a.x, upd.decay, upd.step),

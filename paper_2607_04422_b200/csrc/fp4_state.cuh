@@ -346,8 +346,8 @@ __device__ __forceinline__ uint64_t neg_quotient2(uint64_t m, uint64_t den) {
 // 32-byte sectors, so no sector is touched by two instructions -- with 128-bit pieces at a
 // 64-byte lane stride every sector is looked up twice on loads and written as two partial
 // sectors on stores.
-__device__ __forceinline__ void ldg_f32x8(const float* p, float* v) {
-  asm volatile("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+__device__ __forceinline__ void ld_f32x8(const float* p, float* v) {
+  asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
                : "l"(p));
 }

@@ -284,3 +284,32 @@ def test_single_launch_quantiser_reports_that_it_gave_up(shape, scale):
     oc, os_, osg = oracle.quantize(x_np)
     assert np.float32(ts.item()) == np.float32(osg)
     assert np.array_equal(sf_from_atoms(scales.cpu().numpy(), rows, cols // 16), os_)
+
+
+@pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | 0x2D5A0000, FP4_FLAG_FOUR_SIX, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX | 0x2D5A0000])
+@pytest.mark.parametrize("shape,offset", [((2816, 2688), 0), ((4224, 5760), 0), ((4224, 5760), 4)])
+def test_blocks_of_the_second_pass_wait_for_the_maximum_of_the_whole_tensor(shape, offset, flags):
+    """The second pass starts at the tensor's end while blocks of the first still run: wherever the largest magnitude lies, whoever
+    reads it last, the last rows have its scale."""
+    rows, cols = shape
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    buf = torch.randn(rows * cols + 8, device="cuda", generator=gen)
+    x = buf[offset:offset + rows * cols].view(shape)                 # 4: on a 16-byte, not on a 32-byte boundary
+    codes = torch.empty((rows, cols // 2), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(fp4.fp4_scale_bytes(rows, cols), dtype=torch.uint8, device="cuda")
+    ts = torch.empty(1, device="cuda")
+    widen = np.float32(4 if flags & FP4_FLAG_RHT else 1)
+    sg = widen * np.float32(64) / np.float32(2688)
+    last = x[-128:].cpu().numpy()
+    want_codes, want_scales, _ = oracle.quantize(last, s_g=sg, rht=bool(flags & FP4_FLAG_RHT), mask=flags >> 16,
+                                                 four_six=bool(flags & FP4_FLAG_FOUR_SIX))
+    rng = np.random.default_rng(1)
+    for at in rng.integers(0, (rows - 128) * cols, 48):
+        keep = x.view(-1)[at].clone()
+        x.view(-1)[at] = 64.0
+        fp4.fp4_quantize(x, codes, scales, ts, flags=flags)
+        x.view(-1)[at] = keep
+        assert np.float32(ts.item()) == sg
+        got = sf_from_atoms(scales[-128 * (cols // 16):].cpu().numpy(), 128, cols // 16)
+        assert np.array_equal(got, want_scales), (int(at), mismatch_report(got, want_scales))
+        assert np.array_equal(codes[-128:].cpu().numpy(), want_codes), int(at)

@@ -127,3 +127,21 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
         binding.load_library()
     monkeypatch.undo()
     binding.load_library()
+
+
+def test_chained_kernels_read_nothing_through_the_read_only_path():
+    """A kernel chained to the one before it lives while that one still writes: loads that promise constant memory may be moved ahead
+    of its wait (__ldg, ld.global.nc, pointers to const with __restrict__)."""
+    folder = os.path.join(ROOT, "paper_2607_04422_b200", "csrc")
+    read_only = re.compile(r"__ldg\(|ld\.global\.nc|const\s+\w+\s*\*\s*__restrict__")
+    chained = 0
+    for name in sorted(os.listdir(folder)):
+        with open(os.path.join(folder, name)) as f:
+            code = re.sub(r"//[^\n]*", "", f.read())
+        parts = re.split(r"(?=__global__)", code)
+        assert not read_only.search(parts[0]), name
+        for kernel in parts[1:]:
+            if "pdl_wait()" in kernel:
+                chained += 1
+                assert not read_only.search(kernel), (name, read_only.search(kernel).group(), kernel[:120])
+    assert chained >= 14
