@@ -55,32 +55,36 @@ __device__ __forceinline__ void load_block16(const float* p, bool wide, float (&
 
 // ----------------------------------------------------------------------------------
 // Row quantiser: one thread per block of 16 (64 contiguous bytes, a warp covers 512 consecutive elements of a row); 8-byte code
-// store and 1-byte scale store per thread.  Thread blocks walk the tensor from its end: the amax pass has just read it
-// front to back, so the end is what L2 still holds (74 of 268 MB at most: with 128-bit loads and another block order 37).
-// grid: rows x ceil(cols / 4096) thread blocks.  amax_bits holds the tensor amax on entry (bit pattern).
+// store and 1-byte scale store per thread.  Thread blocks walk the tensor from its end, since the amax pass has just read it front to
+// back.  grid: (strips of 4096 columns, 128, rows / 128), all three counted down, so that the pieces of a row stay together without a
+// division.  amax_bits holds the tensor amax on entry (bit pattern).
 //
-// Bounds: HBM with reads and writes mixed, 5.5 TB/s of it.  With 256-bit loads (every sector looked up once), no 64-bit division for the
-// place and none of the two IEEE divisions per block, whole calls, before / after: 8192 x 8192 92.9 / 91.4 us, 16384 x 8192
-// 179 / 173, 4096 x 4096 29.4 / 28.3, 2048 x 4352 20.5 / 19.1, 8192 x 8192 with the options 116 / 111.  (One cooperative launch in
-// which every block walks the same units in both passes finds 74 MB of 8192 x 8192 in the L2, and is slower all the same:
-// 93.3 us, prefetched a unit ahead or not.)
+// Bounds: HBM with reads and writes mixed, 6 TB/s of it.  The pass finds 36 MB of 8192 x 8192 and of 4096 x 16384 (268 MB) in the L2, the
+// amax pass of a repeated call 50 (dram__bytes_read, caches as they are); strip after strip it found 31 and 21, and whole calls took
+// 8192 x 8192 85.9 us (now 84.5), 4096 x 16384 93.0 (84.3), 5120 x 14464 100.4 (94.7), 11776 x 14592 218 (212).  With 256-bit
+// loads (every sector looked up once), no 64-bit division for the place and none of the two IEEE divisions per block, whole calls, before /
+// after: 8192 x 8192 86.6 / 84.5, 16384 x 8192 168 / 167, 4096 x 4096 23.1 / 22.8, 2048 x 4352 16.6 / 15.2, 8192 x 8192 with the
+// options 106.8 / 100.5.  (One cooperative launch in which every block walks the same units in both passes is slower: 93.3 us at 8192 x
+// 8192 where the two passes took 91.4, prefetched a unit ahead or not.)
 // ----------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_quantize_rows(const float* x, int64_t rows, int64_t cols,
+__device__ __forceinline__ uint32_t row_of_block() { return (gridDim.z - 1 - blockIdx.z) * 128 + (127 - blockIdx.y); }
+__global__ void __launch_bounds__(256) k_quantize_rows(const float* x, int64_t cols,
                                                        uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
                                                        const uint32_t* amax_bits, const bool wide) {
   pdl_launch_dependents();
   pdl_wait();
   const float sg = scale_exact(__uint_as_float(ld_u32(amax_bits)));
   const float six_sg = __fmul_rn(6.0f, sg), rcp_six_sg = __frcp_rn(six_sg);
-  const int64_t r = (int64_t)gridDim.x - 1 - blockIdx.x;
-  const int64_t kb = (int64_t)(gridDim.y - 1 - blockIdx.y) * 256 + threadIdx.x;
-  if (kb >= (cols >> 4)) return;
+  const uint32_t r = row_of_block(), kblocks = (uint32_t)cols >> 4;
+  const uint32_t kb = (gridDim.x - 1 - blockIdx.x) * 256 + threadIdx.x;
+  if (kb >= kblocks) return;
+  const uint64_t b = (uint64_t)r * kblocks + kb;   // block of the tensor
   float v[16];
-  load_block16(x + r * cols + kb * 16, wide, v);
+  load_block16(x + b * 16, wide, v);
   uint32_t lo, hi;
   const uint32_t sb = quantize_block16_fast(v, sg, six_sg, rcp_six_sg, lo, hi);
-  *reinterpret_cast<uint2*>(codes + r * (cols / 2) + kb * 8) = make_uint2(lo, hi);
-  scales[sf_offset(r, kb, cols >> 4)] = (uint8_t)sb;
+  *reinterpret_cast<uint2*>(codes + b * 8) = make_uint2(lo, hi);
+  scales[sf_offset(r, kb, kblocks)] = (uint8_t)sb;
 }
 
 __global__ void k_finish_tensor_scale(float* ts, float widen) {
@@ -90,23 +94,24 @@ __global__ void k_finish_tensor_scale(float* ts, float widen) {
 
 // Row quantiser with the paper-faithful options (Section 3.4): one thread per block of 16
 // (the transform and the two candidate encodings are local to a block), a warp covers 512
-// consecutive elements of a row.  grid: rows x ceil(cols / 4096) thread blocks, row-major.
-__global__ void __launch_bounds__(256) k_quantize_rows_opts(const float* x, int64_t rows, int64_t cols,
+// consecutive elements of a row.  grid: as k_quantize_rows.
+__global__ void __launch_bounds__(256) k_quantize_rows_opts(const float* x, int64_t cols,
                                                             uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
                                                             const uint32_t* amax_bits, const bool wide,
                                                             const QuantOpts q) {
   pdl_launch_dependents();
   pdl_wait();
   const float sg = scale_exact(__fmul_rn(q.widen, __uint_as_float(ld_u32(amax_bits))));
-  const int64_t r = (int64_t)gridDim.x - 1 - blockIdx.x;   // from the end, as k_quantize_rows
-  const int64_t kb = (int64_t)(gridDim.y - 1 - blockIdx.y) * 256 + threadIdx.x;
-  if (kb >= (cols >> 4)) return;
+  const uint32_t r = row_of_block(), kblocks = (uint32_t)cols >> 4;
+  const uint32_t kb = (gridDim.x - 1 - blockIdx.x) * 256 + threadIdx.x;
+  if (kb >= kblocks) return;
+  const uint64_t b = (uint64_t)r * kblocks + kb;   // block of the tensor
   float v[16];
-  load_block16(x + r * cols + kb * 16, wide, v);
+  load_block16(x + b * 16, wide, v);
   uint32_t lo, hi;
   const uint32_t sb = quantize_block16_opts(v, q, sg, lo, hi);
-  *reinterpret_cast<uint2*>(codes + r * (cols / 2) + kb * 8) = make_uint2(lo, hi);
-  scales[sf_offset(r, kb, cols >> 4)] = (uint8_t)sb;
+  *reinterpret_cast<uint2*>(codes + b * 8) = make_uint2(lo, hi);
+  scales[sf_offset(r, kb, kblocks)] = (uint8_t)sb;
 }
 
 // ----------------------------------------------------------------------------------
@@ -323,9 +328,9 @@ cudaError_t launch_quantize(const CUtensorMap* tm, const float* x, int64_t rows,
   pdl_select(true);
   uint32_t* amax = reinterpret_cast<uint32_t*>(tensor_scale);
   launch_chained(k_amax, dim3(grid_for(n4, 256 * 8, sms)), dim3(256), 0, st, reinterpret_cast<const float4*>(x), n4, amax);
-  const dim3 qgrid((unsigned)rows, (unsigned)((cols / 16 + 255) / 256));
-  if (pf) launch_chained(k_quantize_rows_opts, qgrid, dim3(256), 0, st, x, rows, cols, codes, scales, amax, wide, q);
-  else launch_chained(k_quantize_rows, qgrid, dim3(256), 0, st, x, rows, cols, codes, scales, amax, wide);
+  const dim3 qgrid((unsigned)((cols / 16 + 255) / 256), 128, (unsigned)(rows / 128));   // rows: a multiple of 128, at most 2^20
+  if (pf) launch_chained(k_quantize_rows_opts, qgrid, dim3(256), 0, st, x, cols, codes, scales, amax, wide, q);
+  else launch_chained(k_quantize_rows, qgrid, dim3(256), 0, st, x, cols, codes, scales, amax, wide);
   launch_chained(k_finish_tensor_scale, dim3(1), dim3(1), 0, st, tensor_scale, q.widen);
   count_launches(3);
   return cudaGetLastError();

@@ -313,3 +313,26 @@ def test_blocks_of_the_second_pass_wait_for_the_maximum_of_the_whole_tensor(shap
         got = sf_from_atoms(scales[-128 * (cols // 16):].cpu().numpy(), 128, cols // 16)
         assert np.array_equal(got, want_scales), (int(at), mismatch_report(got, want_scales))
         assert np.array_equal(codes[-128:].cpu().numpy(), want_codes), int(at)
+
+
+def test_long_rows_take_no_longer_than_short_ones():
+    # the second pass reads from the tensor's end, where the L2 still holds it, also where a row takes several thread blocks: measured 0.99
+    # times the time of short rows, 1.09 where all rows' last strips of 4096 columns came first
+    calls = []
+    for shape in ((16384, 4096), (4096, 16384)):
+        x = torch.randn(shape, device="cuda")
+        codes = torch.empty((shape[0], shape[1] // 2), dtype=torch.uint8, device="cuda")
+        scales = torch.empty(fp4.fp4_scale_bytes(*shape), dtype=torch.uint8, device="cuda")
+        calls.append((x, codes, scales, torch.empty(1, device="cuda")))
+    times = [[], []]
+    for _ in range(12):
+        for call, t in zip(calls, times):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            fp4.fp4_quantize(*call)
+            e0.record()
+            for _ in range(20):
+                fp4.fp4_quantize(*call)
+            e1.record()
+            torch.cuda.synchronize()
+            t.append(e0.elapsed_time(e1))
+    assert np.median(times[1]) < 1.05 * np.median(times[0]), [np.median(t) for t in times]
