@@ -1197,3 +1197,39 @@ def test_prologue_of_one_cluster_counts_from_zero(tiles):
                     ws_many = torch.full((count * ws.numel(),), fill, dtype=torch.uint8, device="cuda")
                     fp4.fp4_root_ns_batched(Gs * count, many, 0, None, ws_many)
                     assert torch.equal(own, outs[0]) and all(torch.equal(o, outs[0]) for o in many), (shapes, scale, fill)
+
+
+@pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX, FP4_FLAG_STORE_BF16, FP4_FLAG_KEEP_OPERANDS])
+@pytest.mark.parametrize("shapes", [m[0] for m in MIXED], ids=["one-launch", "pairs", "both-sums"])
+def test_shapes_in_one_call_take_fewer_launches_than_on_their_own(shapes, flags):
+    """Whatever the options, matrices of several shapes share launches: fewer than a call per shape takes in all."""
+    def launches(part):
+        Gs = [torch.randn(s, device="cuda") for s in part]
+        outs = [torch.empty_like(g) for g in Gs]
+        ws = torch.empty(fp4.fp4_root_ns_batched_workspace_bytes(part, 3, flags), dtype=torch.uint8, device="cuda")
+        before = fp4.fp4_kernel_launches()
+        fp4.fp4_root_ns_batched(Gs, outs, 3, fp4.NsParams.make(flags=flags, seed=5), ws)
+        torch.cuda.synchronize()
+        assert fp4.fp4_last_device_status(ws) == 0
+        return fp4.fp4_kernel_launches() - before
+
+    groups = {}
+    for s in shapes:
+        groups.setdefault((min(s), max(s)), []).append(s)
+    assert launches(shapes) < sum(launches(part) for part in groups.values())
+
+
+@pytest.mark.parametrize("flags", [0, FP4_FLAG_RHT | FP4_FLAG_FOUR_SIX])
+def test_clusters_beside_the_launches_of_the_other_stream(flags):
+    """FP4_FLAG_OVERLAP_GROUPS with groups of up to 16 blocks (clusters) beside ones that take half of the SMs, in either order."""
+    for shapes in ([(256, 512), (1536, 2048), (384, 640), (1536, 2304)], [(1536, 2048), (256, 512), (1536, 2304), (512, 512), (128, 384)]):
+        Gs = [torch.from_numpy(workloads.gradient_like(*s, seed=i)).cuda() for i, s in enumerate(shapes)]
+        results = []
+        for overlap in (0, FP4_FLAG_OVERLAP_GROUPS):
+            outs = [torch.empty_like(g) for g in Gs]
+            ws = torch.full((fp4.fp4_root_ns_batched_workspace_bytes(shapes, 5, flags),), 0xAB, dtype=torch.uint8, device="cuda")
+            for _ in range(3):
+                fp4.fp4_root_ns_batched(Gs, outs, 5, fp4.NsParams.make(flags=flags | overlap, seed=1), ws)
+            assert fp4.fp4_last_device_status(ws) == 0
+            results.append(outs)
+        assert all(torch.equal(a, b) for a, b in zip(*results))
