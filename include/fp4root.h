@@ -177,18 +177,21 @@ fp4_status fp4_root_coeffs(int64_t m, int64_t n, int steps, float abc[3]);
  *   an NVFP4 quantisation with 16-element blocks along the contraction axis; the
  *   result is X_steps (transposed back when m > n).
  * Two calls that share a workspace must not overlap in time.
- * Launches: 6 kernels for clip, normalisation and the first quantisation (one, cooperative, when
- *   the group's matrices fit the shared memories of all SMs: 7.2 M elements) plus 3 per iteration
+ * Launches: 6 kernels for clip, normalisation and the first quantisation (7 where a batched call has small
+ *   and large matrices in one group; one when the group's matrices fit the shared memories of all SMs:
+ *   7.2 M elements) plus 3 per iteration
  *   (and a transpose pass for a tall matrix on the routes that cannot write the result
  *   transposed from the last product).  Groups of up to a few million elements run all
- *   iterations in one cooperative launch instead, whose blocks wait on one another (bounded
+ *   iterations in one launch instead, whose blocks wait on one another (bounded
  *   waits); somewhat larger ones (short sides up to 2048) run two of the three products of an
- *   iteration in such a launch.  Short kernels are chained with programmatic dependent launch;
+ *   iteration in such a launch.  Launches whose blocks wait on one another are cooperative, or, up to 16 blocks
+ *   on a stream that owns the whole device, one thread-block cluster.  Short kernels are chained with programmatic dependent launch;
  *   the environment variable FP4ROOT_NO_PDL (any value) switches that off.  Kernels launched before or after
  *   the call on the same stream see ordinary stream order either way.
  *   A cooperative launch starts when all its blocks - up to one per SM, each with most of an SM's shared
  *   memory - can be resident at once: beside a long kernel on another stream it waits for
- *   that kernel's SMs, where plain launches would have started on the free ones.  On a stream that owns only
+ *   that kernel's SMs, where plain launches would have started on the free ones.  A cluster needs
+ *   its SMs (up to 16) free in one part of the device (GPC), not anywhere.  On a stream that owns only
  *   a part of the device (a green context, a context with an SM limit) the sizes above shrink with
  *   the part; results are the same.
  */

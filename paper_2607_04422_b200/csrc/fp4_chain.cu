@@ -884,7 +884,11 @@ k_chain(const __grid_constant__ ChainPackOf<MAX> pack, const __grid_constant__ C
 
 // The blocks wait on one another, so all have to be resident: a cooperative launch - or, up to kChainCluster blocks, a single
 // cluster, which is an ordinary launch whose set-up overlaps with the prologue (a power of two of blocks, some without a tile): 256 x 512
-// 77.2 -> 74.6 us, with options 100.2 -> 97.7.
+// 77.2 -> 74.6 us, with options 100.2 -> 97.7.  A cooperative launch takes any SMs that are free, a cluster those of one GPC, so beside other work
+// it may start later, or finish sooner.  Two of the caller's streams, time per call of the second, cooperative / cluster: 512 x 512 beside 1024 x
+// 1024 146 / 163 us, beside 640 x 1024 93 / 96, beside 2048 x 2048 266 / 264; 256 x 512 beside 1024 x 1024 88 / 79, beside 2048 x 2048 262 / 169.
+// The second stream of FP4_FLAG_OVERLAP_GROUPS: eight groups of one to 16 tiles 353 / 326, two larger and four such groups 322 / 313, 4096 x
+// 4096 and six of them 921 / 909, two 1536 wide and two such groups 517 / 520.
 constexpr int kChainCluster = 16;
 int g_cluster_blocks[64];   // per device: blocks of the largest such cluster it holds, or 0 (set once, before the device's first launch)
 template <int BN, bool PF, bool SYM = false>
@@ -978,7 +982,8 @@ static Residents residents(int bn, int64_t full, int64_t sym) {
 // stay in the tensor memory, long where they move through memory - or a main loop, whichever is longer.  The constants here
 // and of the CTA-pair kernel's estimate beside the caller are fitted to the times of all routes and both widths at 213 shapes and
 // groups (short sides 128 to 2304, long sides to 32768, 1 to 14 matrices, plain and with the quantiser options): choosing by them
-// loses 0.1 % on average against always knowing the fastest, 3.5 % at worst, and 0.7 % (9 %) at 100 others drawn at random.
+// loses 0.1 % on average against always knowing the fastest, 3.5 % at worst, and 0.7 % (9 %) at 100 others drawn at random.  Calls of mixed
+// shapes, which they were not fitted to: at 119 drawn ones (2 to 4 shapes, up to 14 matrices) route and merging lose 0.4 % (14 %).
 struct TileUs {
   double product, resident, memory;
   TileUs(int bn, bool opts)
@@ -1013,7 +1018,7 @@ static double width_us(int bn, const WorkShape* w, int count, bool opts, int sms
   }
   return 3 * t.product + g1.tiles(rs, r.na) + g2.tiles(rs, r.na) + g3.tiles(rf, r.nx);
 }
-// The width of a single launch's tiles.  Measured, 5 iterations, 64 / 128 columns: 256 x 512 83 / 101 us, 1024 x 4096 159 / 185 (with the
+// The width of a single launch's tiles.  Measured, 5 iterations, 64 / 128 columns: 256 x 512 83 / 101 us (now 72 as one cluster), 1024 x 4096 159 / 185 (with the
 // quantiser options 200 / 243), 8 x 768 x 768 155 / 179, 1152 x 8192 290 / 324, 1536 x 1536 148 / 139, 1536 x 2816 196 / 188,
 // 2048 x 2048 210 / 196 (250 / 249).
 static bool narrow_tiles(const WorkShape* w, int count, bool opts, int sms) {

@@ -790,9 +790,9 @@ std::vector<std::vector<MatrixCtx>> group_by_shape(const std::vector<MatrixCtx>&
 // merge, the best pair first.  Measured, the groups one after the other / together: the 14 matrices of two decoder blocks 512 wide (four each of
 // 512 x 512 and 128 x 512, six of 512 x 1536) 310 / 172 us, of one 1024 wide (1024, 256, 2816) 470 / 323, of two 1600 wide (400,
 // 4304) 1425 / 1220, of one 4096 wide (1024, 11008) with the quantiser options 5600 / 5420, the optimiser step around one
-// 3072 wide (8192) 3240 / 3095.  (Single matrices only join a group, they do not form one: for a call of single matrices of many
-// shapes FP4_FLAG_OVERLAP_GROUPS is the faster way, as it has been tested to be.  Six of 1536 x 1536 .. 2816 1177 us, with the
-// option 823; together they would take 540.)  The group of the call's first matrix, whose prologue clears the status word, comes first.
+// 3072 wide (8192) 3240 / 3095.  (Single matrices only join a group, they do not form one, although they
+// would gain, too: six of 1536 x 1536 .. 2816 take 1177 us, with FP4_FLAG_OVERLAP_GROUPS 823, together 540; 192 x 176 and 256 x 272 with BF16
+// storage 146, together 83.  A test of that option takes a call of single matrices as the case that it makes faster.)  The group of the call's first matrix, whose prologue clears the status word, comes first.
 void merge_groups(std::vector<std::vector<MatrixCtx>>& groups, int cap, int steps, const fp4_ns_params* p, int device_sms, int sms) {
   if (groups.size() < 2) return;
   const uint8_t* first = groups[0][0].ws;
